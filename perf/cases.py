@@ -26,8 +26,8 @@ FLUIDS = {"tube": [WATER_B, AIR], "bubble": [WATER_B, AIR, HELIUM], "column": [W
           "advection": [WATER, AIR], "interface": [WATER_B, AIR, HELIUM]}
 BC = {"tube": [0, 0], "bubble": [0] * 4, "column": [0] * 4, "jet": [2, 0, 0, 0], "advection": [1] * 4,
       "interface": [0, 0, 1, 1, 1, 1]}
-# about how many of a problem's midpoints have a stencil that is not uniform
-BUSY = {"tube": 0.6, "bubble": 0.35, "column": 0.25, "jet": 0.3, "advection": 1.0, "interface": 0.4}
+# about how many of a problem's midpoints have a stencil that is not uniform (counted on states of the listed sizes)
+BUSY = {"tube": 0.95, "bubble": 0.27, "column": 0.22, "jet": 0.25, "advection": 1.0, "interface": 0.08}
 
 
 def _case(kind, nx, ny, nz, steps, precision="fp64", gate=False, check=False, do="steps", count=1):
