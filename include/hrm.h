@@ -429,6 +429,15 @@ hrm_status hrm_probe_wait_timeout(void* stream, int64_t* expired);
 hrm_status hrm_probe_convert(const double* in_d, const float* in_f, int64_t n, float* narrowed, double* widened,
                              void* stream);
 
+/* Diagnostic (not a step of the method): the library forms part of its FP64
+ * products, quotients and square roots with integer operations beside the FP64
+ * unit. For n elements of device arrays out[i] = a[i] * b[i] (op 0), a[i] / b[i]
+ * (op 1) or sqrt(a[i]) (op 2; b is not read) by those operations -- which must
+ * equal the correctly rounded results bit for bit (NaN for NaN). Enqueued on
+ * `stream`; no synchronisation; HRM_E_INVAL for an unknown op, n < 0 or a NULL
+ * array with n > 0. */
+hrm_status hrm_probe_soft64(int32_t op, const double* a, const double* b, int64_t n, double* out, void* stream);
+
 /* Diagnostic, not a step of the method: the bounded grid barrier of the
  * batched form's persistent kernel, made to run out: 4 blocks wait at a barrier
  * that counts 5 (nothing completes it), each wait limited to limit_ms. Returns

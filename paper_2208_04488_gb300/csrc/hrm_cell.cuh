@@ -22,16 +22,16 @@ __device__ __forceinline__ void cell_prim(const double* W, const DevFluid& f, do
   double S, P;
   mix_SP<double, N>(f, &W[L::AL], S, P);
   const double re = rhoe_tilde<N, D>(W, f);
-  const double p = (re - P) / S;
+  const double p = quot(re - P, S);
 #pragma unroll
   for (int k = 0; k < N; ++k) V[k] = W[k];
 #pragma unroll
-  for (int d = 0; d < D; ++d) V[L::MOM + d] = W[L::MOM + d] / rho;
+  for (int d = 0; d < D; ++d) V[L::MOM + d] = quot(W[L::MOM + d], rho);
   V[L::EN] = p;
 #pragma unroll
   for (int k = 0; k < N - 1; ++k) V[L::AL + k] = W[L::AL + k];
   rc2 = rho_c2(S, P, p);
-  c = sqrt(rc2 / rho);
+  c = rsqrt_r(quot(rc2, rho));
 }
 
 // Order-preserving bits of a non-negative double (IEEE order equals unsigned order).
@@ -51,7 +51,7 @@ __device__ __forceinline__ double c4eq(const double* W, const DevFluid& f, doubl
   for (int k = 0; k < N; ++k) rho += W[k];
   double Y[N];
 #pragma unroll
-  for (int k = 0; k < N; ++k) Y[k] = W[k] / rho;
+  for (int k = 0; k < N; ++k) Y[k] = quot(W[k], rho);
   const double re = rhoe_tilde<N, D>(W, f);
   double cvb = 0.0, cpb = 0.0, qb = 0.0;
 #pragma unroll
@@ -63,23 +63,23 @@ __device__ __forceinline__ double c4eq(const double* W, const DevFluid& f, doubl
   const double pinf1 = f.pinf[l], R1 = f.Rg[l], Rb = cpb - cvb;
   const double Bp = -(re * Rb - pinf1 * cvb - pinf1 * Y[l] * R1);
   const double den = 2.0 * cvb * p + Bp;
-  const double Gam = (-(-(rho * Rb) * p - pinf1 * rho * (Rb - Y[l] * R1)) / den) / rho;
+  const double Gam = quot(quot(-(-(rho * Rb) * p - pinf1 * rho * (Rb - Y[l] * R1)), den), rho);
   if (Gam_out) *Gam_out = Gam;
-  double c2 = Gam * p / rho;
-  const double e = re / rho + qb;
+  double c2 = quot(Gam * p, rho);
+  const double e = quot(re, rho) + qb;
 #pragma unroll
   for (int k = 0; k < N; ++k) {
     const double dre = e - f.q[k];
-    const double dcv = (f.cv[k] - cvb) / rho;
-    const double dRb = (f.Rg[k] - Rb) / rho;
-    const double dY1 = ((k == l ? 1.0 : 0.0) - Y[l]) / rho;
+    const double dcv = quot(f.cv[k] - cvb, rho);
+    const double dRb = quot(f.Rg[k] - Rb, rho);
+    const double dY1 = quot((k == l ? 1.0 : 0.0) - Y[l], rho);
     const double dB = -(dre * Rb + re * dRb - pinf1 * dcv - pinf1 * R1 * dY1);
     const double dC = -(pinf1 * (dre * (Rb - Y[l] * R1) + re * (dRb - R1 * dY1)));
-    const double psi = -(dcv * p * p + dB * p + dC) / den;
+    const double psi = quot(-(dcv * p * p + dB * p + dC), den);
     if (Psi) Psi[k] = psi;
     c2 += Y[k] * psi;
   }
-  return sqrt(c2);
+  return rsqrt_r(c2);
 }
 
 // Four-equation HRM sound speed of a conservative vector: relaxed p, then Eq.
@@ -146,7 +146,7 @@ __device__ __forceinline__ void prim_body(int64_t c, const double* __restrict__ 
     }
     const double cw = c4 ? c4_of_cell<N, D>(w, f) : cs;  // wave speed of the CFL maxima
 #pragma unroll
-    for (int d = 0; d < D; ++d) s[d] = (fabs(v[L::MOM + d]) + cw) / g.dx[d];
+    for (int d = 0; d < D; ++d) s[d] = quot(fabs(v[L::MOM + d]) + cw, g.dx[d]);
   }
 }
 
@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(kCellThreads)
   double rho = 0.0, E = 0.0, ar[N];
 #pragma unroll
   for (int k = 0; k < N; ++k) {
-    const double rhok = (p + f.pinf[k]) / (f.Rg[k] * T);
+    const double rhok = quot(p + f.pinf[k], f.Rg[k] * T);
     ar[k] = al[k] * rhok;
     rho = rho + ar[k];
     E = E + al[k] * (p + f.gamma[k] * f.pinf[k]) * f.inv_gm1[k] + ar[k] * f.q[k];
@@ -299,7 +299,7 @@ __global__ void __launch_bounds__(kCellThreads)
       const double gd = (rho_at(nb[1]) - rho_at(nb[0])) * (0.5 * g.inv_dx[d]);
       g2 += gd * gd;
     }
-    out[c] = sqrt(g2) / r0;
+    out[c] = quot(rsqrt_r(g2), r0);
     return;
   }
   if (field == 6 || field == 7) {
@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(kCellThreads)
     for (int k = 0; k < N - 1; ++k) sa += w[L::AL + k];
 #pragma unroll
     for (int k = 0; k < N; ++k)
-      out[k * nc + c] = field == 7 ? w[k] / r : (k < N - 1 ? w[L::AL + k] : 1.0 - sa);
+      out[k * nc + c] = field == 7 ? quot(w[k], r) : (k < N - 1 ? w[L::AL + k] : 1.0 - sa);
     return;
   }
   if (field == 1 || field == 2) {

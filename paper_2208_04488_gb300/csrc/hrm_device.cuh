@@ -9,6 +9,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "hrm_soft64.cuh"
+
 #define HRM_MAXN 4
 
 namespace hrm {
@@ -154,7 +156,12 @@ __host__ __device__ inline bool patched(const DevGrid& g, int dir) {
 template <typename T> __device__ __forceinline__ T dmin(T a, T b) { return (b < a) ? b : a; }
 template <typename T> __device__ __forceinline__ T dmax(T a, T b) { return (a < b) ? b : a; }
 
-__device__ __forceinline__ double rsqrt_r(double x) { return sqrt(x); }
+// FP64 quotients and square roots on the integer pipes (hrm_soft64.cuh): the bits
+// of the FP64 unit's sequences, which take 137 and 143 of its cycles per warp,
+// at 27 and 30.
+__device__ __forceinline__ double quot(double a, double b) { return soft::div(a, b); }
+__device__ __forceinline__ float quot(float a, float b) { return a / b; }
+__device__ __forceinline__ double rsqrt_r(double x) { return soft::root(x); }
 __device__ __forceinline__ float rsqrt_r(float x) { return sqrtf(x); }
 // tanh|x| = m / (m + 2), m = expm1(2|x|): Taylor series of expm1 below 0.5, else
 // exp(y) = 2^k exp(r) with Cody-Waite reduction (y = k ln2 + r, ln2 split into
@@ -177,14 +184,14 @@ __device__ __forceinline__ double tanh_r(double x) {
       for (int k = 18; k >= 2; --k) s = 1.0 + (y * (1.0 / (double)k)) * s;
       m = y * s;
     } else {
-      const double k = rint(y / kLn2);
+      const double k = rint(quot(y, kLn2));
       const double r = (y - k * kLn2Hi) - k * kLn2Lo;
       double s = 1.0;
 #pragma unroll
       for (int j = 17; j >= 1; --j) s = 1.0 + (r * (1.0 / (double)j)) * s;
       m = ldexp(s, (int)k) - 1.0;
     }
-    t = m / (m + 2.0);
+    t = quot(m, m + 2.0);
   }
   return x < 0.0 ? -t : t;
 }
@@ -232,8 +239,8 @@ __device__ __forceinline__ void mix_SP(const DevFluid& f, const R* al_stored, R&
 // rho c^2 = gbar (p + pbar_inf) = (1 + 1/S) p + P/S
 template <typename R>
 __device__ __forceinline__ R rho_c2(R S, R P, R p) {
-  R gb = R(1) + R(1) / S;
-  return gb * p + P / S;
+  R gb = R(1) + quot(R(1), S);
+  return gb * p + quot(P, S);
 }
 
 // ---------------------------------------------------------------- WENO-IS (App. C)
@@ -295,7 +302,7 @@ __device__ __forceinline__ R weno_is(R um2, R um1, R u0, R up1, R up2, R eps) {
   weno_eta<R>(b0, b1, b01, b2, b3, tau5, eps, e0, e1, e2, e3);
   const R es = e0 + e1 + e2 + e3;
   // sum_k omega_k S_k with omega_k = e_k / es: the normalisation applied once
-  return (e0 * s0 + e1 * s1 + e2 * s2 + e3 * s3) / es;
+  return quot(e0 * s0 + e1 * s1 + e2 * s2 + e3 * s3, es);
 }
 
 // The same interpolation with every nonlinear weight replaced by its linear
@@ -346,8 +353,8 @@ __device__ __forceinline__ R weno_dev(R um2, R um1, R u0, R up1, R up2, R eps) {
   R e0, e1, e2, e3;
   weno_eta<R>(b0, b1, b01, b2, b3, tau5, eps, e0, e1, e2, e3);
   const R es = e0 + e1 + e2 + e3;
-  const R dv[4] = {e0 / es - R(15.0 / 32.0), e1 / es - R(5.0 / 32.0), e2 / es - R(5.0 / 16.0),
-                   e3 / es - R(1.0 / 16.0)};
+  const R dv[4] = {quot(e0, es) - R(15.0 / 32.0), quot(e1, es) - R(5.0 / 32.0), quot(e2, es) - R(5.0 / 16.0),
+                   quot(e3, es) - R(1.0 / 16.0)};
   R mx = R(0);
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
@@ -382,7 +389,7 @@ __device__ __forceinline__ void prim_state(const DevFluid& f, PrimState<R, N, D>
   const R p = s.V[L::EN];
   s.rho = rho;
   s.E = (S * p + P) + R(0.5) * rho * kin + rq;
-  s.c = rsqrt_r(rho_c2(S, P, p) / rho);
+  s.c = rsqrt_r(quot(rho_c2(S, P, p), rho));
 }
 
 // HLLC flux of the flux-source form G (F^HLLC plus the upwind alpha s_* in the
@@ -400,8 +407,8 @@ __device__ __forceinline__ R hllc(const DevFluid& f, PrimState<R, N, D>& Ls, Pri
   const R ubar = R(0.5) * (uL + uR), cbar = R(0.5) * (Ls.c + Rs.c);
   const R sL = dmin(ubar - cbar, uL - Ls.c);
   const R sR = dmax(ubar + cbar, uR + Rs.c);
-  const R ss = (pR - pL + Ls.rho * uL * (sL - uL) - Rs.rho * uR * (sR - uR)) /
-               (Ls.rho * (sL - uL) - Rs.rho * (sR - uR));
+  const R ss = quot(pR - pL + Ls.rho * uL * (sL - uL) - Rs.rho * uR * (sR - uR),
+                    Ls.rho * (sL - uL) - Rs.rho * (sR - uR));
   const int sg = (ss > R(0)) ? 1 : ((ss < R(0)) ? -1 : 0);
   const R wL = (sg > 0) ? R(1) : ((sg < 0) ? R(0) : R(0.5));
   const R wR = R(1) - wL;
@@ -416,7 +423,7 @@ __device__ __forceinline__ R hllc(const DevFluid& f, PrimState<R, N, D>& Ls, Pri
     const R pK = side == 0 ? pL : pR;
     const R sK = side == 0 ? sL : sR;
     const R sfac = side == 0 ? dmin(R(0), sL) : dmax(R(0), sR);
-    const R chi = (sK - uK) / (sK - ss);
+    const R chi = quot(sK - uK, sK - ss);
     // F_K + s_{-/+} (W_{*,K} - W_K), conservative slots
 #pragma unroll
     for (int k = 0; k < N; ++k) {
@@ -431,7 +438,7 @@ __device__ __forceinline__ R hllc(const DevFluid& f, PrimState<R, N, D>& Ls, Pri
       const R ms = (d == DIR) ? chi * K.rho * ss : chi * K.rho * K.V[L::MOM + d];
       G[L::MOM + d] = G[L::MOM + d] + w * (Fm + sfac * (ms - mom));
     }
-    const R Es = chi * (K.E + (ss - uK) * (K.rho * ss + pK / (sK - uK)));
+    const R Es = chi * (K.E + (ss - uK) * (K.rho * ss + quot(pK, sK - uK)));
     G[L::EN] = G[L::EN] + w * ((K.E + pK) * uK + sfac * (Es - K.E));
 #pragma unroll
     for (int k = 0; k < N - 1; ++k) G[L::AL + k] = G[L::AL + k] + w * (K.V[L::AL + k] * ss);

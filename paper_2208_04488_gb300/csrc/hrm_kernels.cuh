@@ -104,7 +104,7 @@ __device__ __forceinline__ double rhoe_tilde(const double* W, const DevFluid& f)
   }
 #pragma unroll
   for (int d = 0; d < D; ++d) kin += W[L::MOM + d] * W[L::MOM + d];
-  return W[L::EN] - 0.5 * kin / rho - rq;
+  return W[L::EN] - quot(0.5 * kin, rho) - rq;
 }
 
 __device__ __forceinline__ double theta_of(double lo, double hi, double eps) {
@@ -461,7 +461,7 @@ __device__ __forceinline__ void face_body(int64_t t, const Nodes6& nd, const dou
     // characteristic projection with the face-averaged state (App. D)
     const R rhob = R(0.5) * (R(Rr[nd.c[2]]) + R(Rr[nd.c[3]]));
     const R cb = R(0.5) * (R(Cc[nd.c[2]]) + R(Cc[nd.c[3]]));
-    const R inv_rc = R(1) / (rhob * cb);
+    const R inv_rc = quot(R(1), rhob * cb);
     const R rc2b = rhob * cb * cb;
     const R eps = R(pr.weno_eps);
     R UL[M], UR[M];
@@ -480,7 +480,7 @@ __device__ __forceinline__ void face_body(int64_t t, const Nodes6& nd, const dou
 #pragma unroll
       for (int j = 0; j < 6; ++j) w6[j] = R(V[k * nc + nd.c[j]]);
       arb[k] = R(0.5) * (w6[2] + w6[3]);
-      const R coef = arb[k] / rc2b;
+      const R coef = quot(arb[k], rc2b);
 #pragma unroll
       for (int j = 0; j < 6; ++j) w6[j] = w6[j] - coef * p6[j];
       UL[1 + k] = weno_sel<R>(lin, w6[0], w6[1], w6[2], w6[3], w6[4], eps);
@@ -510,8 +510,8 @@ __device__ __forceinline__ void face_body(int64_t t, const Nodes6& nd, const dou
     {
       R h[N];
 #pragma unroll
-      for (int k = 0; k < N; ++k) h[k] = arb[k] / (R(2) * cb);
-      const R rc_2 = rhob * cb / R(2);
+      for (int k = 0; k < N; ++k) h[k] = quot(arb[k], R(2) * cb);
+      const R rc_2 = rhob * cb * R(0.5);
 #pragma unroll
       for (int side = 0; side < 2; ++side) {
         const R* U = side == 0 ? UL : UR;
@@ -553,7 +553,7 @@ __device__ __forceinline__ void face_body(int64_t t, const Nodes6& nd, const dou
       auto half = [](R a, R b, R c, R d, R e) -> R {
         const R num = fabs(R(16) * b - a - R(30) * c + R(16) * d - e);
         const R den = fabs(a + R(16) * b + R(30) * c + R(16) * d + e);
-        return den == R(0) ? R(0) : num / den;
+        return den == R(0) ? R(0) : quot(num, den);
       };
       const R sr_ = R(0.5) * (half(r6[1], r6[2], r6[3], r6[4], r6[5]) + half(r6[0], r6[1], r6[2], r6[3], r6[4]));
       const R sp_ = R(0.5) * (half(p6[1], p6[2], p6[3], p6[4], p6[5]) + half(p6[0], p6[1], p6[2], p6[3], p6[4]));
@@ -685,11 +685,11 @@ __device__ __forceinline__ void relax_fast(double* W, const DevFluid& f, double&
   const double A = rho * Cv;
   const double B = fma(pinf1 * rho, Cv + WlR1, -(Re * Rm));
   const double C = -(Re * pinf1 * (Rm - WlR1));
-  const double sq = sqrt(fma(B, B, -4.0 * A * C));
-  const double ps = (B > 0.0) ? (-2.0 * C) / (B + sq) : (sq - B) / (2.0 * A);
+  const double sq = rsqrt_r(fma(B, B, -4.0 * A * C));
+  const double ps = (B > 0.0) ? quot(-2.0 * C, B + sq) : quot(sq - B, 2.0 * A);
   const double ppl = ps + pinf1;
   const double Y = fma(Wl * fma(f.gamma[l], pinf1, ps), f.cv[l], fma(-Wl, f.cv[l], Cv) * ppl);
-  const double z = Re / (rho * Y * ps);
+  const double z = quot(Re, rho * Y * ps);
 #pragma unroll
   for (int k = 0; k < N - 1; ++k)  // alpha_k = rho_k' R_k T* / (p* + p_inf,k), one stiffened gas at most
     W[L::AL + k] = W[k] * f.Rg[k] * (k == l ? ps : ppl) * z;
@@ -720,7 +720,7 @@ __device__ __forceinline__ void relax_cell(double* W, const DevFluid& f, double*
   for (int k = 0; k < N; ++k) rho += W[k];
   double Y[N];
 #pragma unroll
-  for (int k = 0; k < N; ++k) Y[k] = W[k] / rho;
+  for (int k = 0; k < N; ++k) Y[k] = quot(W[k], rho);
   const double re = rhoe_tilde<N, D>(W, f);
   double cvb = 0.0, cpb = 0.0;
 #pragma unroll
@@ -732,14 +732,14 @@ __device__ __forceinline__ void relax_cell(double* W, const DevFluid& f, double*
   const double Ap = cvb;
   const double Bp = -(re * (cpb - cvb) - pinf1 * cvb - pinf1 * Yl * R1);
   const double Cp = -(re * pinf1 * ((cpb - cvb) - Yl * R1));
-  const double sq = sqrt(Bp * Bp - 4.0 * Ap * Cp);
-  const double ps = (Bp > 0.0) ? (-2.0 * Cp) / (Bp + sq) : (sq - Bp) / (2.0 * Ap);
-  const double den = Yl * (ps + f.gamma[l] * pinf1) * f.cv[l] / (ps + pinf1) + cvb - Yl * f.cv[l];
-  const double Ts = (re / rho) / den;
+  const double sq = rsqrt_r(Bp * Bp - 4.0 * Ap * Cp);
+  const double ps = (Bp > 0.0) ? quot(-2.0 * Cp, Bp + sq) : quot(sq - Bp, 2.0 * Ap);
+  const double den = quot(Yl * (ps + f.gamma[l] * pinf1) * f.cv[l], ps + pinf1) + cvb - Yl * f.cv[l];
+  const double Ts = quot(quot(re, rho), den);
 #pragma unroll
   for (int k = 0; k < N - 1; ++k) {
-    const double rhok = (ps + f.pinf[k]) / (f.Rg[k] * Ts);
-    W[L::AL + k] = W[k] / rhok;
+    const double rhok = quot(ps + f.pinf[k], f.Rg[k] * Ts);
+    W[L::AL + k] = quot(W[k], rhok);
   }
   if (pT) {
     pT[0] = ps;
@@ -764,7 +764,7 @@ __device__ __forceinline__ int admissibility_bits(const double* W, const DevFlui
   const double re = rhoe_tilde<N, D>(W, f);
   double S, P;
   mix_SP<double, N>(f, &W[L::AL], S, P);
-  const double p = (re - P) / S;
+  const double p = quot(re - P, S);
   if (!(rho_c2(S, P, p) > 0.0)) b |= 4;
   if (!(re > 0.0)) b |= 8;
   return b;
@@ -957,13 +957,13 @@ __device__ __forceinline__ void update_body(int64_t c, const double* Wn, const d
 #pragma unroll
     for (int m = 0; m < L::NC; ++m) {
       const double df = F[m * nf + fr] - F[m * nf + fl];
-      rhs[m] = rhs[m] - (scale ? df * idx : df / dx);
+      rhs[m] = rhs[m] - (scale ? df * idx : quot(df, dx));
     }
 #pragma unroll
     for (int k = 0; k < N - 1; ++k) {
       const int m = L::AL + k;
       const double df = F[m * nf + fr] - F[(M + k) * nf + fl];
-      rhs[m] = rhs[m] - (scale ? df * idx : df / dx);
+      rhs[m] = rhs[m] - (scale ? df * idx : quot(df, dx));
     }
   }
   if (MODE == 1) {

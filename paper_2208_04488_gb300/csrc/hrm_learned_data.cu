@@ -38,7 +38,7 @@ __device__ double stencil_dev(const Nodes6& nd, const double* __restrict__ V, co
   }
   const double rhob = 0.5 * (Rr[nd.c[2]] + Rr[nd.c[3]]);
   const double cb = 0.5 * (Cc[nd.c[2]] + Cc[nd.c[3]]);
-  const double inv_rc = 1.0 / (rhob * cb);
+  const double inv_rc = quot(1.0, rhob * cb);
   const double rc2b = rhob * cb * cb;
   double mx = 0.0;
   auto both = [&]() {
@@ -58,7 +58,7 @@ __device__ double stencil_dev(const Nodes6& nd, const double* __restrict__ V, co
 #pragma unroll
     for (int j = 0; j < 6; ++j) w6[j] = V[k * nc + nd.c[j]];
     const double arb = 0.5 * (w6[2] + w6[3]);
-    const double coef = arb / rc2b;
+    const double coef = quot(arb, rc2b);
 #pragma unroll
     for (int j = 0; j < 6; ++j) w6[j] = w6[j] - coef * p6[j];
     both();

@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(kThreads)
     cell_prim<N, D>(w, f, v, rho, cs, rc2);
 #pragma unroll
     for (int d = 0; d < D; ++d) {
-      const double s = (fabs(v[L::MOM + d]) + cs) / g.dx[d];
+      const double s = quot(fabs(v[L::MOM + d]) + cs, g.dx[d]);
       mx[d] = (s != s) ? s : (s > mx[d] ? s : mx[d]);  // NaN propagates as the largest value
     }
   }

@@ -74,6 +74,13 @@ __global__ void k_convert(const double* in_d, const float* in_f, int64_t n, floa
   widened[i] = hrm::widen_f32(in_f[i]);
 }
 
+// The integer-pipe FP64 arithmetic, element by element.
+__global__ void k_soft64(int op, const double* a, const double* b, int64_t n, double* out) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  out[i] = op == 0 ? hrm::soft::mul(a[i], b[i]) : (op == 1 ? hrm::soft::div(a[i], b[i]) : hrm::soft::root(a[i]));
+}
+
 // Blocks waiting at a grid barrier that counts one block more than launched.
 __global__ void __launch_bounds__(128) k_barrier_probe(hrm::GridSync* s, uint64_t limit_ns) {
   hrm::grid_barrier(s, gridDim.x + 1u, limit_ns);
@@ -103,6 +110,15 @@ extern "C" hrm_status hrm_probe_convert(const double* in_d, const float* in_f, i
   if (n == 0) return HRM_OK;
   cudaStream_t s = (cudaStream_t)stream;
   k_convert<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(in_d, in_f, n, narrowed, widened);
+  return cudaGetLastError() == cudaSuccess ? HRM_OK : HRM_E_CUDA;
+}
+
+extern "C" hrm_status hrm_probe_soft64(int32_t op, const double* a, const double* b, int64_t n, double* out,
+                                       void* stream) {
+  if (op < 0 || op > 2 || n < 0 || (n > 0 && (!a || !b || !out))) return HRM_E_INVAL;
+  if (n == 0) return HRM_OK;
+  cudaStream_t s = (cudaStream_t)stream;
+  k_soft64<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(op, a, b, n, out);
   return cudaGetLastError() == cudaSuccess ? HRM_OK : HRM_E_CUDA;
 }
 

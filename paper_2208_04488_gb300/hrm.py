@@ -176,6 +176,8 @@ def lib():
     L.hrm_probe_wait_timeout.restype = ctypes.c_int
     L.hrm_probe_convert.argtypes = [_VP, _VP, ctypes.c_int64, _VP, _VP, _VP]
     L.hrm_probe_convert.restype = ctypes.c_int
+    L.hrm_probe_soft64.argtypes = [ctypes.c_int32, _VP, _VP, ctypes.c_int64, _VP, _VP]
+    L.hrm_probe_soft64.restype = ctypes.c_int
     L.hrm_probe_barrier_timeout.argtypes = [_VP, ctypes.c_double, ctypes.POINTER(ctypes.c_int64)]
     L.hrm_probe_barrier_timeout.restype = ctypes.c_int
     L.hrm_step_tau.argtypes = [_VP, _DP]
@@ -233,6 +235,20 @@ def probe_convert(in_d, in_f, stream=None):
     if st != HRM_OK:
         raise HrmError(st, "conversion probe failed")
     return narrowed, widened
+
+
+def probe_soft64(op, a, b, stream=None):
+    """a * b (op 0), a / b (1) or sqrt(a) (2) of two FP64 device tensors of equal
+    length by the library's integer-pipe arithmetic."""
+    import torch
+    assert a.dtype == b.dtype == torch.float64 and a.numel() == b.numel()
+    a, b = a.contiguous(), b.contiguous()
+    out = torch.empty_like(a)
+    st = lib().hrm_probe_soft64(int(op), _VP(a.data_ptr()), _VP(b.data_ptr()), a.numel(), _VP(out.data_ptr()),
+                                _VP(_stream_handle(stream)))
+    if st != HRM_OK:
+        raise HrmError(st, "arithmetic probe failed")
+    return out
 
 
 def params_default(**overrides) -> HrmParams:
