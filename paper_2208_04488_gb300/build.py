@@ -26,6 +26,7 @@ FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", 
          "--expt-relaxed-constexpr"] + (["-DHRM_BOUNDS_CHECK"] if BOUNDS_CHECK else [])
 UNITS = {
     "hrm_cell.cu": ["--fmad=false"],
+    "hrm_sweep.cu": ["--fmad=false"],
     "hrm_face64_d1.cu": ["--fmad=false"],
     "hrm_face64_d2.cu": ["--fmad=false"],
     "hrm_face64_d3.cu": ["--fmad=false"],

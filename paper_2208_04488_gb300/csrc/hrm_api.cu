@@ -48,6 +48,7 @@ struct hrm_ctx {
   mlp::GateBlob* blob = nullptr;   // learned gate weights (hrm_set_detector)
   uint8_t* gate[3] = {nullptr, nullptr, nullptr};  // gate bytes per direction (midpoint grids)
   uint8_t* same = nullptr;         // FP64 form: per cell, the last update left W bit for bit as its source
+  SweepLists lists;                // FP64 form: uniform faces and the midpoints to sweep (hrm_sweep.cuh)
   uint32_t* defer = nullptr;       // precision form: per direction, a worklist of deferred midpoints and its counter
   int64_t defer_cap = 0;           // worklist entries (the largest midpoint grid; 0: no worklist)
   hrm_alloc_fn alloc = nullptr;    // device memory source (hrm_set_allocator at creation; NULL: cudaMalloc)
@@ -257,6 +258,10 @@ GateArgs gate_of(const hrm_ctx* c, int d) {
     g.defer_count = g.defer_list + c->defer_cap;
   }
   if (c->params.learned) g.fixed = c->gate[d];
+  if (c->params.precision == HRM_FP64) {
+    g.list = c->lists.list[d];
+    g.list_cnt = c->lists.cnt + kSweepCounts * d;
+  }
   if (c->params.learned == 1 && defer_sweep(c)) {  // the network inside the sweep
     g.net = c->blob;
     g.R32 = c->R32;
@@ -264,6 +269,16 @@ GateArgs gate_of(const hrm_ctx* c, int d) {
     g.out_gate = c->gate[d];
   }
   return g;
+}
+
+// FP64 form: uniform faces and the lists of the other midpoints of Wsrc; full: the
+// uniform faces' fluxes into the flux planes as well.
+int enqueue_mark(hrm_ctx* c, cudaStream_t s, const double* Wsrc, bool full) {
+  if (c->params.precision != HRM_FP64) return 0;
+  SweepLists l = c->lists;
+  for (int d = 0; d < c->D; ++d) l.F[d] = full ? c->F[d] : nullptr;
+  launch_mark64(c->N, c->D, Wsrc, c->V, c->dg, l, c->params.scheme == HRM_SCHEME_HLLC1, s);
+  return 2;
 }
 
 // With the learned detector, its gate kernel runs before each sweep, except in
@@ -316,6 +331,7 @@ int enqueue_stage(hrm_ctx* c, cudaStream_t s, const double* Wsrc, double* Wout, 
       });
       ++k;
     }
+  k += enqueue_mark(c, s, Wsrc, false);
   // the sweeps: independent (each reads the primitives and writes its own flux
   // planes), so directions d > 0 run on their own streams beside direction 0
   const bool fork = c->D > 1 && c->par[1];
@@ -352,7 +368,8 @@ int enqueue_stage(hrm_ctx* c, cudaStream_t s, const double* Wsrc, double* Wout, 
                        count, c->P32, r32_target(c), s, tau_next ? 1 : 0);
     else
       c->fk->update(0, c->params.precision == HRM_FP32, c->Wn, Wsrc, Wout, c->F[0], c->F[1], c->F[2], c->dg,
-                    c->fl, c->st, a, b, relax, count, same_out ? same : nullptr, s);
+                    c->fl, c->st, a, b, relax, count, same_out ? same : nullptr,
+                    c->params.precision == HRM_FP64 ? c->lists.uni : nullptr, c->V, s);
   });
   ++k;
   return k;
@@ -746,6 +763,15 @@ hrm_status hrm_create(hrm_ctx** out, const hrm_grid* grid, int32_t N, const doub
     if ((int64_t)nf > c->defer_cap) c->defer_cap = (int64_t)nf;
   }
   if ((s = cuda_check(c, ctx_malloc(c, &c->same, (size_t)c->nc), "alloc unchanged-cell flags"))) return bail(s);
+  if ((s = cuda_check(c, ctx_malloc(c, &c->lists.eq, (size_t)c->nint), "alloc equality flags"))) return bail(s);
+  if ((s = cuda_check(c, ctx_malloc(c, &c->lists.uni, (size_t)c->nint), "alloc uniform-face flags"))) return bail(s);
+  if ((s = cuda_check(c, ctx_malloc(c, &c->lists.cnt, sizeof(uint32_t) * kSweepCounters), "alloc sweep counters")))
+    return bail(s);
+  if (c->defer_cap >= (int64_t)0xffffffffll)  // (its flux planes alone would exceed the device)
+    return bail(fail(c, HRM_E_NOMEM, "2^32 - 1 midpoints or more in one direction"));
+  for (int d = 0; d < D; ++d)
+    if ((s = cuda_check(c, ctx_malloc(c, &c->lists.list[d], sizeof(uint32_t) * (size_t)face_total(c->dg, d)), "alloc midpoint list")))
+      return bail(s);
   // worklist of the precision form's deferred midpoints (32-bit entries; none
   // beyond 2^32 - 1 midpoints, where the sweep keeps its fallbacks inline)
   if (c->defer_cap < (int64_t)0xffffffffll) {
@@ -792,6 +818,10 @@ void hrm_destroy(hrm_ctx* c) {
   ctx_free(c, c->Wn);
   ctx_free(c, c->Ws);
   ctx_free(c, c->same);
+  ctx_free(c, c->lists.eq);
+  ctx_free(c, c->lists.uni);
+  ctx_free(c, c->lists.cnt);
+  for (int d = 0; d < 3; ++d) ctx_free(c, c->lists.list[d]);
   ctx_free(c, c->defer);
   ctx_free(c, c->V);
   ctx_free(c, c->AUX);
@@ -1173,6 +1203,7 @@ hrm_status hrm_rhs(hrm_ctx* c, const double* lam, double* rhs) {
     launch_prim32(c->N, c->D, c->Wn, c->P32, r32_target(c), c->dg, c->fl, c->st, 0, c->stream);
   else
     c->ck->prim(c->Wn, c->V, c->AUX, p32_target(c), r32_target(c), c->dg, c->fl, c->st, 0, nullptr, c->stream);
+  c->launches += enqueue_mark(c, c->stream, c->Wn, true);
   for (int d = 0; d < c->D; ++d) {
     if (separate_gate(c)) {
       launch_gate(c->N, c->D, d, c->P32, c->R32, c->dg, c->blob, gate_logit_threshold(c), c->gate[d],
@@ -1183,7 +1214,7 @@ hrm_status hrm_rhs(hrm_ctx* c, const double* lam, double* rhs) {
                    gate_of(c, d), c->stream);
   }
   c->fk->update(1, 0, c->Wn, c->Wn, out, c->F[0], c->F[1], c->F[2], c->dg, c->fl, c->st, 0.0, 1.0, 0, 0,
-                nullptr, c->stream);
+                nullptr, nullptr, nullptr, c->stream);
   c->launches += 2 + c->D * sweep_kernels(c);
   if ((s = last_launch(c, "rhs"))) return s;
   // (the update writes interior cells only: the stage state's slices stay)

@@ -7,6 +7,7 @@
 
 #include "hrm_cell.cuh"
 #include "hrm_face32.cuh"
+#include "hrm_face64.cuh"
 #include "hrm_sync.cuh"
 
 namespace hrm {
@@ -112,7 +113,8 @@ __device__ __forceinline__ void stage_face(const BatchInst& I, int64_t t, int sr
                                             I.st->lam[DIR], false, xs))
       face32_full<N, D, DIR>(t, nd, I, src, pr, xs);
   } else {
-    face_body<double, N, D, DIR>(t, nd, pick(I, src), I.V, I.AUX, I.F[DIR], I.g, I.f, pr, I.st->lam[DIR]);
+    face_body<N, D, DIR>(t, nd, pick(I, src), I.V, I.AUX, I.F[DIR], I.g, I.f, pr, I.st->lam[DIR],
+                         reinterpret_cast<double*>(xs));
   }
 }
 
@@ -155,7 +157,9 @@ __device__ __forceinline__ void stage_update(const BatchInst& I, const WorkItem&
 
 template <int D, bool FP32>
 __device__ __forceinline__ void batch_stage(const StageArgs& A) {
-  __shared__ float xs[2 * Lay<3, D>::M * kBatchFace32Threads];  // the FP32 bodies' column (largest N)
+  // the bodies' column (largest N): 2 x M floats, or kFaceCol doubles
+  __shared__ __align__(16) float xs[FP32 ? 2 * Lay<3, D>::M * kBatchFace32Threads : 2 * kFaceCol<3, D>];
+  static_assert(kBatchFace32Threads == kFaceThreads, "column stride of the bodies");
   const unsigned int nb = gridDim.x;
   const bool stamper = blockIdx.x == 0 && threadIdx.x == 0;
   unsigned long long* stamp = A.sync->stamp[A.stage];

@@ -12,7 +12,7 @@ namespace hrm {
 // Primitive variables of a conservative vector (Sec. 2): rho = sum alpha_k rho_k,
 // u_d = rho u_d / rho, p from the mixture EOS p/(gbar-1) + gbar pbar_inf/(gbar-1) =
 // rho (e - qbar), rho c^2 = gbar (p + pbar_inf), c = sqrt(rho c^2 / rho).
-template <int N, int D>
+template <int N, int D, bool SOFT = false>
 __device__ __forceinline__ void cell_prim(const double* W, const DevFluid& f, double* V, double& rho,
                                           double& c, double& rc2) {
   using L = Lay<N, D>;
@@ -20,7 +20,7 @@ __device__ __forceinline__ void cell_prim(const double* W, const DevFluid& f, do
 #pragma unroll
   for (int k = 0; k < N; ++k) rho += W[k];
   double S, P;
-  mix_SP<double, N>(f, &W[L::AL], S, P);
+  mix_SP<double, N, SOFT>(f, &W[L::AL], S, P);
   const double re = rhoe_tilde<N, D>(W, f);
   const double p = quot(re - P, S);
 #pragma unroll
@@ -113,7 +113,7 @@ __device__ __forceinline__ void prim_body(int64_t c, const double* __restrict__ 
     double w[M], v[M], rho, cs, rc2;
 #pragma unroll
     for (int m = 0; m < M; ++m) w[m] = W[m * nc + c];
-    cell_prim<N, D>(w, f, v, rho, cs, rc2);
+    cell_prim<N, D, true>(w, f, v, rho, cs, rc2);
 #pragma unroll
     for (int m = 0; m < M; ++m) V[m * nc + c] = v[m];
     AUX[c] = cs;

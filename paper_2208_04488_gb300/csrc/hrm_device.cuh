@@ -75,6 +75,38 @@ __device__ __forceinline__ int64_t hrm_checked_index(const DevGrid& g, int64_t i
 #define HRM_IDX(g, i, n) (i)
 #endif
 
+// Indices of cell c of a plane (x fastest). 32-bit divisions where they do: the
+// 64-bit ones take about four times the instructions.
+__device__ __forceinline__ void plane_index(int64_t c, int64_t n0, int64_t n1, int64_t* ijk) {
+  if ((uint64_t)c <= 0xffffffffull && (uint64_t)n0 <= 0xffffffffull && (uint64_t)n1 <= 0xffffffffull) {
+    const uint32_t u = (uint32_t)c, r = u / (uint32_t)n0, k = r / (uint32_t)n1;
+    ijk[0] = u - r * (uint32_t)n0;
+    ijk[1] = r - k * (uint32_t)n1;
+    ijk[2] = k;
+    return;
+  }
+  const int64_t r = c / n0;
+  ijk[0] = c % n0;
+  ijk[1] = r % n1;
+  ijk[2] = r / n1;
+}
+__device__ __forceinline__ void cell_index(const DevGrid& g, int64_t c, int64_t* ijk) {
+  plane_index(c, g.n[0], g.n[1], ijk);
+}
+
+// Work of the list-driven sweeps (hrm_sweep.cuh): one byte per cell each for eq
+// and uni, a list of midpoints per direction with kSweepCounts counters (entries,
+// entries taken); F: the flux planes where the uniform faces' fluxes are wanted
+// as well.
+constexpr int kSweepCounts = 4, kSweepCounters = 3 * kSweepCounts;
+struct SweepLists {
+  uint8_t* eq = nullptr;
+  uint8_t* uni = nullptr;
+  uint32_t* list[3] = {nullptr, nullptr, nullptr};
+  uint32_t* cnt = nullptr;
+  double* F[3] = {nullptr, nullptr, nullptr};
+};
+
 struct DevParams {
   int32_t limiters, blend, scheme, qexp;
   double eps_ar, eps_a, eps_rhoe, hs_ar, hs_a, hs_rc2, hs_rhoe, weno_eps, Cs;
@@ -162,6 +194,18 @@ template <typename T> __device__ __forceinline__ T dmax(T a, T b) { return (a < 
 __device__ __forceinline__ double quot(double a, double b) { return soft::div(a, b); }
 __device__ __forceinline__ float quot(float a, float b) { return a / b; }
 __device__ __forceinline__ double rsqrt_r(double x) { return soft::root(x); }
+// FP64 products on the integer pipes, for the bodies whose adds keep the FP64 unit
+// busy meanwhile: the bits of a * b.
+__device__ __forceinline__ double prod(double a, double b) { return soft::mul(a, b); }
+__device__ __forceinline__ float prod(float a, float b) { return a * b; }
+// x times a power of two
+__device__ __forceinline__ double halved(double x) { return soft::scale<-1>(x); }
+__device__ __forceinline__ float halved(float x) { return 0.5f * x; }
+// 0 + x: a negative zero becomes a positive one
+__device__ __forceinline__ double plus_zero(double x) {
+  return (((uint32_t)__double2hiint(x) & 0x7fffffffu) | (uint32_t)__double2loint(x)) == 0u ? 0.0 : x;
+}
+__device__ __forceinline__ float plus_zero(float x) { return 0.f + x; }
 __device__ __forceinline__ float rsqrt_r(float x) { return sqrtf(x); }
 // tanh|x| = m / (m + 2), m = expm1(2|x|): Taylor series of expm1 below 0.5, else
 // exp(y) = 2^k exp(r) with Cody-Waite reduction (y = k ln2 + r, ln2 split into
@@ -173,7 +217,9 @@ __device__ __forceinline__ double tanh_r(double x) {
   constexpr double kLn2Lo = 1.9082149292705877e-10;
   const double ax = fabs(x);
   double t;
-  if (ax > 22.0) {
+  if (ax < 0x1p-55) {
+    t = ax;  // every s below rounds to 1, m to 2 ax and m + 2 to 2
+  } else if (ax > 22.0) {
     t = 1.0;
   } else {
     const double y = 2.0 * ax;
@@ -220,7 +266,9 @@ struct Lay {
 // ---------------------------------------------------------------- mixture rules (Sec. 2)
 
 // S = 1/(gbar - 1), P = gbar pbar_inf / (gbar - 1) from the N-1 stored alphas.
-template <typename R, int N>
+// SOFT: FP64 products on the integer pipes (where many warps share the FP64 unit;
+// a lone warp's chain is shorter without).
+template <typename R, int N, bool SOFT = false>
 __device__ __forceinline__ void mix_SP(const DevFluid& f, const R* al_stored, R& S, R& P) {
   R sum = R(0);
   S = R(0);
@@ -231,8 +279,9 @@ __device__ __forceinline__ void mix_SP(const DevFluid& f, const R* al_stored, R&
 #pragma unroll
   for (int k = 0; k < N; ++k) {
     R a = (k < N - 1) ? al_stored[k] : last;
-    S = S + a * inv_gm1_of(f, k, R());
-    P = P + a * gpinf_gm1_of(f, k, R());
+    S = S + (SOFT ? prod(a, inv_gm1_of(f, k, R())) : a * inv_gm1_of(f, k, R()));
+    const R gp = gpinf_gm1_of(f, k, R());
+    if (gp != R(0)) P = P + (SOFT ? prod(a, gp) : a * gp);  // (a zero term adds nothing)
   }
 }
 
@@ -240,7 +289,7 @@ __device__ __forceinline__ void mix_SP(const DevFluid& f, const R* al_stored, R&
 template <typename R>
 __device__ __forceinline__ R rho_c2(R S, R P, R p) {
   R gb = R(1) + quot(R(1), S);
-  return gb * p + quot(P, S);
+  return prod(gb, p) + quot(P, S);
 }
 
 // ---------------------------------------------------------------- WENO-IS (App. C)
@@ -373,42 +422,80 @@ struct PrimState {
   R rho, E, c;
 };
 
+// rc2 (nullable) receives rho c^2.
 template <typename R, int N, int D>
-__device__ __forceinline__ void prim_state(const DevFluid& f, PrimState<R, N, D>& s) {
+__device__ __forceinline__ void prim_state(const DevFluid& f, PrimState<R, N, D>& s, R* rc2_out = nullptr) {
   using L = Lay<N, D>;
-  R rho = R(0), rq = R(0), kin = R(0);
+  R rho = R(0), kin = R(0);
 #pragma unroll
-  for (int k = 0; k < N; ++k) {
-    rho = rho + s.V[k];
-    rq = rq + s.V[k] * q_of(f, k, R());
-  }
+  for (int k = 0; k < N; ++k) rho = rho + s.V[k];
 #pragma unroll
   for (int d = 0; d < D; ++d) kin = kin + s.V[L::MOM + d] * s.V[L::MOM + d];
   R S, P;
   mix_SP<R, N>(f, &s.V[L::AL], S, P);
   const R p = s.V[L::EN];
   s.rho = rho;
-  s.E = (S * p + P) + R(0.5) * rho * kin + rq;
-  s.c = rsqrt_r(quot(rho_c2(S, P, p), rho));
+  s.E = (S * p + P) + R(0.5) * rho * kin;
+  if (f.has_q) {
+    R rq = R(0);
+#pragma unroll
+    for (int k = 0; k < N; ++k) rq = rq + s.V[k] * q_of(f, k, R());
+    s.E = s.E + rq;
+  }
+  const R rc2 = rho_c2(S, P, p);
+  s.c = rsqrt_r(quot(rc2, rho));
+  if (rc2_out) *rc2_out = rc2;
+}
+
+// Wave speeds and s_* of HLLC (Sec. 4.1.1) between two states given by normal
+// velocity, pressure, density and sound speed.
+template <typename R>
+__device__ __forceinline__ R hllc_speeds(R uL, R uR, R pL, R pR, R rhoL, R rhoR, R cL, R cR, R& sL, R& sR) {
+  const R ubar = R(0.5) * (uL + uR), cbar = R(0.5) * (cL + cR);
+  sL = dmin(ubar - cbar, uL - cL);
+  sR = dmax(ubar + cbar, uR + cR);
+  return quot(pR - pL + rhoL * uL * (sL - uL) - rhoR * uR * (sR - uR), rhoL * (sL - uL) - rhoR * (sR - uR));
+}
+
+// Star flux of one side, F_K + s_{-/+} (W_{*,K} - W_K) and the upwind alpha s_*,
+// each slot given to put(m, value): V(m) primitives, s the side's own wave speed,
+// sfac = min(0, s_L) or max(0, s_R).
+template <typename R, int N, int D, int DIR, typename GetV, typename Put>
+__device__ __forceinline__ void hllc_side(GetV V, R rho, R E, R s, R sfac, R ss, Put put) {
+  using L = Lay<N, D>;
+  const R u = V(L::MOM + DIR), p = V(L::EN);
+  const R chi = quot(s - u, s - ss);
+#pragma unroll
+  for (int k = 0; k < N; ++k) {
+    const R wk = V(k);
+    put(k, wk * u + sfac * (chi * wk - wk));
+  }
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    const R v = V(L::MOM + d), mom = rho * v;
+    R Fm = mom * u;
+    if (d == DIR) Fm = Fm + p;
+    const R ms = (d == DIR) ? chi * rho * ss : chi * rho * v;
+    put(L::MOM + d, Fm + sfac * (ms - mom));
+  }
+  const R Es = chi * (E + (ss - u) * (rho * ss + quot(p, s - u)));
+  put(L::EN, (E + p) * u + sfac * (Es - E));
+#pragma unroll
+  for (int k = 0; k < N - 1; ++k) put(L::AL + k, V(L::AL + k) * ss);
 }
 
 // HLLC flux of the flux-source form G (F^HLLC plus the upwind alpha s_* in the
 // alpha slots) and s_*, from two primitive states. At s_* = 0 the two star
 // fluxes are averaged ((1 +- sign)/2 with sign(0) = 0).
 template <typename R, int N, int D, int DIR>
-__device__ __forceinline__ R hllc(const DevFluid& f, PrimState<R, N, D>& Ls, PrimState<R, N, D>& Rs,
-                                  R* G) {
+__device__ __forceinline__ R hllc(const DevFluid& f, PrimState<R, N, D>& Ls, PrimState<R, N, D>& Rs, R* G) {
   using L = Lay<N, D>;
   constexpr int M = L::M;
   prim_state<R, N, D>(f, Ls);
   prim_state<R, N, D>(f, Rs);
-  const R uL = Ls.V[L::MOM + DIR], uR = Rs.V[L::MOM + DIR];
-  const R pL = Ls.V[L::EN], pR = Rs.V[L::EN];
-  const R ubar = R(0.5) * (uL + uR), cbar = R(0.5) * (Ls.c + Rs.c);
-  const R sL = dmin(ubar - cbar, uL - Ls.c);
-  const R sR = dmax(ubar + cbar, uR + Rs.c);
-  const R ss = quot(pR - pL + Ls.rho * uL * (sL - uL) - Rs.rho * uR * (sR - uR),
-                    Ls.rho * (sL - uL) - Rs.rho * (sR - uR));
+  R sL, sR;
+  const R ss = hllc_speeds<R>(Ls.V[L::MOM + DIR], Rs.V[L::MOM + DIR], Ls.V[L::EN], Rs.V[L::EN], Ls.rho, Rs.rho, Ls.c,
+                              Rs.c, sL, sR);
   const int sg = (ss > R(0)) ? 1 : ((ss < R(0)) ? -1 : 0);
   const R wL = (sg > 0) ? R(1) : ((sg < 0) ? R(0) : R(0.5));
   const R wR = R(1) - wL;
@@ -417,31 +504,11 @@ __device__ __forceinline__ R hllc(const DevFluid& f, PrimState<R, N, D>& Ls, Pri
 #pragma unroll
   for (int side = 0; side < 2; ++side) {
     if ((side == 0 && sg < 0) || (side == 1 && sg > 0)) continue;
-    PrimState<R, N, D>& K = side == 0 ? Ls : Rs;
+    const PrimState<R, N, D>& K = side == 0 ? Ls : Rs;
     const R w = side == 0 ? wL : wR;
-    const R uK = side == 0 ? uL : uR;
-    const R pK = side == 0 ? pL : pR;
-    const R sK = side == 0 ? sL : sR;
-    const R sfac = side == 0 ? dmin(R(0), sL) : dmax(R(0), sR);
-    const R chi = quot(sK - uK, sK - ss);
-    // F_K + s_{-/+} (W_{*,K} - W_K), conservative slots
-#pragma unroll
-    for (int k = 0; k < N; ++k) {
-      const R wk = K.V[k];
-      G[k] = G[k] + w * (wk * uK + sfac * (chi * wk - wk));
-    }
-#pragma unroll
-    for (int d = 0; d < D; ++d) {
-      const R mom = K.rho * K.V[L::MOM + d];
-      R Fm = mom * uK;
-      if (d == DIR) Fm = Fm + pK;
-      const R ms = (d == DIR) ? chi * K.rho * ss : chi * K.rho * K.V[L::MOM + d];
-      G[L::MOM + d] = G[L::MOM + d] + w * (Fm + sfac * (ms - mom));
-    }
-    const R Es = chi * (K.E + (ss - uK) * (K.rho * ss + quot(pK, sK - uK)));
-    G[L::EN] = G[L::EN] + w * ((K.E + pK) * uK + sfac * (Es - K.E));
-#pragma unroll
-    for (int k = 0; k < N - 1; ++k) G[L::AL + k] = G[L::AL + k] + w * (K.V[L::AL + k] * ss);
+    hllc_side<R, N, D, DIR>([&](int m) { return K.V[m]; }, K.rho, K.E, side == 0 ? sL : sR,
+                            side == 0 ? dmin(R(0), sL) : dmax(R(0), sR), ss,
+                            [&](int m, R v) { G[m] = G[m] + w * v; });
   }
   return ss;
 }

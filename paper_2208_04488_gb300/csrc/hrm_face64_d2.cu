@@ -1,7 +1,7 @@
 // FP64 per-midpoint and per-cell-update kernels for D = 2, N = 2..3 species.
 // Built without FMA contraction: the FP64 path evaluates the method's
 // expressions in the same order and rounding as written, operation by operation.
-#include "hrm_kernels.cuh"
+#include "hrm_face64.cuh"
 #include "hrm_launch.h"
 
 namespace hrm {
@@ -18,15 +18,16 @@ void face_l(int precision, const double* W, const double* V, const double* AUX, 
       face32_d2(N, DIR, W, V, AUX, P32, out, g, f, p, st, gate, s);
       return;
     }
-    k_face<double, N, kD, DIR><<<lane_patch_grid(g, DIR), kFaceThreads, 0, s>>>(W, V, AUX, out, g, f, p, st,
-                                                                                gate.fixed);
+    k_face<N, kD, DIR><<<list_grid(g, DIR, 3), kFaceThreads, 0, s>>>(W, V, AUX, out, g, f, p, st, gate.fixed,
+                                                                     gate.list, gate.list_cnt);
   }
 }
 
 template <int N>
 void update_l(int mode, int fast, const double* Wn, const double* Wsrc, double* Wout, const double* F0,
               const double* F1, const double* F2, const DevGrid& g, const DevFluid& f, StepState* st, double a,
-              double b, int relax, int count, uint8_t* same, cudaStream_t s) {
+              double b, int relax, int count, uint8_t* same, const uint8_t* uni,
+              const double* V, cudaStream_t s) {
   if (fast && mode == 0) {
     update32_d2(N, Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count, s);
     return;
@@ -36,7 +37,7 @@ void update_l(int mode, int fast, const double* Wn, const double* Wsrc, double* 
     k_update<N, kD, 1><<<gr, kCellThreads, 0, s>>>(Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count);
   else
     k_update<N, kD, 0><<<gr, kCellThreads, 0, s>>>(Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count,
-                                                   same);
+                                                   same, uni, V);
 }
 
 template <int N>

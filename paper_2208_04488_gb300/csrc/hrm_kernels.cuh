@@ -270,33 +270,6 @@ __device__ __forceinline__ void flux_limit(const double* Wi, const double* Wj, c
   G = hs ? H : Gss;
 }
 
-// True when the flux limiter provably leaves G unchanged: every checked quantity
-// of the high-order half-cell states W_i^{+}, W_{i+1}^{-} (alpha_k rho_k, all N
-// alpha_k, rho e~) is at or above both its limiter threshold and its hard-switch
-// threshold. Then no theta trigger fires (a_high >= eps >= min(eps, a_low)) and
-// no hard switch either, whatever the first-order states, so the first-order
-// flux is not needed. The states are those flux_limit forms, bit for bit; NaN
-// fails the test.
-template <int N, int D>
-__device__ __forceinline__ bool flux_limit_noop(const double* Wi, const double* Wj, const double* Fi,
-                                                const double* Fj, double lam, const FluxPack<N, D>& G,
-                                                const DevFluid& f, const DevParams& pr) {
-  using L = Lay<N, D>;
-  constexpr int M = L::M;
-  double Wp[M], Wm[M], ap[N], am[N];
-  half_state<N, D>(Wi, Fi, G, -2.0 * lam, true, Wp);
-  half_state<N, D>(Wj, Fj, G, 2.0 * lam, false, Wm);
-  all_alpha_W<N, D>(Wp, ap);
-  all_alpha_W<N, D>(Wm, am);
-  const double tar = pr.eps_ar > pr.hs_ar ? pr.eps_ar : pr.hs_ar;
-  const double ta = pr.eps_a > pr.hs_a ? pr.eps_a : pr.hs_a;
-  const double tre = pr.eps_rhoe > pr.hs_rhoe ? pr.eps_rhoe : pr.hs_rhoe;
-  bool ok = rhoe_tilde<N, D>(Wp, f) >= tre && rhoe_tilde<N, D>(Wm, f) >= tre;
-#pragma unroll
-  for (int k = 0; k < N; ++k) ok = ok && Wp[k] >= tar && Wm[k] >= tar && ap[k] >= ta && am[k] >= ta;
-  return ok;
-}
-
 // ---------------------------------------------------------------- per-midpoint kernel
 
 // Loads of the six node cells i-2..i+3 of a midpoint.
@@ -333,9 +306,9 @@ template <int DIR>
 __device__ __forceinline__ bool face_nodes(const DevGrid& g, int64_t t, Nodes6& nd) {
   const int64_t f0 = g.n[0] + (DIR == 0), f1 = g.n[1] + (DIR == 1), f2 = g.n[2] + (DIR == 2);
   if (t >= f0 * f1 * f2) return false;
-  const int64_t i0 = t % f0;
-  const int64_t r = t / f0;
-  const int64_t i1 = r % f1, i2 = r / f1;
+  int64_t ijk[3];
+  plane_index(t, f0, f1, ijk);
+  const int64_t i0 = ijk[0], i1 = ijk[1], i2 = ijk[2];
   const int64_t fp = DIR == 0 ? i0 : (DIR == 1 ? i1 : i2);
   const bool dlo = g.bc[2 * DIR] == 2, dhi = g.bc[2 * DIR + 1] == 2;
   // cell of the Dirichlet slice that continues this line
@@ -377,274 +350,6 @@ __device__ __forceinline__ bool uniform_nodes(const double* __restrict__ W, int6
       if (j != 2) same &= __double_as_longlong(W[m * nc + nd.c[j]]) == b;
   }
   return same;
-}
-
-// Outputs of a midpoint: M + N - 1 planes over the face grid of the direction --
-// the NC conservative flux slots, the N-1 alpha slots of G^-_{i+1/2} (planes
-// AL..M-1) and the N-1 alpha slots of G^+_{i+1/2} (planes M..M+N-2).
-// One midpoint t of direction DIR (t inside the face grid); lam = lambda_DIR.
-// lin: the midpoint is gated smooth -- the WENO-IS weights are replaced by the
-// linear weights d_k; everything else is unchanged.
-template <typename R, int N, int D, int DIR>
-__device__ __forceinline__ void face_body(int64_t t, const Nodes6& nd, const double* __restrict__ W,
-                                          const double* __restrict__ V, const double* __restrict__ AUX,
-                                          double* __restrict__ out, const DevGrid& g, const DevFluid& f,
-                                          const DevParams& pr, double lam, bool lin = false) {
-  using L = Lay<N, D>;
-  constexpr int M = L::M;
-  const int64_t nc = g.ncells;
-  const int64_t nf = face_count<DIR>(g);
-  const double* __restrict__ Cc = AUX;           // sound speed
-  const double* __restrict__ Rr = AUX + nc;      // mixture density
-  const double* __restrict__ RC2 = AUX + 2 * nc; // rho c^2
-
-  // node states i and i+1 (FP64)
-  double Vi[M], Vj[M], Wi[M], Wj[M];
-#pragma unroll
-  for (int m = 0; m < M; ++m) {
-    Vi[m] = V[m * nc + nd.c[2]];
-    Vj[m] = V[m * nc + nd.c[3]];
-    Wi[m] = W[m * nc + nd.c[2]];
-    Wj[m] = W[m * nc + nd.c[3]];
-  }
-
-  // first-order HLLC flux and u_* from the node states (Sec. 4.1.1), evaluated
-  // where it is used: the first-order scheme, and the flux limiter where it may act
-  FluxPack<N, D> H;
-  auto first_order = [&]() {
-    PrimState<double, N, D> a, b;
-#pragma unroll
-    for (int m = 0; m < M; ++m) {
-      a.V[m] = Vi[m];
-      b.V[m] = Vj[m];
-    }
-    double GH[M];
-    const double uH = hllc<double, N, D, DIR>(f, a, b, GH);
-#pragma unroll
-    for (int m = 0; m < L::NC; ++m) H.Gc[m] = GH[m];
-#pragma unroll
-    for (int k = 0; k < N - 1; ++k) {
-      H.gm[k] = GH[L::AL + k] - uH * Vi[L::AL + k];
-      H.gp[k] = GH[L::AL + k] - uH * Vj[L::AL + k];
-    }
-  };
-
-  FluxPack<N, D> G;
-  if (pr.scheme == 1) {
-    first_order();
-    G = H;
-  } else if (uniform_nodes<N, D>(W, nc, nd)) {
-    // six bit-identical node states: in exact arithmetic every step below returns
-    // the node's physical flux with zero alpha slots -- constants are reproduced
-    // by the interpolation (App. C), the HLLC flux of equal states is their flux
-    // (Sec. 4.1.1), the HCS weights sum to one, alpha u - u alpha = 0 (Eq. G_pm),
-    // and the node state is the limiters' own candidate (Sec. 4.3.2)
-    const double un = Vi[L::MOM + DIR], p = Vi[L::EN];
-#pragma unroll
-    for (int k = 0; k < N; ++k) G.Gc[k] = Wi[k] * un;
-#pragma unroll
-    for (int d = 0; d < D; ++d) G.Gc[L::MOM + d] = Wi[L::MOM + d] * un;
-    G.Gc[L::MOM + DIR] = G.Gc[L::MOM + DIR] + p;
-    G.Gc[L::EN] = (Wi[L::EN] + p) * un;
-#pragma unroll
-    for (int k = 0; k < N - 1; ++k) {
-      G.gm[k] = 0.0;
-      G.gp[k] = 0.0;
-    }
-  } else {
-    R p6[6], u6[6];
-#pragma unroll
-    for (int j = 0; j < 6; ++j) {
-      p6[j] = R(V[L::EN * nc + nd.c[j]]);
-      u6[j] = R(V[(L::MOM + DIR) * nc + nd.c[j]]);
-    }
-    // characteristic projection with the face-averaged state (App. D)
-    const R rhob = R(0.5) * (R(Rr[nd.c[2]]) + R(Rr[nd.c[3]]));
-    const R cb = R(0.5) * (R(Cc[nd.c[2]]) + R(Cc[nd.c[3]]));
-    const R inv_rc = quot(R(1), rhob * cb);
-    const R rc2b = rhob * cb * cb;
-    const R eps = R(pr.weno_eps);
-    R UL[M], UR[M];
-    R w6[6];
-#pragma unroll
-    for (int j = 0; j < 6; ++j) w6[j] = u6[j] - inv_rc * p6[j];
-    UL[0] = weno_sel<R>(lin, w6[0], w6[1], w6[2], w6[3], w6[4], eps);
-    UR[0] = weno_sel<R>(lin, w6[5], w6[4], w6[3], w6[2], w6[1], eps);
-#pragma unroll
-    for (int j = 0; j < 6; ++j) w6[j] = u6[j] + inv_rc * p6[j];
-    UL[M - 1] = weno_sel<R>(lin, w6[0], w6[1], w6[2], w6[3], w6[4], eps);
-    UR[M - 1] = weno_sel<R>(lin, w6[5], w6[4], w6[3], w6[2], w6[1], eps);
-    R arb[N];
-#pragma unroll
-    for (int k = 0; k < N; ++k) {
-#pragma unroll
-      for (int j = 0; j < 6; ++j) w6[j] = R(V[k * nc + nd.c[j]]);
-      arb[k] = R(0.5) * (w6[2] + w6[3]);
-      const R coef = quot(arb[k], rc2b);
-#pragma unroll
-      for (int j = 0; j < 6; ++j) w6[j] = w6[j] - coef * p6[j];
-      UL[1 + k] = weno_sel<R>(lin, w6[0], w6[1], w6[2], w6[3], w6[4], eps);
-      UR[1 + k] = weno_sel<R>(lin, w6[5], w6[4], w6[3], w6[2], w6[1], eps);
-    }
-    {
-      int t_ = 0;
-#pragma unroll
-      for (int d = 0; d < D; ++d) {
-        if (d == DIR) continue;
-#pragma unroll
-        for (int j = 0; j < 6; ++j) w6[j] = R(V[(L::MOM + d) * nc + nd.c[j]]);
-        UL[N + 1 + t_] = weno_sel<R>(lin, w6[0], w6[1], w6[2], w6[3], w6[4], eps);
-        UR[N + 1 + t_] = weno_sel<R>(lin, w6[5], w6[4], w6[3], w6[2], w6[1], eps);
-        ++t_;
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < N - 1; ++k) {
-#pragma unroll
-      for (int j = 0; j < 6; ++j) w6[j] = R(V[(L::AL + k) * nc + nd.c[j]]);
-      UL[N + D + k] = weno_sel<R>(lin, w6[0], w6[1], w6[2], w6[3], w6[4], eps);
-      UR[N + D + k] = weno_sel<R>(lin, w6[5], w6[4], w6[3], w6[2], w6[1], eps);
-    }
-    // back to primitive variables, V~ = R U~
-    PrimState<R, N, D> sl, sr;
-    {
-      R h[N];
-#pragma unroll
-      for (int k = 0; k < N; ++k) h[k] = quot(arb[k], R(2) * cb);
-      const R rc_2 = rhob * cb * R(0.5);
-#pragma unroll
-      for (int side = 0; side < 2; ++side) {
-        const R* U = side == 0 ? UL : UR;
-        R* Vt = side == 0 ? sl.V : sr.V;
-#pragma unroll
-        for (int k = 0; k < N; ++k) Vt[k] = (-h[k]) * U[0] + U[1 + k] + h[k] * U[M - 1];
-        Vt[L::MOM + DIR] = R(0.5) * U[0] + R(0.5) * U[M - 1];
-        int t_ = 0;
-#pragma unroll
-        for (int d = 0; d < D; ++d) {
-          if (d == DIR) continue;
-          Vt[L::MOM + d] = U[N + 1 + t_];
-          ++t_;
-        }
-        Vt[L::EN] = (-rc_2) * U[0] + rc_2 * U[M - 1];
-#pragma unroll
-        for (int k = 0; k < N - 1; ++k) Vt[L::AL + k] = U[N + D + k];
-      }
-    }
-    // positivity-preserving interpolation limiter (Sec. 4.3.2)
-    if (pr.limiters) {
-      interp_limit<R, N, D>(sl.V, Vi, RC2[nd.c[2]], f, pr);
-      interp_limit<R, N, D>(sr.V, Vj, RC2[nd.c[3]], f, pr);
-    }
-    // high-order midpoint flux G~ and velocity u~
-    R Gt[M];
-    const R ut = hllc<R, N, D, DIR>(f, sl, sr, Gt);
-    // explicit HCS reconstruction (Eqs. reconstructed_G, reconstructed_vel)
-    constexpr double psi = 256.0 / 175.0;
-    constexpr double a1 = 75.0 * psi / 128.0 - 37.0 / 60.0;
-    constexpr double a2 = 25.0 * psi / 256.0 - 2.0 / 15.0;
-    constexpr double a3 = 3.0 * psi / 256.0 - 1.0 / 60.0;
-    // shock sensor (Sec. 4.3.1) on rho and p
-    R sig = R(0);
-    if (pr.blend) {
-      R r6[6];
-#pragma unroll
-      for (int j = 0; j < 6; ++j) r6[j] = R(Rr[nd.c[j]]);
-      auto half = [](R a, R b, R c, R d, R e) -> R {
-        const R num = fabs(R(16) * b - a - R(30) * c + R(16) * d - e);
-        const R den = fabs(a + R(16) * b + R(30) * c + R(16) * d + e);
-        return den == R(0) ? R(0) : quot(num, den);
-      };
-      const R sr_ = R(0.5) * (half(r6[1], r6[2], r6[3], r6[4], r6[5]) + half(r6[0], r6[1], r6[2], r6[3], r6[4]));
-      const R sp_ = R(0.5) * (half(p6[1], p6[2], p6[3], p6[4], p6[5]) + half(p6[0], p6[1], p6[2], p6[3], p6[4]));
-      const R prod = sr_ * sp_;
-      R pw = prod;
-      for (int e = 1; e < pr.qexp; ++e) pw = pw * prod;
-      sig = tanh_r(R(pr.Cs) * pw);
-    }
-    const R one_m = R(1) - sig;
-    const R uhcs = R(psi) * ut - R(a1) * (u6[2] + u6[3]) + R(a2) * (u6[1] + u6[4]) - R(a3) * (u6[0] + u6[5]);
-    const double uhat = (double)(sig * ut + one_m * uhcs);
-    // node fluxes G of the flux-source form at the six nodes, slot by slot
-#pragma unroll
-    for (int m = 0; m < M; ++m) {
-      R Gn[6];
-#pragma unroll
-      for (int j = 0; j < 6; ++j) {
-        const double un = (double)u6[j];
-        double v;
-        if (m < L::MOM) {
-          v = W[m * nc + nd.c[j]] * un;
-        } else if (m < L::EN) {
-          v = W[m * nc + nd.c[j]] * un + ((m - L::MOM) == DIR ? (double)p6[j] : 0.0);
-        } else if (m == L::EN) {
-          v = (W[m * nc + nd.c[j]] + (double)p6[j]) * un;
-        } else {
-          v = W[m * nc + nd.c[j]] * un;
-        }
-        Gn[j] = R(v);
-      }
-      const R ghcs = R(psi) * Gt[m] - R(a1) * (Gn[2] + Gn[3]) + R(a2) * (Gn[1] + Gn[4]) - R(a3) * (Gn[0] + Gn[5]);
-      const double gh = (double)(sig * Gt[m] + one_m * ghcs);
-      if (m < L::NC) {
-        G.Gc[m] = gh;
-      } else {
-        // quasi-conservative alpha slots (Eq. G_pm, high-order form)
-        G.gm[m - L::AL] = gh - uhat * Vi[m];
-        G.gp[m - L::AL] = gh - uhat * Vj[m];
-      }
-    }
-
-    if (pr.limiters) {
-      double Fi[L::NC], Fj[L::NC];
-      node_flux<N, D, DIR>(Wi, Vi, Fi);
-      node_flux<N, D, DIR>(Wj, Vj, Fj);
-      if (!flux_limit_noop<N, D>(Wi, Wj, Fi, Fj, lam, G, f, pr)) {
-        first_order();
-        flux_limit<N, D>(Wi, Wj, Fi, Fj, lam, G, H, f, pr);
-      }
-    }
-  }
-#pragma unroll
-  for (int m = 0; m < L::NC; ++m) out[m * nf + t] = G.Gc[m];
-#pragma unroll
-  for (int k = 0; k < N - 1; ++k) {
-    out[(L::AL + k) * nf + t] = G.gm[k];
-    out[(M + k) * nf + t] = G.gp[k];
-  }
-}
-
-// Midpoint of this thread in a sweep of a 2D or 3D grid launched over
-// lane_patch_grid blocks: a block takes 32 x 4 midpoints (along x, then y; z
-// from the block index) and each warp an 8 x 4 patch of them. Uniform and
-// non-uniform stencils come in bands a few midpoints wide along the material
-// interfaces and wave fronts; a warp of 32 midpoints along one row crossing such
-// a band holds a few non-uniform lanes, which run the whole midpoint body, and
-// an 8 x 4 patch holds more of the band and fewer idle lanes. Past the end of
-// the grid: the midpoint count (no midpoint).
-template <int DIR>
-__device__ __forceinline__ int64_t lane_patch_midpoint(const DevGrid& g) {
-  static_assert(kFaceThreads == 128, "four warps per block");
-  const int64_t f0 = g.n[0] + (DIR == 0), f1 = g.n[1] + (DIR == 1), f2 = g.n[2] + (DIR == 2);
-  const int64_t nbx = (f0 + 31) / 32, nby = (f1 + 3) / 4, b = blockIdx.x;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t i0 = (b % nbx) * 32 + w * 8 + (lane & 7);
-  const int64_t i1 = ((b / nbx) % nby) * 4 + (lane >> 3);
-  const int64_t i2 = b / (nbx * nby);
-  if (i0 >= f0 || i1 >= f1 || i2 >= f2) return f0 * f1 * f2;
-  return (i2 * f1 + i1) * f0 + i0;
-}
-
-template <typename R, int N, int D, int DIR>
-__global__ void __launch_bounds__(kFaceThreads)
-    k_face(const double* __restrict__ W, const double* __restrict__ V, const double* __restrict__ AUX,
-           double* __restrict__ out, DevGrid g, DevFluid f, DevParams pr, const StepState* __restrict__ st,
-           const uint8_t* __restrict__ gate) {
-  const int64_t t = D >= 2 ? lane_patch_midpoint<DIR>(g) : (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  Nodes6 nd;
-  if (!face_nodes<DIR>(g, t, nd)) return;
-  const bool lin = gate != nullptr && gate[t] != 0;
-  face_body<R, N, D, DIR>(t, nd, W, V, AUX, out, g, f, pr, st->lam[DIR], lin);
 }
 
 // ---------------------------------------------------------------- thermal relaxation (Sec. 4.2)
@@ -796,9 +501,9 @@ __device__ __forceinline__ void fast_combine(int64_t c, const double* Wn, const 
   using L = Lay<N, D>;
   constexpr int M = L::M;
   const int64_t nc = g.ncells;
-  const int64_t i0 = c % g.n[0];
-  const int64_t r = c / g.n[0];
-  const int64_t i1 = r % g.n[1], i2 = r / g.n[1];
+  int64_t ijk[3];
+  cell_index(g, c, ijk);
+  const int64_t i0 = ijk[0], i1 = ijk[1], i2 = ijk[2];
   double acc[M];
 #pragma unroll
   for (int m = 0; m < M; ++m) acc[m] = Ws[m];
@@ -841,9 +546,9 @@ __device__ __forceinline__ bool faces_unchanged(int64_t c, const double* __restr
                                                 const DevGrid& g) {
   using L = Lay<N, D>;
   constexpr int M = L::M;
-  const int64_t i0 = c % g.n[0];
-  const int64_t r = c / g.n[0];
-  const int64_t i1 = r % g.n[1], i2 = r / g.n[1];
+  int64_t ijk[3];
+  cell_index(g, c, ijk);
+  const int64_t i0 = ijk[0], i1 = ijk[1], i2 = ijk[2];
   auto bits = [](double x) { return (unsigned long long)__double_as_longlong(x); };
   auto same_finite = [&](double x, double y) {
     const unsigned long long bx = bits(x);
@@ -892,25 +597,44 @@ __device__ __forceinline__ bool stage_keeps_cell(int64_t c, const double* Wn, co
   return same;
 }
 
+// Flux of a uniform face from the state of one of its cells: the node's physical
+// flux F^d (NC conservative slots; the alpha slots are zero).
+template <int N, int D>
+__device__ __forceinline__ void uniform_flux64(int64_t c, int d, const double* __restrict__ W,
+                                               const double* __restrict__ V, int64_t nc, double* G) {
+  using L = Lay<N, D>;
+  const double un = V[(L::MOM + d) * nc + c], p = V[L::EN * nc + c];
+#pragma unroll
+  for (int m = 0; m < L::EN; ++m) {
+    G[m] = prod(W[m * nc + c], un);
+    if (m == L::MOM + d) G[m] = G[m] + p;
+  }
+  G[L::EN] = prod(W[L::EN * nc + c] + p, un);
+}
+
 // RHS_i = -sum_d (G^{d,-}_{i+1/2} - G^{d,+}_{i-1/2}) / dx_d (Eq. semi_W_G_pm_eqn),
 // then W_out = a W^n + b (W_src + dt RHS) (SSP-RK stage in Shu-Osher form),
 // optionally followed by the thermal relaxation and the admissibility count.
 // MODE 1 writes RHS instead of the combination. In-place (W_out == W_src or W^n)
 // is allowed: each thread reads its own cell before writing it.
 // FAST (precision form): reciprocal of dx and of rho instead of divisions.
+// uni (nullable): the cell's uniform faces (k_mark), whose flux is formed here
+// from W_src and its primitives V and not read.
 // One interior cell c < nint (Dirichlet slices keep their state).
 template <int N, int D, int MODE, bool FAST = false>
 __device__ __forceinline__ void update_body(int64_t c, const double* Wn, const double* Wsrc, double* Wout,
                                             const double* __restrict__ F0, const double* __restrict__ F1,
                                             const double* __restrict__ F2, const DevGrid& g, const DevFluid& f,
                                             StepState* st, double dt, double a, double b, int relax, int count,
-                                            uint8_t* __restrict__ same = nullptr) {
+                                            uint8_t* __restrict__ same = nullptr,
+                                            const uint8_t* __restrict__ uni = nullptr,
+                                            const double* __restrict__ V = nullptr) {
   using L = Lay<N, D>;
   constexpr int M = L::M;
   const int64_t nc = g.ncells;
-  const int64_t i0 = c % g.n[0];
-  const int64_t r = c / g.n[0];
-  const int64_t i1 = r % g.n[1], i2 = r / g.n[1];
+  int64_t ijk[3];
+  cell_index(g, c, ijk);
+  const int64_t i0 = ijk[0], i1 = ijk[1], i2 = ijk[2];
   double Ws[M];
 #pragma unroll
   for (int m = 0; m < M; ++m) Ws[m] = Wsrc[m * nc + c];
@@ -936,12 +660,17 @@ __device__ __forceinline__ void update_body(int64_t c, const double* Wn, const d
   double rhs[M];
 #pragma unroll
   for (int m = 0; m < M; ++m) rhs[m] = 0.0;
-  // Faces all bit-equal: every difference is +0, its quotient by dx too, and
-  // the sums below would leave rhs at +0 -- the divisions are left out.
-  const bool flat = faces_unchanged<N, D>(c, F0, F1, F2, g);
+  const unsigned ub = uni ? uni[c] : 0u;
+  // flat: every flux difference is exactly +0 (the two faces' values bit-equal and finite)
+  bool flat = true;
+  auto differ = [](double x, double y) {
+    const long long bx = __double_as_longlong(x);
+    return (bx != __double_as_longlong(y)) | (((uint32_t)(bx >> 32) & 0x7ff00000u) == 0x7ff00000u);
+  };
 #pragma unroll
   for (int d = 0; d < D; ++d) {
-    if (flat) break;
+    const unsigned u = ub >> (2 * d) & 3u;
+    if (u == 3u) continue;  // both faces uniform: the cell's own flux twice, and rhs - 0 / dx = rhs
     const double* F = d == 0 ? F0 : (d == 1 ? F1 : F2);
     const int64_t f0 = g.n[0] + (d == 0), f1 = g.n[1] + (d == 1), f2 = g.n[2] + (d == 2);
     const int64_t nf = f0 * f1 * f2;
@@ -952,17 +681,17 @@ __device__ __forceinline__ void update_body(int64_t c, const double* Wn, const d
     // df / dx and df * (1/dx) are the same correctly rounded number: the product
     // then stands for the quotient at no change of any result
     const bool scale = FAST || (__double_as_longlong(dx) & 0xFFFFFFFFFFFFFll) == 0;
+    double own[L::NC];
+    if (u) uniform_flux64<N, D>(c, d, Wsrc, V, nc, own);
     // G^-_{i+1/2} - G^+_{i-1/2}: the alpha slots of the right face use alpha_i
     // (planes AL..), those of the left face alpha_i as its right neighbour (planes M..)
 #pragma unroll
-    for (int m = 0; m < L::NC; ++m) {
-      const double df = F[m * nf + fr] - F[m * nf + fl];
-      rhs[m] = rhs[m] - (scale ? df * idx : quot(df, dx));
-    }
-#pragma unroll
-    for (int k = 0; k < N - 1; ++k) {
-      const int m = L::AL + k;
-      const double df = F[m * nf + fr] - F[(M + k) * nf + fl];
+    for (int m = 0; m < M; ++m) {
+      const double fo = m < L::NC ? own[m < L::NC ? m : 0] : 0.0;
+      const double vl = (u & 1u) ? fo : F[(m < L::NC ? m : M + m - L::AL) * nf + fl];
+      const double vr = (u & 2u) ? fo : F[m * nf + fr];
+      flat = flat & !differ(vl, vr);
+      const double df = vr - vl;
       rhs[m] = rhs[m] - (scale ? df * idx : quot(df, dx));
     }
   }
@@ -1011,11 +740,12 @@ template <int N, int D, int MODE, bool FAST = false>
 __global__ void __launch_bounds__(kCellThreads)
     k_update(const double* Wn, const double* Wsrc, double* Wout, const double* __restrict__ F0,
              const double* __restrict__ F1, const double* __restrict__ F2, DevGrid g, DevFluid f,
-             StepState* st, double a, double b, int relax, int count, uint8_t* __restrict__ same = nullptr) {
+             StepState* st, double a, double b, int relax, int count, uint8_t* __restrict__ same = nullptr,
+             const uint8_t* __restrict__ uni = nullptr, const double* __restrict__ V = nullptr) {
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= g.nint) return;
   update_body<N, D, MODE, FAST>(c, Wn, Wsrc, Wout, F0, F1, F2, g, f, st, MODE == 1 ? 0.0 : st->dt, a, b, relax,
-                                count, same);
+                                count, same, uni, V);
 }
 
 }  // namespace hrm

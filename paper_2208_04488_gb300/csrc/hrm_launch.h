@@ -48,6 +48,9 @@ struct GateArgs {
   const float* R32 = nullptr;
   float zthr = 0.f;
   uint8_t* out_gate = nullptr;
+  // FP64 form: the midpoints to sweep and their counters (SweepLists of the direction)
+  const uint32_t* list = nullptr;
+  uint32_t* list_cnt = nullptr;
 };
 
 // Stream of the deferred-midpoint kernel: gate.side (forked from s after the
@@ -73,10 +76,11 @@ struct FaceKernels {
                   const GateArgs& gate, cudaStream_t);
   // mode 0: RK combination, mode 1: write the RHS; fast: precision-form variant;
   // same (nullable; FP64 RK combination): per interior cell, set to 1 where
-  // W_out equals W_src bit for bit, else 0
+  // W_out equals W_src bit for bit, else 0; uni (nullable; FP64 RK combination):
+  // the cells' uniform faces, whose fluxes are formed from W_src and V
   void (*update)(int mode, int fast, const double* Wn, const double* Wsrc, double* Wout, const double* F0,
                  const double* F1, const double* F2, const DevGrid&, const DevFluid&, StepState*, double a,
-                 double b, int relax, int count, uint8_t* same, cudaStream_t);
+                 double b, int relax, int count, uint8_t* same, const uint8_t* uni, const double* V, cudaStream_t);
 };
 
 const CellKernels* cell_kernels(int N, int D);
@@ -155,11 +159,20 @@ inline unsigned patch_grid(const DevGrid& g, int dir) {
   return (unsigned)(dir == 1 ? nbx * ((f1 + 3) / 4) * f2 : nbx * f1 * ((f2 + 3) / 4));
 }
 
-// Blocks of kFaceThreads covering the midpoints of direction dir of a 2D or 3D
-// grid in the layout of lane_patch_midpoint (32 x 4 midpoints per block).
-inline unsigned lane_patch_grid(const DevGrid& g, int dir) {
-  const long long f0 = g.n[0] + (dir == 0), f1 = g.n[1] + (dir == 1), f2 = g.n[2] + (dir == 2);
-  return (unsigned)(((f0 + 31) / 32) * ((f1 + 3) / 4) * f2);
+// Uniform faces and the lists of the other midpoints of a stage's source state,
+// FP64 form (hrm_sweep.cuh): two launches. all: every midpoint is listed.
+void launch_mark64(int N, int D, const double* W, const double* V, const DevGrid& g, const SweepLists& lists, int all,
+                   cudaStream_t s);
+
+// Blocks of kFaceThreads of a list-driven sweep: what is resident at per_sm blocks
+// on each SM, or fewer where the whole midpoint grid needs no more.
+inline unsigned list_grid(const DevGrid& g, int dir, int per_sm) {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const long long f = (g.n[0] + (dir == 0)) * (g.n[1] + (dir == 1)) * (g.n[2] + (dir == 2));
+  const long long all = (f + 127) / 128, fit = (long long)(sms > 0 ? sms : 1) * per_sm;
+  return (unsigned)(all < fit ? all : fit);
 }
 
 // Smallest float not below x (thresholds of the FP32 screens).

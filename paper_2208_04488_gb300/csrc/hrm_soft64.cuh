@@ -119,6 +119,8 @@ HRM_SOFT double mul_in(double a, double b) {
 // and one comparison completes the 54-bit quotient. A quotient of two 53-bit
 // numbers never lies halfway between two others, so the bit below the last
 // decides the rounding.
+// EXP: the result times 2^EXP (exponents are added up in the upper word anyway).
+template <int EXP = 0>
 HRM_SOFT double div_in(double a, double b) {
   const uint32_t ah = hi_of(a), al = lo_of(a), bh = hi_of(b), bl = lo_of(b);
   const uint64_t A = (uint64_t)((ah & 0xfffffu) | kOne) << 32 | al;
@@ -139,7 +141,7 @@ HRM_SOFT double div_in(double a, double b) {
   uint64_t q = ((uint64_t)d0 << 31) + ((uint64_t)d1 << 12) + d2 + (R >= B ? 1u : 0u);
   const uint32_t one = (uint32_t)(q >> 54);  // A >= B
   q = (q + 1u + one) >> (1u + one);
-  const uint32_t ex = (ah & 0xfff00000u) - (bh & 0xfff00000u) + (1021u << 20) + (one << 20);
+  const uint32_t ex = (ah & 0xfff00000u) - (bh & 0xfff00000u) + ((uint32_t)(1021 + EXP) << 20) + (one << 20);
   return pack((uint32_t)(q >> 32) + ex, (uint32_t)q);
 }
 
@@ -194,6 +196,22 @@ HRM_SOFT double mul(double a, double b) {
       ((((hi_of(a) & ~kSign) | lo_of(a)) == 0u) | (((hi_of(b) & ~kSign) | lo_of(b)) == 0u)))
     return pack((hi_of(a) ^ hi_of(b)) & kSign, 0u);
   return a * b;
+}
+
+// a 2^EXP, EXP small: the exponent field of a normal number moves.
+template <int EXP>
+HRM_SOFT double scale(double a) {
+  const uint32_t h = hi_of(a), e = h & kExp;
+  if (e - (16u << 20) < (2000u << 20)) return pack(h + ((uint32_t)EXP << 20), lo_of(a));
+  if (((h & ~kSign) | lo_of(a)) == 0u) return a;
+  return a * (EXP < 0 ? 1.0 / (double)(1 << (EXP < 0 ? -EXP : 0)) : (double)(1 << (EXP > 0 ? EXP : 0)));
+}
+
+// Whether x is zero or of a magnitude within [2^LO, 2^HI).
+template <int LO, int HI>
+HRM_SOFT bool within(double x) {
+  const uint32_t h = hi_of(x);
+  return ((h & kExp) - ((uint32_t)(1023 + LO) << 20) < ((uint32_t)(HI - LO) << 20)) | (((h & ~kSign) | lo_of(x)) == 0u);
 }
 
 // sqrt(a) for any operand, likewise.

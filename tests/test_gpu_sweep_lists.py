@@ -1,0 +1,65 @@
+"""List-driven sweeps: uniform faces are found by comparing neighbouring cells and
+only the other midpoints run the midpoint body. On grids around the sizes of the
+blocks and warps that build the lists, in every dimension and with every kind of
+side, a uniform state with a few disturbed cells -- the corners, the middle, or
+none -- must step exactly as the oracle, which tests every midpoint's six nodes."""
+import numpy as np
+import pytest
+
+from paper_2208_04488_gb300 import problems as P
+
+pytestmark = pytest.mark.gpu
+
+GRIDS = [[3], [7], [255], [256], [257], [33, 3], [5, 64], [257, 4], [3, 4, 5], [9, 3, 8]]
+
+
+@pytest.fixture(scope="module")
+def hrm():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2208_04488_gb300 import build, hrm as H
+    build.build()
+    return H
+
+
+def disturbed(n, bc, where, N=3):
+    """A uniform moving state with disturbed cells (and a boundary state of its own on Dirichlet sides)."""
+    D, cells = len(n), int(np.prod(n))
+    fl = [P.BENCH_WATER, P.BENCH_AIR, P.BENCH_HELIUM][:N]
+    gamma, pinf, cv, q = P._species(fl)
+    one = np.ones(cells)
+    prim = P._assemble(N, D, [0.3 * one, 0.5 * one][:N - 1], [(20.0 - 15.0 * d) * one for d in range(D)], 1.2e5 * one, 310.0 * one)
+    at = {"none": [], "first": [0], "last": [cells - 1], "middle": [cells // 2], "ends": [0, cells // 3, cells - 1]}[where]
+    for i, c in enumerate(at):
+        prim[0, c] += 0.05 * (i + 1)
+        prim[N - 1 + (i % D), c] += 3.0
+        prim[N + D - 1, c] *= 1.01
+    pr = P.Problem("disturbed", gamma, pinf, cv, q, list(n), [0.0] * D, [1.0 + 0.3 * d for d in range(D)], [bc] * (2 * D), prim,
+                   cfl=0.4)
+    if bc == 2:  # half of the sides continue the interior state, the others differ
+        for b in range(2 * D):
+            ns = cells // n[b // 2]
+            s = P._assemble(N, D, [np.full(ns, 0.3), np.full(ns, 0.5)][:N - 1],
+                            [np.full(ns, 20.0 - 15.0 * d) for d in range(D)], np.full(ns, 1.2e5), np.full(ns, 310.0))
+            if b % 2:
+                s[N + D, : (ns + 1) // 2] += 5.0
+            pr.boundary[b] = s
+    return pr
+
+
+@pytest.mark.parametrize("n", GRIDS, ids=lambda n: "x".join(map(str, n)))
+@pytest.mark.parametrize("bc", [0, 1, 2], ids=["transmissive", "periodic", "dirichlet"])
+@pytest.mark.parametrize("where", ["none", "first", "last", "middle", "ends"])
+def test_step_and_rhs_equal_the_oracle(hrm, orc, n, bc, where):
+    import torch
+    pr = disturbed(n, bc, where)
+    f, g, W = orc.setup(pr)
+    s = hrm.Solver.from_problem(pr, params=hrm.params_default(cfl=0.4, check=0))
+    dt, _ = orc.dt(f, g, W, 0.4)
+    lam = orc.lambdas(f, g, W, dt)
+    rhs = s.rhs(lam, torch.empty((pr.M, pr.ncells), dtype=torch.float64, device="cuda")).cpu().numpy()
+    np.testing.assert_array_equal(rhs, orc.rhs(f, orc.make_params(), g, W, lam))
+    s.step(dt, 3)
+    np.testing.assert_array_equal(s.get(hrm.FIELD_W), orc.step(f, orc.make_params(), g, W, dt, 3))
+    s.close()
