@@ -48,9 +48,9 @@ struct hrm_ctx {
   mlp::GateBlob* blob = nullptr;   // learned gate weights (hrm_set_detector)
   uint8_t* gate[3] = {nullptr, nullptr, nullptr};  // gate bytes per direction (midpoint grids)
   uint8_t* same = nullptr;         // FP64 form: per cell, the last update left W bit for bit as its source
-  SweepLists lists;                // FP64 form: uniform faces and the midpoints to sweep (hrm_sweep.cuh)
+  SweepLists lists;                // uniform faces and the midpoints to sweep (hrm_sweep.cuh)
   uint32_t* defer = nullptr;       // precision form: per direction, a worklist of deferred midpoints and its counter
-  int64_t defer_cap = 0;           // worklist entries (the largest midpoint grid; 0: no worklist)
+  int64_t defer_cap = 0;           // worklist entries per direction (the largest midpoint grid)
   hrm_alloc_fn alloc = nullptr;    // device memory source (hrm_set_allocator at creation; NULL: cudaMalloc)
   hrm_free_fn dealloc = nullptr;
   void* alloc_user = nullptr;
@@ -245,7 +245,7 @@ float* r32_target(hrm_ctx* c) { return c->params.learned == 1 ? c->R32 : nullptr
 // without the FP64 fallbacks inline), except with the first-order scheme or the
 // screens off.
 bool defer_sweep(const hrm_ctx* c) {
-  return c->params.precision == HRM_FP32 && c->defer && c->params.scheme == HRM_SCHEME_WCNS && c->params.screen;
+  return c->params.precision == HRM_FP32 && c->params.scheme == HRM_SCHEME_WCNS && c->params.screen;
 }
 
 // Kernels one sweep launches.
@@ -254,14 +254,11 @@ int sweep_kernels(const hrm_ctx* c) { return defer_sweep(c) ? 2 : 1; }
 GateArgs gate_of(const hrm_ctx* c, int d) {
   GateArgs g;
   if (defer_sweep(c)) {
-    g.defer_list = c->defer + (size_t)d * (size_t)(c->defer_cap + 1);
-    g.defer_count = g.defer_list + c->defer_cap;
+    g.defer_list = c->defer + (size_t)d * (size_t)c->defer_cap;
   }
   if (c->params.learned) g.fixed = c->gate[d];
-  if (c->params.precision == HRM_FP64) {
-    g.list = c->lists.list[d];
-    g.list_cnt = c->lists.cnt + kSweepCounts * d;
-  }
+  g.list = c->lists.list[d];
+  g.list_cnt = c->lists.cnt + kSweepCounts * d;
   if (c->params.learned == 1 && defer_sweep(c)) {  // the network inside the sweep
     g.net = c->blob;
     g.R32 = c->R32;
@@ -271,13 +268,17 @@ GateArgs gate_of(const hrm_ctx* c, int d) {
   return g;
 }
 
-// FP64 form: uniform faces and the lists of the other midpoints of Wsrc; full: the
-// uniform faces' fluxes into the flux planes as well.
+// Uniform faces and the lists of the other midpoints of Wsrc (its primitives or
+// FP32 planes are up to date); full: the uniform faces' fluxes into the flux
+// planes as well.
 int enqueue_mark(hrm_ctx* c, cudaStream_t s, const double* Wsrc, bool full) {
-  if (c->params.precision != HRM_FP64) return 0;
   SweepLists l = c->lists;
-  for (int d = 0; d < c->D; ++d) l.F[d] = full ? c->F[d] : nullptr;
-  launch_mark64(c->N, c->D, Wsrc, c->V, c->dg, l, c->params.scheme == HRM_SCHEME_HLLC1, s);
+  const bool fp32 = c->params.precision == HRM_FP32;
+  for (int d = 0; d < c->D; ++d) {
+    l.F[d] = full ? c->F[d] : nullptr;
+    l.gate[d] = c->params.learned == 1 && defer_sweep(c) ? c->gate[d] : nullptr;
+  }
+  launch_mark(c->N, c->D, Wsrc, c->V, fp32 ? c->P32 : nullptr, c->dg, l, c->params.scheme == HRM_SCHEME_HLLC1, s);
   return 2;
 }
 
@@ -331,7 +332,7 @@ int enqueue_stage(hrm_ctx* c, cudaStream_t s, const double* Wsrc, double* Wout, 
       });
       ++k;
     }
-  k += enqueue_mark(c, s, Wsrc, false);
+  k += enqueue_mark(c, s, Wsrc, c->params.precision == HRM_FP32 && !fuse_next);
   // the sweeps: independent (each reads the primitives and writes its own flux
   // planes), so directions d > 0 run on their own streams beside direction 0
   const bool fork = c->D > 1 && c->par[1];
@@ -365,7 +366,7 @@ int enqueue_stage(hrm_ctx* c, cudaStream_t s, const double* Wsrc, double* Wout, 
   traced(c, s, HRM_KERNEL_UPDATE, [&] {
     if (fuse_next)
       launch_update32p(c->N, c->D, c->Wn, Wsrc, Wout, c->F[0], c->F[1], c->F[2], c->dg, c->fl, c->st, a, b, relax,
-                       count, c->P32, r32_target(c), s, tau_next ? 1 : 0);
+                       count, c->P32, r32_target(c), c->lists.uni, s, tau_next ? 1 : 0);
     else
       c->fk->update(0, c->params.precision == HRM_FP32, c->Wn, Wsrc, Wout, c->F[0], c->F[1], c->F[2], c->dg,
                     c->fl, c->st, a, b, relax, count, same_out ? same : nullptr,
@@ -772,22 +773,13 @@ hrm_status hrm_create(hrm_ctx** out, const hrm_grid* grid, int32_t N, const doub
   for (int d = 0; d < D; ++d)
     if ((s = cuda_check(c, ctx_malloc(c, &c->lists.list[d], sizeof(uint32_t) * (size_t)face_total(c->dg, d)), "alloc midpoint list")))
       return bail(s);
-  // worklist of the precision form's deferred midpoints (32-bit entries; none
-  // beyond 2^32 - 1 midpoints, where the sweep keeps its fallbacks inline)
-  if (c->defer_cap < (int64_t)0xffffffffll) {
-    if ((s = cuda_check(c, ctx_malloc(c, &c->defer, sizeof(uint32_t) * (size_t)D * (size_t)(c->defer_cap + 1)),
-                        "alloc worklist")))
-      return bail(s);
-    for (int d = 0; d < D; ++d) {
-      if ((s = cuda_check(c, cudaStreamCreateWithFlags(&c->side[d], cudaStreamNonBlocking), "side stream")))
-        return bail(s);
-      if ((s = cuda_check(c, cudaEventCreateWithFlags(&c->ev_fast[d], cudaEventDisableTiming), "event")))
-        return bail(s);
-      if ((s = cuda_check(c, cudaEventCreateWithFlags(&c->ev_fix[d], cudaEventDisableTiming), "event")))
-        return bail(s);
-    }
-  } else {
-    c->defer_cap = 0;
+  // worklist of the precision form's deferred midpoints
+  if ((s = cuda_check(c, ctx_malloc(c, &c->defer, sizeof(uint32_t) * (size_t)D * (size_t)c->defer_cap), "alloc worklist")))
+    return bail(s);
+  for (int d = 0; d < D; ++d) {
+    if ((s = cuda_check(c, cudaStreamCreateWithFlags(&c->side[d], cudaStreamNonBlocking), "side stream"))) return bail(s);
+    if ((s = cuda_check(c, cudaEventCreateWithFlags(&c->ev_fast[d], cudaEventDisableTiming), "event"))) return bail(s);
+    if ((s = cuda_check(c, cudaEventCreateWithFlags(&c->ev_fix[d], cudaEventDisableTiming), "event"))) return bail(s);
   }
   if (D > 1) {
     if ((s = cuda_check(c, cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming), "event"))) return bail(s);

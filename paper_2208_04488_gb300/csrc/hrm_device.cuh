@@ -96,8 +96,8 @@ __device__ __forceinline__ void cell_index(const DevGrid& g, int64_t c, int64_t*
 
 // Work of the list-driven sweeps (hrm_sweep.cuh): one byte per cell each for eq
 // and uni, a list of midpoints per direction with kSweepCounts counters (entries,
-// entries taken); F: the flux planes where the uniform faces' fluxes are wanted
-// as well.
+// groups of 32 taken, deferred midpoints); F: the flux planes where the uniform
+// faces' fluxes are wanted as well; gate: the gate bytes where they are.
 constexpr int kSweepCounts = 4, kSweepCounters = 3 * kSweepCounts;
 struct SweepLists {
   uint8_t* eq = nullptr;
@@ -105,7 +105,20 @@ struct SweepLists {
   uint32_t* list[3] = {nullptr, nullptr, nullptr};
   uint32_t* cnt = nullptr;
   double* F[3] = {nullptr, nullptr, nullptr};
+  uint8_t* gate[3] = {nullptr, nullptr, nullptr};
 };
+
+// Next group of 32 entries of a list for this warp (every lane calls it): the
+// entry of this lane, or an index past the end. False when the list is done.
+__device__ __forceinline__ bool next_entries(uint32_t* __restrict__ cnt, uint32_t n, uint32_t& i) {
+  const int lane = threadIdx.x & 31;
+  uint32_t k = 0;
+  __syncwarp();
+  if (lane == 0) k = atomicAdd(&cnt[1], 1u);
+  k = __shfl_sync(0xffffffffu, k, 0);
+  i = k * 32u + (uint32_t)lane;
+  return k < n / 32u + (n % 32u ? 1u : 0u);
+}
 
 struct DevParams {
   int32_t limiters, blend, scheme, qexp;
@@ -172,16 +185,6 @@ struct StepState {
   int wn_relaxed;  // nonzero: every interior cell of W^n came out of the form's relaxation (set by the host)
   int planes_tau;  // nonzero: the FP32 planes and tau_bits already hold W^n's (set by the host)
 };
-
-// Whether the midpoints of direction dir go to blocks in patches of 32 along x
-// by 4 along dir (one warp per row), so that a block's four warps read 9 rows
-// of nodes instead of 24 and share them in L1: always for z (z neighbours lie a
-// whole plane apart); for y on rows of at most 1024 cells (measured: the FP32
-// step 1.2 % faster at 1024 x 512, 1.6 % slower at 2048 x 1024, where the
-// linear layout's concurrently running blocks already share the rows in L2).
-__host__ __device__ inline bool patched(const DevGrid& g, int dir) {
-  return dir == 2 || (dir == 1 && g.n[0] <= 1024);
-}
 
 // ---------------------------------------------------------------- small helpers
 

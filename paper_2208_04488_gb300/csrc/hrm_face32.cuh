@@ -483,36 +483,6 @@ __device__ __forceinline__ bool uniform_stencil(const float* __restrict__ P32, i
   return same;
 }
 
-// Midpoint t of a uniform stencil: the node's physical flux from the
-// conservative planes (the HCS node-flux expression at node i), zero alpha slots.
-template <int N, int D, int DIR>
-__device__ __forceinline__ void uniform_flux(int64_t t, const Nodes6& nd, const float* __restrict__ P32,
-                                             double* __restrict__ out, const DevGrid& g) {
-  using L = Lay<N, D>;
-  using Q = P32Lay<N, D>;
-  constexpr int M = L::M;
-  const int64_t nc = g.ncells;
-  const int64_t nf = face_count<DIR>(g);
-  auto ld = [&](int plane) -> float { return P32[(int64_t)plane * nc + nd.c[2]]; };
-  const float un = ld(L::MOM + DIR), pn = ld(L::EN);
-#pragma unroll
-  for (int m = 0; m < L::NC; ++m) {
-    float v;
-    if (m < L::MOM)
-      v = ld(m) * un;
-    else if (m < L::EN)
-      v = ld(Q::MOM + (m - L::MOM)) * un + ((m - L::MOM) == DIR ? pn : 0.f);
-    else
-      v = (ld(Q::E) + pn) * un;
-    out[m * nf + t] = widen_f32(v);
-  }
-#pragma unroll
-  for (int k = 0; k < N - 1; ++k) {
-    out[(L::AL + k) * nf + t] = 0.0;
-    out[(M + k) * nf + t] = 0.0;
-  }
-}
-
 // Appends index t to a worklist where `need` (all lanes of the warp call it;
 // warp-aggregated: one atomic per warp; order not significant).
 __device__ __forceinline__ void defer_push(bool need, int64_t t, uint32_t* __restrict__ list,
@@ -539,7 +509,7 @@ __device__ __forceinline__ void update32p_cell(int64_t c, const double* Wn, cons
                                                const double* __restrict__ F2, const DevGrid& g, const DevFluid& f,
                                                StepState* st, double a, double b, int relax, int count,
                                                float* __restrict__ P32, float* __restrict__ R32,
-                                               double* s = nullptr) {
+                                               double* s = nullptr, const uint8_t* __restrict__ uni = nullptr) {
   using L = Lay<N, D>;
   using Q = P32Lay<N, D>;
   constexpr int M = L::M;
@@ -553,7 +523,15 @@ __device__ __forceinline__ void update32p_cell(int64_t c, const double* Wn, cons
 #pragma unroll
   for (int m = 0; m < M; ++m) Ws[m] = Wsrc[m * nc + c];
   const bool with_wn = a != 0.0;
-  if ((!relax || st->wn_relaxed) && stage_keeps_cell<N, D>(c, Wn, Ws, F0, F1, F2, g, with_wn)) {
+  const unsigned ub = uni ? uni[c] : 0u;
+  bool keep = !relax || st->wn_relaxed;
+  if (uni) {
+    // all faces uniform: no flux difference
+    keep = keep && ub == (1u << 2 * D) - 1u && (!with_wn || same_state<N, D>(c, Wn, Ws, nc));
+  } else {
+    keep = keep && stage_keeps_cell<N, D>(c, Wn, Ws, F0, F1, F2, g, with_wn);
+  }
+  if (keep) {
     // W_out = W_src exactly, and the planes already hold those of W_src
     if (Wout != Wsrc && !(with_wn && Wout == Wn)) {
 #pragma unroll
@@ -568,7 +546,7 @@ __device__ __forceinline__ void update32p_cell(int64_t c, const double* Wn, cons
     }
     return;
   }
-  fast_combine<N, D>(c, Wn, Ws, F0, F1, F2, g, st->dt, a, b, Wo);
+  fast_combine<N, D>(c, Wn, Ws, F0, F1, F2, g, st->dt, a, b, Wo, ub, P32);
   double rho, Re;
   if (relax)
     relax_fast<N, D>(Wo, f, rho, Re);
@@ -587,11 +565,11 @@ __global__ void __launch_bounds__(kCellThreads)
     k_update32p(const double* Wn, const double* Wsrc, double* Wout, const double* __restrict__ F0,
                 const double* __restrict__ F1, const double* __restrict__ F2, DevGrid g, DevFluid f,
                 StepState* st, double a, double b, int relax, int count, float* __restrict__ P32,
-                float* __restrict__ R32, int tau = 0) {
+                float* __restrict__ R32, int tau, const uint8_t* __restrict__ uni) {
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (!tau) {
     if (c >= g.nint) return;
-    update32p_cell<N, D>(c, Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count, P32, R32);
+    update32p_cell<N, D>(c, Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count, P32, R32, nullptr, uni);
     return;
   }
   // a step's last stage (tau): the next step's planes and CFL maxima as well,
@@ -600,7 +578,8 @@ __global__ void __launch_bounds__(kCellThreads)
   double s[D];
 #pragma unroll
   for (int d = 0; d < D; ++d) s[d] = 0.0;
-  if (c < g.nint) update32p_cell<N, D>(c, Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count, P32, R32, s);
+  if (c < g.nint)
+    update32p_cell<N, D>(c, Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count, P32, R32, s, uni);
   block_tau_max<D>(s, st->tau_bits);
 }
 
@@ -985,25 +964,30 @@ __device__ __forceinline__ bool face32_body(int64_t t, const Nodes6& nd, const d
   return true;
 }
 
-// Screened sweep without the FP64 fallbacks (about a third of the full body's
-// code and at most 80 registers, so six blocks per SM, with some values
-// spilled; seven or more blocks changed the compiler's FP32 contraction):
-// midpoints whose screens fail are appended to `list` (warp-aggregated; order
-// not significant) for k_face32_fix. *count must be 0 at launch; list holds one
-// entry per midpoint.
+// Screened sweep over the list of direction DIR (k_mark) without the FP64
+// fallbacks (about a third of the full body's code and at most 80 registers, so
+// six blocks per SM, with some values spilled; seven or more blocks changed the
+// compiler's FP32 contraction): midpoints whose screens fail are appended to
+// `deferred` (warp-aggregated; order not significant), counted in cnt[2], for
+// k_face32_fix.
 template <int N, int D, int DIR>
 __global__ void __launch_bounds__(kFaceThreads, 6)
     k_face32_fast(const double* __restrict__ W, const float* __restrict__ P32, double* __restrict__ out, DevGrid g,
                   DevFluid f, DevParams pr, const StepState* __restrict__ st, const uint8_t* __restrict__ gate,
-                  uint32_t* __restrict__ list, uint32_t* __restrict__ count) {
-  const int64_t t = patch_midpoint<DIR>(g);
-  Nodes6 nd;
-  bool need = false;
-  if (face_nodes<DIR>(g, t, nd)) {
-    const bool lin = gate != nullptr && gate[t] != 0;
-    need = !face32_body<N, D, DIR, true>(t, nd, W, nullptr, nullptr, P32, out, g, f, pr, st->lam[DIR], lin);
+                  const uint32_t* __restrict__ list, uint32_t* __restrict__ cnt, uint32_t* __restrict__ deferred) {
+  const uint32_t n = cnt[0];
+  uint32_t i;
+  while (next_entries(cnt, n, i)) {
+    const int64_t t = i < n ? (int64_t)list[i] : 0;
+    Nodes6 nd;
+    bool need = false;
+    if (i < n && face_nodes<DIR>(g, t, nd)) {
+      const bool lin = gate != nullptr && gate[t] != 0;
+      need = !face32_body<N, D, DIR, true>(t, nd, W, nullptr, nullptr, P32, out, g, f, pr, st->lam[DIR], lin, nullptr,
+                                           true);
+    }
+    defer_push(need, t, deferred, &cnt[2]);
   }
-  defer_push(need, t, list, count);
 }
 
 // The midpoints a k_face32_fast launch deferred, with the full body (FP64
@@ -1024,20 +1008,27 @@ __global__ void __launch_bounds__(kFaceThreads, 2)
     Nodes6 nd;
     if (!face_nodes<DIR>(g, t, nd)) continue;
     const bool lin = gate != nullptr && gate[t] != 0;
-    face32_body<N, D, DIR>(t, nd, W, nullptr, nullptr, P32, out, g, f, pr, st->lam[DIR], lin);
+    face32_body<N, D, DIR>(t, nd, W, nullptr, nullptr, P32, out, g, f, pr, st->lam[DIR], lin, nullptr, true);
   }
 }
 
+// The same list with the full body in one kernel (screens off, first-order scheme).
 template <int N, int D, int DIR>
 __global__ void __launch_bounds__(kFaceThreads, 3)
     k_face32(const double* __restrict__ W, const double* __restrict__ V, const double* __restrict__ AUX,
              const float* __restrict__ P32, double* __restrict__ out, DevGrid g, DevFluid f, DevParams pr,
-             const StepState* __restrict__ st, const uint8_t* __restrict__ gate) {
-  const int64_t t = patch_midpoint<DIR>(g);
-  Nodes6 nd;
-  if (!face_nodes<DIR>(g, t, nd)) return;
-  const bool lin = gate != nullptr && gate[t] != 0;
-  face32_body<N, D, DIR>(t, nd, W, V, AUX, P32, out, g, f, pr, st->lam[DIR], lin);
+             const StepState* __restrict__ st, const uint8_t* __restrict__ gate, const uint32_t* __restrict__ list,
+             uint32_t* __restrict__ cnt) {
+  const uint32_t n = cnt[0];
+  uint32_t i;
+  while (next_entries(cnt, n, i)) {
+    if (i >= n) continue;
+    const int64_t t = list[i];
+    Nodes6 nd;
+    if (!face_nodes<DIR>(g, t, nd)) continue;
+    const bool lin = gate != nullptr && gate[t] != 0;
+    face32_body<N, D, DIR>(t, nd, W, V, AUX, P32, out, g, f, pr, st->lam[DIR], lin, nullptr, true);
+  }
 }
 
 }  // namespace hrm

@@ -14,21 +14,20 @@ void launch(const double* W, const double* V, const double* AUX, const float* P3
             const DevFluid& f, const DevParams& p, const StepState* st, const GateArgs& gate, cudaStream_t s) {
   if constexpr (DIR < kD) {
     if (gate.defer_list) {
-      cudaMemsetAsync(gate.defer_count, 0, sizeof(uint32_t), s);
       if (gate.net)
-        k_face32_net<N, kD, DIR><<<patch_grid(g, DIR), kFaceThreads, 0, s>>>(
-            W, P32, gate.R32, out, g, f, p, st, static_cast<const mlp::GateBlob*>(gate.net), gate.zthr,
-            gate.out_gate, gate.defer_list, gate.defer_count);
+        k_face32_net<N, kD, DIR><<<list_grid(g, DIR, 6), kFaceThreads, 0, s>>>(
+            W, P32, gate.R32, out, g, f, p, st, static_cast<const mlp::GateBlob*>(gate.net), gate.zthr, gate.out_gate,
+            gate.list, gate.list_cnt, gate.defer_list);
       else
-        k_face32_fast<N, kD, DIR><<<patch_grid(g, DIR), kFaceThreads, 0, s>>>(
-            W, P32, out, g, f, p, st, gate.fixed, gate.defer_list, gate.defer_count);
+        k_face32_fast<N, kD, DIR><<<list_grid(g, DIR, 6), kFaceThreads, 0, s>>>(
+            W, P32, out, g, f, p, st, gate.fixed, gate.list, gate.list_cnt, gate.defer_list);
       const cudaStream_t sf = fix_stream(gate, s);
       k_face32_fix<N, kD, DIR><<<kFixBlocks, kFixThreads, 0, sf>>>(W, P32, out, g, f, p, st, gate.fixed,
-                                                                    gate.defer_list, gate.defer_count);
+                                                                    gate.defer_list, gate.list_cnt + 2);
       fix_done(gate);
     } else {
-      k_face32<N, kD, DIR><<<patch_grid(g, DIR), kFaceThreads, 0, s>>>(W, V, AUX, P32, out, g, f, p, st,
-                                                                                gate.fixed);
+      k_face32<N, kD, DIR><<<list_grid(g, DIR, 3), kFaceThreads, 0, s>>>(W, V, AUX, P32, out, g, f, p, st, gate.fixed,
+                                                                         gate.list, gate.list_cnt);
     }
   }
 }
@@ -47,14 +46,14 @@ void update32_d1(int N, const double* Wn, const double* Wsrc, double* Wout, cons
 
 void update32p_d1(int N, const double* Wn, const double* Wsrc, double* Wout, const double* F0, const double* F1,
                   const double* F2, const DevGrid& g, const DevFluid& f, StepState* st, double a, double b, int relax,
-                  int count, float* P32, float* R32, int tau, cudaStream_t s) {
+                  int count, float* P32, float* R32, int tau, const uint8_t* uni, cudaStream_t s) {
   const unsigned gr = grid_for(g.nint, kCellThreads);
   if (N == 2)
     k_update32p<2, kD><<<gr, kCellThreads, 0, s>>>(Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count, P32, R32,
-                                                    tau);
+                                                    tau, uni);
   else if (N == 3)
     k_update32p<3, kD><<<gr, kCellThreads, 0, s>>>(Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count, P32, R32,
-                                                    tau);
+                                                    tau, uni);
 }
 
 void face32_d1(int N, int dir, const double* W, const double* V, const double* AUX, const float* P32, double* out,

@@ -464,21 +464,14 @@ __global__ void __launch_bounds__(kFaceThreads, 3)
            const uint8_t* __restrict__ gate, const uint32_t* __restrict__ list, uint32_t* __restrict__ cnt) {
   __shared__ double col[kFaceCol<N, D>];
   const uint32_t n = cnt[0];
-  const int lane = threadIdx.x & 31;
-  for (;;) {
-    uint32_t i = 0;
-    if (lane == 0) i = atomicAdd(&cnt[1], 1u);
-    i = __shfl_sync(0xffffffffu, i, 0);
-    if (i >= (n + 31u) / 32u) break;
-    if (i * 32u + lane < n) {
-      const int64_t t = list[i * 32u + lane];
-      Nodes6 nd;
-      if (face_nodes<DIR>(g, t, nd)) {
-        const bool lin = gate != nullptr && gate[t] != 0;
-        face_body<N, D, DIR, true>(t, nd, W, V, AUX, out, g, f, pr, st->lam[DIR], col, lin);
-      }
-    }
-    __syncwarp();
+  uint32_t i;
+  while (next_entries(cnt, n, i)) {
+    Nodes6 nd;
+    if (i >= n) continue;
+    const int64_t t = list[i];
+    if (!face_nodes<DIR>(g, t, nd)) continue;
+    const bool lin = gate != nullptr && gate[t] != 0;
+    face_body<N, D, DIR, true>(t, nd, W, V, AUX, out, g, f, pr, st->lam[DIR], col, lin);
   }
 }
 

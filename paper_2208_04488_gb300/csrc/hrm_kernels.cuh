@@ -277,31 +277,6 @@ struct Nodes6 {
   int64_t c[6];
 };
 
-// Midpoint of this thread in a sweep launched over patch_grid blocks of
-// kFaceThreads: linear, or patched as above. Past the end of a row or of the
-// grid: the midpoint count (no midpoint).
-template <int DIR>
-__device__ __forceinline__ int64_t patch_midpoint(const DevGrid& g) {
-  static_assert(kFaceThreads == 128, "four warps per patch");
-  const int64_t f0 = g.n[0] + (DIR == 0), f1 = g.n[1] + (DIR == 1), f2 = g.n[2] + (DIR == 2);
-  if (!patched(g, DIR)) return (int64_t)blockIdx.x * kFaceThreads + threadIdx.x;
-  const int64_t nbx = (f0 + 31) / 32, b = blockIdx.x;
-  const int64_t bx = b % nbx, rest = b / nbx;
-  const int w = threadIdx.x >> 5;
-  int64_t i1, i2;
-  if (DIR == 1) {
-    const int64_t nby = (f1 + 3) / 4;
-    i1 = (rest % nby) * 4 + w;
-    i2 = rest / nby;
-  } else {
-    i1 = rest % f1;
-    i2 = (rest / f1) * 4 + w;
-  }
-  const int64_t i0 = bx * 32 + (threadIdx.x & 31);
-  if (i0 >= f0 || i1 >= f1 || i2 >= f2) return f0 * f1 * f2;
-  return (i2 * f1 + i1) * f0 + i0;
-}
-
 template <int DIR>
 __device__ __forceinline__ bool face_nodes(const DevGrid& g, int64_t t, Nodes6& nd) {
   const int64_t f0 = g.n[0] + (DIR == 0), f1 = g.n[1] + (DIR == 1), f2 = g.n[2] + (DIR == 2);
@@ -487,17 +462,40 @@ __device__ __forceinline__ void count_bits(StepState* st, int b) {
 // The precision form's FP64 arithmetic writes its multiply-adds as explicit
 // fma(): its translation units are built without FMA contraction, so that every
 // FP32 expression rounds as written whichever kernel it is inlined into.
+// Flux of a uniform face in the precision form, from the FP32 planes of one of
+// its cells (the HCS node-flux expression): NC slots, the alpha slots are zero.
+// Planes as in P32Lay: V, then c, rho, rho c^2, rho u_d, E.
+template <int N, int D>
+__device__ __forceinline__ void uniform_flux32(int64_t c, int d, const float* __restrict__ P32, int64_t nc, double* G) {
+  using L = Lay<N, D>;
+  const float un = P32[(L::MOM + d) * nc + c], pn = P32[L::EN * nc + c];
+#pragma unroll
+  for (int m = 0; m < L::NC; ++m) {
+    float v;
+    if (m < L::MOM)
+      v = P32[m * nc + c] * un;
+    else if (m < L::EN)
+      v = P32[(L::M + 3 + (m - L::MOM)) * nc + c] * un + ((m - L::MOM) == d ? pn : 0.f);
+    else
+      v = (P32[(L::M + 3 + D) * nc + c] + pn) * un;
+    G[m] = widen_f32(v);
+  }
+}
+
 // Precision form: W_out = a W^n + b (W_src + dt RHS) of one interior cell c,
 // with W_src + dt RHS accumulated directly and dt/dx_d folded into one
 // coefficient per direction (one multiply-add per slot and direction). Ws: the
 // cell's W_src, already loaded. The SSP-RK stages that combine with W^n have
 // b = 1 - a, so their combination is formed as acc + a (W^n - acc): two
-// operations as before, and exactly acc when W^n equals acc.
+// operations as before, and exactly acc when W^n equals acc. ub: the cell's
+// uniform faces (k_mark), whose flux comes from the cell's own planes P32; two
+// of them leave acc as it is (acc + cd 0 with cd < 0).
 template <int N, int D>
 __device__ __forceinline__ void fast_combine(int64_t c, const double* Wn, const double* Ws,
                                              const double* __restrict__ F0, const double* __restrict__ F1,
                                              const double* __restrict__ F2, const DevGrid& g, double dt, double a,
-                                             double b, double* Wo) {
+                                             double b, double* Wo, unsigned ub = 0u,
+                                             const float* __restrict__ P32 = nullptr) {
   using L = Lay<N, D>;
   constexpr int M = L::M;
   const int64_t nc = g.ncells;
@@ -509,20 +507,24 @@ __device__ __forceinline__ void fast_combine(int64_t c, const double* Wn, const 
   for (int m = 0; m < M; ++m) acc[m] = Ws[m];
 #pragma unroll
   for (int d = 0; d < D; ++d) {
+    const unsigned u = ub >> (2 * d) & 3u;
+    if (u == 3u) continue;
     const double* F = d == 0 ? F0 : (d == 1 ? F1 : F2);
     const int64_t f0 = g.n[0] + (d == 0), f1 = g.n[1] + (d == 1), f2 = g.n[2] + (d == 2);
     const int64_t nf = f0 * f1 * f2;
     const int64_t fl = HRM_IDX(g, (i2 * f1 + i1) * f0 + i0, nf);
     const int64_t fr = HRM_IDX(g, fl + (d == 0 ? 1 : (d == 1 ? f0 : f0 * f1)), nf);
     const double cd = -dt * g.inv_dx[d];
+    double own[L::NC];
+    if (u) uniform_flux32<N, D>(c, d, P32, nc, own);
     // G^-_{i+1/2} - G^+_{i-1/2}: the alpha slots of the right face use alpha_i
     // (planes AL..), those of the left face alpha_i as its right neighbour (planes M..)
 #pragma unroll
-    for (int m = 0; m < L::NC; ++m) acc[m] = fma(cd, F[m * nf + fr] - F[m * nf + fl], acc[m]);
-#pragma unroll
-    for (int k = 0; k < N - 1; ++k) {
-      const int m = L::AL + k;
-      acc[m] = fma(cd, F[m * nf + fr] - F[(M + k) * nf + fl], acc[m]);
+    for (int m = 0; m < M; ++m) {
+      const double fo = m < L::NC ? own[m < L::NC ? m : 0] : 0.0;
+      const double vl = (u & 1u) ? fo : F[(m < L::NC ? m : M + m - L::AL) * nf + fl];
+      const double vr = (u & 2u) ? fo : F[m * nf + fr];
+      acc[m] = fma(cd, vr - vl, acc[m]);
     }
   }
   if (a == 0.0 && b == 1.0) {
@@ -570,6 +572,18 @@ __device__ __forceinline__ bool faces_unchanged(int64_t c, const double* __restr
   return same;
 }
 
+// Whether W_src of cell c is W^n bit for bit, with no component -0.
+template <int N, int D>
+__device__ __forceinline__ bool same_state(int64_t c, const double* Wn, const double* Ws, int64_t nc) {
+  bool same = true;
+#pragma unroll
+  for (int m = 0; m < Lay<N, D>::M; ++m) {
+    const unsigned long long bs = (unsigned long long)__double_as_longlong(Ws[m]);
+    same = same & (bs == (unsigned long long)__double_as_longlong(Wn[m * nc + c])) & (bs != 0x8000000000000000ull);
+  }
+  return same;
+}
+
 // Precision form: whether a stage returns cell c exactly as it is, so that its
 // arithmetic can be left out. Every flux difference G^-_{i+1/2} - G^+_{i-1/2}
 // is exactly zero when the two faces' values are bit-equal and finite; a stage
@@ -583,18 +597,8 @@ template <int N, int D>
 __device__ __forceinline__ bool stage_keeps_cell(int64_t c, const double* Wn, const double* Ws,
                                                  const double* __restrict__ F0, const double* __restrict__ F1,
                                                  const double* __restrict__ F2, const DevGrid& g, bool with_wn) {
-  constexpr int M = Lay<N, D>::M;
   const int64_t nc = g.ncells;
-  bool same = faces_unchanged<N, D>(c, F0, F1, F2, g);
-  if (with_wn) {
-#pragma unroll
-    for (int m = 0; m < M; ++m) {
-      const unsigned long long bs = (unsigned long long)__double_as_longlong(Ws[m]);
-      same = same & (bs == (unsigned long long)__double_as_longlong(Wn[m * nc + c])) &
-             (bs != 0x8000000000000000ull);
-    }
-  }
-  return same;
+  return faces_unchanged<N, D>(c, F0, F1, F2, g) && (!with_wn || same_state<N, D>(c, Wn, Ws, nc));
 }
 
 // Flux of a uniform face from the state of one of its cells: the node's physical

@@ -31,9 +31,8 @@ struct GateArgs {
   const uint8_t* fixed = nullptr;
   // precision form with screens: the sweep defers midpoints whose screens fail
   // to a second kernel through this worklist (one entry per midpoint of the
-  // direction) and counter; nullptr: one kernel with the fallbacks inline
+  // direction; counted in list_cnt[2]); nullptr: one kernel with the fallbacks inline
   uint32_t* defer_list = nullptr;
-  uint32_t* defer_count = nullptr;
   // optional: run the deferred midpoints on `side` (after ev_fast, recorded on
   // the sweep's stream) and record ev_fix there, so that they overlap the next
   // sweep; the caller joins ev_fix before the update
@@ -48,7 +47,7 @@ struct GateArgs {
   const float* R32 = nullptr;
   float zthr = 0.f;
   uint8_t* out_gate = nullptr;
-  // FP64 form: the midpoints to sweep and their counters (SweepLists of the direction)
+  // the midpoints to sweep and their counters (SweepLists of the direction)
   const uint32_t* list = nullptr;
   uint32_t* list_cnt = nullptr;
 };
@@ -113,22 +112,23 @@ void face32_d3(int N, int dir, const double* W, const double* V, const double* A
 // hrm_face32_dD.cu).
 void update32p_d1(int N, const double* Wn, const double* Wsrc, double* Wout, const double* F0, const double* F1,
                   const double* F2, const DevGrid&, const DevFluid&, StepState*, double a, double b, int relax,
-                  int count, float* P32, float* R32, int tau, cudaStream_t);
+                  int count, float* P32, float* R32, int tau, const uint8_t* uni, cudaStream_t);
 void update32p_d2(int N, const double* Wn, const double* Wsrc, double* Wout, const double* F0, const double* F1,
                   const double* F2, const DevGrid&, const DevFluid&, StepState*, double a, double b, int relax,
-                  int count, float* P32, float* R32, int tau, cudaStream_t);
+                  int count, float* P32, float* R32, int tau, const uint8_t* uni, cudaStream_t);
 void update32p_d3(int N, const double* Wn, const double* Wsrc, double* Wout, const double* F0, const double* F1,
                   const double* F2, const DevGrid&, const DevFluid&, StepState*, double a, double b, int relax,
-                  int count, float* P32, float* R32, int tau, cudaStream_t);
+                  int count, float* P32, float* R32, int tau, const uint8_t* uni, cudaStream_t);
+// uni (nullable): the cells' uniform faces (k_mark; their fluxes are not read);
 // tau: also accumulate the CFL maxima of W_out into st->tau_bits (a step's last
 // stage; grids without Dirichlet slices, five-equation sound speed).
 inline void launch_update32p(int N, int D, const double* Wn, const double* Wsrc, double* Wout, const double* F0,
                              const double* F1, const double* F2, const DevGrid& g, const DevFluid& f, StepState* st,
-                             double a, double b, int relax, int count, float* P32, float* R32, cudaStream_t s,
-                             int tau = 0) {
-  if (D == 1) update32p_d1(N, Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count, P32, R32, tau, s);
-  if (D == 2) update32p_d2(N, Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count, P32, R32, tau, s);
-  if (D == 3) update32p_d3(N, Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count, P32, R32, tau, s);
+                             double a, double b, int relax, int count, float* P32, float* R32, const uint8_t* uni,
+                             cudaStream_t s, int tau = 0) {
+  if (D == 1) update32p_d1(N, Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count, P32, R32, tau, uni, s);
+  if (D == 2) update32p_d2(N, Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count, P32, R32, tau, uni, s);
+  if (D == 3) update32p_d3(N, Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count, P32, R32, tau, uni, s);
 }
 
 // Primitive kernel of the precision form (FP32 planes only; hrm_face32_dD.cu).
@@ -150,19 +150,11 @@ void launch_set_dt(StepState* st, double dt, cudaStream_t s);
 
 inline unsigned grid_for(long long n, int threads) { return (unsigned)((n + threads - 1) / threads); }
 
-// Blocks of kFaceThreads covering the midpoints of direction dir in the layout
-// of patch_midpoint (linear, or patches of 32 x 4 where patched(g, dir)).
-inline unsigned patch_grid(const DevGrid& g, int dir) {
-  const long long f0 = g.n[0] + (dir == 0), f1 = g.n[1] + (dir == 1), f2 = g.n[2] + (dir == 2);
-  if (!patched(g, dir)) return grid_for(f0 * f1 * f2, 128);
-  const long long nbx = (f0 + 31) / 32;
-  return (unsigned)(dir == 1 ? nbx * ((f1 + 3) / 4) * f2 : nbx * f1 * ((f2 + 3) / 4));
-}
-
-// Uniform faces and the lists of the other midpoints of a stage's source state,
-// FP64 form (hrm_sweep.cuh): two launches. all: every midpoint is listed.
-void launch_mark64(int N, int D, const double* W, const double* V, const DevGrid& g, const SweepLists& lists, int all,
-                   cudaStream_t s);
+// Uniform faces and the lists of the other midpoints of a stage's source state
+// (hrm_sweep.cuh): two launches. P32 NULL: the FP64 form, from W and V; else the
+// precision form, from its FP32 planes. all: every midpoint is listed.
+void launch_mark(int N, int D, const double* W, const double* V, const float* P32, const DevGrid& g,
+                 const SweepLists& lists, int all, cudaStream_t s);
 
 // Blocks of kFaceThreads of a list-driven sweep: what is resident at per_sm blocks
 // on each SM, or fewer where the whole midpoint grid needs no more.

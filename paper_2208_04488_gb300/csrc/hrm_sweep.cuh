@@ -11,7 +11,7 @@
 // nodes equal, so such faces are neither written nor read.
 #pragma once
 
-#include "hrm_kernels.cuh"
+#include "hrm_face32.cuh"
 #include "hrm_launch.h"
 
 namespace hrm {
@@ -31,24 +31,35 @@ __device__ __forceinline__ int64_t neighbour(const DevGrid& g, int d, const int6
   return c + (bc_map(g, d, j) - ijk[d]) * stride;
 }
 
-// eq[c], bit d: every plane of W finite and bit for bit the same in cell c and
-// the cell after it along d; bit 3 + d, for the first cell of a line: in cell c
-// and the ghost cell before it. Thread 0 clears the lists' counters.
-template <int N, int D>
+// eq[c], bit d: every plane finite and the same in cell c and the cell after it
+// along d; bit 3 + d, for the first cell of a line: in cell c and the ghost cell
+// before it. T double: the M planes of W, bit for bit (the FP64 form's uniform
+// stencils); T float: the precision form's FP32 planes, by value. Thread by thread
+// the lists' counters are cleared.
+template <int N, int D, typename T>
 __global__ void __launch_bounds__(kCellThreads)
-    k_equal(const double* __restrict__ W, DevGrid g, uint8_t* __restrict__ eq, uint32_t* __restrict__ cnt) {
+    k_equal(const T* __restrict__ W, DevGrid g, uint8_t* __restrict__ eq, uint32_t* __restrict__ cnt) {
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (c < kSweepCounters) cnt[c] = 0u;
   if (c >= g.nint) return;
-  constexpr int M = Lay<N, D>::M;
+  constexpr int M = sizeof(T) == 8 ? Lay<N, D>::M : P32Lay<N, D>::PLANES;
+  auto same_value = [](T x, T y) {
+    if constexpr (sizeof(T) == 8)
+      return __double_as_longlong(x) == __double_as_longlong(y);
+    else
+      return x == y;
+  };
   int64_t ijk[3];
   cell_index(g, c, ijk);
-  long long w[M];
+  T w[M];
   bool fin = true;
 #pragma unroll
   for (int m = 0; m < M; ++m) {
-    w[m] = __double_as_longlong(W[m * g.ncells + c]);
-    fin = fin & (((uint32_t)(w[m] >> 32) & 0x7ff00000u) != 0x7ff00000u);
+    w[m] = W[m * g.ncells + c];
+    if constexpr (sizeof(T) == 8)
+      fin = fin & (((uint32_t)__double2hiint(w[m]) & 0x7ff00000u) != 0x7ff00000u);
+    else
+      fin = fin & ((__float_as_uint(w[m]) & 0x7f800000u) != 0x7f800000u);
   }
   unsigned bits = 0;
 #pragma unroll
@@ -57,7 +68,7 @@ __global__ void __launch_bounds__(kCellThreads)
       o = HRM_IDX(g, o, g.ncells);
       bool s = fin;
 #pragma unroll
-      for (int m = 0; m < M; ++m) s = s & (__double_as_longlong(W[m * g.ncells + o]) == w[m]);
+      for (int m = 0; m < M; ++m) s = s & same_value(W[m * g.ncells + o], w[m]);
       return s;
     };
     if (same(neighbour<D, false>(g, d, ijk, c))) bits |= 1u << d;
@@ -70,10 +81,12 @@ __global__ void __launch_bounds__(kCellThreads)
 // of direction d are uniform (no face is with `all`, the first-order scheme). The
 // other midpoints go to lists.list[d] in the order of their cells, one atomic per
 // block and direction. With lists.F (every midpoint's flux wanted) the uniform
-// faces' fluxes are written too.
-template <int N, int D>
+// faces' fluxes are written too, and with lists.gate their gate bytes. FP32: the
+// precision form (P32), else the FP64 form (W, V).
+template <int N, int D, bool FP32>
 __global__ void __launch_bounds__(kCellThreads)
-    k_mark(const double* __restrict__ W, const double* __restrict__ V, DevGrid g, SweepLists lists, int all) {
+    k_mark(const double* __restrict__ W, const double* __restrict__ V, const float* __restrict__ P32, DevGrid g,
+           SweepLists lists, int all) {
   using L = Lay<N, D>;
   constexpr int kWarps = kCellThreads / 32;
   __shared__ uint32_t base[D][kWarps];
@@ -88,17 +101,22 @@ __global__ void __launch_bounds__(kCellThreads)
     for (int d = 0; d < D; ++d) {
       const int64_t stride = d == 0 ? 1 : (d == 1 ? g.n[0] : g.n[0] * g.n[1]);
       const int64_t n = g.n[d], i = ijk[d];
-      const bool per = g.bc[2 * d] == 1;
       bool pair[6];  // cells i + j - 3 and i + j - 2 equal
+      if (i >= 3 && i + 2 < n) {
 #pragma unroll
-      for (int j = 0; j < 6; ++j) {
-        int64_t q = i + j - 3;
-        if (per) q = q < 0 ? q + n : (q >= n ? q - n : q);
-        const bool low = q == -1;
-        pair[j] = true;
-        if (q >= -1 && q < n) {
-          const unsigned e = lists.eq[HRM_IDX(g, c + ((low ? 0 : q) - i) * stride, g.nint)];
-          pair[j] = (e >> (low ? 3 + d : d)) & 1u;
+        for (int j = 0; j < 6; ++j) pair[j] = (lists.eq[HRM_IDX(g, c + (j - 3) * stride, g.nint)] >> d) & 1u;
+      } else {
+        const bool per = g.bc[2 * d] == 1;
+#pragma unroll
+        for (int j = 0; j < 6; ++j) {
+          int64_t q = i + j - 3;
+          if (per) q = q < 0 ? q + n : (q >= n ? q - n : q);
+          const bool low = q == -1;
+          pair[j] = true;
+          if (q >= -1 && q < n) {
+            const unsigned e = lists.eq[HRM_IDX(g, c + ((low ? 0 : q) - i) * stride, g.nint)];
+            pair[j] = (e >> (low ? 3 + d : d)) & 1u;
+          }
         }
       }
       const bool mid = pair[1] & pair[2] & pair[3] & pair[4];
@@ -139,10 +157,17 @@ __global__ void __launch_bounds__(kCellThreads)
     if (lo[d]) lists.list[d][p] = (uint32_t)t;
     if (hi[d]) lists.list[d][p + (lo[d] ? 1u : 0u)] = (uint32_t)up;
     const bool last = ijk[d] == g.n[d] - 1 && !hi[d];
+    if (lists.gate[d]) {
+      if (!lo[d]) lists.gate[d][t] = 2;
+      if (last) lists.gate[d][up] = 2;
+    }
     if (lists.F[d] && (!lo[d] || last)) {
       const int64_t nf = f0 * f1 * (g.n[2] + (d == 2));
       double G[L::NC];
-      uniform_flux64<N, D>(c, d, W, V, g.ncells, G);
+      if constexpr (FP32)
+        uniform_flux32<N, D>(c, d, P32, g.ncells, G);
+      else
+        uniform_flux64<N, D>(c, d, W, V, g.ncells, G);
 #pragma unroll
       for (int m = 0; m < L::M + N - 1; ++m) {
         const double v = m < L::NC ? G[m < L::NC ? m : 0] : 0.0;

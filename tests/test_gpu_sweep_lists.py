@@ -63,3 +63,22 @@ def test_step_and_rhs_equal_the_oracle(hrm, orc, n, bc, where):
     s.step(dt, 3)
     np.testing.assert_array_equal(s.get(hrm.FIELD_W), orc.step(f, orc.make_params(), g, W, dt, 3))
     s.close()
+
+
+@pytest.mark.parametrize("n", GRIDS, ids=lambda n: "x".join(map(str, n)))
+@pytest.mark.parametrize("bc", [0, 1, 2], ids=["transmissive", "periodic", "dirichlet"])
+@pytest.mark.parametrize("where", ["none", "ends"])
+def test_precision_form_step_equals_its_stages(hrm, n, bc, where):
+    """The step's updates form uniform faces' fluxes from the cell's own planes; the
+    stages taken one at a time write and read every midpoint's flux."""
+    pr = disturbed(n, bc, where)
+    prm = hrm.params_default(cfl=0.4, check=0, precision=hrm.FP32)
+    a, b = hrm.Solver.from_problem(pr, params=prm), hrm.Solver.from_problem(pr, params=prm)
+    for _ in range(3):
+        a.step(0.0, 1)
+        b.begin_step(b.step_tau())
+        for k in range(b.stages()):
+            b.stage(k)
+    np.testing.assert_array_equal(a.get(hrm.FIELD_W), b.get(hrm.FIELD_W))
+    a.close()
+    b.close()
