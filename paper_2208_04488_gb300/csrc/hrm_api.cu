@@ -304,9 +304,10 @@ bool fuse_last(const hrm_ctx* c) {
 // FP64 form within one step: same_out, the update marks the cells whose state it
 // leaves bit for bit as in Wsrc; same_in, the primitive pass keeps those cells'
 // primitives (the previous stage's update marked them, nothing wrote W since).
+// src_relaxed: Wsrc came out of the previous stage's relaxation.
 int enqueue_stage(hrm_ctx* c, cudaStream_t s, const double* Wsrc, double* Wout, double a, double b, int relax,
                   int count, bool first, bool prim_done = false, bool fuse_next = false, bool tau_next = false,
-                  bool same_in = false, bool same_out = false) {
+                  bool same_in = false, bool same_out = false, bool src_relaxed = false) {
   uint8_t* same = c->params.precision == HRM_FP64 ? c->same : nullptr;
   int k = 0;
   float* p32 = p32_target(c);
@@ -366,11 +367,11 @@ int enqueue_stage(hrm_ctx* c, cudaStream_t s, const double* Wsrc, double* Wout, 
   traced(c, s, HRM_KERNEL_UPDATE, [&] {
     if (fuse_next)
       launch_update32p(c->N, c->D, c->Wn, Wsrc, Wout, c->F[0], c->F[1], c->F[2], c->dg, c->fl, c->st, a, b, relax,
-                       count, c->P32, r32_target(c), c->lists.uni, s, tau_next ? 1 : 0);
+                       count, c->P32, r32_target(c), c->lists.uni, src_relaxed ? 1 : 0, s, tau_next ? 1 : 0);
     else
       c->fk->update(0, c->params.precision == HRM_FP32, c->Wn, Wsrc, Wout, c->F[0], c->F[1], c->F[2], c->dg,
                     c->fl, c->st, a, b, relax, count, same_out ? same : nullptr,
-                    c->params.precision == HRM_FP64 ? c->lists.uni : nullptr, c->V, s);
+                    c->params.precision == HRM_FP64 ? c->lists.uni : nullptr, c->V, src_relaxed ? 1 : 0, s);
   });
   ++k;
   return k;
@@ -391,12 +392,12 @@ int enqueue_step(hrm_ctx* c, cudaStream_t s) {
       break;
     case HRM_RK2:
       k += enqueue_stage(c, s, c->Wn, c->Ws, 0.0, 1.0, rs, 0, true, false, fp32, false, false, true);
-      k += enqueue_stage(c, s, c->Ws, c->Wn, 0.5, 0.5, rf, ck, false, fp32, fl, fl, true, false);
+      k += enqueue_stage(c, s, c->Ws, c->Wn, 0.5, 0.5, rf, ck, false, fp32, fl, fl, true, false, rs);
       break;
     default:
       k += enqueue_stage(c, s, c->Wn, c->Ws, 0.0, 1.0, rs, 0, true, false, fp32, false, false, true);
-      k += enqueue_stage(c, s, c->Ws, c->Ws, 0.75, 0.25, rs, 0, false, fp32, fp32, false, true, true);
-      k += enqueue_stage(c, s, c->Ws, c->Wn, 1.0 / 3.0, 2.0 / 3.0, rf, ck, false, fp32, fl, fl, true, false);
+      k += enqueue_stage(c, s, c->Ws, c->Ws, 0.75, 0.25, rs, 0, false, fp32, fp32, false, true, true, rs);
+      k += enqueue_stage(c, s, c->Ws, c->Wn, 1.0 / 3.0, 2.0 / 3.0, rf, ck, false, fp32, fl, fl, true, false, rs);
       break;
   }
   return k;
@@ -1206,7 +1207,7 @@ hrm_status hrm_rhs(hrm_ctx* c, const double* lam, double* rhs) {
                    gate_of(c, d), c->stream);
   }
   c->fk->update(1, 0, c->Wn, c->Wn, out, c->F[0], c->F[1], c->F[2], c->dg, c->fl, c->st, 0.0, 1.0, 0, 0,
-                nullptr, nullptr, nullptr, c->stream);
+                nullptr, nullptr, nullptr, 0, c->stream);
   c->launches += 2 + c->D * sweep_kernels(c);
   if ((s = last_launch(c, "rhs"))) return s;
   // (the update writes interior cells only: the stage state's slices stay)

@@ -193,10 +193,12 @@ template <typename T> __device__ __forceinline__ T dmax(T a, T b) { return (a < 
 
 // FP64 quotients and square roots on the integer pipes (hrm_soft64.cuh): the bits
 // of the FP64 unit's sequences, which take 137 and 143 of its cycles per warp,
-// at 27 and 30.
-__device__ __forceinline__ double quot(double a, double b) { return soft::div(a, b); }
+// at 27 and 30. Out of line: a body has a dozen to two dozen of them, and the
+// instruction fetch of as many copies costs more than the calls (measured 1-3 %
+// of a pass on most workloads).
+static __device__ __noinline__ double quot(double a, double b) { return soft::div(a, b); }
 __device__ __forceinline__ float quot(float a, float b) { return a / b; }
-__device__ __forceinline__ double rsqrt_r(double x) { return soft::root(x); }
+static __device__ __noinline__ double rsqrt_r(double x) { return soft::root(x); }
 // FP64 products on the integer pipes, for the bodies whose adds keep the FP64 unit
 // busy meanwhile: the bits of a * b.
 __device__ __forceinline__ double prod(double a, double b) { return soft::mul(a, b); }

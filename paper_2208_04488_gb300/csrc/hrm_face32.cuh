@@ -509,7 +509,8 @@ __device__ __forceinline__ void update32p_cell(int64_t c, const double* Wn, cons
                                                const double* __restrict__ F2, const DevGrid& g, const DevFluid& f,
                                                StepState* st, double a, double b, int relax, int count,
                                                float* __restrict__ P32, float* __restrict__ R32,
-                                               double* s = nullptr, const uint8_t* __restrict__ uni = nullptr) {
+                                               double* s = nullptr, const uint8_t* __restrict__ uni = nullptr,
+                                               int src_relaxed = 0) {
   using L = Lay<N, D>;
   using Q = P32Lay<N, D>;
   constexpr int M = L::M;
@@ -524,18 +525,30 @@ __device__ __forceinline__ void update32p_cell(int64_t c, const double* Wn, cons
   for (int m = 0; m < M; ++m) Ws[m] = Wsrc[m * nc + c];
   const bool with_wn = a != 0.0;
   const unsigned ub = uni ? uni[c] : 0u;
-  bool keep = !relax || st->wn_relaxed;
+  // Unchanged cells (see stage_keeps_cell; here no flux difference means that all
+  // faces are uniform). From a step's second relaxed stage on (src_relaxed) W_src
+  // came out of relax_fast: then its conserved variables being W^n's is enough,
+  // for the relaxation forms W_src's volume fractions again.
+  bool keep, by_src = false;
   if (uni) {
-    // all faces uniform: no flux difference
-    keep = keep && ub == (1u << 2 * D) - 1u && (!with_wn || same_state<N, D>(c, Wn, Ws, nc));
+    keep = ub == (1u << 2 * D) - 1u;
+    if (keep && with_wn) {
+      by_src = relax && src_relaxed && same_state<N, D>(c, Wn, Ws, nc, L::NC);
+      keep = by_src || ((!relax || st->wn_relaxed) && same_state<N, D>(c, Wn, Ws, nc));
+    } else {
+      keep = keep && (!relax || st->wn_relaxed);
+    }
   } else {
-    keep = keep && stage_keeps_cell<N, D>(c, Wn, Ws, F0, F1, F2, g, with_wn);
+    keep = (!relax || st->wn_relaxed) && stage_keeps_cell<N, D>(c, Wn, Ws, F0, F1, F2, g, with_wn);
   }
   if (keep) {
     // W_out = W_src exactly, and the planes already hold those of W_src
     if (Wout != Wsrc && !(with_wn && Wout == Wn)) {
 #pragma unroll
       for (int m = 0; m < M; ++m) Wout[m * nc + c] = Ws[m];
+    } else if (by_src && Wout == Wn) {
+#pragma unroll
+      for (int k = 0; k < N - 1; ++k) Wout[(L::AL + k) * nc + c] = Ws[L::AL + k];
     }
     if (count) count_bits(st, admissibility_bits<N, D>(Ws, f));
     if (s) {
@@ -565,11 +578,12 @@ __global__ void __launch_bounds__(kCellThreads)
     k_update32p(const double* Wn, const double* Wsrc, double* Wout, const double* __restrict__ F0,
                 const double* __restrict__ F1, const double* __restrict__ F2, DevGrid g, DevFluid f,
                 StepState* st, double a, double b, int relax, int count, float* __restrict__ P32,
-                float* __restrict__ R32, int tau, const uint8_t* __restrict__ uni) {
+                float* __restrict__ R32, int tau, const uint8_t* __restrict__ uni, int src_relaxed) {
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (!tau) {
     if (c >= g.nint) return;
-    update32p_cell<N, D>(c, Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count, P32, R32, nullptr, uni);
+    update32p_cell<N, D>(c, Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count, P32, R32, nullptr, uni,
+                         src_relaxed);
     return;
   }
   // a step's last stage (tau): the next step's planes and CFL maxima as well,
@@ -579,7 +593,8 @@ __global__ void __launch_bounds__(kCellThreads)
 #pragma unroll
   for (int d = 0; d < D; ++d) s[d] = 0.0;
   if (c < g.nint)
-    update32p_cell<N, D>(c, Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count, P32, R32, s, uni);
+    update32p_cell<N, D>(c, Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count, P32, R32, s, uni,
+                         src_relaxed);
   block_tau_max<D>(s, st->tau_bits);
 }
 

@@ -28,7 +28,7 @@ template <int N>
 void update_l(int mode, int fast, const double* Wn, const double* Wsrc, double* Wout, const double* F0,
               const double* F1, const double* F2, const DevGrid& g, const DevFluid& f, StepState* st, double a,
               double b, int relax, int count, uint8_t* same, const uint8_t* uni,
-              const double* V, cudaStream_t s) {
+              const double* V, int src_relaxed, cudaStream_t s) {
   if (fast && mode == 0) {
     update32_d1(N, Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count, s);
     return;
@@ -38,7 +38,7 @@ void update_l(int mode, int fast, const double* Wn, const double* Wsrc, double* 
     k_update<N, kD, 1><<<gr, kCellThreads, 0, s>>>(Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count);
   else
     k_update<N, kD, 0><<<gr, kCellThreads, 0, s>>>(Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count,
-                                                   same, uni, V);
+                                                   same, uni, V, src_relaxed);
 }
 
 template <int N>

@@ -572,12 +572,15 @@ __device__ __forceinline__ bool faces_unchanged(int64_t c, const double* __restr
   return same;
 }
 
-// Whether W_src of cell c is W^n bit for bit, with no component -0.
+// Whether the first `slots` components of W_src of cell c are W^n's bit for bit,
+// with none -0.
 template <int N, int D>
-__device__ __forceinline__ bool same_state(int64_t c, const double* Wn, const double* Ws, int64_t nc) {
+__device__ __forceinline__ bool same_state(int64_t c, const double* Wn, const double* Ws, int64_t nc,
+                                           int slots = Lay<N, D>::M) {
   bool same = true;
 #pragma unroll
   for (int m = 0; m < Lay<N, D>::M; ++m) {
+    if (m >= slots) continue;
     const unsigned long long bs = (unsigned long long)__double_as_longlong(Ws[m]);
     same = same & (bs == (unsigned long long)__double_as_longlong(Wn[m * nc + c])) & (bs != 0x8000000000000000ull);
   }
@@ -632,7 +635,7 @@ __device__ __forceinline__ void update_body(int64_t c, const double* Wn, const d
                                             StepState* st, double dt, double a, double b, int relax, int count,
                                             uint8_t* __restrict__ same = nullptr,
                                             const uint8_t* __restrict__ uni = nullptr,
-                                            const double* __restrict__ V = nullptr) {
+                                            const double* __restrict__ V = nullptr, int src_relaxed = 0) {
   using L = Lay<N, D>;
   constexpr int M = L::M;
   const int64_t nc = g.ncells;
@@ -713,21 +716,28 @@ __device__ __forceinline__ void update_body(int64_t c, const double* Wn, const d
     for (int m = 0; m < M; ++m) Wo[m] = a * Wn[m * nc + c] + b * (Ws[m] + dt * rhs[m]);
   }
   // relax_cell recomputes the volume fractions from the conserved variables
-  // alone: where those are bit-equal to W^n's and W^n came out of relax_cell
-  // (the host's flag), it would return W^n's volume fractions, taken directly.
+  // alone: where those are bit-equal to a state's that came out of relax_cell --
+  // W_src from the second relaxed stage of a step on (src_relaxed), W^n by the
+  // host's flag -- it would return that state's volume fractions, taken directly.
   bool keep = false;
-  if (relax && flat && st->wn_relaxed) {
-    keep = true;
+  if (relax && flat) {
+    auto conserved_as = [&](auto value) {
+      bool k = true;
 #pragma unroll
-    for (int m = 0; m < L::NC; ++m)
-      keep = keep & (__double_as_longlong(Wo[m]) == __double_as_longlong(Wn[m * nc + c]));
-  }
-  if (keep) {
+      for (int m = 0; m < L::NC; ++m) k = k & (__double_as_longlong(Wo[m]) == __double_as_longlong(value(m)));
+      return k;
+    };
+    if (src_relaxed && conserved_as([&](int m) { return Ws[m]; })) {
+      keep = true;
 #pragma unroll
-    for (int k = 0; k < N - 1; ++k) Wo[L::AL + k] = Wn[(L::AL + k) * nc + c];
-  } else if (relax) {
-    relax_cell<N, D, FAST>(Wo, f);
+      for (int k = 0; k < N - 1; ++k) Wo[L::AL + k] = Ws[L::AL + k];
+    } else if (st->wn_relaxed && conserved_as([&](int m) { return Wn[m * nc + c]; })) {
+      keep = true;
+#pragma unroll
+      for (int k = 0; k < N - 1; ++k) Wo[L::AL + k] = Wn[(L::AL + k) * nc + c];
+    }
   }
+  if (relax && !keep) relax_cell<N, D, FAST>(Wo, f);
   if (count) count_bits(st, admissibility_bits<N, D>(Wo, f));
   if (same) {
     // the next stage's primitive pass keeps this cell's V and AUX where W_out is W_src
@@ -745,11 +755,11 @@ __global__ void __launch_bounds__(kCellThreads)
     k_update(const double* Wn, const double* Wsrc, double* Wout, const double* __restrict__ F0,
              const double* __restrict__ F1, const double* __restrict__ F2, DevGrid g, DevFluid f,
              StepState* st, double a, double b, int relax, int count, uint8_t* __restrict__ same = nullptr,
-             const uint8_t* __restrict__ uni = nullptr, const double* __restrict__ V = nullptr) {
+             const uint8_t* __restrict__ uni = nullptr, const double* __restrict__ V = nullptr, int src_relaxed = 0) {
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= g.nint) return;
   update_body<N, D, MODE, FAST>(c, Wn, Wsrc, Wout, F0, F1, F2, g, f, st, MODE == 1 ? 0.0 : st->dt, a, b, relax,
-                                count, same, uni, V);
+                                count, same, uni, V, src_relaxed);
 }
 
 }  // namespace hrm

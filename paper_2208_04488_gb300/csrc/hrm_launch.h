@@ -76,10 +76,11 @@ struct FaceKernels {
   // mode 0: RK combination, mode 1: write the RHS; fast: precision-form variant;
   // same (nullable; FP64 RK combination): per interior cell, set to 1 where
   // W_out equals W_src bit for bit, else 0; uni (nullable; FP64 RK combination):
-  // the cells' uniform faces, whose fluxes are formed from W_src and V
+  // the cells' uniform faces, whose fluxes are formed from W_src and V; src_relaxed:
+  // every interior cell of W_src came out of the form's relaxation
   void (*update)(int mode, int fast, const double* Wn, const double* Wsrc, double* Wout, const double* F0,
                  const double* F1, const double* F2, const DevGrid&, const DevFluid&, StepState*, double a,
-                 double b, int relax, int count, uint8_t* same, const uint8_t* uni, const double* V, cudaStream_t);
+                 double b, int relax, int count, uint8_t* same, const uint8_t* uni, const double* V, int src_relaxed, cudaStream_t);
 };
 
 const CellKernels* cell_kernels(int N, int D);
@@ -112,23 +113,26 @@ void face32_d3(int N, int dir, const double* W, const double* V, const double* A
 // hrm_face32_dD.cu).
 void update32p_d1(int N, const double* Wn, const double* Wsrc, double* Wout, const double* F0, const double* F1,
                   const double* F2, const DevGrid&, const DevFluid&, StepState*, double a, double b, int relax,
-                  int count, float* P32, float* R32, int tau, const uint8_t* uni, cudaStream_t);
+                  int count, float* P32, float* R32, int tau, const uint8_t* uni, int src_relaxed,
+                  cudaStream_t);
 void update32p_d2(int N, const double* Wn, const double* Wsrc, double* Wout, const double* F0, const double* F1,
                   const double* F2, const DevGrid&, const DevFluid&, StepState*, double a, double b, int relax,
-                  int count, float* P32, float* R32, int tau, const uint8_t* uni, cudaStream_t);
+                  int count, float* P32, float* R32, int tau, const uint8_t* uni, int src_relaxed,
+                  cudaStream_t);
 void update32p_d3(int N, const double* Wn, const double* Wsrc, double* Wout, const double* F0, const double* F1,
                   const double* F2, const DevGrid&, const DevFluid&, StepState*, double a, double b, int relax,
-                  int count, float* P32, float* R32, int tau, const uint8_t* uni, cudaStream_t);
+                  int count, float* P32, float* R32, int tau, const uint8_t* uni, int src_relaxed,
+                  cudaStream_t);
 // uni (nullable): the cells' uniform faces (k_mark; their fluxes are not read);
 // tau: also accumulate the CFL maxima of W_out into st->tau_bits (a step's last
 // stage; grids without Dirichlet slices, five-equation sound speed).
 inline void launch_update32p(int N, int D, const double* Wn, const double* Wsrc, double* Wout, const double* F0,
                              const double* F1, const double* F2, const DevGrid& g, const DevFluid& f, StepState* st,
                              double a, double b, int relax, int count, float* P32, float* R32, const uint8_t* uni,
-                             cudaStream_t s, int tau = 0) {
-  if (D == 1) update32p_d1(N, Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count, P32, R32, tau, uni, s);
-  if (D == 2) update32p_d2(N, Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count, P32, R32, tau, uni, s);
-  if (D == 3) update32p_d3(N, Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count, P32, R32, tau, uni, s);
+                             int src_relaxed, cudaStream_t s, int tau = 0) {
+  if (D == 1) update32p_d1(N, Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count, P32, R32, tau, uni, src_relaxed, s);
+  if (D == 2) update32p_d2(N, Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count, P32, R32, tau, uni, src_relaxed, s);
+  if (D == 3) update32p_d3(N, Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count, P32, R32, tau, uni, src_relaxed, s);
 }
 
 // Primitive kernel of the precision form (FP32 planes only; hrm_face32_dD.cu).
