@@ -74,6 +74,8 @@ struct hrm_ctx {
   BatchInst* p_inst = nullptr;     // this context as a one-instance batch
   WorkItem* p_cells = nullptr;
   WorkItem* p_tiles = nullptr;
+  uint64_t* p_listed = nullptr;    // its listed and deferred midpoints
+  uint64_t* p_deferred = nullptr;
   int p_ncell = 0, p_ntiles = 0, p_grid = 0;
   GridSync* p_sync = nullptr;
   unsigned int p_expired_seen = 0;
@@ -412,8 +414,8 @@ bool persistent_eligible(const hrm_ctx* c) {
          (c->N == 2 || c->N == 3);
 }
 
-// Device tables of the persistent step: this context as one instance, its
-// cells in items of 1024, its midpoints of both directions in tiles of 128.
+// Device tables of the persistent step: this context as one instance, its cells
+// in items, its midpoints of both directions in tiles of 128.
 hrm_status setup_persistent(hrm_ctx* c) {
   if (c->p_inst) return HRM_OK;
   BatchInst I;
@@ -429,7 +431,12 @@ hrm_status setup_persistent(hrm_ctx* c) {
   I.P32 = c->P32;
   I.st = c->st;
   std::vector<WorkItem> cells, tiles;
-  constexpr int64_t kCellItem = 1024;
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  c->p_grid = sms * batch_stage32_fit();
+  if (c->p_grid <= 0) return fail(c, HRM_E_CUDA, "persistent stage kernel: no resident block fits an SM");
+  const int64_t kCellItem = default_cell_tile(c->nint, c->p_grid);
   for (int64_t x = 0; x < c->nint; x += kCellItem) cells.push_back({0, 0, x, std::min<int64_t>(x + kCellItem, c->nint)});
   for (int d = 0; d < 2; ++d) {
     const int64_t nf = (c->dg.n[0] + (d == 0)) * (c->dg.n[1] + (d == 1));
@@ -441,6 +448,9 @@ hrm_status setup_persistent(hrm_ctx* c) {
   if ((s = cuda_check(c, ctx_malloc(c, &c->p_cells, sizeof(WorkItem) * cells.size()), "alloc items"))) return s;
   if ((s = cuda_check(c, ctx_malloc(c, &c->p_tiles, sizeof(WorkItem) * tiles.size()), "alloc tiles"))) return s;
   if ((s = cuda_check(c, ctx_malloc(c, &c->p_sync, sizeof(GridSync)), "alloc grid sync"))) return s;
+  const size_t listed = sizeof(uint64_t) * (size_t)(face_total(c->dg, 0) + face_total(c->dg, 1));
+  if ((s = cuda_check(c, ctx_malloc(c, &c->p_listed, listed), "alloc midpoint list"))) return s;
+  if ((s = cuda_check(c, ctx_malloc(c, &c->p_deferred, listed), "alloc deferred list"))) return s;
   if ((s = cuda_check(c, cudaMemcpyAsync(c->p_inst, &I, sizeof I, cudaMemcpyHostToDevice, c->stream), "copy instance")))
     return s;
   if ((s = cuda_check(c, cudaMemcpyAsync(c->p_cells, cells.data(), sizeof(WorkItem) * cells.size(),
@@ -453,11 +463,7 @@ hrm_status setup_persistent(hrm_ctx* c) {
   if ((s = cuda_check(c, cudaStreamSynchronize(c->stream), "persistent set-up"))) return s;
   c->p_ncell = (int)cells.size();
   c->p_ntiles = (int)tiles.size();
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  c->p_grid = sms * batch_stage32_fit();
-  return c->p_grid > 0 ? HRM_OK : fail(c, HRM_E_CUDA, "persistent stage kernel: no resident block fits an SM");
+  return HRM_OK;
 }
 
 // The three stage launches of one persistent step (SSP-RK3, Shu-Osher form).
@@ -484,6 +490,10 @@ hrm_status enqueue_persistent_step(hrm_ctx* c, cudaStream_t s) {
     A.pr = c->dp;
     A.sync = c->p_sync;
     A.limit_ns = 2000000000ull;
+    A.listed = c->p_listed;
+    A.deferred = c->p_deferred;
+    // the segments of this context's species count (the others stay empty)
+    A.seg[1] = A.seg[3] = face_total(c->dg, 0);
     A.stage = k;
     A.update = 1;
     hrm_status st;
@@ -829,6 +839,8 @@ void hrm_destroy(hrm_ctx* c) {
   ctx_free(c, c->p_cells);
   ctx_free(c, c->p_tiles);
   ctx_free(c, c->p_sync);
+  ctx_free(c, c->p_listed);
+  ctx_free(c, c->p_deferred);
   for (int i = 0; i < 2 * kMaxProf; ++i)
     if (c->prof_ev[i]) cudaEventDestroy(c->prof_ev[i]);
   if (c->cap) cudaStreamDestroy(c->cap);

@@ -43,7 +43,7 @@ constexpr int kBatchFace32Threads = 128;  // threads of the persistent kernel: o
 // ---------------------------------------------------------------- persistent stage kernel
 // One launch per RK stage for every instance: the primitive phase, at the first
 // stage the step scalars of every instance, the midpoint phase over
-// 128-midpoint tiles of both directions, the update phase -- separated by the
+// 128-midpoint tiles of both directions (stage_midpoints), the update phase -- separated by the
 // bounded grid barrier of hrm_sync.cuh. Blocks take work items from one queue
 // per phase; the cell items are grouped by species count and the tiles by
 // species count and direction, so that neighbouring items run the same code.
@@ -69,6 +69,12 @@ struct StageArgs {
   DevParams pr;
   GridSync* sync;
   uint64_t limit_ns;      // time limit of one barrier wait
+  // listed midpoints: (instance << 40 | midpoint), one segment per species count
+  // and direction starting at seg[key], and those deferred to the full body
+  // (key << 62 | instance << 40 | midpoint)
+  uint64_t* listed;
+  uint64_t* deferred;
+  int64_t seg[4];
   int stage;              // 0..2: slot of the phase stamps
   int update;             // 1: the update phase runs in this launch (0: the caller runs it after)
 };
@@ -104,18 +110,144 @@ __device__ __noinline__ void face32_full(int64_t t, const Nodes6& nd, const Batc
                                       I.st->lam[DIR], false, xs);
 }
 
+// Whether midpoint t of the tile is uniform, and if so its flux: the node's
+// physical flux with zero alpha slots.
 template <int N, int D, int DIR, bool FP32>
-__device__ __forceinline__ void stage_face(const BatchInst& I, int64_t t, int src, const DevParams& pr, float* xs) {
+__device__ __forceinline__ bool stage_uniform(const BatchInst& I, int64_t t, int src) {
+  using L = Lay<N, D>;
   Nodes6 nd;
-  if (!face_nodes<DIR>(I.g, t, nd)) return;
+  if (!face_nodes<DIR>(I.g, t, nd)) return true;
+  const double* W = pick(I, src);
+  const int64_t nc = I.g.ncells;
+  double G[L::NC];
   if constexpr (FP32) {
-    if (!face32_body<N, D, DIR, true, true>(t, nd, pick(I, src), nullptr, nullptr, I.P32, I.F[DIR], I.g, I.f, pr,
-                                            I.st->lam[DIR], false, xs))
-      face32_full<N, D, DIR>(t, nd, I, src, pr, xs);
+    if (!uniform_stencil<N, D>(I.P32, nc, nd)) return false;
+    uniform_flux32<N, D>(nd.c[2], DIR, I.P32, nc, G);
+  } else {
+    if (!uniform_nodes<N, D>(W, nc, nd)) return false;
+    uniform_flux64<N, D>(nd.c[2], DIR, W, I.V, nc, G);
+  }
+  const int64_t nf = face_count<DIR>(I.g);
+#pragma unroll
+  for (int m = 0; m < L::M + N - 1; ++m) I.F[DIR][m * nf + t] = m < L::NC ? G[m < L::NC ? m : 0] : 0.0;
+  return true;
+}
+
+// The body of listed midpoint t; false where the precision form's screens leave it
+// to the full body.
+template <int N, int D, int DIR, bool FP32>
+__device__ __forceinline__ bool stage_face(const BatchInst& I, int64_t t, int src, const DevParams& pr, float* xs) {
+  Nodes6 nd;
+  if (!face_nodes<DIR>(I.g, t, nd)) return true;
+  if constexpr (FP32) {
+    return face32_body<N, D, DIR, true, true>(t, nd, pick(I, src), nullptr, nullptr, I.P32, I.F[DIR], I.g, I.f, pr,
+                                              I.st->lam[DIR], false, xs);
   } else {
     face_body<N, D, DIR>(t, nd, pick(I, src), I.V, I.AUX, I.F[DIR], I.g, I.f, pr, I.st->lam[DIR],
                          reinterpret_cast<double*>(xs));
+    return true;
   }
+}
+
+// The midpoint phase, in three steps between grid barriers: every midpoint of the
+// tiles is tested for a uniform stencil and listed if it has none, by species
+// count and direction; warps take the listed ones 32 at a time; and in the
+// precision form those that its screens defer go to one lane of a warp each,
+// spread over the grid (each is a long FP64 chain, and in line it kept its block
+// from its next tile). False when a barrier ran out.
+template <int D, bool FP32>
+__device__ __forceinline__ bool stage_midpoints(const StageArgs& A, float* xs) {
+  constexpr uint64_t kMidpoint = (1ull << 40) - 1ull;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  __shared__ unsigned int wbase[kBatchFace32Threads / 32];
+  for (int it = next_item(A.sync, 1); it < A.ntiles; it = next_item(A.sync, 1)) {
+    const WorkItem w = A.tiles[it];
+    const BatchInst& I = A.insts[w.inst];
+    const int64_t t = w.begin + threadIdx.x;
+    const int key = (I.N - 2) * 2 + w.pad;
+    bool uni = true;
+    if (t < w.end) {
+      if (key == 0)
+        uni = stage_uniform<2, D, 0, FP32>(I, t, A.src);
+      else if (key == 1)
+        uni = stage_uniform<2, D, 1, FP32>(I, t, A.src);
+      else if (key == 2)
+        uni = stage_uniform<3, D, 0, FP32>(I, t, A.src);
+      else
+        uni = stage_uniform<3, D, 1, FP32>(I, t, A.src);
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, !uni);
+    if (lane == 0) wbase[warp] = __popc(m);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      unsigned int n = 0;
+      for (int k = 0; k < kBatchFace32Threads / 32; ++k) n += wbase[k];
+      unsigned int b = n ? atomicAdd(&A.sync->listed[key], n) : 0u;
+      for (int k = 0; k < kBatchFace32Threads / 32; ++k) {
+        const unsigned int c = wbase[k];
+        wbase[k] = b;
+        b += c;
+      }
+    }
+    __syncthreads();
+    if (!uni)
+      A.listed[A.seg[key] + wbase[warp] + __popc(m & ((1u << lane) - 1u))] = (uint64_t)w.inst << 40 | (uint64_t)t;
+  }
+  if (!grid_barrier(A.sync, gridDim.x, A.limit_ns)) return false;
+  {
+    volatile const unsigned int* listed = A.sync->listed;
+    unsigned int n[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) n[k] = listed[k];
+    for (;;) {
+      unsigned int g = 0;
+      __syncwarp();
+      if (lane == 0) g = atomicAdd(&A.sync->queue[3], 1u);
+      g = __shfl_sync(0xffffffffu, g, 0);
+      int key = 0;
+      while (key < 4 && g >= (n[key] + 31u) / 32u) {
+        g -= (n[key] + 31u) / 32u;
+        ++key;
+      }
+      if (key == 4) break;
+      const unsigned int i = g * 32u + lane;
+      bool done = true;
+      uint64_t e = 0;
+      if (i < n[key]) {
+        e = A.listed[A.seg[key] + i];
+        const BatchInst& I = A.insts[e >> 40];
+        const int64_t t = (int64_t)(e & kMidpoint);
+        if (key == 0)
+          done = stage_face<2, D, 0, FP32>(I, t, A.src, A.pr, xs);
+        else if (key == 1)
+          done = stage_face<2, D, 1, FP32>(I, t, A.src, A.pr, xs);
+        else if (key == 2)
+          done = stage_face<3, D, 0, FP32>(I, t, A.src, A.pr, xs);
+        else
+          done = stage_face<3, D, 1, FP32>(I, t, A.src, A.pr, xs);
+      }
+      if (!done) A.deferred[atomicAdd(&A.sync->deferred, 1u)] = (uint64_t)key << 62 | e;
+    }
+  }
+  if (!grid_barrier(A.sync, gridDim.x, A.limit_ns)) return false;
+  if constexpr (FP32) {
+    const unsigned int n = *(volatile const unsigned int*)&A.sync->deferred;
+    const unsigned int warps = gridDim.x * (kBatchFace32Threads / 32);
+    const unsigned int first = blockIdx.x + gridDim.x * warp;
+    for (uint64_t i = first + (uint64_t)lane * warps; i < n; i += 32ull * warps) {
+      const uint64_t e = A.deferred[i];
+      const int key = (int)(e >> 62);
+      const BatchInst& I = A.insts[e >> 40 & ((1ull << 22) - 1ull)];
+      const int64_t t = (int64_t)(e & kMidpoint);
+      Nodes6 nd;
+      if (key == 0 && face_nodes<0>(I.g, t, nd)) face32_full<2, D, 0>(t, nd, I, A.src, A.pr, xs);
+      if (key == 1 && face_nodes<1>(I.g, t, nd)) face32_full<2, D, 1>(t, nd, I, A.src, A.pr, xs);
+      if (key == 2 && face_nodes<0>(I.g, t, nd)) face32_full<3, D, 0>(t, nd, I, A.src, A.pr, xs);
+      if (key == 3 && face_nodes<1>(I.g, t, nd)) face32_full<3, D, 1>(t, nd, I, A.src, A.pr, xs);
+    }
+    if (n && !grid_barrier(A.sync, gridDim.x, A.limit_ns)) return false;
+  }
+  return true;
 }
 
 template <int N, int D, bool FP32>
@@ -182,23 +314,8 @@ __device__ __forceinline__ void batch_stage(const StageArgs& A) {
     if (!grid_barrier(A.sync, nb, A.limit_ns)) return;
   }
   if (stamper) stamp[2] = tc::global_ns();
-  for (int it = next_item(A.sync, 1); it < A.ntiles; it = next_item(A.sync, 1)) {
-    const WorkItem w = A.tiles[it];
-    const BatchInst& I = A.insts[w.inst];
-    const int64_t t = w.begin + threadIdx.x;
-    if (t >= w.end) continue;
-    const int key = I.N * 2 + w.pad;
-    if (key == 4)
-      stage_face<2, D, 0, FP32>(I, t, A.src, A.pr, xs);
-    else if (key == 5)
-      stage_face<2, D, 1, FP32>(I, t, A.src, A.pr, xs);
-    else if (key == 6)
-      stage_face<3, D, 0, FP32>(I, t, A.src, A.pr, xs);
-    else
-      stage_face<3, D, 1, FP32>(I, t, A.src, A.pr, xs);
-  }
+  if (!stage_midpoints<D, FP32>(A, xs)) return;
   if (A.update) {
-    if (!grid_barrier(A.sync, nb, A.limit_ns)) return;
     if (stamper) stamp[3] = tc::global_ns();
     for (int it = next_item(A.sync, 2); it < A.ncell_items; it = next_item(A.sync, 2)) {
       const WorkItem w = A.cells[it];
@@ -215,6 +332,18 @@ __device__ __forceinline__ void batch_stage(const StageArgs& A) {
     __threadfence();
     if (atomicAdd(&A.sync->done, 1u) == nb - 1u) stamp[4] = tc::global_ns();
   }
+}
+
+// Cells per item of the per-cell phases for `blocks` resident blocks: at least two
+// items per block, so that no block runs a long item while others have none, and
+// at most 4096 (a block takes 128 cells at a time). With 4096 cells always, 24
+// instances of 6000 cells kept 48 of 912 blocks busy; with this rule and the
+// midpoint phase's lists a stage launch over them takes 0.24 ms against 0.65, and
+// over 8 FP64 instances of 3000 cells 0.30 against 0.79; 64 instances of 11.35 M
+// cells 10.2 ms per FP32 step against 12.8 and 93.7 per FP64 step against 115.
+inline int default_cell_tile(int64_t cells, int64_t blocks) {
+  const int64_t t = (cells / (2 * blocks) + 127) / 128 * 128;
+  return (int)(t < 128 ? 128 : (t > 4096 ? 4096 : t));
 }
 
 // Persistent stage launchers for D = 2 (FP64: hrm_batch64_d2.cu, precision

@@ -22,7 +22,7 @@ using namespace hrm;
 namespace {
 
 struct Shape {
-  int cell_tile = 4096;   // cells per work item of the per-cell phases
+  int cell_tile = 4096;   // cells per work item of the per-cell phases (default_cell_tile at creation)
   int blocks_per_sm = 0;  // persistent grid = SMs x blocks_per_sm (0: all that fit)
 };
 
@@ -45,6 +45,9 @@ struct hrm_batch {
   int ncell_items = 0;
   WorkItem* d_tiles = nullptr;   // 128-midpoint tiles, grouped by species count and direction (in pad)
   int ntiles = 0;
+  uint64_t* d_listed = nullptr;  // the stage's non-uniform midpoints, a segment per species count and direction
+  uint64_t* d_deferred = nullptr;  // precision form: those left to the full body
+  int64_t seg[5] = {};           // segment starts
   GridSync* sync = nullptr;      // queues and barrier of the persistent launches
   unsigned int expired_seen = 0; // barrier waits that ran out, as last reported
   Shape shape;
@@ -159,6 +162,9 @@ hrm_status enqueue_stage(hrm_batch* b, cudaStream_t s, int stage) {
   A.pr = b->dp;
   A.sync = b->sync;
   A.limit_ns = kBarrierLimitNs;
+  A.listed = b->d_listed;
+  A.deferred = b->d_deferred;
+  for (int k = 0; k < 4; ++k) A.seg[k] = b->seg[k];
   A.stage = stage;
   A.update = 1;
   hrm_status st;
@@ -245,6 +251,8 @@ void hrm_batch_destroy(hrm_batch* b) {
   cudaFree(b->d_cells);
   cudaFree(b->d_tiles);
   cudaFree(b->sync);
+  cudaFree(b->d_listed);
+  cudaFree(b->d_deferred);
   if (b->cap) cudaStreamDestroy(b->cap);
   delete b;
 }
@@ -379,6 +387,22 @@ hrm_status hrm_batch_create(hrm_batch** out, int32_t ninst, const hrm_instance* 
   if ((s = bcuda(b, cudaMemcpy(b->d_insts, b->host.data(), sizeof(BatchInst) * ninst, cudaMemcpyHostToDevice),
                  "copy instances")))
     return bail(s);
+  // midpoints by species count and direction: the list's segments
+  for (int k = 0; k < 4; ++k) {
+    b->seg[k + 1] = b->seg[k];
+    for (int i = 0; i < ninst; ++i)
+      if (b->N[i] == 2 + k / 2) {
+        const DevGrid& g = b->host[i].g;
+        b->seg[k + 1] += (g.n[0] + (k % 2 == 0)) * (g.n[1] + (k % 2 == 1));
+      }
+  }
+  if (ninst >= 1 << 22 || b->seg[4] >= (int64_t)0xffffffffll)
+    return bail(bfail(b, HRM_E_NOMEM, "more midpoints or instances than the work lists address"));
+  if ((s = bcuda(b, cudaMalloc(&b->d_listed, sizeof(uint64_t) * (size_t)b->seg[4]), "alloc midpoint list"))) return bail(s);
+  if (p.precision == HRM_FP32 &&
+      (s = bcuda(b, cudaMalloc(&b->d_deferred, sizeof(uint64_t) * (size_t)b->seg[4]), "alloc deferred list")))
+    return bail(s);
+  b->shape.cell_tile = default_cell_tile(b->total_cells, grid_blocks(b));
   if ((s = build_items(b))) return bail(s);
   *out = b;
   return HRM_OK;

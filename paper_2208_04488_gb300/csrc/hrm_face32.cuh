@@ -459,20 +459,14 @@ __global__ void __launch_bounds__(kCellThreads)
   block_tau_max<D>(s, st->tau_bits);
 }
 
-// True when every FP32 plane holds the same value at the six nodes of a
-// midpoint (a NaN anywhere makes it false). One pass without branches, so
-// that many loads are in flight at once: measured on the 1024x512
-// shock-bubble, rounds of four planes with an exit after each, or
-// short-circuit compares (each load waiting for the previous compare), made
-// the check cost as much as the work it saves. PARTIAL: four planes per loop
-// trip instead of all of them unrolled, for the batched stage kernel, whose
-// register budget is shared with every phase (fully unrolled there, the
-// check's loads spilled: 16.6 against 11.8 ms per batched step). The result
-// is the same either way.
-template <int N, int D, bool PARTIAL = false>
+// True when every FP32 plane holds the same value at the six nodes of a midpoint
+// (a NaN anywhere makes it false). Four planes per loop trip: the batched stage
+// kernel that calls it shares its register budget with every phase (fully
+// unrolled, the loads spilled).
+template <int N, int D>
 __device__ __forceinline__ bool uniform_stencil(const float* __restrict__ P32, int64_t nc, const Nodes6& nd) {
   bool same = true;
-#pragma unroll(PARTIAL ? 4 : P32Lay<N, D>::PLANES)
+#pragma unroll 4
   for (int q = 0; q < P32Lay<N, D>::PLANES; ++q) {
     const float* p = P32 + (int64_t)q * nc;
     float v[6];
@@ -604,13 +598,13 @@ __global__ void __launch_bounds__(kCellThreads)
 // Returns true when the midpoint's outputs were written.
 // XSMEM: the per-thread column of biased values lives in `xs` (the caller's
 // shared memory, 2 x M x kFaceThreads floats) instead of a static array of its own.
-// nonuniform: the caller has found the stencil not uniform (uniform_stencil).
+// The stencil is known not to be uniform (uniform_flux32 otherwise).
 template <int N, int D, int DIR, bool DEFER = false, bool XSMEM = false>
 __device__ __forceinline__ bool face32_body(int64_t t, const Nodes6& nd, const double* __restrict__ W,
                                             const double* __restrict__ V, const double* __restrict__ AUX,
                                             const float* __restrict__ P32, double* __restrict__ out,
                                             const DevGrid& g, const DevFluid& f, const DevParams& pr, double lam,
-                                            bool lin = false, float* xs = nullptr, bool nonuniform = false) {
+                                            bool lin = false, float* xs = nullptr) {
   using L = Lay<N, D>;
   using Q = P32Lay<N, D>;
   constexpr int M = L::M;
@@ -657,39 +651,6 @@ __device__ __forceinline__ bool face32_body(int64_t t, const Nodes6& nd, const d
     load_node(3, Vj, nullptr);
     first_order(Vi, Vj, G);
   } else {
-    // Uniform stencil: the scheme's midpoint flux is then the node's physical
-    // flux with zero alpha slots, in exact arithmetic. WENO-IS reproduces a
-    // constant (App. C), so both interpolated states equal the node state; the
-    // HLLC flux of two equal states is their physical flux (Sec. 4.1.1); the HCS
-    // weights psi - 2 a1 + 2 a2 - 2 a3 sum to one, so any sensor blend returns
-    // it; the node state is a limiter's first-order candidate as well, so both
-    // positivity limiters, whatever their theta or hard switch, return it
-    // (Sec. 4.3.2); and with no alpha differences the quasi-conservative alpha
-    // slots vanish. Here that value is formed directly (the node flux of the
-    // conservative planes, as the HCS term reads it) instead of through rounded
-    // steps that would only cancel; every FP32 sweep takes the same exit, so
-    // they stay bit-identical to one another.
-    if (!nonuniform && uniform_stencil<N, D, XSMEM>(P32, nc, nd)) {
-      // (uniform_flux, written out here: as a call the sweep spills more)
-      const float un = ld(L::MOM + DIR, 2), pn = ld(L::EN, 2);
-#pragma unroll
-      for (int m = 0; m < L::NC; ++m) {
-        float v;
-        if (m < L::MOM)
-          v = ld(m, 2) * un;
-        else if (m < L::EN)
-          v = ld(Q::MOM + (m - L::MOM), 2) * un + ((m - L::MOM) == DIR ? pn : 0.f);
-        else
-          v = (ld(Q::E, 2) + pn) * un;
-        out[m * nf + t] = widen_f32(v);
-      }
-#pragma unroll
-      for (int k = 0; k < N - 1; ++k) {
-        out[(L::AL + k) * nf + t] = 0.0;
-        out[(M + k) * nf + t] = 0.0;
-      }
-      return true;
-    }
     float p6[6], u6[6];
 #pragma unroll
     for (int j = 0; j < 6; ++j) {
@@ -998,8 +959,7 @@ __global__ void __launch_bounds__(kFaceThreads, 6)
     bool need = false;
     if (i < n && face_nodes<DIR>(g, t, nd)) {
       const bool lin = gate != nullptr && gate[t] != 0;
-      need = !face32_body<N, D, DIR, true>(t, nd, W, nullptr, nullptr, P32, out, g, f, pr, st->lam[DIR], lin, nullptr,
-                                           true);
+      need = !face32_body<N, D, DIR, true>(t, nd, W, nullptr, nullptr, P32, out, g, f, pr, st->lam[DIR], lin);
     }
     defer_push(need, t, deferred, &cnt[2]);
   }
@@ -1023,7 +983,7 @@ __global__ void __launch_bounds__(kFaceThreads, 2)
     Nodes6 nd;
     if (!face_nodes<DIR>(g, t, nd)) continue;
     const bool lin = gate != nullptr && gate[t] != 0;
-    face32_body<N, D, DIR>(t, nd, W, nullptr, nullptr, P32, out, g, f, pr, st->lam[DIR], lin, nullptr, true);
+    face32_body<N, D, DIR>(t, nd, W, nullptr, nullptr, P32, out, g, f, pr, st->lam[DIR], lin);
   }
 }
 
@@ -1042,7 +1002,7 @@ __global__ void __launch_bounds__(kFaceThreads, 3)
     Nodes6 nd;
     if (!face_nodes<DIR>(g, t, nd)) continue;
     const bool lin = gate != nullptr && gate[t] != 0;
-    face32_body<N, D, DIR>(t, nd, W, V, AUX, P32, out, g, f, pr, st->lam[DIR], lin, nullptr, true);
+    face32_body<N, D, DIR>(t, nd, W, V, AUX, P32, out, g, f, pr, st->lam[DIR], lin);
   }
 }
 

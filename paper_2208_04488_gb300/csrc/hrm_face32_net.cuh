@@ -47,8 +47,7 @@ __global__ void __launch_bounds__(kFaceThreads, 6)
     if (in) {
       const bool lin = z > zthr;
       gate[t] = lin ? 1 : 0;
-      need = !face32_body<N, D, DIR, true>(t, nd, W, nullptr, nullptr, P32, out, g, f, pr, st->lam[DIR], lin, nullptr,
-                                           true);
+      need = !face32_body<N, D, DIR, true>(t, nd, W, nullptr, nullptr, P32, out, g, f, pr, st->lam[DIR], lin);
     }
     defer_push(need, t, deferred, &cnt[2]);
   }

@@ -138,8 +138,9 @@ __device__ __forceinline__ bool interp_limit_noop(const double* Vt, double rc2, 
 // and the N-1 alpha slots of G^+_{i+1/2} (planes M..M+N-2).
 // lin: the midpoint is gated smooth -- the WENO-IS weights are replaced by the
 // linear weights d_k; everything else is unchanged. col: kFaceCol doubles of
-// shared memory. LISTED: the six node states are known to differ (k_mark).
-template <int N, int D, int DIR, bool LISTED = false>
+// shared memory. The six node states are known to differ (a uniform stencil takes
+// the node's flux, uniform_flux64).
+template <int N, int D, int DIR>
 __device__ __forceinline__ void face_body(int64_t t, const Nodes6& nd, const double* __restrict__ W,
                                           const double* __restrict__ V, const double* __restrict__ AUX,
                                           double* __restrict__ out, const DevGrid& g, const DevFluid& f,
@@ -188,23 +189,6 @@ __device__ __forceinline__ void face_body(int64_t t, const Nodes6& nd, const dou
     store(H);
     return;
   }
-  if (!LISTED && uniform_nodes<N, D>(W, nc, nd)) {
-    // six bit-identical node states: in exact arithmetic every step below returns
-    // the node's physical flux with zero alpha slots -- constants are reproduced
-    // by the interpolation (App. C), the HLLC flux of equal states is their flux
-    // (Sec. 4.1.1), the HCS weights sum to one, alpha u - u alpha = 0 (Eq. G_pm),
-    // and the node state is the limiters' own candidate (Sec. 4.3.2)
-    FluxPack<N, D> G;
-    uniform_flux64<N, D>(nd.c[2], DIR, W, V, nc, G.Gc);
-#pragma unroll
-    for (int k = 0; k < N - 1; ++k) {
-      G.gm[k] = 0.0;
-      G.gp[k] = 0.0;
-    }
-    store(G);
-    return;
-  }
-
   double p6[6], u6[6];
 #pragma unroll
   for (int j = 0; j < 6; ++j) {
@@ -471,7 +455,7 @@ __global__ void __launch_bounds__(kFaceThreads, 3)
     const int64_t t = list[i];
     if (!face_nodes<DIR>(g, t, nd)) continue;
     const bool lin = gate != nullptr && gate[t] != 0;
-    face_body<N, D, DIR, true>(t, nd, W, V, AUX, out, g, f, pr, st->lam[DIR], col, lin);
+    face_body<N, D, DIR>(t, nd, W, V, AUX, out, g, f, pr, st->lam[DIR], col, lin);
   }
 }
 

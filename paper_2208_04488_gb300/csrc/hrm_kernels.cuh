@@ -462,8 +462,10 @@ __device__ __forceinline__ void count_bits(StepState* st, int b) {
 // The precision form's FP64 arithmetic writes its multiply-adds as explicit
 // fma(): its translation units are built without FMA contraction, so that every
 // FP32 expression rounds as written whichever kernel it is inlined into.
-// Flux of a uniform face in the precision form, from the FP32 planes of one of
-// its cells (the HCS node-flux expression): NC slots, the alpha slots are zero.
+// The same flux in the precision form, where every FP32 plane holds the same value
+// at the six nodes (uniform_stencil), from the planes of one of the cells (the HCS
+// node-flux expression). Formed directly instead of through rounded steps that
+// would only cancel; every FP32 sweep takes it, so they stay bit-identical.
 // Planes as in P32Lay: V, then c, rho, rho c^2, rho u_d, E.
 template <int N, int D>
 __device__ __forceinline__ void uniform_flux32(int64_t c, int d, const float* __restrict__ P32, int64_t nc, double* G) {
@@ -604,8 +606,12 @@ __device__ __forceinline__ bool stage_keeps_cell(int64_t c, const double* Wn, co
   return faces_unchanged<N, D>(c, F0, F1, F2, g) && (!with_wn || same_state<N, D>(c, Wn, Ws, nc));
 }
 
-// Flux of a uniform face from the state of one of its cells: the node's physical
-// flux F^d (NC conservative slots; the alpha slots are zero).
+// Flux of a midpoint whose six node states are bit-identical, from the state of
+// one of its cells: the node's physical flux F^d (NC conservative slots; the alpha
+// slots are zero). In exact arithmetic every step of the midpoint body returns it:
+// constants are reproduced by the interpolation (App. C), the HLLC flux of equal
+// states is their flux (Sec. 4.1.1), the HCS weights sum to one, alpha u - u alpha
+// = 0 (Eq. G_pm), and the node state is the limiters' own candidate (Sec. 4.3.2).
 template <int N, int D>
 __device__ __forceinline__ void uniform_flux64(int64_t c, int d, const double* __restrict__ W,
                                                const double* __restrict__ V, int64_t nc, double* G) {

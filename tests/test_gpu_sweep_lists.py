@@ -82,3 +82,19 @@ def test_precision_form_step_equals_its_stages(hrm, n, bc, where):
     np.testing.assert_array_equal(a.get(hrm.FIELD_W), b.get(hrm.FIELD_W))
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("where", ["none", "ends"])
+def test_batch_of_small_instances_equals_single_contexts(hrm, precision, where):
+    """The stage kernel's lists over instances smaller than a warp's, a tile's or a
+    work item's share, of both species counts."""
+    ps = [disturbed(n, bc, where, N) for n in ([3, 3], [33, 3], [5, 64], [257, 4]) for bc in (0, 1) for N in (2, 3)]
+    prm = hrm.params_default(cfl=0.4, check=0, precision=hrm.FP64 if precision == "fp64" else hrm.FP32)
+    b = hrm.BatchSolver(ps, params=prm)
+    b.step(3)
+    for i, pr in enumerate(ps):
+        s = hrm.Solver.from_problem(pr, params=prm)
+        s.step(0.0, 3)
+        np.testing.assert_array_equal(b.get(i), s.get(hrm.FIELD_W))
+        s.close()
