@@ -19,7 +19,7 @@ void face_l(int precision, const double* W, const double* V, const double* AUX, 
       return;
     }
     const long long nf = (g.n[0] + (DIR == 0)) * (g.n[1] + (DIR == 1)) * (g.n[2] + (DIR == 2));
-    k_face<N, kD, DIR><<<list_grid(g, DIR, 3), kFaceThreads, 0, s>>>(W, V, AUX, out, g, f, p, st, gate.fixed,
+    k_face<N, kD, DIR><<<list_grid(g, DIR, 3, 8), kFaceThreads, 0, s>>>(W, V, AUX, out, g, f, p, st, gate.fixed,
                                                                      gate.list, gate.list_cnt);
   }
 }

@@ -18,7 +18,7 @@ void face_l(int precision, const double* W, const double* V, const double* AUX, 
       face32_d3(N, DIR, W, V, AUX, P32, out, g, f, p, st, gate, s);
       return;
     }
-    k_face<N, kD, DIR><<<list_grid(g, DIR, 3), kFaceThreads, 0, s>>>(W, V, AUX, out, g, f, p, st, gate.fixed,
+    k_face<N, kD, DIR><<<list_grid(g, DIR, 3, 8), kFaceThreads, 0, s>>>(W, V, AUX, out, g, f, p, st, gate.fixed,
                                                                      gate.list, gate.list_cnt);
   }
 }

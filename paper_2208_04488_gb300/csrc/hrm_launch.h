@@ -161,13 +161,14 @@ void launch_mark(int N, int D, const double* W, const double* V, const float* P3
                  const SweepLists& lists, int all, cudaStream_t s);
 
 // Blocks of kFaceThreads of a list-driven sweep: what is resident at per_sm blocks
-// on each SM, or fewer where the whole midpoint grid needs no more.
-inline unsigned list_grid(const DevGrid& g, int dir, int per_sm) {
+// on each SM, or fewer where the whole midpoint grid needs no more at `lanes`
+// threads per midpoint.
+inline unsigned list_grid(const DevGrid& g, int dir, int per_sm, int lanes = 1) {
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const long long f = (g.n[0] + (dir == 0)) * (g.n[1] + (dir == 1)) * (g.n[2] + (dir == 2));
-  const long long all = (f + 127) / 128, fit = (long long)(sms > 0 ? sms : 1) * per_sm;
+  const long long all = (f * lanes + 127) / 128, fit = (long long)(sms > 0 ? sms : 1) * per_sm;
   return (unsigned)(all < fit ? all : fit);
 }
 
