@@ -59,6 +59,9 @@ struct hrm_ctx {
   // in 2D and 3D the sweeps of one stage run concurrently: direction d > 0 on par[d]
   cudaStream_t par[3] = {nullptr, nullptr, nullptr};
   cudaEvent_t ev_fork = nullptr, ev_join[3] = {};
+  // precision form: the unchanged cells are finished beside the sweeps here
+  cudaStream_t keep = nullptr;
+  cudaEvent_t ev_mark = nullptr, ev_keep = nullptr;
   int gate_set[3] = {0, 0, 0};     // fixed gate provided (hrm_set_gate)
   int gate_blocks = 0;             // persistent blocks of the gate kernel
   const CellKernels* ck = nullptr;
@@ -336,6 +339,16 @@ int enqueue_stage(hrm_ctx* c, cudaStream_t s, const double* Wsrc, double* Wout, 
       ++k;
     }
   k += enqueue_mark(c, s, Wsrc, c->params.precision == HRM_FP32 && !fuse_next);
+  Update32Args up{};
+  if (fuse_next) {
+    up = {c->Wn, Wsrc, Wout, c->F[0], c->F[1], c->F[2], c->st, a, b, relax, count, c->P32, r32_target(c),
+          c->lists.uni, src_relaxed ? 1 : 0};
+    cudaEventRecord(c->ev_mark, s);
+    cudaStreamWaitEvent(c->keep, c->ev_mark, 0);
+    launch_update32p(c->N, c->D, up, c->dg, c->fl, tau_next ? 1 : 0, c->lists, 0, c->keep);
+    cudaEventRecord(c->ev_keep, c->keep);
+    ++k;
+  }
   // the sweeps: independent (each reads the primitives and writes its own flux
   // planes), so directions d > 0 run on their own streams beside direction 0
   const bool fork = c->D > 1 && c->par[1];
@@ -366,10 +379,10 @@ int enqueue_stage(hrm_ctx* c, cudaStream_t s, const double* Wsrc, double* Wout, 
   });
   if (defer_sweep(c))
     for (int d = 0; d < c->D; ++d) cudaStreamWaitEvent(s, c->ev_fix[d], 0);
+  if (fuse_next) cudaStreamWaitEvent(s, c->ev_keep, 0);
   traced(c, s, HRM_KERNEL_UPDATE, [&] {
     if (fuse_next)
-      launch_update32p(c->N, c->D, c->Wn, Wsrc, Wout, c->F[0], c->F[1], c->F[2], c->dg, c->fl, c->st, a, b, relax,
-                       count, c->P32, r32_target(c), c->lists.uni, src_relaxed ? 1 : 0, s, tau_next ? 1 : 0);
+      launch_update32p(c->N, c->D, up, c->dg, c->fl, tau_next ? 1 : 0, c->lists, 1, s);
     else
       c->fk->update(0, c->params.precision == HRM_FP32, c->Wn, Wsrc, Wout, c->F[0], c->F[1], c->F[2], c->dg,
                     c->fl, c->st, a, b, relax, count, same_out ? same : nullptr,
@@ -777,6 +790,8 @@ hrm_status hrm_create(hrm_ctx** out, const hrm_grid* grid, int32_t N, const doub
   if ((s = cuda_check(c, ctx_malloc(c, &c->same, (size_t)c->nc), "alloc unchanged-cell flags"))) return bail(s);
   if ((s = cuda_check(c, ctx_malloc(c, &c->lists.eq, (size_t)c->nint), "alloc equality flags"))) return bail(s);
   if ((s = cuda_check(c, ctx_malloc(c, &c->lists.uni, (size_t)c->nint), "alloc uniform-face flags"))) return bail(s);
+  if ((s = cuda_check(c, ctx_malloc(c, &c->lists.cells, sizeof(uint32_t) * (size_t)c->nint), "alloc cell list")))
+    return bail(s);
   if ((s = cuda_check(c, ctx_malloc(c, &c->lists.cnt, sizeof(uint32_t) * kSweepCounters), "alloc sweep counters")))
     return bail(s);
   if (c->defer_cap >= (int64_t)0xffffffffll)  // (its flux planes alone would exceed the device)
@@ -792,6 +807,9 @@ hrm_status hrm_create(hrm_ctx** out, const hrm_grid* grid, int32_t N, const doub
     if ((s = cuda_check(c, cudaEventCreateWithFlags(&c->ev_fast[d], cudaEventDisableTiming), "event"))) return bail(s);
     if ((s = cuda_check(c, cudaEventCreateWithFlags(&c->ev_fix[d], cudaEventDisableTiming), "event"))) return bail(s);
   }
+  if ((s = cuda_check(c, cudaStreamCreateWithFlags(&c->keep, cudaStreamNonBlocking), "update stream"))) return bail(s);
+  if ((s = cuda_check(c, cudaEventCreateWithFlags(&c->ev_mark, cudaEventDisableTiming), "event"))) return bail(s);
+  if ((s = cuda_check(c, cudaEventCreateWithFlags(&c->ev_keep, cudaEventDisableTiming), "event"))) return bail(s);
   if (D > 1) {
     if ((s = cuda_check(c, cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming), "event"))) return bail(s);
     for (int d = 1; d < D; ++d) {
@@ -823,6 +841,7 @@ void hrm_destroy(hrm_ctx* c) {
   ctx_free(c, c->same);
   ctx_free(c, c->lists.eq);
   ctx_free(c, c->lists.uni);
+  ctx_free(c, c->lists.cells);
   ctx_free(c, c->lists.cnt);
   for (int d = 0; d < 3; ++d) ctx_free(c, c->lists.list[d]);
   ctx_free(c, c->defer);
@@ -852,6 +871,9 @@ void hrm_destroy(hrm_ctx* c) {
     if (c->ev_fix[d]) cudaEventDestroy(c->ev_fix[d]);
   }
   if (c->ev_fork) cudaEventDestroy(c->ev_fork);
+  if (c->keep) cudaStreamDestroy(c->keep);
+  if (c->ev_mark) cudaEventDestroy(c->ev_mark);
+  if (c->ev_keep) cudaEventDestroy(c->ev_keep);
   delete c;
 }
 

@@ -277,8 +277,9 @@ __device__ __forceinline__ void stage_update(const BatchInst& I, const WorkItem&
     if constexpr (FP32) {
       if (A.fuse_next) {
         // as k_update32p: combination, relaxation, store, next stage's FP32 planes
-        update32p_cell<N, D>(c, I.Wn, Wsrc, Wout, I.F[0], I.F[1], I.F[2], I.g, I.f, I.st, A.a, A.b, A.relax, 0,
-                             I.P32, nullptr);
+        const Update32Args U{I.Wn, Wsrc, Wout, I.F[0], I.F[1], I.F[2], I.st, A.a, A.b, A.relax, 0, I.P32, nullptr,
+                             nullptr, 0};
+        if (!update32p_keep<N, D>(c, U, I.g, I.f, nullptr)) update32p_change<N, D>(c, U, I.g, I.f, nullptr);
         continue;
       }
     }

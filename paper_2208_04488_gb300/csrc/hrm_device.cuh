@@ -96,13 +96,15 @@ __device__ __forceinline__ void cell_index(const DevGrid& g, int64_t c, int64_t*
 
 // Work of the list-driven sweeps (hrm_sweep.cuh): one byte per cell each for eq
 // and uni, a list of midpoints per direction with kSweepCounts counters (entries,
-// groups of 32 taken, deferred midpoints); F: the flux planes where the uniform
+// groups of 32 taken, deferred midpoints); cells: the cells that the stage's update
+// changes, with the fourth set of counters; F: the flux planes where the uniform
 // faces' fluxes are wanted as well; gate: the gate bytes where they are.
-constexpr int kSweepCounts = 4, kSweepCounters = 3 * kSweepCounts;
+constexpr int kSweepCounts = 4, kSweepCounters = 4 * kSweepCounts;
 struct SweepLists {
   uint8_t* eq = nullptr;
   uint8_t* uni = nullptr;
   uint32_t* list[3] = {nullptr, nullptr, nullptr};
+  uint32_t* cells = nullptr;
   uint32_t* cnt = nullptr;
   double* F[3] = {nullptr, nullptr, nullptr};
   uint8_t* gate[3] = {nullptr, nullptr, nullptr};
@@ -118,6 +120,29 @@ __device__ __forceinline__ bool next_entries(uint32_t* __restrict__ cnt, uint32_
   k = __shfl_sync(0xffffffffu, k, 0);
   i = k * 32u + (uint32_t)lane;
   return k < n / 32u + (n % 32u ? 1u : 0u);
+}
+
+// Appends value to a list where `need`, in thread order within the block, with one
+// atomic per block of at most 1024 threads (every thread calls it).
+__device__ __forceinline__ void block_append(bool need, uint32_t value, uint32_t* __restrict__ list,
+                                             uint32_t* __restrict__ count) {
+  __shared__ uint32_t base[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  const unsigned m = __ballot_sync(0xffffffffu, need);
+  if (lane == 0) base[warp] = __popc(m);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    uint32_t n = 0;
+    for (int w = 0; w < warps; ++w) n += base[w];
+    uint32_t b = n ? atomicAdd(count, n) : 0u;
+    for (int w = 0; w < warps; ++w) {
+      const uint32_t k = base[w];
+      base[w] = b;
+      b += k;
+    }
+  }
+  __syncthreads();
+  if (need) list[base[warp] + __popc(m & ((1u << lane) - 1u))] = value;
 }
 
 struct DevParams {

@@ -5,6 +5,7 @@
 #pragma once
 
 #include "hrm_cell.cuh"
+#include "hrm_launch.h"
 
 namespace hrm {
 
@@ -497,99 +498,118 @@ __device__ __forceinline__ void defer_push(bool need, int64_t t, uint32_t* __res
 // in place of a separate k_prim32 pass over W_out. Interior cells only: the
 // planes of Dirichlet slices keep what the stage's first primitive pass wrote
 // (their states do not change).
+// The cell's five-equation CFL speeds (|u_d| + c) / dx_d, as k_prim32 forms them.
+template <int D>
+__device__ __forceinline__ void speeds32(const DevGrid& g, const float* u, float cs, double* s) {
+#pragma unroll
+  for (int d = 0; d < D; ++d) s[d] = widen_f32((fabsf(u[d]) + cs) * narrow_f64(g.inv_dx[d]));
+}
+
+// Cells that the stage returns as they are (see stage_keeps_cell; with uni no flux
+// difference means that all faces are uniform): done here, and true. From a step's
+// second relaxed stage on W_src's conserved variables being W^n's is enough, for
+// the relaxation forms W_src's volume fractions again. s (nullable): CFL speeds.
 template <int N, int D>
-__device__ __forceinline__ void update32p_cell(int64_t c, const double* Wn, const double* Wsrc, double* Wout,
-                                               const double* __restrict__ F0, const double* __restrict__ F1,
-                                               const double* __restrict__ F2, const DevGrid& g, const DevFluid& f,
-                                               StepState* st, double a, double b, int relax, int count,
-                                               float* __restrict__ P32, float* __restrict__ R32,
-                                               double* s = nullptr, const uint8_t* __restrict__ uni = nullptr,
-                                               int src_relaxed = 0) {
+__device__ __forceinline__ bool update32p_keep(int64_t c, const Update32Args& A, const DevGrid& g, const DevFluid& f,
+                                               double* s) {
   using L = Lay<N, D>;
   using Q = P32Lay<N, D>;
   constexpr int M = L::M;
   const int64_t nc = g.ncells;
-  // the cell's five-equation CFL speeds (|u_d| + c) / dx_d, as k_prim32 forms them
-  auto speeds = [&](const float* u, float cs) {
+  const bool with_wn = A.a != 0.0;
+  if (A.uni && A.uni[c] != (1u << 2 * D) - 1u) return false;
+  const bool by_wn = !A.relax || A.st->wn_relaxed, by_source = with_wn && A.relax && A.src_relaxed;
+  if (!by_wn && !(A.uni && by_source)) return false;
+  double Ws[M];
 #pragma unroll
-    for (int d = 0; d < D; ++d) s[d] = widen_f32((fabsf(u[d]) + cs) * narrow_f64(g.inv_dx[d]));
-  };
-  double Ws[M], Wo[M];
-#pragma unroll
-  for (int m = 0; m < M; ++m) Ws[m] = Wsrc[m * nc + c];
-  const bool with_wn = a != 0.0;
-  const unsigned ub = uni ? uni[c] : 0u;
-  // Unchanged cells (see stage_keeps_cell; here no flux difference means that all
-  // faces are uniform). From a step's second relaxed stage on (src_relaxed) W_src
-  // came out of relax_fast: then its conserved variables being W^n's is enough,
-  // for the relaxation forms W_src's volume fractions again.
-  bool keep, by_src = false;
-  if (uni) {
-    keep = ub == (1u << 2 * D) - 1u;
-    if (keep && with_wn) {
-      by_src = relax && src_relaxed && same_state<N, D>(c, Wn, Ws, nc, L::NC);
-      keep = by_src || ((!relax || st->wn_relaxed) && same_state<N, D>(c, Wn, Ws, nc));
-    } else {
-      keep = keep && (!relax || st->wn_relaxed);
-    }
-  } else {
-    keep = (!relax || st->wn_relaxed) && stage_keeps_cell<N, D>(c, Wn, Ws, F0, F1, F2, g, with_wn);
+  for (int m = 0; m < M; ++m) Ws[m] = A.Wsrc[m * nc + c];
+  bool by_src = false;
+  if (A.uni) {
+    by_src = by_source && same_state<N, D>(c, A.Wn, Ws, nc, L::NC);
+    if (!by_src && !(by_wn && (!with_wn || same_state<N, D>(c, A.Wn, Ws, nc)))) return false;
+  } else if (!stage_keeps_cell<N, D>(c, A.Wn, Ws, A.F0, A.F1, A.F2, g, with_wn)) {
+    return false;
   }
-  if (keep) {
-    // W_out = W_src exactly, and the planes already hold those of W_src
-    if (Wout != Wsrc && !(with_wn && Wout == Wn)) {
+  // W_out = W_src exactly, and the planes already hold those of W_src
+  if (A.Wout != A.Wsrc && !(with_wn && A.Wout == A.Wn)) {
 #pragma unroll
-      for (int m = 0; m < M; ++m) Wout[m * nc + c] = Ws[m];
-    } else if (by_src && Wout == Wn) {
+    for (int m = 0; m < M; ++m) A.Wout[m * nc + c] = Ws[m];
+  } else if (by_src && A.Wout == A.Wn) {
 #pragma unroll
-      for (int k = 0; k < N - 1; ++k) Wout[(L::AL + k) * nc + c] = Ws[L::AL + k];
-    }
-    if (count) count_bits(st, admissibility_bits<N, D>(Ws, f));
-    if (s) {
-      float u[D];
-#pragma unroll
-      for (int d = 0; d < D; ++d) u[d] = P32[(int64_t)(L::MOM + d) * nc + c];
-      speeds(u, P32[(int64_t)Q::C * nc + c]);
-    }
-    return;
+    for (int k = 0; k < N - 1; ++k) A.Wout[(L::AL + k) * nc + c] = Ws[L::AL + k];
   }
-  fast_combine<N, D>(c, Wn, Ws, F0, F1, F2, g, st->dt, a, b, Wo, ub, P32);
-  double rho, Re;
-  if (relax)
-    relax_fast<N, D>(Wo, f, rho, Re);
-  else
-    rho_Re<N, D>(Wo, f, rho, Re);
-  if (count) count_bits(st, admissibility_bits<N, D>(Wo, f));
+  if (A.count) count_bits(A.st, admissibility_bits<N, D>(Ws, f));
+  if (s) {
+    float u[D];
 #pragma unroll
-  for (int m = 0; m < M; ++m) Wout[m * nc + c] = Wo[m];
-  float u[D], cs;
-  prim32_store<N, D>(c, Wo, rho, Re, P32, R32, nc, f, u, cs);
-  if (s) speeds(u, cs);
+    for (int d = 0; d < D; ++d) u[d] = A.P32[(int64_t)(L::MOM + d) * nc + c];
+    speeds32<D>(g, u, A.P32[(int64_t)Q::C * nc + c], s);
+  }
+  return true;
 }
 
+// Any other cell.
+template <int N, int D, bool SOFT = false>
+__device__ __forceinline__ void update32p_change(int64_t c, const Update32Args& A, const DevGrid& g, const DevFluid& f,
+                                                 double* s) {
+  constexpr int M = Lay<N, D>::M;
+  const int64_t nc = g.ncells;
+  double Ws[M], Wo[M];
+#pragma unroll
+  for (int m = 0; m < M; ++m) Ws[m] = A.Wsrc[m * nc + c];
+  fast_combine<N, D>(c, A.Wn, Ws, A.F0, A.F1, A.F2, g, A.st->dt, A.a, A.b, Wo, A.uni ? A.uni[c] : 0u, A.P32);
+  double rho, Re;
+  if (A.relax)
+    relax_fast<N, D, SOFT>(Wo, f, rho, Re);
+  else
+    rho_Re<N, D>(Wo, f, rho, Re);
+  if (A.count) count_bits(A.st, admissibility_bits<N, D>(Wo, f));
+#pragma unroll
+  for (int m = 0; m < M; ++m) A.Wout[m * nc + c] = Wo[m];
+  float u[D], cs;
+  prim32_store<N, D>(c, Wo, rho, Re, A.P32, A.R32, nc, f, u, cs);
+  if (s) speeds32<D>(g, u, cs, s);
+}
+
+// The update in two kernels. k_keep32 finishes the cells that the stage leaves
+// unchanged and lists the others; what it needs is known before the sweeps, so it
+// runs beside them (it is bound by memory, they by latency). k_update32p then
+// takes the listed cells, 32 to a warp: they come in bands (fronts, interfaces)
+// that are often narrower than a warp, and a warp pays the FP64 work of all its
+// lanes. One kernel over all cells took 3.1 ms per launch on the 256^3 interface's
+// stages 2 and 3, with 10 of 32 lanes active in the changed cells' warps; now the
+// listed cells take 0.9 to 1.0 ms after the sweeps.
+// tau: a step's last stage, the next step's CFL maxima as well, which k_prim32 then
+// leaves as they are (grids without Dirichlet slices, whose cells these kernels do
+// not cover).
 template <int N, int D>
 __global__ void __launch_bounds__(kCellThreads)
-    k_update32p(const double* Wn, const double* Wsrc, double* Wout, const double* __restrict__ F0,
-                const double* __restrict__ F1, const double* __restrict__ F2, DevGrid g, DevFluid f,
-                StepState* st, double a, double b, int relax, int count, float* __restrict__ P32,
-                float* __restrict__ R32, int tau, const uint8_t* __restrict__ uni, int src_relaxed) {
-  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (!tau) {
-    if (c >= g.nint) return;
-    update32p_cell<N, D>(c, Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count, P32, R32, nullptr, uni,
-                         src_relaxed);
-    return;
-  }
-  // a step's last stage (tau): the next step's planes and CFL maxima as well,
-  // which k_prim32 then leaves as they are (grids without Dirichlet slices,
-  // whose cells this kernel does not cover)
+    k_keep32(Update32Args A, DevGrid g, DevFluid f, int tau, uint32_t* __restrict__ cells, uint32_t* __restrict__ cnt) {
+  const int64_t c = (int64_t)blockIdx.x * kCellThreads + threadIdx.x;
   double s[D];
 #pragma unroll
   for (int d = 0; d < D; ++d) s[d] = 0.0;
-  if (c < g.nint)
-    update32p_cell<N, D>(c, Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count, P32, R32, s, uni,
-                         src_relaxed);
-  block_tau_max<D>(s, st->tau_bits);
+  const bool changed = c < g.nint && !update32p_keep<N, D>(c, A, g, f, tau ? s : nullptr);
+  block_append(changed, (uint32_t)c, cells, cnt);
+  if (tau) block_tau_max<D>(s, A.st->tau_bits);
+}
+
+template <int N, int D>
+__global__ void __launch_bounds__(kCellThreads, 3)
+    k_update32p(Update32Args A, DevGrid g, DevFluid f, int tau, const uint32_t* __restrict__ cells,
+                uint32_t* __restrict__ cnt) {
+  double s[D], sc[D];
+#pragma unroll
+  for (int d = 0; d < D; ++d) s[d] = sc[d] = 0.0;
+  const uint32_t n = cnt[0];
+  uint32_t i;
+  while (next_entries(cnt, n, i)) {
+    if (i >= n) continue;
+    update32p_change<N, D, true>(cells[i], A, g, f, tau ? sc : nullptr);
+#pragma unroll
+    for (int d = 0; d < D; ++d) s[d] = (sc[d] != sc[d]) ? sc[d] : (sc[d] > s[d] ? sc[d] : s[d]);
+  }
+  if (tau) block_tau_max<D>(s, A.st->tau_bits);
 }
 
 // DEFER: where a screen fails (or for the first-order scheme) return false

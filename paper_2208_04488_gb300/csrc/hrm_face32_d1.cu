@@ -44,17 +44,22 @@ void update32_d1(int N, const double* Wn, const double* Wsrc, double* Wout, cons
     k_update<3, kD, 0, true><<<gr, kCellThreads, 0, s>>>(Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count);
 }
 
-void update32p_d1(int N, const double* Wn, const double* Wsrc, double* Wout, const double* F0, const double* F1,
-                  const double* F2, const DevGrid& g, const DevFluid& f, StepState* st, double a, double b, int relax,
-                  int count, float* P32, float* R32, int tau, const uint8_t* uni, int src_relaxed,
-                  cudaStream_t s) {
-  const unsigned gr = grid_for(g.nint, kCellThreads);
+void update32p_d1(int N, const Update32Args& A, const DevGrid& g, const DevFluid& f, int tau, const SweepLists& lists,
+                  int phase, cudaStream_t s) {
+  uint32_t* cnt = lists.cnt + 3 * kSweepCounts;
+  if (phase == 0) {
+    const unsigned gr = grid_for(g.nint, kCellThreads);
+    if (N == 2)
+      k_keep32<2, kD><<<gr, kCellThreads, 0, s>>>(A, g, f, tau, lists.cells, cnt);
+    else if (N == 3)
+      k_keep32<3, kD><<<gr, kCellThreads, 0, s>>>(A, g, f, tau, lists.cells, cnt);
+    return;
+  }
+  const unsigned gr = resident_grid(g.nint, kCellThreads, 3);
   if (N == 2)
-    k_update32p<2, kD><<<gr, kCellThreads, 0, s>>>(Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count, P32, R32,
-                                                    tau, uni, src_relaxed);
+    k_update32p<2, kD><<<gr, kCellThreads, 0, s>>>(A, g, f, tau, lists.cells, cnt);
   else if (N == 3)
-    k_update32p<3, kD><<<gr, kCellThreads, 0, s>>>(Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count, P32, R32,
-                                                    tau, uni, src_relaxed);
+    k_update32p<3, kD><<<gr, kCellThreads, 0, s>>>(A, g, f, tau, lists.cells, cnt);
 }
 
 void face32_d1(int N, int dir, const double* W, const double* V, const double* AUX, const float* P32, double* out,

@@ -341,8 +341,10 @@ __device__ __forceinline__ bool uniform_nodes(const double* __restrict__ W, int6
 // Eq. T_relax_e gives T* = R_e (p* + p_inf,1) / (rho Y), and the relaxed volume
 // fractions alpha_k = alpha_k rho_k R_k T* / (p* + p_inf,k) share one division
 // z = R_e / (rho Y p*). Two divisions and one square root per cell. Returns rho
-// and R_e for a primitive evaluation that follows.
-template <int N, int D>
+// and R_e for a primitive evaluation that follows. SOFT: products on the integer
+// pipes (where the registers allow three blocks of 256 per SM, 1-4 % of a pass; in
+// the batched stage kernel's 80 registers they cost 2 %).
+template <int N, int D, bool SOFT = false>
 __device__ __forceinline__ void relax_fast(double* W, const DevFluid& f, double& rho_out, double& Re_out,
                                            double* pT = nullptr) {
   using L = Lay<N, D>;
@@ -360,19 +362,22 @@ __device__ __forceinline__ void relax_fast(double* W, const DevFluid& f, double&
   }
 #pragma unroll
   for (int d = 0; d < D; ++d) m2 = fma(W[L::MOM + d], W[L::MOM + d], m2);
-  const double Re = fma(rho, W[L::EN] - rq, -0.5 * m2);
-  const double pinf1 = f.pinf[l], Wl = W[l], WlR1 = Wl * f.Rg[l];
-  const double A = rho * Cv;
-  const double B = fma(pinf1 * rho, Cv + WlR1, -(Re * Rm));
-  const double C = -(Re * pinf1 * (Rm - WlR1));
-  const double sq = rsqrt_r(fma(B, B, -4.0 * A * C));
-  const double ps = (B > 0.0) ? quot(-2.0 * C, B + sq) : quot(sq - B, 2.0 * A);
+  auto mul = [](double x, double y) { return SOFT ? prod(x, y) : x * y; };
+  const double Re = fma(rho, W[L::EN] - rq, -halved(m2));
+  const double pinf1 = f.pinf[l], Wl = W[l], WlR1 = mul(Wl, f.Rg[l]);
+  const double A = mul(rho, Cv);
+  const double B = fma(mul(pinf1, rho), Cv + WlR1, -mul(Re, Rm));
+  const double C = -mul(mul(Re, pinf1), Rm - WlR1);
+  const double sq = rsqrt_r(fma(B, B, mul(soft::scale<2>(-A), C)));
+  const bool pos = B > 0.0;
+  const double ps = quot(pos ? soft::scale<1>(-C) : sq - B, pos ? B + sq : soft::scale<1>(A));
   const double ppl = ps + pinf1;
-  const double Y = fma(Wl * fma(f.gamma[l], pinf1, ps), f.cv[l], fma(-Wl, f.cv[l], Cv) * ppl);
-  const double z = quot(Re, rho * Y * ps);
+  const double Y = fma(mul(Wl, fma(f.gamma[l], pinf1, ps)), f.cv[l], mul(fma(-Wl, f.cv[l], Cv), ppl));
+  const double z = quot(Re, mul(mul(rho, Y), ps));
 #pragma unroll
-  for (int k = 0; k < N - 1; ++k)  // alpha_k = rho_k' R_k T* / (p* + p_inf,k), one stiffened gas at most
-    W[L::AL + k] = W[k] * f.Rg[k] * (k == l ? ps : ppl) * z;
+  for (int k = 0; k < N - 1; ++k)
+    // alpha_k = rho_k' R_k T* / (p* + p_inf,k), one stiffened gas at most
+    W[L::AL + k] = mul(mul(mul(W[k], f.Rg[k]), k == l ? ps : ppl), z);
   if (pT) {
     pT[0] = ps;
     pT[1] = z * ps * ppl;
@@ -405,20 +410,22 @@ __device__ __forceinline__ void relax_cell(double* W, const DevFluid& f, double*
   double cvb = 0.0, cpb = 0.0;
 #pragma unroll
   for (int k = 0; k < N; ++k) {
-    cvb += Y[k] * f.cv[k];
-    cpb += Y[k] * f.cp[k];
+    cvb += prod(Y[k], f.cv[k]);
+    cpb += prod(Y[k], f.cp[k]);
   }
   const double pinf1 = f.pinf[l], R1 = f.Rg[l], Yl = Y[l];
-  const double Ap = cvb;
-  const double Bp = -(re * (cpb - cvb) - pinf1 * cvb - pinf1 * Yl * R1);
-  const double Cp = -(re * pinf1 * ((cpb - cvb) - Yl * R1));
-  const double sq = rsqrt_r(Bp * Bp - 4.0 * Ap * Cp);
-  const double ps = (Bp > 0.0) ? quot(-2.0 * Cp, Bp + sq) : quot(sq - Bp, 2.0 * Ap);
-  const double den = quot(Yl * (ps + f.gamma[l] * pinf1) * f.cv[l], ps + pinf1) + cvb - Yl * f.cv[l];
+  const double Ap = cvb, Rb = cpb - cvb, YR = prod(Yl, R1);
+  const double Bp = -(prod(re, Rb) - prod(pinf1, cvb) - prod(prod(pinf1, Yl), R1));
+  const double Cp = -prod(prod(re, pinf1), Rb - YR);
+  const double sq = rsqrt_r(prod(Bp, Bp) - prod(soft::scale<2>(Ap), Cp));
+  const bool pos = Bp > 0.0;
+  const double ps = quot(pos ? soft::scale<1>(-Cp) : sq - Bp, pos ? Bp + sq : soft::scale<1>(Ap));
+  const double pl = ps + pinf1;
+  const double den = quot(prod(prod(Yl, ps + prod(f.gamma[l], pinf1)), f.cv[l]), pl) + cvb - prod(Yl, f.cv[l]);
   const double Ts = quot(quot(re, rho), den);
 #pragma unroll
   for (int k = 0; k < N - 1; ++k) {
-    const double rhok = quot(ps + f.pinf[k], f.Rg[k] * Ts);
+    const double rhok = quot(ps + f.pinf[k], prod(f.Rg[k], Ts));
     W[L::AL + k] = quot(W[k], rhok);
   }
   if (pT) {

@@ -109,30 +109,37 @@ void face32_d3(int N, int dir, const double* W, const double* V, const double* A
                const DevGrid&, const DevFluid&, const DevParams&, const StepState*, const GateArgs& gate,
                cudaStream_t);
 
-// Precision-form update fused with the next stage's FP32 planes (k_update32p;
-// hrm_face32_dD.cu).
-void update32p_d1(int N, const double* Wn, const double* Wsrc, double* Wout, const double* F0, const double* F1,
-                  const double* F2, const DevGrid&, const DevFluid&, StepState*, double a, double b, int relax,
-                  int count, float* P32, float* R32, int tau, const uint8_t* uni, int src_relaxed,
+// Precision-form update fused with the next stage's FP32 planes (hrm_face32_dD.cu):
+// phase 0 finishes the unchanged cells and lists the others (any time after the
+// lists were built, beside the sweeps), phase 1 updates the listed ones. tau: also
+// accumulate the CFL maxima of W_out into st->tau_bits (a step's last stage; grids
+// without Dirichlet slices, five-equation sound speed).
+struct Update32Args {
+  const double* Wn;
+  const double* Wsrc;
+  double* Wout;
+  const double* F0;
+  const double* F1;
+  const double* F2;
+  StepState* st;
+  double a, b;
+  int relax, count;
+  float* P32;
+  float* R32;
+  const uint8_t* uni;  // nullable: the cells' uniform faces (k_mark; their fluxes are not read)
+  int src_relaxed;     // W_src came out of the form's relaxation (a step's second relaxed stage on)
+};
+void update32p_d1(int N, const Update32Args& A, const DevGrid&, const DevFluid&, int tau, const SweepLists&, int phase,
                   cudaStream_t);
-void update32p_d2(int N, const double* Wn, const double* Wsrc, double* Wout, const double* F0, const double* F1,
-                  const double* F2, const DevGrid&, const DevFluid&, StepState*, double a, double b, int relax,
-                  int count, float* P32, float* R32, int tau, const uint8_t* uni, int src_relaxed,
+void update32p_d2(int N, const Update32Args& A, const DevGrid&, const DevFluid&, int tau, const SweepLists&, int phase,
                   cudaStream_t);
-void update32p_d3(int N, const double* Wn, const double* Wsrc, double* Wout, const double* F0, const double* F1,
-                  const double* F2, const DevGrid&, const DevFluid&, StepState*, double a, double b, int relax,
-                  int count, float* P32, float* R32, int tau, const uint8_t* uni, int src_relaxed,
+void update32p_d3(int N, const Update32Args& A, const DevGrid&, const DevFluid&, int tau, const SweepLists&, int phase,
                   cudaStream_t);
-// uni (nullable): the cells' uniform faces (k_mark; their fluxes are not read);
-// tau: also accumulate the CFL maxima of W_out into st->tau_bits (a step's last
-// stage; grids without Dirichlet slices, five-equation sound speed).
-inline void launch_update32p(int N, int D, const double* Wn, const double* Wsrc, double* Wout, const double* F0,
-                             const double* F1, const double* F2, const DevGrid& g, const DevFluid& f, StepState* st,
-                             double a, double b, int relax, int count, float* P32, float* R32, const uint8_t* uni,
-                             int src_relaxed, cudaStream_t s, int tau = 0) {
-  if (D == 1) update32p_d1(N, Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count, P32, R32, tau, uni, src_relaxed, s);
-  if (D == 2) update32p_d2(N, Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count, P32, R32, tau, uni, src_relaxed, s);
-  if (D == 3) update32p_d3(N, Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count, P32, R32, tau, uni, src_relaxed, s);
+inline void launch_update32p(int N, int D, const Update32Args& A, const DevGrid& g, const DevFluid& f, int tau,
+                             const SweepLists& lists, int phase, cudaStream_t s) {
+  if (D == 1) update32p_d1(N, A, g, f, tau, lists, phase, s);
+  if (D == 2) update32p_d2(N, A, g, f, tau, lists, phase, s);
+  if (D == 3) update32p_d3(N, A, g, f, tau, lists, phase, s);
 }
 
 // Primitive kernel of the precision form (FP32 planes only; hrm_face32_dD.cu).
@@ -160,16 +167,20 @@ inline unsigned grid_for(long long n, int threads) { return (unsigned)((n + thre
 void launch_mark(int N, int D, const double* W, const double* V, const float* P32, const DevGrid& g,
                  const SweepLists& lists, int all, cudaStream_t s);
 
-// Blocks of kFaceThreads of a list-driven sweep: what is resident at per_sm blocks
-// on each SM, or fewer where the whole midpoint grid needs no more at `lanes`
-// threads per midpoint.
-inline unsigned list_grid(const DevGrid& g, int dir, int per_sm, int lanes = 1) {
+// Blocks for up to n items of a list that its warps take from a counter: what is
+// resident at per_sm blocks on each SM, or fewer where n needs no more.
+inline unsigned resident_grid(long long n, int threads, int per_sm) {
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const long long f = (g.n[0] + (dir == 0)) * (g.n[1] + (dir == 1)) * (g.n[2] + (dir == 2));
-  const long long all = (f * lanes + 127) / 128, fit = (long long)(sms > 0 ? sms : 1) * per_sm;
+  const long long all = (n + threads - 1) / threads, fit = (long long)(sms > 0 ? sms : 1) * per_sm;
   return (unsigned)(all < fit ? all : fit);
+}
+
+// Blocks of kFaceThreads of a list-driven sweep at `lanes` threads per midpoint.
+inline unsigned list_grid(const DevGrid& g, int dir, int per_sm, int lanes = 1) {
+  const long long f = (g.n[0] + (dir == 0)) * (g.n[1] + (dir == 1)) * (g.n[2] + (dir == 2));
+  return resident_grid(f * lanes, 128, per_sm);
 }
 
 // Smallest float not below x (thresholds of the FP32 screens).
