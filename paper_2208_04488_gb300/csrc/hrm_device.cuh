@@ -241,6 +241,10 @@ __device__ __forceinline__ float rsqrt_r(float x) { return sqrtf(x); }
 // exp(y) = 2^k exp(r) with Cody-Waite reduction (y = k ln2 + r, ln2 split into
 // a 32-bit head and its tail) and the Taylor series of exp(r); 1 above 22.
 // Built without contraction, every rounding is fixed by the expression order.
+__constant__ const double kInverse[19] = {0.0,        1.0,        1.0 / 2.0,  1.0 / 3.0,  1.0 / 4.0,  1.0 / 5.0,  1.0 / 6.0,
+                                          1.0 / 7.0,  1.0 / 8.0,  1.0 / 9.0,  1.0 / 10.0, 1.0 / 11.0, 1.0 / 12.0,
+                                          1.0 / 13.0, 1.0 / 14.0, 1.0 / 15.0, 1.0 / 16.0, 1.0 / 17.0, 1.0 / 18.0};
+template <bool SOFT>
 __device__ __forceinline__ double tanh_r(double x) {
   constexpr double kLn2 = 0.6931471805599453;
   constexpr double kLn2Hi = 0.6931471803691238;
@@ -253,25 +257,29 @@ __device__ __forceinline__ double tanh_r(double x) {
     t = 1.0;
   } else {
     const double y = 2.0 * ax;
-    double m;
-    if (y < 0.5) {
-      double s = 1.0;
+    const bool small = y < 0.5;
+    const double k = small ? 0.0 : rint(quot(y, kLn2));
+    const double r = small ? y : (y - k * kLn2Hi) - k * kLn2Lo;
+    // both series are s = 1 + (r / j) s from the last term down: expm1 to j = 2,
+    // exp to j = 1. SOFT: one loop, its products beside the FP64 unit (unrolled for
+    // either branch they were a tenth of a midpoint's FP64 instructions); else
+    // unrolled, the shorter chain for a lone warp.
+    double s = 1.0;
+    if constexpr (SOFT) {
+#pragma unroll 1
+      for (int j = small ? 18 : 17; j >= (small ? 2 : 1); --j) s = 1.0 + prod(prod(r, kInverse[j]), s);
+    } else if (small) {
 #pragma unroll
-      for (int k = 18; k >= 2; --k) s = 1.0 + (y * (1.0 / (double)k)) * s;
-      m = y * s;
+      for (int j = 18; j >= 2; --j) s = 1.0 + (r * (1.0 / (double)j)) * s;
     } else {
-      const double k = rint(quot(y, kLn2));
-      const double r = (y - k * kLn2Hi) - k * kLn2Lo;
-      double s = 1.0;
 #pragma unroll
       for (int j = 17; j >= 1; --j) s = 1.0 + (r * (1.0 / (double)j)) * s;
-      m = ldexp(s, (int)k) - 1.0;
     }
+    const double m = small ? y * s : ldexp(s, (int)k) - 1.0;
     t = quot(m, m + 2.0);
   }
   return x < 0.0 ? -t : t;
 }
-__device__ __forceinline__ float tanh_r(float x) { return tanhf(x); }
 
 // Index of cell j (may lie in the 3 ghost layers) along direction d under the
 // boundary condition of that side: transmissive copies the first interior cell

@@ -24,6 +24,17 @@
 
 namespace hrm {
 
+// 1, 2, 4 and 1/4 in registers, unknown to the compiler (read from memory once per
+// thread).
+struct FmaUnits {
+  double one, two, four, quarter;
+};
+__device__ const double kFmaUnits[4] = {1.0, 2.0, 4.0, 0.25};
+__device__ __forceinline__ FmaUnits load_units() {
+  const volatile double* p = kFmaUnits;
+  return {p[0], p[1], p[2], p[3]};
+}
+
 // WENO-IS (App. C) of weno_is, value by value the same, on the stencil (a, b, c,
 // d, e) = u_{i-2} .. u_{i+2}; a3, c3, d3: three times a, c, d; b0 = (c - d)^2.
 // For values that are zero or of a magnitude within [2^-200, 2^80) and eps
@@ -31,33 +42,39 @@ namespace hrm {
 // With x_k the sub-stencil sums of S_k = x_k / 2, / 2, / 8, / 8 and p_k the
 // products of eta_k = (15 p_0, 5 p_1, 10 p_2, 2 p_3) / 32, the powers of two move
 // through the roundings: sum eta_k S_k / sum eta_k = V / ES / 4 below.
+// Additions go through an FMA with a multiplier in registers (FmaUnits): the FP64
+// unit takes a DFMA of three registers every 16 cycles, but a DADD, a DMUL or a
+// DFMA with a constant operand only every 19 (measured).
 __device__ __forceinline__ double weno_side(double a, double b, double c, double d, double e, double a3, double c3,
-                                            double d3, double b0, double eps) {
+                                            double d3, double b0, double eps, const FmaUnits& u) {
   using soft::mul_in;
   auto sq = [](double x) { return mul_in<true, false>(x, x); };      // of any sign
   auto pos = [](double x, double y) { return mul_in<false, false>(x, y); };
   auto any = [](double x, double y) { return mul_in<true, true>(x, y); };
+  auto add = [&](double x, double y) { return fma(x, u.one, y); };
+  auto sub = [&](double x, double y) { return fma(x, u.one, -y); };
   constexpr double k = 13.0 / 12.0;
   // k t^2 + t'^2 / 4 as ((k t) t) + ((t' / 4) t'): the last product is exact in the FMA
-  auto beta = [&](double t, double tt) { return fma(0.25, sq(tt), mul_in<true, false>(any(k, t), t)); };
-  const double x0 = c + d;
-  const double x1 = c3 - b;
-  const double x2 = fma(2.0, d3, c3) - e;
-  const double x3 = (a3 - any(10.0, b)) + any(15.0, c);
-  const double b1 = sq(b - c);
-  const double b01 = beta(fma(-2.0, c, b) + d, b - d);
-  const double b2 = beta(fma(-2.0, d, c) + e, fma(-4.0, d, c3) + e);
-  const double b3 = beta(fma(-2.0, b, a) + c, fma(-4.0, b, a) + c3);
-  const double tau = beta(fma(-4.0, b, fma(2.0, c3, fma(-4.0, d, e))) + a, fma(2.0, b, fma(-2.0, d, e)) - a);
-  const double A = b0 + eps, B = b1 + eps, C = b01 + eps, g2 = b2 + eps, g3 = b3 + eps;
+  auto beta = [&](double t, double tt) { return fma(u.quarter, sq(tt), mul_in<true, false>(any(k, t), t)); };
+  const double x0 = add(c, d);
+  const double x1 = sub(c3, b);
+  const double x2 = sub(fma(u.two, d3, c3), e);
+  const double x3 = add(sub(a3, any(10.0, b)), any(15.0, c));
+  const double b1 = sq(sub(b, c));
+  const double b01 = beta(add(fma(u.two, -c, b), d), sub(b, d));
+  const double b2 = beta(add(fma(u.two, -d, c), e), add(fma(u.four, -d, c3), e));
+  const double b3 = beta(add(fma(u.two, -b, a), c), add(fma(u.four, -b, a), c3));
+  const double tau = beta(add(fma(u.four, -b, fma(u.two, c3, fma(u.four, -d, e))), a),
+                          sub(fma(u.two, b, fma(u.two, -d, e)), a));
+  const double A = add(b0, eps), B = add(b1, eps), C = add(b01, eps), g2 = add(b2, eps), g3 = add(b3, eps);
   const double t2 = sq(tau);
   const double g23 = pos(g2, g3), ABC = pos(pos(A, B), C);
-  const double E0 = pos(15.0, pos(pos(A, C) + t2, pos(B, g23)));
-  const double E1 = pos(5.0, pos(pos(B, C) + t2, pos(A, g23)));
-  const double E2 = pos(5.0, pos(g2 + tau, pos(ABC, g3)));
-  const double E3 = pos(g3 + tau, pos(ABC, g2));
-  const double ES = fma(2.0, E3, fma(2.0, E2, E0 + E1));
-  const double V = fma(2.0, any(E0, x0) + any(E1, x1), any(E2, x2)) + any(E3, x3);
+  const double E0 = pos(15.0, pos(add(pos(A, C), t2), pos(B, g23)));
+  const double E1 = pos(5.0, pos(add(pos(B, C), t2), pos(A, g23)));
+  const double E2 = pos(5.0, pos(add(g2, tau), pos(ABC, g3)));
+  const double E3 = pos(add(g3, tau), pos(ABC, g2));
+  const double ES = fma(u.two, E3, fma(u.two, E2, add(E0, E1)));
+  const double V = add(fma(u.two, add(any(E0, x0), any(E1, x1)), any(E2, x2)), any(E3, x3));
   return (((uint32_t)__double2hiint(V) & 0x7ff00000u) == 0u) ? V : soft::div_in<-2>(V, ES);
 }
 
@@ -72,7 +89,8 @@ __device__ __forceinline__ double linear_side(double a, double b, double c, doub
 
 // Both biased values at x_{i+1/2} of one characteristic field from its six node
 // values; lin: the linear weights (gated midpoint).
-__device__ __forceinline__ void weno_both(const double* v, double eps, bool lin, double& left, double& right) {
+__device__ __forceinline__ void weno_both(const double* v, double eps, bool lin, const FmaUnits& units, double& left,
+                                          double& right) {
   bool in = (eps >= 0x1p-60) & (eps <= 0x1p170);
 #pragma unroll
   for (int j = 0; j < 6; ++j) in = in & soft::within<-200, 80>(v[j]);
@@ -98,7 +116,7 @@ __device__ __forceinline__ void weno_both(const double* v, double eps, bool lin,
     const double a = s ? v[5] : v[0], b = s ? v[4] : v[1], c = s ? v[3] : v[2], d = s ? v[2] : v[3], e = s ? v[1] : v[4];
     const double c3 = s ? t3 : t2, d3 = s ? t2 : t3;
     const double x = lin ? linear_side(a, b, c, d, e, triple(a), c3, d3)
-                         : weno_side(a, b, c, d, e, triple(a), c3, d3, b0, eps);
+                         : weno_side(a, b, c, d, e, triple(a), c3, d3, b0, eps, units);
     if (s == 0)
       left = cl ? left : x;
     else
@@ -217,6 +235,8 @@ __device__ __forceinline__ void face_body(int64_t t, const Nodes6& nd, const dou
   const double cb = halved(Cc[nd.c[2]] + Cc[nd.c[3]]);
   const double rc = prod(rhob, cb);
   {
+    // (a lone warp's DADD takes the same 64 cycles: no loads there)
+    const FmaUnits units = LANES == 1 ? load_units() : FmaUnits{1.0, 2.0, 4.0, 0.25};
     const double inv_rc = quot(1.0, rc);
     const double rc2b = prod(rc, cb);
 #pragma unroll 1
@@ -239,7 +259,7 @@ __device__ __forceinline__ void face_body(int64_t t, const Nodes6& nd, const dou
         }
       }
       double left, right;
-      weno_both(w6, pr.weno_eps, lin, left, right);
+      weno_both(w6, pr.weno_eps, lin, units, left, right);
       slot(0, fi) = left;
       slot(1, fi) = right;
     }
@@ -333,7 +353,7 @@ __device__ __forceinline__ void face_body(int64_t t, const Nodes6& nd, const dou
     const double pw1 = (0.5 * (slot(1, 0) + slot(1, 1))) * (0.5 * (slot(1, 2) + slot(1, 3)));
     double pw = pw1;
     for (int e = 1; e < pr.qexp; ++e) pw = pw * pw1;
-    sig = tanh_r(pr.Cs * pw);
+    sig = tanh_r<LANES == 1>(pr.Cs * pw);
   }
   group_sync();
   const double one_m = 1.0 - sig;
@@ -497,12 +517,11 @@ __global__ void __launch_bounds__(kFaceThreads, 3)
            const uint8_t* __restrict__ gate, const uint32_t* __restrict__ list, uint32_t* __restrict__ cnt) {
   __shared__ double col[kFaceCol<N, D>];
   const uint32_t n = cnt[0];
-  uint32_t i;
   if (n <= kSplitMax) {
     const uint32_t warps = gridDim.x * (kFaceThreads / 32), per = 32 / kSplitLanes;
     for (uint32_t k = blockIdx.x + gridDim.x * (threadIdx.x >> 5); k * per < n; k += warps) {
       Nodes6 nd;
-      i = k * per + (threadIdx.x & 31) / kSplitLanes;
+      const uint32_t i = k * per + (threadIdx.x & 31) / kSplitLanes;
       if (i >= n) continue;
       const int64_t t = list[i];
       if (!face_nodes<DIR>(g, t, nd)) continue;
@@ -511,6 +530,7 @@ __global__ void __launch_bounds__(kFaceThreads, 3)
     }
     return;
   }
+  uint32_t i;
   while (next_entries(cnt, n, i)) {
     Nodes6 nd;
     if (i >= n) continue;
