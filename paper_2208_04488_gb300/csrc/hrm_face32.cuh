@@ -97,15 +97,19 @@ __device__ __forceinline__ float weno_increment(float a, float b, float d, float
 }
 
 // Interpolation limiter of the precision form: partial densities from FP32,
-// volume fractions carried in FP64 (at, the N-1 stored ones); theta in FP64.
+// volume fractions carried in FP64 (at, the N-1 stored ones); theta in FP64. Wn:
+// the node's conservative state, which holds its partial densities and volume
+// fractions; its other primitives and rho c^2 are formed only where rho c^2 of the
+// midpoint lies below the hard switch's threshold, or the switch acts (a deferred
+// midpoint is one lane's chain, and they were a fifth of it).
 template <int N, int D>
-__device__ __forceinline__ void interp_limit32(float* Vt, double* at, const double* Vn, double rc2n,
-                                               const DevFluid& f, const DevParams& pr) {
+__device__ __forceinline__ void interp_limit32(float* Vt, double* at, const double* Wn, const DevFluid& f,
+                                               const DevParams& pr) {
   using L = Lay<N, D>;
   constexpr int M = L::M;
 #pragma unroll
   for (int k = 0; k < N; ++k) {
-    const double lo = Vn[k], hi = (double)Vt[k];
+    const double lo = Wn[k], hi = (double)Vt[k];
     const double tgt = dmin(pr.eps_ar, lo);
     double th = 1.0;
     if (hi < tgt) th = (tgt - lo) / (hi - lo);
@@ -117,7 +121,7 @@ __device__ __forceinline__ void interp_limit32(float* Vt, double* at, const doub
 #pragma unroll
     for (int k = 0; k < N - 1; ++k) {
       alt[k] = at[k];
-      aln[k] = Vn[L::AL + k];
+      aln[k] = Wn[L::AL + k];
       st += alt[k];
       sn += aln[k];
     }
@@ -144,17 +148,22 @@ __device__ __forceinline__ void interp_limit32(float* Vt, double* at, const doub
   }
 #pragma unroll
   for (int k = 0; k < N; ++k) {
-    hs |= (double)Vt[k] < dmin(pr.hs_ar, Vn[k]);
+    hs |= (double)Vt[k] < dmin(pr.hs_ar, Wn[k]);
     hs |= alt[k] < dmin(pr.hs_a, aln[k]);
   }
   double S, P;
   mix_SP<double, N>(f, alt, S, P);
-  hs |= rho_c2(S, P, (double)Vt[L::EN]) < dmin(pr.hs_rc2, rc2n);
-  if (hs) {
+  const double rc2 = rho_c2(S, P, (double)Vt[L::EN]);
+  if (hs || rc2 < pr.hs_rc2) {
+    double Vn[M], rho, c, rc2n;
+    cell_prim<N, D>(Wn, f, Vn, rho, c, rc2n);
+    hs |= rc2 < dmin(pr.hs_rc2, rc2n);
+    if (hs) {
 #pragma unroll
-    for (int m = 0; m < M; ++m) Vt[m] = (float)Vn[m];
+      for (int m = 0; m < M; ++m) Vt[m] = (float)Vn[m];
 #pragma unroll
-    for (int k = 0; k < N - 1; ++k) at[k] = Vn[L::AL + k];
+      for (int k = 0; k < N - 1; ++k) at[k] = Wn[L::AL + k];
+    }
   }
 #pragma unroll
   for (int k = 0; k < N - 1; ++k) Vt[L::AL + k] = (float)at[k];
@@ -631,17 +640,16 @@ __device__ __forceinline__ bool face32_body(int64_t t, const Nodes6& nd, const d
   const int64_t nc = g.ncells;
   const int64_t nf = face_count<DIR>(g);
   auto ld = [&](int plane, int j) -> float { return P32[(int64_t)plane * nc + nd.c[j]]; };
-  // node state j in FP64 from W (the FP64 limiters' inputs where a screen fails);
-  // returns rho c^2
-  auto load_node = [&](int j, double* Vn, double* Wn) -> double {
-    double w[M], rho, cs, rc2;
+  // node state j in FP64 from W, and its primitives (the FP64 limiters' inputs
+  // where a screen fails)
+  auto load_state = [&](int j, double* Wn) {
 #pragma unroll
-    for (int m = 0; m < M; ++m) {
-      w[m] = W[m * nc + nd.c[j]];
-      if (Wn) Wn[m] = w[m];
-    }
-    cell_prim<N, D>(w, f, Vn, rho, cs, rc2);
-    return rc2;
+    for (int m = 0; m < M; ++m) Wn[m] = W[m * nc + nd.c[j]];
+  };
+  auto load_node = [&](int j, double* Vn, double* Wn) {
+    double rho, cs, rc2;
+    load_state(j, Wn);
+    cell_prim<N, D>(Wn, f, Vn, rho, cs, rc2);
   };
   // first-order HLLC in FP32 from the node states, alpha slots in FP64
   auto first_order = [&](const double* Vi, const double* Vj, FluxPack<N, D>& H) {
@@ -666,9 +674,9 @@ __device__ __forceinline__ bool face32_body(int64_t t, const Nodes6& nd, const d
   FluxPack<N, D> G;
   if (pr.scheme == 1) {
     if constexpr (DEFER) return false;
-    double Vi[M], Vj[M];
-    load_node(2, Vi, nullptr);
-    load_node(3, Vj, nullptr);
+    double Vi[M], Vj[M], Wi[M], Wj[M];
+    load_node(2, Vi, Wi);
+    load_node(3, Vj, Wj);
     first_order(Vi, Vj, G);
   } else {
     float p6[6], u6[6];
@@ -831,26 +839,26 @@ __device__ __forceinline__ bool face32_body(int64_t t, const Nodes6& nd, const d
       // does not depend on whether the screen ran)
       if (!(pr.screen && interp_screen32<N, D>(sl.V, at_L, f, pr))) {
         if constexpr (DEFER) return false;
-        double Vn[M], a0[NA], a1[NA];
-        const double rc2n = load_node(2, Vn, nullptr);
+        double Wn[M], a0[NA], a1[NA];
+        load_state(2, Wn);
 #pragma unroll
-        for (int k = 0; k < N - 1; ++k) a0[k] = a1[k] = Vn[L::AL + k] + (double)incL[k];
-        interp_limit32<N, D>(sl.V, a1, Vn, rc2n, f, pr);
+        for (int k = 0; k < N - 1; ++k) a0[k] = a1[k] = Wn[L::AL + k] + (double)incL[k];
+        interp_limit32<N, D>(sl.V, a1, Wn, f, pr);
 #pragma unroll
         for (int k = 0; k < N - 1; ++k) {
           if (a1[k] != a0[k])
-            dL[k] = ff_of(a1[k] - Vn[L::AL + k]);
+            dL[k] = ff_of(a1[k] - Wn[L::AL + k]);
           else
             sl.V[L::AL + k] = UL[N + D + k];
         }
       }
       if (!(pr.screen && interp_screen32<N, D>(sr.V, at_R, f, pr))) {
         if constexpr (DEFER) return false;
-        double Vn[M], a0[NA], a1[NA];
-        const double rc2n = load_node(3, Vn, nullptr);
+        double Wn[M], a0[NA], a1[NA];
+        load_state(3, Wn);
 #pragma unroll
-        for (int k = 0; k < N - 1; ++k) a0[k] = a1[k] = Vn[L::AL + k] + (double)incR[k];
-        interp_limit32<N, D>(sr.V, a1, Vn, rc2n, f, pr);
+        for (int k = 0; k < N - 1; ++k) a0[k] = a1[k] = Wn[L::AL + k] + (double)incR[k];
+        interp_limit32<N, D>(sr.V, a1, Wn, f, pr);
 #pragma unroll
         for (int k = 0; k < N - 1; ++k) {
           if (a1[k] != a0[k])
