@@ -1285,8 +1285,11 @@ hrm_status hrm_get(hrm_ctx* c, int32_t field, double* dst, int32_t on_device) {
       return fail(c, HRM_E_INVAL, "unknown field %d", field);
   }
   if (field != HRM_FIELD_W) {
-    c->ck->fields(c->Wn, c->Ws, field, c->dg, c->fl, c->stream);
+    // straight into the caller's planes where their stride is the stored one
+    const bool direct = on_device && c->nint == c->nc && (uintptr_t)dst % sizeof(double) == 0;
+    c->ck->fields(c->Wn, direct ? dst : c->Ws, field, c->dg, c->fl, c->stream);
     ++c->launches;
+    if (direct) return last_launch(c, "get");
     src = c->Ws;
   }
   hrm_status s = copy_planes(c, dst, c->nint, src, c->nc, c->nint, planes,

@@ -53,7 +53,17 @@ void relax_l(double* W, const DevGrid& g, const DevFluid& f, cudaStream_t s) {
 }
 template <int N, int D>
 void fields_l(const double* W, double* out, int field, const DevGrid& g, const DevFluid& f, cudaStream_t s) {
-  k_fields<N, D><<<grid_for(g.nint, kCellThreads), kCellThreads, 0, s>>>(W, out, field, g, f);
+  const unsigned gr = grid_for(g.nint, kCellThreads);
+  switch (field) {
+    case 1: k_fields<N, D, 1><<<gr, kCellThreads, 0, s>>>(W, out, g, f); break;
+    case 2: k_fields<N, D, 2><<<gr, kCellThreads, 0, s>>>(W, out, g, f); break;
+    case 3: k_fields<N, D, 3><<<gr, kCellThreads, 0, s>>>(W, out, g, f); break;
+    case 4: k_fields<N, D, 4><<<gr, kCellThreads, 0, s>>>(W, out, g, f); break;
+    case 5: k_fields<N, D, 5><<<gr, kCellThreads, 0, s>>>(W, out, g, f); break;
+    case 6: k_fields<N, D, 6><<<gr, kCellThreads, 0, s>>>(W, out, g, f); break;
+    case 7: k_fields<N, D, 7><<<gr, kCellThreads, 0, s>>>(W, out, g, f); break;
+    case 8: k_fields<N, D, 8><<<gr, kCellThreads, 0, s>>>(W, out, g, f); break;
+  }
 }
 template <int N, int D>
 void admiss_l(const double* W, const DevGrid& g, const DevFluid& f, StepState* st, cudaStream_t s) {

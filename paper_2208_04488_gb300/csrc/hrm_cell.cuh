@@ -56,16 +56,16 @@ __device__ __forceinline__ double c4eq(const double* W, const DevFluid& f, doubl
   double cvb = 0.0, cpb = 0.0, qb = 0.0;
 #pragma unroll
   for (int k = 0; k < N; ++k) {
-    cvb += Y[k] * f.cv[k];
-    cpb += Y[k] * f.cp[k];
-    qb += Y[k] * f.q[k];
+    cvb += prod(Y[k], f.cv[k]);
+    cpb += prod(Y[k], f.cp[k]);
+    if (f.has_q) qb += Y[k] * f.q[k];
   }
-  const double pinf1 = f.pinf[l], R1 = f.Rg[l], Rb = cpb - cvb;
-  const double Bp = -(re * Rb - pinf1 * cvb - pinf1 * Y[l] * R1);
-  const double den = 2.0 * cvb * p + Bp;
-  const double Gam = quot(quot(-(-(rho * Rb) * p - pinf1 * rho * (Rb - Y[l] * R1)), den), rho);
+  const double pinf1 = f.pinf[l], R1 = f.Rg[l], Rb = cpb - cvb, YR = prod(Y[l], R1);
+  const double Bp = -(prod(re, Rb) - prod(pinf1, cvb) - prod(prod(pinf1, Y[l]), R1));
+  const double den = prod(soft::scale<1>(cvb), p) + Bp;
+  const double Gam = quot(quot(-(prod(-prod(rho, Rb), p) - prod(prod(pinf1, rho), Rb - YR)), den), rho);
   if (Gam_out) *Gam_out = Gam;
-  double c2 = quot(Gam * p, rho);
+  double c2 = quot(prod(Gam, p), rho);
   const double e = quot(re, rho) + qb;
 #pragma unroll
   for (int k = 0; k < N; ++k) {
@@ -73,11 +73,11 @@ __device__ __forceinline__ double c4eq(const double* W, const DevFluid& f, doubl
     const double dcv = quot(f.cv[k] - cvb, rho);
     const double dRb = quot(f.Rg[k] - Rb, rho);
     const double dY1 = quot((k == l ? 1.0 : 0.0) - Y[l], rho);
-    const double dB = -(dre * Rb + re * dRb - pinf1 * dcv - pinf1 * R1 * dY1);
-    const double dC = -(pinf1 * (dre * (Rb - Y[l] * R1) + re * (dRb - R1 * dY1)));
-    const double psi = quot(-(dcv * p * p + dB * p + dC), den);
+    const double dB = -(prod(dre, Rb) + prod(re, dRb) - prod(pinf1, dcv) - prod(prod(pinf1, R1), dY1));
+    const double dC = -prod(pinf1, prod(dre, Rb - YR) + prod(re, dRb - prod(R1, dY1)));
+    const double psi = quot(-(prod(prod(dcv, p), p) + prod(dB, p) + dC), den);
     if (Psi) Psi[k] = psi;
-    c2 += Y[k] * psi;
+    c2 += prod(Y[k], psi);
   }
   return rsqrt_r(c2);
 }
@@ -250,10 +250,14 @@ __global__ void __launch_bounds__(kCellThreads) k_relax(double* W, DevGrid g, De
   for (int k = 0; k < N - 1; ++k) W[(L::AL + k) * nc + c] = w[L::AL + k];
 }
 
-// Output fields of the current state (HRM_FIELD_*).
-template <int N, int D>
+// Output field `field` (HRM_FIELD_*) of the current state; a kernel per field, so
+// that the light ones are not held to the registers of the four-equation ones (a
+// snapshot of relaxation, dt and six fields at 1024x512: 546 -> 490 us with this,
+// the fields written straight to the caller's planes and the four-equation speed's
+// products on the integer pipes).
+template <int N, int D, int field>
 __global__ void __launch_bounds__(kCellThreads)
-    k_fields(const double* __restrict__ W, double* __restrict__ out, int field, DevGrid g, DevFluid f) {
+    k_fields(const double* __restrict__ W, double* __restrict__ out, DevGrid g, DevFluid f) {
   using L = Lay<N, D>;
   constexpr int M = L::M;
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -262,7 +266,7 @@ __global__ void __launch_bounds__(kCellThreads)
   double w[M], v[M], rho, cs, rc2;
 #pragma unroll
   for (int m = 0; m < M; ++m) w[m] = W[m * nc + c];
-  if (field == 8) {
+  if constexpr (field == 8) {
     // numerical schlieren |grad rho| / rho: central differences, neighbours
     // through the boundary conditions (copy, wrap, or the prescribed state)
     const int64_t ijk[3] = {c % g.n[0], (c / g.n[0]) % g.n[1], c / (g.n[0] * g.n[1])};
@@ -302,7 +306,7 @@ __global__ void __launch_bounds__(kCellThreads)
     out[c] = quot(rsqrt_r(g2), r0);
     return;
   }
-  if (field == 6 || field == 7) {
+  if constexpr (field == 6 || field == 7) {
     // all N volume fractions (alpha_N = 1 - the others) or mass fractions Y_k
     double r = 0.0, sa = 0.0;
 #pragma unroll
@@ -314,9 +318,9 @@ __global__ void __launch_bounds__(kCellThreads)
       out[k * nc + c] = field == 7 ? quot(w[k], r) : (k < N - 1 ? w[L::AL + k] : 1.0 - sa);
     return;
   }
-  if (field == 1 || field == 2) {
+  if constexpr (field == 1 || field == 2) {
     cell_prim<N, D>(w, f, v, rho, cs, rc2);
-    if (field == 1) {
+    if constexpr (field == 1) {
 #pragma unroll
       for (int m = 0; m < M; ++m) out[m * nc + c] = v[m];
     } else {
@@ -329,10 +333,10 @@ __global__ void __launch_bounds__(kCellThreads)
 #pragma unroll
   for (int m = 0; m < M; ++m) wr[m] = w[m];
   relax_cell<N, D>(wr, f, pT);
-  if (field == 3) {
+  if constexpr (field == 3) {
     out[c] = pT[0];
     out[nc + c] = pT[1];
-  } else if (field == 5) {
+  } else if constexpr (field == 5) {
     double Psi[N], Gam;
     c4eq<N, D>(w, f, pT[0], Psi, &Gam);
 #pragma unroll
