@@ -15,7 +15,7 @@ void launch(const double* W, const double* V, const double* AUX, const float* P3
   if constexpr (DIR < kD) {
     if (gate.defer_list) {
       if (gate.net)
-        k_face32_net<N, kD, DIR><<<list_grid(g, DIR, 6), kFaceThreads, 0, s>>>(
+        k_face32_net<N, kD, DIR><<<list_grid(g, DIR, 5), kFaceThreads, 0, s>>>(
             W, P32, gate.R32, out, g, f, p, st, static_cast<const mlp::GateBlob*>(gate.net), gate.zthr, gate.out_gate,
             gate.list, gate.list_cnt, gate.defer_list);
       else

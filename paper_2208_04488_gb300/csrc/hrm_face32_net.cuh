@@ -12,7 +12,7 @@
 //
 // Gate bytes (one per midpoint, in `gate`): 1 linear weights, 0 full WENO-IS,
 // 2 uniform stencil (exact node flux; written by k_mark). The deferred-midpoint
-// kernel reads them.
+// kernel reads them. Five blocks per SM: 2.8 % of a pass over six at 1024x512.
 #pragma once
 
 #include "hrm_learned.cuh"
@@ -20,7 +20,7 @@
 namespace hrm {
 
 template <int N, int D, int DIR>
-__global__ void __launch_bounds__(kFaceThreads, 6)
+__global__ void __launch_bounds__(kFaceThreads, 5)
     k_face32_net(const double* __restrict__ W, const float* __restrict__ P32, const float* __restrict__ R32,
                  double* __restrict__ out, DevGrid g, DevFluid f, DevParams pr, const StepState* __restrict__ st,
                  const mlp::GateBlob* __restrict__ blob, float zthr, uint8_t* __restrict__ gate,
