@@ -33,9 +33,9 @@ sys.path.insert(0, ROOT)
 # DRAM traffic per launch of the dominant kernels, dram__bytes_read.sum + dram__bytes_write.sum from one
 # ncu capture on this workload (profiles/k_face_fp64_shock_bubble_1024x512.md and
 # profiles/k_face32_shock_bubble_1024x512.md); to be re-taken whenever those kernels change.
-TRAFFIC_BYTES = {"k_face_fp64": 82.78e6, "k_face32": 73.09e6}
+TRAFFIC_BYTES = {"k_face_fp64": 9.06e6, "k_face32": 6.07e6}
 # FP64-pipe activity of the FP64 sweep in the same ncu capture (fraction of peak sustained)
-FP64_PIPE_ACTIVE = {"k_face_fp64": 0.716}
+FP64_PIPE_ACTIVE = {"k_face_fp64": 0.769}
 METRIC = "cell-updates/s (FP64 plain vs FP32+learned) at stated L1 err; % of roofline"
 UNIT = "cell-updates/s"
 WORKLOAD = "2D three-species shock-bubble, 1024x512 cells, Mach 1.5 shock, water+air+helium, SSP-RK3, CFL 0.4"
@@ -731,11 +731,10 @@ def main():
         # the precision form's sweep finishes a uniform stencil exactly (the node
         # flux) without the method's arithmetic: the share of such midpoints, as
         # the learned form's sweep reports it in its gate bytes (byte 2) at the
-        # end of the same steps, and the sweep's compulsory bytes per launch (the
-        # FP32 planes of the cells read once, the FP64 flux planes written once)
+        # end of the same steps, and the bytes a launch moves (ncu capture: the
+        # sweep reads and writes at listed, non-uniform midpoints only)
         uni = (learned_runs["fp32_learned"].get("gated_uniform") if learned_runs is not None else None)
-        nfx = (pr.n[0] + 1) * int(np.prod(pr.n[1:]))
-        bytes32 = 4 * (pr.M + 4 + pr.D + pr.N - 1) * pr.ncells + 8 * (pr.M + pr.N - 1) * nfx
+        bytes32 = TRAFFIC_BYTES["k_face32"]
         learned_block = None
         if learned_runs is not None:
             faces_g = gated_face_flops(pr, pr.cfl, W_fp64)
@@ -791,10 +790,10 @@ def main():
                                                        "FP64 sweep: the method's arithmetic at non-uniform "
                                                        "midpoints, the node flux at uniform ones (the sweep "
                                                        "takes that flux where its FP32 planes are uniform); "
-                                                       "the sweep is bound by the latency of its non-uniform "
-                                                       "warps, not by the FP32 pipe (ncu: FMA pipe 13-14 %)",
+                                                       "the sweep is bound by the latency of its body, "
+                                                       "not by the FP32 pipe (ncu: FMA pipe 19-23 %)",
                                       "uniform_share": uni,
-                                      "hbm": {"compulsory_bytes_per_launch": bytes32,
+                                      "hbm": {"traffic_bytes_per_launch": bytes32,
                                               "achieved_gbs": bytes32 / (tf32 / n32) / 1e9,
                                               "peak_gbs": pk.get("hbm_gbs"),
                                               "frac": (bytes32 / (tf32 / n32) / 1e9 / pk["hbm_gbs"]
