@@ -791,7 +791,7 @@ hrm_status hrm_create(hrm_ctx** out, const hrm_grid* grid, int32_t N, const doub
   if (c->defer_cap >= (int64_t)0xffffffffll)  // (its flux planes alone would exceed the device)
     return bail(fail(c, HRM_E_NOMEM, "2^32 - 1 midpoints or more in one direction"));
   // the lists, their counters and flags, and the worklist of the precision form's deferred midpoints: one
-  // allocation (a new context pays for each one; eight of them took 0.1 ms at 250x250)
+  // allocation (a new context pays for each)
   size_t used = 0;
   auto reserve = [&](size_t bytes) {
     const size_t at = used;

@@ -501,15 +501,34 @@ __device__ __forceinline__ void face_body(int64_t t, const Nodes6& nd, const dou
 // Sweep of direction DIR over its list (k_mark), a warp of 32 entries at a time
 // taken from a counter: every lane then runs the whole body (the FP64 unit's time
 // does not depend on the active lanes), and the warps end within one entry of one
-// another. Three blocks per SM. Lists of at most kSplitMax entries leave the chip
-// mostly idle so, each SM having a warp or two that issue an FP64 instruction
-// every 64 cycles; there kSplitLanes lanes share an entry, the groups dealt out to
-// the first warp of every block, then to the second ones. Measured per step (smooth
-// advection, both sweeps of n midpoints): n = 900 311 -> 174 us, 3025 445 -> 222,
-// 5625 458 -> 341, 8100 470 -> 412, 12100 473 -> 529; 400-cell tube 305 -> 189
-// (4 lanes 216, 16 lanes 255).
-constexpr int kSplitLanes = 8;
-constexpr uint32_t kSplitMax = 8192;
+// another. Three blocks per SM. Shorter lists leave each SM a warp or two that
+// issue an FP64 instruction every 64 cycles; there several lanes share an entry,
+// the groups dealt out to the first warp of every block, then to the second ones.
+// Measured us per step (both sweeps of n listed midpoints each) with 8 | 4 | 2 | 1
+// lanes, three species: n = 4704 443 | 429 | 537 | 661, 8256 606 | 439 | 507 | 701,
+// 12880 815 | 582 | 606 | 758, 20100 1307 | 1028 | 710 | 835, 32896 2048 | 1500 |
+// 1083 | 1043; two: 3080 228 | 228 | 260 | 411, 5256 341 | 351 | 369 | 445, 12210
+// 559 | 420 | 435 | 478, 17030 757 | 633 | 462 | 484, 25760 965 | 701 | 497 | 481.
+constexpr uint32_t kSplit8 = 4608, kSplit4 = 13312, kSplit2 = 20480;
+
+template <int N, int D, int DIR, int LANES>
+__device__ __forceinline__ void sweep_split(const double* __restrict__ W, const double* __restrict__ V,
+                                            const double* __restrict__ AUX, double* __restrict__ out, const DevGrid& g,
+                                            const DevFluid& f, const DevParams& pr, const StepState* __restrict__ st,
+                                            const uint8_t* __restrict__ gate, const uint32_t* __restrict__ list,
+                                            uint32_t n, double* col) {
+  const uint32_t warps = gridDim.x * (kFaceThreads / 32), per = 32 / LANES;
+  for (uint32_t k = blockIdx.x + gridDim.x * (threadIdx.x >> 5); k * per < n; k += warps) {
+    Nodes6 nd;
+    const uint32_t i = k * per + (threadIdx.x & 31) / LANES;
+    if (i >= n) continue;
+    const int64_t t = list[i];
+    if (!face_nodes<DIR>(g, t, nd)) continue;
+    const bool lin = gate != nullptr && gate[t] != 0;
+    face_body<N, D, DIR, LANES>(t, nd, W, V, AUX, out, g, f, pr, st->lam[DIR], col, lin);
+  }
+}
+
 template <int N, int D, int DIR>
 __global__ void __launch_bounds__(kFaceThreads, 3)
     k_face(const double* __restrict__ W, const double* __restrict__ V, const double* __restrict__ AUX,
@@ -517,19 +536,9 @@ __global__ void __launch_bounds__(kFaceThreads, 3)
            const uint8_t* __restrict__ gate, const uint32_t* __restrict__ list, uint32_t* __restrict__ cnt) {
   __shared__ double col[kFaceCol<N, D>];
   const uint32_t n = cnt[0];
-  if (n <= kSplitMax) {
-    const uint32_t warps = gridDim.x * (kFaceThreads / 32), per = 32 / kSplitLanes;
-    for (uint32_t k = blockIdx.x + gridDim.x * (threadIdx.x >> 5); k * per < n; k += warps) {
-      Nodes6 nd;
-      const uint32_t i = k * per + (threadIdx.x & 31) / kSplitLanes;
-      if (i >= n) continue;
-      const int64_t t = list[i];
-      if (!face_nodes<DIR>(g, t, nd)) continue;
-      const bool lin = gate != nullptr && gate[t] != 0;
-      face_body<N, D, DIR, kSplitLanes>(t, nd, W, V, AUX, out, g, f, pr, st->lam[DIR], col, lin);
-    }
-    return;
-  }
+  if (n <= kSplit8) return sweep_split<N, D, DIR, 8>(W, V, AUX, out, g, f, pr, st, gate, list, n, col);
+  if (n <= kSplit4) return sweep_split<N, D, DIR, 4>(W, V, AUX, out, g, f, pr, st, gate, list, n, col);
+  if (n <= kSplit2) return sweep_split<N, D, DIR, 2>(W, V, AUX, out, g, f, pr, st, gate, list, n, col);
   uint32_t i;
   while (next_entries(cnt, n, i)) {
     Nodes6 nd;

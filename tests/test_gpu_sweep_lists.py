@@ -98,3 +98,38 @@ def test_batch_of_small_instances_equals_single_contexts(hrm, precision, where):
         s.step(0.0, 3)
         np.testing.assert_array_equal(b.get(i), s.get(hrm.FIELD_W))
         s.close()
+
+
+@pytest.mark.parametrize("n", [[70], [40, 24], [130, 80], [12, 10, 9]], ids=lambda n: "x".join(map(str, n)))
+@pytest.mark.parametrize("low", [-140, -330], ids=["2^-465", "subnormal"])
+def test_decaying_velocities_equal_the_oracle(hrm, orc, n, low):
+    """Velocities of every exponent down to zero beside ordinary ones, alone and within one stencil."""
+    pr = disturbed(n, 0, "ends")
+    rng = np.random.default_rng(20)
+    D, cells = len(n), int(np.prod(n))
+    for d in range(D):
+        exponent = rng.uniform(low, 1.0, cells) if d else np.linspace(1.0, low, cells) + rng.uniform(-9.0, 0.0, cells)
+        u = rng.choice([-1.0, 1.0], cells) * 10.0 ** exponent
+        pr.prim[pr.N - 1 + d] = np.where(rng.random(cells) < 0.1, 0.0, u)
+    f, g, W = orc.setup(pr)
+    s = hrm.Solver.from_problem(pr, params=hrm.params_default(cfl=0.4, check=0))
+    dt, _ = orc.dt(f, g, W, 0.4)
+    W1 = orc.step(f, orc.make_params(), g, W, dt, 2)
+    s.step(dt, 2)
+    np.testing.assert_array_equal(s.get(hrm.FIELD_W), W1)
+    s.close()
+
+
+@pytest.mark.parametrize("cells", [4607, 4608, 13311, 13312, 20479, 20480])
+def test_shared_midpoints_equal_the_oracle(hrm, orc, cells):
+    """Lists around the lengths at which 8, 4, 2 and 1 lanes take a midpoint (no stencil is uniform)."""
+    pr = disturbed([cells], 0, "none")
+    rng = np.random.default_rng(cells)
+    pr.prim[0] += 0.01 * rng.random(cells)
+    pr.prim[pr.N - 1] += rng.random(cells)
+    f, g, W = orc.setup(pr)
+    s = hrm.Solver.from_problem(pr, params=hrm.params_default(cfl=0.4, check=0))
+    dt, _ = orc.dt(f, g, W, 0.4)
+    s.step(dt, 2)
+    np.testing.assert_array_equal(s.get(hrm.FIELD_W), orc.step(f, orc.make_params(), g, W, dt, 2))
+    s.close()
