@@ -99,6 +99,9 @@ __device__ __forceinline__ void cell_index(const DevGrid& g, int64_t c, int64_t*
 // groups of 32 taken, deferred midpoints); cells: the cells that the stage's update
 // changes, with the fourth set of counters; F: the flux planes where the uniform
 // faces' fluxes are wanted as well; gate: the gate bytes where they are.
+// A cell between two uniform faces takes its own flux twice, whose difference is
+// zero unless the flux is not finite: such cells carry kFluxOverflow in uni.
+constexpr unsigned kFluxOverflow = 0x40u;
 constexpr int kSweepCounts = 4, kSweepCounters = 4 * kSweepCounts;
 struct SweepLists {
   uint8_t* eq = nullptr;

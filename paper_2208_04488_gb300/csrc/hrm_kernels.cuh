@@ -498,7 +498,8 @@ __device__ __forceinline__ void uniform_flux32(int64_t c, int d, const float* __
 // b = 1 - a, so their combination is formed as acc + a (W^n - acc): two
 // operations as before, and exactly acc when W^n equals acc. ub: the cell's
 // uniform faces (k_mark), whose flux comes from the cell's own planes P32; two
-// of them leave acc as it is (acc + cd 0 with cd < 0).
+// of them leave acc as it is (acc + cd 0 with cd < 0), unless their flux or cd is
+// not finite.
 template <int N, int D>
 __device__ __forceinline__ void fast_combine(int64_t c, const double* Wn, const double* Ws,
                                              const double* __restrict__ F0, const double* __restrict__ F1,
@@ -517,13 +518,13 @@ __device__ __forceinline__ void fast_combine(int64_t c, const double* Wn, const 
 #pragma unroll
   for (int d = 0; d < D; ++d) {
     const unsigned u = ub >> (2 * d) & 3u;
-    if (u == 3u) continue;
+    const double cd = -dt * g.inv_dx[d];
+    if (u == 3u && !(ub & kFluxOverflow) && ((uint32_t)__double2hiint(cd) & 0x7ff00000u) != 0x7ff00000u) continue;
     const double* F = d == 0 ? F0 : (d == 1 ? F1 : F2);
     const int64_t f0 = g.n[0] + (d == 0), f1 = g.n[1] + (d == 1), f2 = g.n[2] + (d == 2);
     const int64_t nf = f0 * f1 * f2;
     const int64_t fl = HRM_IDX(g, (i2 * f1 + i1) * f0 + i0, nf);
     const int64_t fr = HRM_IDX(g, fl + (d == 0 ? 1 : (d == 1 ? f0 : f0 * f1)), nf);
-    const double cd = -dt * g.inv_dx[d];
     double own[L::NC];
     if (u) uniform_flux32<N, D>(c, d, P32, nc, own);
     // G^-_{i+1/2} - G^+_{i-1/2}: the alpha slots of the right face use alpha_i
@@ -690,7 +691,8 @@ __device__ __forceinline__ void update_body(int64_t c, const double* Wn, const d
 #pragma unroll
   for (int d = 0; d < D; ++d) {
     const unsigned u = ub >> (2 * d) & 3u;
-    if (u == 3u) continue;  // both faces uniform: the cell's own flux twice, and rhs - 0 / dx = rhs
+    // both faces uniform: the cell's own flux twice, and rhs - 0 / dx = rhs
+    if (u == 3u && !(ub & kFluxOverflow)) continue;
     const double* F = d == 0 ? F0 : (d == 1 ? F1 : F2);
     const int64_t f0 = g.n[0] + (d == 0), f1 = g.n[1] + (d == 1), f2 = g.n[2] + (d == 2);
     const int64_t nf = f0 * f1 * f2;

@@ -10,10 +10,10 @@ void mark(const double* W, const double* V, const float* P32, const DevGrid& g, 
           cudaStream_t s) {
   const unsigned gr = grid_for(g.nint, kCellThreads);
   if (P32) {
-    k_equal<N, D, float><<<gr, kCellThreads, 0, s>>>(P32, g, lists.eq, lists.cnt);
+    k_equal<N, D, float><<<gr, kCellThreads, 0, s>>>(P32, nullptr, g, lists.eq, lists.cnt);
     k_mark<N, D, true><<<gr, kCellThreads, 0, s>>>(W, V, P32, g, lists, all);
   } else {
-    k_equal<N, D, double><<<gr, kCellThreads, 0, s>>>(W, g, lists.eq, lists.cnt);
+    k_equal<N, D, double><<<gr, kCellThreads, 0, s>>>(W, V, g, lists.eq, lists.cnt);
     k_mark<N, D, false><<<gr, kCellThreads, 0, s>>>(W, V, P32, g, lists, all);
   }
 }

@@ -31,14 +31,19 @@ __device__ __forceinline__ int64_t neighbour(const DevGrid& g, int d, const int6
   return c + (bc_map(g, d, j) - ijk[d]) * stride;
 }
 
-// eq[c], bit d: every plane finite and the same in cell c and the cell after it
-// along d; bit 3 + d, for the first cell of a line: in cell c and the ghost cell
-// before it. T double: the M planes of W, bit for bit (the FP64 form's uniform
-// stencils); T float: the precision form's FP32 planes, by value. Thread by thread
-// the lists' counters are cleared.
+// eq[c], bit d: every plane the same in cell c and the cell after it along d; bit
+// 3 + d, for the first cell of a line: in cell c and the ghost cell before it; bit
+// 6 (kFluxOverflow): the cell's physical flux may not be finite. T double: the M
+// planes of W, bit for bit (the FP64 form's uniform stencils; its velocities and
+// pressure from V); T float: the precision form's FP32 planes, by value. Thread by
+// thread the lists' counters are cleared.
+// Bit 6 by exponents: every factor of a flux term, p included, lies below 2^(a+1)
+// and every velocity below 2^(b+1) for their largest exponents a and b, so the
+// terms and their sums (E + p and + p) lie below 2^(a + b + 4).
 template <int N, int D, typename T>
 __global__ void __launch_bounds__(kCellThreads)
-    k_equal(const T* __restrict__ W, DevGrid g, uint8_t* __restrict__ eq, uint32_t* __restrict__ cnt) {
+    k_equal(const T* __restrict__ W, const double* __restrict__ V, DevGrid g, uint8_t* __restrict__ eq,
+            uint32_t* __restrict__ cnt) {
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (c < kSweepCounters) cnt[c] = 0u;
   if (c >= g.nint) return;
@@ -51,22 +56,36 @@ __global__ void __launch_bounds__(kCellThreads)
   };
   int64_t ijk[3];
   cell_index(g, c, ijk);
+  constexpr int kBias = sizeof(T) == 8 ? 1023 : 127, kMant = sizeof(T) == 8 ? 20 : 23;
+  auto magnitude = [](T x) -> uint32_t {  // ordered as |x|, exponent field on top
+    if constexpr (sizeof(T) == 8)
+      return (uint32_t)__double2hiint(x) & 0x7fffffffu;
+    else
+      return __float_as_uint(x) & 0x7fffffffu;
+  };
   T w[M];
-  bool fin = true;
+  uint32_t hw = 0, hu = 0;
 #pragma unroll
   for (int m = 0; m < M; ++m) {
     w[m] = W[m * g.ncells + c];
-    if constexpr (sizeof(T) == 8)
-      fin = fin & (((uint32_t)__double2hiint(w[m]) & 0x7ff00000u) != 0x7ff00000u);
-    else
-      fin = fin & ((__float_as_uint(w[m]) & 0x7f800000u) != 0x7f800000u);
+    hw = max(hw, magnitude(w[m]));
   }
-  unsigned bits = 0;
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    constexpr int u = Lay<N, D>::MOM;
+    if constexpr (sizeof(T) == 8)
+      hu = max(hu, magnitude(V[(u + d) * g.ncells + c]));
+    else
+      hu = max(hu, magnitude(w[u + d]));
+  }
+  if constexpr (sizeof(T) == 8) hw = max(hw, magnitude(V[Lay<N, D>::EN * g.ncells + c]));
+  const int ew = (int)(hw >> kMant), eu = (int)(hu >> kMant);  // 2 kBias + 1 for infinities and NaN
+  unsigned bits = (ew > 2 * kBias - 4 || eu > 2 * kBias || ew + eu > 3 * kBias - 4) ? kFluxOverflow : 0u;
 #pragma unroll
   for (int d = 0; d < D; ++d) {
     auto same = [&](int64_t o) {
       o = HRM_IDX(g, o, g.ncells);
-      bool s = fin;
+      bool s = true;
 #pragma unroll
       for (int m = 0; m < M; ++m) s = s & same_value(W[m * g.ncells + o], w[m]);
       return s;
@@ -78,7 +97,8 @@ __global__ void __launch_bounds__(kCellThreads)
 }
 
 // uni[c], bits 2 d and 2 d + 1: the faces of cell c on the low and the high side
-// of direction d are uniform (no face is with `all`, the first-order scheme). The
+// of direction d are uniform (no face is with `all`, the first-order scheme); bit
+// kFluxOverflow as in eq[c]. The
 // other midpoints go to lists.list[d] in the order of their cells, one atomic per
 // block and direction. With lists.F (every midpoint's flux wanted) the uniform
 // faces' fluxes are written too, and with lists.gate their gate bytes. FP32: the
@@ -123,7 +143,7 @@ __global__ void __launch_bounds__(kCellThreads)
       uni |= (unsigned)(pair[0] & mid) << (2 * d) | (unsigned)(mid & pair[5]) << (2 * d + 1);
     }
   }
-  if (in) lists.uni[c] = (uint8_t)uni;
+  if (in) lists.uni[c] = (uint8_t)(uni | (lists.eq[c] & kFluxOverflow));
   uint32_t at[D];
   bool lo[D], hi[D];
 #pragma unroll
