@@ -18,6 +18,7 @@
 #include "hrm_batch.cuh"
 #include "hrm_launch.h"
 #include "hrm_learned.h"
+#include "hrm_target.h"
 
 using namespace hrm;
 
@@ -35,6 +36,7 @@ struct hrm_ctx {
   DevFluid fl{};
   DevGrid dg{};
   DevParams dp{};
+  int device = 0;                  // device of the context (current at creation)
   cudaStream_t stream = nullptr;   // caller's stream: every call is ordered on it
   cudaStream_t cap = nullptr;      // private stream used only to capture the step graph
   double* Wn = nullptr;            // state W^n (M planes)
@@ -766,6 +768,7 @@ hrm_status hrm_create(hrm_ctx** out, const hrm_grid* grid, int32_t N, const doub
   c->fk = face_kernels(N, D);
   if (!c->ck || !c->fk) return bail(fail(c, HRM_E_INVAL, "no kernels for N=%d D=%d", N, D));
   c->stream = (cudaStream_t)cuda_stream;
+  cudaGetDevice(&c->device);
   c->alloc = g_alloc;
   c->dealloc = g_free;
   c->alloc_user = g_alloc_user;
@@ -1288,8 +1291,15 @@ hrm_status hrm_get(hrm_ctx* c, int32_t field, double* dst, int32_t on_device) {
       return fail(c, HRM_E_INVAL, "unknown field %d", field);
   }
   if (field != HRM_FIELD_W) {
-    // straight into the caller's planes where their stride is the stored one
-    const bool direct = on_device && c->nint == c->nc && (uintptr_t)dst % sizeof(double) == 0;
+    // straight into the caller's planes where their stride is the stored one and a
+    // kernel may store there
+    bool direct = on_device && c->nint == c->nc;
+    if (direct) {
+      cudaPointerAttributes at{};
+      const bool got = cudaPointerGetAttributes(&at, dst) == cudaSuccess;
+      if (!got) cudaGetLastError();
+      direct = kernel_target(dst, got, at, c->device);
+    }
     c->ck->fields(c->Wn, direct ? dst : c->Ws, field, c->dg, c->fl, c->stream);
     ++c->launches;
     if (direct) return last_launch(c, "get");
