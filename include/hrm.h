@@ -491,14 +491,15 @@ hrm_status hrm_batch_step(hrm_batch* b, int32_t nsteps);
 hrm_status hrm_batch_time(hrm_batch* b, int32_t i, double* t, int64_t* steps);
 /* Admissibility counters summed over the instances (as hrm_admissibility). */
 hrm_status hrm_batch_admissibility(hrm_batch* b, int64_t counts[4]);
-/* Launch shape of the persistent stage kernel: cells per work item of its
- * per-cell phases (>= 256) and blocks per SM (1 .. the most that can be
+/* Launch shape of the persistent stage kernel: most cells per work item of its
+ * per-cell phases (>= 256; 4096 in a new batch; fewer where the batch is too small
+ * to leave every resident block two items of that size) and blocks per SM (1 .. the most that can be
  * resident; 0 or larger values: all that fit). face_threads and face_tile are
  * accepted and ignored (midpoints go in tiles of 128, one thread each). */
 hrm_status hrm_batch_set_launch(hrm_batch* b, int32_t face_threads, int32_t face_tile, int32_t cell_tile,
                                 int32_t blocks_per_sm);
 /* Autotuner: times steps_per_trial steps of the batch itself for each candidate
- * launch shape (cells per item {1024, 4096, 16384} x blocks per SM 1 .. the most
+ * launch shape (most cells per item {1024, 4096, 16384} x blocks per SM 1 .. the most
  * resident), restores the states after every trial, keeps the fastest and
  * writes it to best[4] (128, 128, cell_tile, blocks_per_sm). */
 hrm_status hrm_batch_tune(hrm_batch* b, int32_t steps_per_trial, int32_t* best);

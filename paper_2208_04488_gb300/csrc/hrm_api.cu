@@ -452,7 +452,7 @@ hrm_status setup_persistent(hrm_ctx* c) {
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   c->p_grid = sms * batch_stage32_fit();
   if (c->p_grid <= 0) return fail(c, HRM_E_CUDA, "persistent stage kernel: no resident block fits an SM");
-  const int64_t kCellItem = default_cell_tile(c->nint, c->p_grid);
+  const int64_t kCellItem = cell_tile(4096, c->nint, c->p_grid);
   for (int64_t x = 0; x < c->nint; x += kCellItem) cells.push_back({0, 0, x, std::min<int64_t>(x + kCellItem, c->nint)});
   for (int d = 0; d < 2; ++d) {
     const int64_t nf = (c->dg.n[0] + (d == 0)) * (c->dg.n[1] + (d == 1));

@@ -9,6 +9,7 @@
 #include "hrm_face32.cuh"
 #include "hrm_face64.cuh"
 #include "hrm_sync.cuh"
+#include "hrm_tiles.h"
 
 namespace hrm {
 
@@ -333,18 +334,6 @@ __device__ __forceinline__ void batch_stage(const StageArgs& A) {
     __threadfence();
     if (atomicAdd(&A.sync->done, 1u) == nb - 1u) stamp[4] = tc::global_ns();
   }
-}
-
-// Cells per item of the per-cell phases for `blocks` resident blocks: at least two
-// items per block, so that no block runs a long item while others have none, and
-// at most 4096 (a block takes 128 cells at a time). With 4096 cells always, 24
-// instances of 6000 cells kept 48 of 912 blocks busy; with this rule and the
-// midpoint phase's lists a stage launch over them takes 0.24 ms against 0.65, and
-// over 8 FP64 instances of 3000 cells 0.30 against 0.79; 64 instances of 11.35 M
-// cells 10.2 ms per FP32 step against 12.8 and 93.7 per FP64 step against 115.
-inline int default_cell_tile(int64_t cells, int64_t blocks) {
-  const int64_t t = (cells / (2 * blocks) + 127) / 128 * 128;
-  return (int)(t < 128 ? 128 : (t > 4096 ? 4096 : t));
 }
 
 // Persistent stage launchers for D = 2 (FP64: hrm_batch64_d2.cu, precision

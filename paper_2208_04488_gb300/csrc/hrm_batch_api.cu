@@ -22,7 +22,7 @@ using namespace hrm;
 namespace {
 
 struct Shape {
-  int cell_tile = 4096;   // cells per work item of the per-cell phases (default_cell_tile at creation)
+  int cell_tile = 4096;   // most cells per work item of the per-cell phases (cell_tile of hrm_tiles.h)
   int blocks_per_sm = 0;  // persistent grid = SMs x blocks_per_sm (0: all that fit)
 };
 
@@ -90,18 +90,23 @@ void drop_graph(hrm_batch* b) {
   b->graph_kernels = 0;
 }
 
-// Work items: every instance's cells in chunks of cell_tile, grouped by species
+int grid_blocks(const hrm_batch* b) {
+  const int per_sm = b->shape.blocks_per_sm > 0 ? std::min(b->shape.blocks_per_sm, b->fit) : b->fit;
+  return b->sms * per_sm;
+}
+
+// Work items: every instance's cells in chunks (cell_tile), grouped by species
 // count; tiles of 128 midpoints of every instance and direction, grouped by
 // species count and direction (the direction in WorkItem::pad). No item spans
 // two instances.
 hrm_status build_items(hrm_batch* b) {
   std::vector<WorkItem> cells, tiles;
+  const int64_t tile = cell_tile(b->shape.cell_tile, b->total_cells, grid_blocks(b));
   for (int gN = 2; gN <= 3; ++gN)
     for (int i = 0; i < b->ninst; ++i) {
       if (b->N[i] != gN) continue;
       const DevGrid& g = b->host[i].g;
-      for (int64_t c = 0; c < g.ncells; c += b->shape.cell_tile)
-        cells.push_back({i, 0, c, std::min<int64_t>(c + b->shape.cell_tile, g.ncells)});
+      for (int64_t c = 0; c < g.ncells; c += tile) cells.push_back({i, 0, c, std::min<int64_t>(c + tile, g.ncells)});
     }
   for (int gN = 2; gN <= 3; ++gN)
     for (int d = 0; d < 2; ++d)
@@ -129,11 +134,6 @@ hrm_status build_items(hrm_batch* b) {
   b->ntiles = (int)tiles.size();
   drop_graph(b);
   return HRM_OK;
-}
-
-int grid_blocks(const hrm_batch* b) {
-  const int per_sm = b->shape.blocks_per_sm > 0 ? std::min(b->shape.blocks_per_sm, b->fit) : b->fit;
-  return b->sms * per_sm;
 }
 
 // One RK stage: reset the phase queues and the barrier count, then the
@@ -402,7 +402,6 @@ hrm_status hrm_batch_create(hrm_batch** out, int32_t ninst, const hrm_instance* 
   if (p.precision == HRM_FP32 &&
       (s = bcuda(b, cudaMalloc(&b->d_deferred, sizeof(uint64_t) * (size_t)b->seg[4]), "alloc deferred list")))
     return bail(s);
-  b->shape.cell_tile = default_cell_tile(b->total_cells, grid_blocks(b));
   if ((s = build_items(b))) return bail(s);
   *out = b;
   return HRM_OK;
