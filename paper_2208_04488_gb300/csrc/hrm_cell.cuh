@@ -11,15 +11,14 @@ namespace hrm {
 
 // Primitive variables of a conservative vector (Sec. 2): rho = sum alpha_k rho_k,
 // u_d = rho u_d / rho, p from the mixture EOS p/(gbar-1) + gbar pbar_inf/(gbar-1) =
-// rho (e - qbar), rho c^2 = gbar (p + pbar_inf), c = sqrt(rho c^2 / rho).
+// rho (e - qbar); S and P of the mixture rules.
 template <int N, int D, bool SOFT = false>
-__device__ __forceinline__ void cell_prim(const double* W, const DevFluid& f, double* V, double& rho,
-                                          double& c, double& rc2) {
+__device__ __forceinline__ void cell_vars(const double* W, const DevFluid& f, double* V, double& rho, double& S,
+                                          double& P) {
   using L = Lay<N, D>;
   rho = 0.0;
 #pragma unroll
   for (int k = 0; k < N; ++k) rho += W[k];
-  double S, P;
   mix_SP<double, N, SOFT>(f, &W[L::AL], S, P);
   const double re = rhoe_tilde<N, D>(W, f);
   const double p = quot(re - P, S);
@@ -30,7 +29,16 @@ __device__ __forceinline__ void cell_prim(const double* W, const DevFluid& f, do
   V[L::EN] = p;
 #pragma unroll
   for (int k = 0; k < N - 1; ++k) V[L::AL + k] = W[L::AL + k];
-  rc2 = rho_c2(S, P, p);
+}
+
+// The same with rho c^2 = gbar (p + pbar_inf) and c = sqrt(rho c^2 / rho). (Callers
+// that need neither take cell_vars: the compiler leaves no out-of-line quotient out.)
+template <int N, int D, bool SOFT = false>
+__device__ __forceinline__ void cell_prim(const double* W, const DevFluid& f, double* V, double& rho,
+                                          double& c, double& rc2) {
+  double S, P;
+  cell_vars<N, D, SOFT>(W, f, V, rho, S, P);
+  rc2 = rho_c2(S, P, V[Lay<N, D>::EN]);
   c = rsqrt_r(quot(rc2, rho));
 }
 
@@ -86,11 +94,8 @@ __device__ __forceinline__ double c4eq(const double* W, const DevFluid& f, doubl
 // 4_eqn_sos (the CFL speed option params.cfl_sound = 1).
 template <int N, int D>
 __device__ __forceinline__ double c4_of_cell(const double* w, const DevFluid& f) {
-  double wr[Lay<N, D>::M], pT[2];
-#pragma unroll
-  for (int m = 0; m < Lay<N, D>::M; ++m) wr[m] = w[m];
-  relax_cell<N, D>(wr, f, pT);
-  return c4eq<N, D>(w, f, pT[0]);
+  double rho, re, cvb, Yl;
+  return c4eq<N, D>(w, f, relaxed_p<N, D>(w, f, rho, re, cvb, Yl));
 }
 
 // Per cell: V (M planes), AUX = (c, rho, rho c^2). With `tau`, also the running
@@ -263,7 +268,7 @@ __global__ void __launch_bounds__(kCellThreads)
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t nc = g.ncells;
   if (c >= g.nint) return;
-  double w[M], v[M], rho, cs, rc2;
+  double w[M];
 #pragma unroll
   for (int m = 0; m < M; ++m) w[m] = W[m * nc + c];
   if constexpr (field == 8) {
@@ -318,32 +323,36 @@ __global__ void __launch_bounds__(kCellThreads)
       out[k * nc + c] = field == 7 ? quot(w[k], r) : (k < N - 1 ? w[L::AL + k] : 1.0 - sa);
     return;
   }
-  if constexpr (field == 1 || field == 2) {
-    cell_prim<N, D>(w, f, v, rho, cs, rc2);
-    if constexpr (field == 1) {
+  double rho;
+  if constexpr (field == 1) {
+    double v[M], S, P;
+    cell_vars<N, D>(w, f, v, rho, S, P);
 #pragma unroll
-      for (int m = 0; m < M; ++m) out[m * nc + c] = v[m];
-    } else {
-      out[c] = cs;
-    }
-    return;
-  }
-  double pT[2];
-  double wr[M];
+    for (int m = 0; m < M; ++m) out[m * nc + c] = v[m];
+  } else if constexpr (field == 2) {  // c of cell_prim
+    double S, P;
+    rho = 0.0;
 #pragma unroll
-  for (int m = 0; m < M; ++m) wr[m] = w[m];
-  relax_cell<N, D>(wr, f, pT);
-  if constexpr (field == 3) {
-    out[c] = pT[0];
-    out[nc + c] = pT[1];
-  } else if constexpr (field == 5) {
-    double Psi[N], Gam;
-    c4eq<N, D>(w, f, pT[0], Psi, &Gam);
-#pragma unroll
-    for (int k = 0; k < N; ++k) out[k * nc + c] = Psi[k];
-    out[N * nc + c] = Gam;
+    for (int k = 0; k < N; ++k) rho += w[k];
+    mix_SP<double, N>(f, &w[L::AL], S, P);
+    out[c] = rsqrt_r(quot(rho_c2(S, P, quot(rhoe_tilde<N, D>(w, f) - P, S)), rho));
+  } else if constexpr (field == 3) {
+    double ps, Ts;
+    relaxed_pT<N, D>(w, f, ps, Ts);
+    out[c] = ps;
+    out[nc + c] = Ts;
   } else {
-    out[c] = c4eq<N, D>(w, f, pT[0]);
+    double re, cvb, Yl;
+    const double ps = relaxed_p<N, D>(w, f, rho, re, cvb, Yl);
+    if constexpr (field == 5) {
+      double Psi[N], Gam;
+      c4eq<N, D>(w, f, ps, Psi, &Gam);
+#pragma unroll
+      for (int k = 0; k < N; ++k) out[k * nc + c] = Psi[k];
+      out[N * nc + c] = Gam;
+    } else {
+      out[c] = c4eq<N, D>(w, f, ps);
+    }
   }
 }
 

@@ -155,9 +155,9 @@ __device__ __forceinline__ void interp_limit32(float* Vt, double* at, const doub
   mix_SP<double, N>(f, alt, S, P);
   const double rc2 = rho_c2(S, P, (double)Vt[L::EN]);
   if (hs || rc2 < pr.hs_rc2) {
-    double Vn[M], rho, c, rc2n;
-    cell_prim<N, D>(Wn, f, Vn, rho, c, rc2n);
-    hs |= rc2 < dmin(pr.hs_rc2, rc2n);
+    double Vn[M], rho, Sn, Pn;
+    cell_vars<N, D>(Wn, f, Vn, rho, Sn, Pn);
+    hs |= rc2 < dmin(pr.hs_rc2, rho_c2(Sn, Pn, Vn[L::EN]));
     if (hs) {
 #pragma unroll
       for (int m = 0; m < M; ++m) Vt[m] = (float)Vn[m];
@@ -647,12 +647,12 @@ __device__ __forceinline__ bool face32_body(int64_t t, const Nodes6& nd, const d
     for (int m = 0; m < M; ++m) Wn[m] = W[m * nc + nd.c[j]];
   };
   auto load_node = [&](int j, double* Vn, double* Wn) {
-    double rho, cs, rc2;
+    double rho, S, P;
     load_state(j, Wn);
-    cell_prim<N, D>(Wn, f, Vn, rho, cs, rc2);
+    cell_vars<N, D>(Wn, f, Vn, rho, S, P);
   };
-  // first-order HLLC in FP32 from the node states, alpha slots in FP64
-  auto first_order = [&](const double* Vi, const double* Vj, FluxPack<N, D>& H) {
+  // first-order HLLC in FP32 from the node states, alpha slots in FP64 (Wi, Wj)
+  auto first_order = [&](const double* Wi, const double* Wj, FluxPack<N, D>& H) {
     PrimState<float, N, D> a, b;
 #pragma unroll
     for (int m = 0; m < M; ++m) {
@@ -665,19 +665,19 @@ __device__ __forceinline__ bool face32_body(int64_t t, const Nodes6& nd, const d
     for (int m = 0; m < L::NC; ++m) H.Gc[m] = (double)GH[m];
 #pragma unroll
     for (int k = 0; k < N - 1; ++k) {
-      const double ga = alpha_flux(Vi[L::AL + k], Vj[L::AL + k], uH);
-      H.gm[k] = ga - uH * Vi[L::AL + k];
-      H.gp[k] = ga - uH * Vj[L::AL + k];
+      const double ga = alpha_flux(Wi[L::AL + k], Wj[L::AL + k], uH);
+      H.gm[k] = ga - uH * Wi[L::AL + k];
+      H.gp[k] = ga - uH * Wj[L::AL + k];
     }
   };
 
   FluxPack<N, D> G;
   if (pr.scheme == 1) {
     if constexpr (DEFER) return false;
-    double Vi[M], Vj[M], Wi[M], Wj[M];
-    load_node(2, Vi, Wi);
-    load_node(3, Vj, Wj);
-    first_order(Vi, Vj, G);
+    double Wi[M], Wj[M];
+    load_state(2, Wi);
+    load_state(3, Wj);
+    first_order(Wi, Wj, G);
   } else {
     float p6[6], u6[6];
 #pragma unroll
@@ -951,7 +951,7 @@ __device__ __forceinline__ bool face32_body(int64_t t, const Nodes6& nd, const d
       load_node(2, Vi, Wi);
       load_node(3, Vj, Wj);
       FluxPack<N, D> H;
-      first_order(Vi, Vj, H);
+      first_order(Wi, Wj, H);
       double Fi[L::NC], Fj[L::NC];
       node_flux<N, D, DIR>(Wi, Vi, Fi);
       node_flux<N, D, DIR>(Wj, Vj, Fj);

@@ -345,8 +345,7 @@ __device__ __forceinline__ bool uniform_nodes(const double* __restrict__ W, int6
 // pipes (where the registers allow three blocks of 256 per SM, 1-4 % of a pass; in
 // the batched stage kernel's 80 registers they cost 2 %).
 template <int N, int D, bool SOFT = false>
-__device__ __forceinline__ void relax_fast(double* W, const DevFluid& f, double& rho_out, double& Re_out,
-                                           double* pT = nullptr) {
+__device__ __forceinline__ void relax_fast(double* W, const DevFluid& f, double& rho_out, double& Re_out) {
   using L = Lay<N, D>;
   const int l = f.liq;
   double rho = 0.0, Cv = 0.0, Rm = 0.0, rq = 0.0, m2 = 0.0;
@@ -378,59 +377,69 @@ __device__ __forceinline__ void relax_fast(double* W, const DevFluid& f, double&
   for (int k = 0; k < N - 1; ++k)
     // alpha_k = rho_k' R_k T* / (p* + p_inf,k), one stiffened gas at most
     W[L::AL + k] = mul(mul(mul(W[k], f.Rg[k]), k == l ? ps : ppl), z);
-  if (pT) {
-    pT[0] = ps;
-    pT[1] = z * ps * ppl;
-  }
   rho_out = rho;
   Re_out = Re;
 }
 
-// Infinite-rate thermal relaxation of one cell: keeps alpha_k rho_k, rho u, E and
-// replaces the stored alpha_k by rho Y_k / rho_k(p*, T*). p* is the positive root of
-// A_p p^2 + B_p p + C_p = 0 (Eqs. Ap_Bp_Cp_1-3, p_relax) in the cancellation-free
-// form, T* from Eq. T_relax_e. Species `liq` is the stiffened gas.
-// FAST (precision form): relax_fast.
-template <int N, int D, bool FAST = false>
-__device__ __forceinline__ void relax_cell(double* W, const DevFluid& f, double* pT = nullptr) {
-  if constexpr (FAST) {
-    double rho, Re;
-    relax_fast<N, D>(W, f, rho, Re, pT);
-    return;
-  }
-  using L = Lay<N, D>;
+// Relaxed pressure p* of one cell: the positive root of A_p p^2 + B_p p + C_p = 0
+// (Eqs. Ap_Bp_Cp_1-3, p_relax) in the cancellation-free form; its rho, rho e~, c_v
+// and Y of species `liq`, the stiffened gas. (Callers that need no more stop here:
+// the compiler leaves no out-of-line quotient out.)
+template <int N, int D>
+__device__ __forceinline__ double relaxed_p(const double* W, const DevFluid& f, double& rho, double& re, double& cvb,
+                                            double& Yl) {
   const int l = f.liq;
-  double rho = 0.0;
+  rho = 0.0;
 #pragma unroll
   for (int k = 0; k < N; ++k) rho += W[k];
   double Y[N];
 #pragma unroll
   for (int k = 0; k < N; ++k) Y[k] = quot(W[k], rho);
-  const double re = rhoe_tilde<N, D>(W, f);
-  double cvb = 0.0, cpb = 0.0;
+  re = rhoe_tilde<N, D>(W, f);
+  cvb = 0.0;
+  double cpb = 0.0;
 #pragma unroll
   for (int k = 0; k < N; ++k) {
     cvb += prod(Y[k], f.cv[k]);
     cpb += prod(Y[k], f.cp[k]);
   }
-  const double pinf1 = f.pinf[l], R1 = f.Rg[l], Yl = Y[l];
+  Yl = Y[l];
+  const double pinf1 = f.pinf[l], R1 = f.Rg[l];
   const double Ap = cvb, Rb = cpb - cvb, YR = prod(Yl, R1);
   const double Bp = -(prod(re, Rb) - prod(pinf1, cvb) - prod(prod(pinf1, Yl), R1));
   const double Cp = -prod(prod(re, pinf1), Rb - YR);
   const double sq = rsqrt_r(prod(Bp, Bp) - prod(soft::scale<2>(Ap), Cp));
   const bool pos = Bp > 0.0;
-  const double ps = quot(pos ? soft::scale<1>(-Cp) : sq - Bp, pos ? Bp + sq : soft::scale<1>(Ap));
-  const double pl = ps + pinf1;
+  return quot(pos ? soft::scale<1>(-Cp) : sq - Bp, pos ? Bp + sq : soft::scale<1>(Ap));
+}
+
+// p* and T* (Eq. T_relax_e).
+template <int N, int D>
+__device__ __forceinline__ void relaxed_pT(const double* W, const DevFluid& f, double& ps, double& Ts) {
+  const int l = f.liq;
+  double rho, re, cvb, Yl;
+  ps = relaxed_p<N, D>(W, f, rho, re, cvb, Yl);
+  const double pinf1 = f.pinf[l], pl = ps + pinf1;
   const double den = quot(prod(prod(Yl, ps + prod(f.gamma[l], pinf1)), f.cv[l]), pl) + cvb - prod(Yl, f.cv[l]);
-  const double Ts = quot(quot(re, rho), den);
+  Ts = quot(quot(re, rho), den);
+}
+
+// Infinite-rate thermal relaxation of one cell: keeps alpha_k rho_k, rho u, E and
+// replaces the stored alpha_k by rho Y_k / rho_k(p*, T*). FAST (precision form):
+// relax_fast.
+template <int N, int D, bool FAST = false>
+__device__ __forceinline__ void relax_cell(double* W, const DevFluid& f) {
+  if constexpr (FAST) {
+    double rho, Re;
+    relax_fast<N, D>(W, f, rho, Re);
+    return;
+  }
+  double ps, Ts;
+  relaxed_pT<N, D>(W, f, ps, Ts);
 #pragma unroll
   for (int k = 0; k < N - 1; ++k) {
     const double rhok = quot(ps + f.pinf[k], prod(f.Rg[k], Ts));
-    W[L::AL + k] = quot(W[k], rhok);
-  }
-  if (pT) {
-    pT[0] = ps;
-    pT[1] = Ts;
+    W[Lay<N, D>::AL + k] = quot(W[k], rhok);
   }
 }
 
