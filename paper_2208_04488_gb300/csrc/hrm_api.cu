@@ -256,16 +256,36 @@ bool defer_sweep(const hrm_ctx* c) {
   return c->params.precision == HRM_FP32 && c->params.scheme == HRM_SCHEME_WCNS && c->params.screen;
 }
 
+// Whether a stage lists its non-uniform midpoints (hrm_sweep.cuh); else every sweep
+// covers all midpoints and tests the six nodes itself, and the update reads every
+// flux. The first-order scheme has no uniform stencils, and up to these sizes the
+// list kernels (two more in the chain of each stage, 3 to 4 us each) cost more than
+// full warps and fewer fluxes give back. whole: the precision form's stage one at a
+// time and its RHS, whose update reads every flux in any case.
+// Measured us per step, lists | none, on the developed shock-bubble and the smooth
+// advection (no uniform stencil): precision form 128x64 196 | 174, 90x90 120 | 101;
+// 256x128 218 | 199, 300x300 234 | 225; 512x256 298 | 313, 1024x512 557 | 760, but
+// 512x512 advection 530 | 460. One stage at a time 512x256 425 | 382, 512x512
+// advection 623 | 545; 1024x512 734 | 833. FP64 128x64 443 | 419, 90x90 386 | 366,
+// 128x128 442 | 421; 256x128 1049 | 1087, 32^3 593 | 646, 1024x512 5794 | 10765.
+constexpr int64_t kListedCells32 = 65536, kListedCells32Whole = 262144, kListedCells64 = 16384;
+bool listed(const hrm_ctx* c, bool whole) {
+  if (c->params.scheme != HRM_SCHEME_WCNS) return false;
+  if (c->params.precision == HRM_FP64) return c->nint > kListedCells64;
+  return c->nint > (whole ? kListedCells32Whole : kListedCells32);
+}
+
 // Kernels one sweep launches.
 int sweep_kernels(const hrm_ctx* c) { return defer_sweep(c) ? 2 : 1; }
 
-GateArgs gate_of(const hrm_ctx* c, int d) {
+// lists: whether the stage has them
+GateArgs gate_of(const hrm_ctx* c, int d, bool lists) {
   GateArgs g;
   if (defer_sweep(c)) {
     g.defer_list = c->defer + (size_t)d * (size_t)c->defer_cap;
   }
   if (c->params.learned) g.fixed = c->gate[d];
-  g.list = c->lists.list[d];
+  g.list = lists ? c->lists.list[d] : nullptr;
   g.list_cnt = c->lists.cnt + kSweepCounts * d;
   if (c->params.learned == 1 && defer_sweep(c)) {  // the network inside the sweep
     g.net = c->blob;
@@ -278,15 +298,18 @@ GateArgs gate_of(const hrm_ctx* c, int d) {
 
 // Uniform faces and the lists of the other midpoints of Wsrc (its primitives or
 // FP32 planes are up to date); full: the uniform faces' fluxes into the flux
-// planes as well.
-int enqueue_mark(hrm_ctx* c, cudaStream_t s, const double* Wsrc, bool full) {
+// planes as well. Without lists only the counters of deferred midpoints are cleared.
+int enqueue_mark(hrm_ctx* c, cudaStream_t s, const double* Wsrc, bool lists, bool full) {
+  if (!lists) {
+    if (defer_sweep(c)) cudaMemsetAsync(c->lists.cnt, 0, sizeof(uint32_t) * kSweepCounters, s);
+    return 0;
+  }
   SweepLists l = c->lists;
-  const bool fp32 = c->params.precision == HRM_FP32;
   for (int d = 0; d < c->D; ++d) {
     l.F[d] = full ? c->F[d] : nullptr;
     l.gate[d] = c->params.learned == 1 && defer_sweep(c) ? c->gate[d] : nullptr;
   }
-  launch_mark(c->N, c->D, Wsrc, c->V, fp32 ? c->P32 : nullptr, c->dg, l, c->params.scheme == HRM_SCHEME_HLLC1, s);
+  launch_mark(c->N, c->D, Wsrc, c->V, c->params.precision == HRM_FP32 ? c->P32 : nullptr, c->dg, l, s);
   return 2;
 }
 
@@ -341,16 +364,19 @@ int enqueue_stage(hrm_ctx* c, cudaStream_t s, const double* Wsrc, double* Wout, 
       });
       ++k;
     }
-  k += enqueue_mark(c, s, Wsrc, c->params.precision == HRM_FP32 && !fuse_next);
+  const bool whole = c->params.precision == HRM_FP32 && !fuse_next, lists = listed(c, whole);
+  k += enqueue_mark(c, s, Wsrc, lists, whole);
   Update32Args up{};
   if (fuse_next) {
     up = {c->Wn, Wsrc, Wout, c->F[0], c->F[1], c->F[2], c->st, a, b, relax, count, c->P32, r32_target(c),
-          c->lists.uni, src_relaxed ? 1 : 0};
-    cudaEventRecord(c->ev_mark, s);
-    cudaStreamWaitEvent(c->keep, c->ev_mark, 0);
-    launch_update32p(c->N, c->D, up, c->dg, c->fl, tau_next ? 1 : 0, c->lists, 0, c->keep);
-    cudaEventRecord(c->ev_keep, c->keep);
-    ++k;
+          lists ? c->lists.uni : nullptr, src_relaxed ? 1 : 0};
+    if (up.uni) {
+      cudaEventRecord(c->ev_mark, s);
+      cudaStreamWaitEvent(c->keep, c->ev_mark, 0);
+      launch_update32p(c->N, c->D, up, c->dg, c->fl, tau_next ? 1 : 0, c->lists, 0, c->keep);
+      cudaEventRecord(c->ev_keep, c->keep);
+      ++k;
+    }
   }
   // the sweeps: independent (each reads the primitives and writes its own flux
   // planes), so directions d > 0 run on their own streams beside direction 0
@@ -362,7 +388,7 @@ int enqueue_stage(hrm_ctx* c, cudaStream_t s, const double* Wsrc, double* Wout, 
     }
     for (int d = 0; d < c->D; ++d) {
       const cudaStream_t sd = (fork && d > 0) ? c->par[d] : s;
-      GateArgs ga = gate_of(c, d);
+      GateArgs ga = gate_of(c, d, lists);
       if (ga.defer_list) {  // the deferred midpoints run beside the next sweep
         ga.side = c->side[d];
         ga.ev_fast = c->ev_fast[d];
@@ -382,14 +408,14 @@ int enqueue_stage(hrm_ctx* c, cudaStream_t s, const double* Wsrc, double* Wout, 
   });
   if (defer_sweep(c))
     for (int d = 0; d < c->D; ++d) cudaStreamWaitEvent(s, c->ev_fix[d], 0);
-  if (fuse_next) cudaStreamWaitEvent(s, c->ev_keep, 0);
+  if (up.uni) cudaStreamWaitEvent(s, c->ev_keep, 0);
   traced(c, s, HRM_KERNEL_UPDATE, [&] {
     if (fuse_next)
       launch_update32p(c->N, c->D, up, c->dg, c->fl, tau_next ? 1 : 0, c->lists, 1, s);
     else
       c->fk->update(0, c->params.precision == HRM_FP32, c->Wn, Wsrc, Wout, c->F[0], c->F[1], c->F[2], c->dg,
                     c->fl, c->st, a, b, relax, count, same_out ? same : nullptr,
-                    c->params.precision == HRM_FP64 ? c->lists.uni : nullptr, c->V, src_relaxed ? 1 : 0, s);
+                    c->params.precision == HRM_FP64 && lists ? c->lists.uni : nullptr, c->V, src_relaxed ? 1 : 0, s);
   });
   ++k;
   return k;
@@ -1236,7 +1262,8 @@ hrm_status hrm_rhs(hrm_ctx* c, const double* lam, double* rhs) {
     launch_prim32(c->N, c->D, c->Wn, c->P32, r32_target(c), c->dg, c->fl, c->st, 0, c->stream);
   else
     c->ck->prim(c->Wn, c->V, c->AUX, p32_target(c), r32_target(c), c->dg, c->fl, c->st, 0, nullptr, c->stream);
-  c->launches += enqueue_mark(c, c->stream, c->Wn, true);
+  const bool lists = listed(c, true);
+  c->launches += enqueue_mark(c, c->stream, c->Wn, lists, true);
   for (int d = 0; d < c->D; ++d) {
     if (separate_gate(c)) {
       launch_gate(c->N, c->D, d, c->P32, c->R32, c->dg, c->blob, gate_logit_threshold(c), c->gate[d],
@@ -1244,7 +1271,7 @@ hrm_status hrm_rhs(hrm_ctx* c, const double* lam, double* rhs) {
       ++c->launches;
     }
     c->fk->face[d](c->params.precision, c->Wn, c->V, c->AUX, c->P32, c->F[d], c->dg, c->fl, c->dp, c->st,
-                   gate_of(c, d), c->stream);
+                   gate_of(c, d, lists), c->stream);
   }
   c->fk->update(1, 0, c->Wn, c->Wn, out, c->F[0], c->F[1], c->F[2], c->dg, c->fl, c->st, 0.0, 1.0, 0, 0,
                 nullptr, nullptr, nullptr, 0, c->stream);

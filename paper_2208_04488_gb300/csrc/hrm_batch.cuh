@@ -122,7 +122,7 @@ __device__ __forceinline__ bool stage_uniform(const BatchInst& I, int64_t t, int
   const int64_t nc = I.g.ncells;
   double G[L::NC];
   if constexpr (FP32) {
-    if (!uniform_stencil<N, D>(I.P32, nc, nd)) return false;
+    if (!uniform_stencil<N, D, 4>(I.P32, nc, nd)) return false;
     uniform_flux32<N, D>(nd.c[2], DIR, I.P32, nc, G);
   } else {
     if (!uniform_nodes<N, D>(W, nc, nd)) return false;

@@ -470,13 +470,13 @@ __global__ void __launch_bounds__(kCellThreads)
 }
 
 // True when every FP32 plane holds the same value at the six nodes of a midpoint
-// (a NaN anywhere makes it false). Four planes per loop trip: the batched stage
-// kernel that calls it shares its register budget with every phase (fully
-// unrolled, the loads spilled).
-template <int N, int D>
+// (a NaN anywhere makes it false). UNROLL planes per loop trip: four in the batched
+// stage kernel, which shares its register budget with every phase (fully unrolled,
+// the loads spilled); all of them elsewhere, so that many loads are in flight.
+template <int N, int D, int UNROLL = P32Lay<N, D>::PLANES>
 __device__ __forceinline__ bool uniform_stencil(const float* __restrict__ P32, int64_t nc, const Nodes6& nd) {
   bool same = true;
-#pragma unroll 4
+#pragma unroll(UNROLL)
   for (int q = 0; q < P32Lay<N, D>::PLANES; ++q) {
     const float* p = P32 + (int64_t)q * nc;
     float v[6];
@@ -485,6 +485,21 @@ __device__ __forceinline__ bool uniform_stencil(const float* __restrict__ P32, i
     same = same & (v[0] == v[2]) & (v[1] == v[2]) & (v[3] == v[2]) & (v[4] == v[2]) & (v[5] == v[2]);
   }
   return same;
+}
+
+// Sweeps without a list test every midpoint's own six nodes: whether t is uniform,
+// and if so its flux (the node's, from the planes) written.
+template <int N, int D, int DIR>
+__device__ __forceinline__ bool uniform_midpoint32(int64_t t, const Nodes6& nd, const float* __restrict__ P32,
+                                                   double* __restrict__ out, const DevGrid& g) {
+  using L = Lay<N, D>;
+  if (!uniform_stencil<N, D>(P32, g.ncells, nd)) return false;
+  double G[L::NC];
+  uniform_flux32<N, D>(nd.c[2], DIR, P32, g.ncells, G);
+  const int64_t nf = face_count<DIR>(g);
+#pragma unroll
+  for (int m = 0; m < L::M + N - 1; ++m) out[m * nf + t] = m < L::NC ? G[m < L::NC ? m : 0] : 0.0;
+  return true;
 }
 
 // Appends index t to a worklist where `need` (all lanes of the warp call it;
@@ -600,6 +615,17 @@ __global__ void __launch_bounds__(kCellThreads)
   for (int d = 0; d < D; ++d) s[d] = 0.0;
   const bool changed = c < g.nint && !update32p_keep<N, D>(c, A, g, f, tau ? s : nullptr);
   block_append(changed, (uint32_t)c, cells, cnt);
+  if (tau) block_tau_max<D>(s, A.st->tau_bits);
+}
+
+// Without lists, over all cells after the sweeps.
+template <int N, int D>
+__global__ void __launch_bounds__(kCellThreads) k_update32p_all(Update32Args A, DevGrid g, DevFluid f, int tau) {
+  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  double s[D];
+#pragma unroll
+  for (int d = 0; d < D; ++d) s[d] = 0.0;
+  if (c < g.nint && !update32p_keep<N, D>(c, A, g, f, tau ? s : nullptr)) update32p_change<N, D>(c, A, g, f, tau ? s : nullptr);
   if (tau) block_tau_max<D>(s, A.st->tau_bits);
 }
 
@@ -974,11 +1000,26 @@ __device__ __forceinline__ bool face32_body(int64_t t, const Nodes6& nd, const d
 // compiler's FP32 contraction): midpoints whose screens fail are appended to
 // `deferred` (warp-aggregated; order not significant), counted in cnt[2], for
 // k_face32_fix.
-template <int N, int D, int DIR>
-__global__ void __launch_bounds__(kFaceThreads, 6)
+// Not LISTED: every midpoint of the direction, a thread each. Small grids, whose few
+// warps wait for one another's latency: four blocks of 128 registers, which spill
+// little (us per step with six: 128x64 187 -> 175, 256x128 205 -> 196, 512x256 384 ->
+// 313).
+template <int N, int D, int DIR, bool LISTED>
+__global__ void __launch_bounds__(kFaceThreads, LISTED ? 6 : 4)
     k_face32_fast(const double* __restrict__ W, const float* __restrict__ P32, double* __restrict__ out, DevGrid g,
                   DevFluid f, DevParams pr, const StepState* __restrict__ st, const uint8_t* __restrict__ gate,
                   const uint32_t* __restrict__ list, uint32_t* __restrict__ cnt, uint32_t* __restrict__ deferred) {
+  if constexpr (!LISTED) {
+    const int64_t t = (int64_t)blockIdx.x * kFaceThreads + threadIdx.x;
+    Nodes6 nd;
+    bool need = false;
+    if (face_nodes<DIR>(g, t, nd) && !uniform_midpoint32<N, D, DIR>(t, nd, P32, out, g)) {
+      const bool lin = gate != nullptr && gate[t] != 0;
+      need = !face32_body<N, D, DIR, true>(t, nd, W, nullptr, nullptr, P32, out, g, f, pr, st->lam[DIR], lin);
+    }
+    defer_push(need, t, deferred, &cnt[2]);
+    return;
+  }
   const uint32_t n = cnt[0];
   uint32_t i;
   while (next_entries(cnt, n, i)) {
@@ -1015,13 +1056,22 @@ __global__ void __launch_bounds__(kFaceThreads, 2)
   }
 }
 
-// The same list with the full body in one kernel (screens off, first-order scheme).
-template <int N, int D, int DIR>
+// The same with the full body in one kernel (screens off, first-order scheme).
+template <int N, int D, int DIR, bool LISTED>
 __global__ void __launch_bounds__(kFaceThreads, 3)
     k_face32(const double* __restrict__ W, const double* __restrict__ V, const double* __restrict__ AUX,
              const float* __restrict__ P32, double* __restrict__ out, DevGrid g, DevFluid f, DevParams pr,
              const StepState* __restrict__ st, const uint8_t* __restrict__ gate, const uint32_t* __restrict__ list,
              uint32_t* __restrict__ cnt) {
+  if constexpr (!LISTED) {
+    const int64_t t = (int64_t)blockIdx.x * kFaceThreads + threadIdx.x;
+    Nodes6 nd;
+    if (!face_nodes<DIR>(g, t, nd)) return;
+    if (pr.scheme == 0 && uniform_midpoint32<N, D, DIR>(t, nd, P32, out, g)) return;
+    const bool lin = gate != nullptr && gate[t] != 0;
+    face32_body<N, D, DIR>(t, nd, W, V, AUX, P32, out, g, f, pr, st->lam[DIR], lin);
+    return;
+  }
   const uint32_t n = cnt[0];
   uint32_t i;
   while (next_entries(cnt, n, i)) {

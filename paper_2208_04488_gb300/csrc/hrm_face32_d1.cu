@@ -9,26 +9,38 @@ namespace {
 
 constexpr int kD = 1;
 
+// Blocks of the sweep with the network, of the screened one and of the full one.
+template <int N, int DIR, bool LISTED>
+void launch_as(unsigned net, unsigned fast, unsigned full, const double* W, const double* V, const double* AUX,
+               const float* P32, double* out, const DevGrid& g, const DevFluid& f, const DevParams& p, const StepState* st,
+               const GateArgs& gate, cudaStream_t s) {
+  if (!gate.defer_list) {
+    k_face32<N, kD, DIR, LISTED><<<full, kFaceThreads, 0, s>>>(W, V, AUX, P32, out, g, f, p, st, gate.fixed, gate.list,
+                                                               gate.list_cnt);
+    return;
+  }
+  if (gate.net)
+    k_face32_net<N, kD, DIR, LISTED><<<net, kFaceThreads, 0, s>>>(
+        W, P32, gate.R32, out, g, f, p, st, static_cast<const mlp::GateBlob*>(gate.net), gate.zthr, gate.out_gate,
+        gate.list, gate.list_cnt, gate.defer_list);
+  else
+    k_face32_fast<N, kD, DIR, LISTED><<<fast, kFaceThreads, 0, s>>>(W, P32, out, g, f, p, st, gate.fixed, gate.list,
+                                                                    gate.list_cnt, gate.defer_list);
+  const cudaStream_t sf = fix_stream(gate, s);
+  k_face32_fix<N, kD, DIR><<<kFixBlocks, kFixThreads, 0, sf>>>(W, P32, out, g, f, p, st, gate.fixed, gate.defer_list,
+                                                                gate.list_cnt + 2);
+  fix_done(gate);
+}
+
 template <int N, int DIR>
 void launch(const double* W, const double* V, const double* AUX, const float* P32, double* out, const DevGrid& g,
             const DevFluid& f, const DevParams& p, const StepState* st, const GateArgs& gate, cudaStream_t s) {
   if constexpr (DIR < kD) {
-    if (gate.defer_list) {
-      if (gate.net)
-        k_face32_net<N, kD, DIR><<<list_grid(g, DIR, 5), kFaceThreads, 0, s>>>(
-            W, P32, gate.R32, out, g, f, p, st, static_cast<const mlp::GateBlob*>(gate.net), gate.zthr, gate.out_gate,
-            gate.list, gate.list_cnt, gate.defer_list);
-      else
-        k_face32_fast<N, kD, DIR><<<list_grid(g, DIR, 6), kFaceThreads, 0, s>>>(
-            W, P32, out, g, f, p, st, gate.fixed, gate.list, gate.list_cnt, gate.defer_list);
-      const cudaStream_t sf = fix_stream(gate, s);
-      k_face32_fix<N, kD, DIR><<<kFixBlocks, kFixThreads, 0, sf>>>(W, P32, out, g, f, p, st, gate.fixed,
-                                                                    gate.defer_list, gate.list_cnt + 2);
-      fix_done(gate);
-    } else {
-      k_face32<N, kD, DIR><<<list_grid(g, DIR, 3), kFaceThreads, 0, s>>>(W, V, AUX, P32, out, g, f, p, st, gate.fixed,
-                                                                         gate.list, gate.list_cnt);
-    }
+    if (gate.list)
+      launch_as<N, DIR, true>(list_grid(g, DIR, 5), list_grid(g, DIR, 6), list_grid(g, DIR, 3), W, V, AUX, P32, out, g, f, p, st,
+                              gate, s);
+    else
+      launch_as<N, DIR, false>(all_grid(g, DIR), all_grid(g, DIR), all_grid(g, DIR), W, V, AUX, P32, out, g, f, p, st, gate, s);
   }
 }
 
@@ -53,6 +65,14 @@ void update32p_d1(int N, const Update32Args& A, const DevGrid& g, const DevFluid
       k_keep32<2, kD><<<gr, kCellThreads, 0, s>>>(A, g, f, tau, lists.cells, cnt);
     else if (N == 3)
       k_keep32<3, kD><<<gr, kCellThreads, 0, s>>>(A, g, f, tau, lists.cells, cnt);
+    return;
+  }
+  if (!A.uni) {
+    const unsigned th = cell_threads(g.nint), gr = grid_for(g.nint, th);
+    if (N == 2)
+      k_update32p_all<2, kD><<<gr, th, 0, s>>>(A, g, f, tau);
+    else if (N == 3)
+      k_update32p_all<3, kD><<<gr, th, 0, s>>>(A, g, f, tau);
     return;
   }
   const unsigned gr = resident_grid(g.nint, kCellThreads, 3);

@@ -124,6 +124,40 @@ __device__ __forceinline__ void weno_both(const double* v, double eps, bool lin,
   }
 }
 
+// First-order HLLC flux and u_* of a midpoint from its two node states (Sec. 4.1.1).
+template <int N, int D, int DIR>
+__device__ __forceinline__ void first_order64(const Nodes6& nd, const double* __restrict__ V, int64_t nc, const DevFluid& f,
+                                              FluxPack<N, D>& H) {
+  using L = Lay<N, D>;
+  PrimState<double, N, D> a, b;
+#pragma unroll
+  for (int m = 0; m < L::M; ++m) {
+    a.V[m] = V[m * nc + nd.c[2]];
+    b.V[m] = V[m * nc + nd.c[3]];
+  }
+  double GH[L::M];
+  const double uH = hllc<double, N, D, DIR>(f, a, b, GH);
+#pragma unroll
+  for (int m = 0; m < L::NC; ++m) H.Gc[m] = GH[m];
+#pragma unroll
+  for (int k = 0; k < N - 1; ++k) {
+    H.gm[k] = GH[L::AL + k] - uH * a.V[L::AL + k];
+    H.gp[k] = GH[L::AL + k] - uH * b.V[L::AL + k];
+  }
+}
+
+template <int N, int D, int DIR>
+__device__ __forceinline__ void store_flux64(int64_t t, const FluxPack<N, D>& G, double* __restrict__ out, int64_t nf) {
+  using L = Lay<N, D>;
+#pragma unroll
+  for (int m = 0; m < L::NC; ++m) out[m * nf + t] = G.Gc[m];
+#pragma unroll
+  for (int k = 0; k < N - 1; ++k) {
+    out[(L::AL + k) * nf + t] = G.gm[k];
+    out[(L::M + k) * nf + t] = G.gp[k];
+  }
+}
+
 // Column of a thread in the shared memory of a block of kFaceThreads: the biased
 // values of the two sides, then the midpoint states with their rho, E and c, then
 // the midpoint flux; 2 sides x (M + 3) slots.
@@ -184,42 +218,6 @@ __device__ __forceinline__ void face_body(int64_t t, const Nodes6& nd, const dou
     if constexpr (LANES > 1) __syncwarp(((1u << LANES) - 1u) << ((threadIdx.x & 31) / LANES * LANES));
   };
 
-  // first-order HLLC flux and u_* from the node states (Sec. 4.1.1), evaluated
-  // where it is used: the first-order scheme, and the flux limiter where it may act
-  auto first_order = [&](FluxPack<N, D>& H) {
-    PrimState<double, N, D> a, b;
-#pragma unroll
-    for (int m = 0; m < M; ++m) {
-      a.V[m] = V[m * nc + nd.c[2]];
-      b.V[m] = V[m * nc + nd.c[3]];
-    }
-    double GH[M];
-    const double uH = hllc<double, N, D, DIR>(f, a, b, GH);
-#pragma unroll
-    for (int m = 0; m < L::NC; ++m) H.Gc[m] = GH[m];
-#pragma unroll
-    for (int k = 0; k < N - 1; ++k) {
-      H.gm[k] = GH[L::AL + k] - uH * a.V[L::AL + k];
-      H.gp[k] = GH[L::AL + k] - uH * b.V[L::AL + k];
-    }
-  };
-  auto store = [&](const FluxPack<N, D>& G) {
-    if (sub != 0) return;
-#pragma unroll
-    for (int m = 0; m < L::NC; ++m) out[m * nf + t] = G.Gc[m];
-#pragma unroll
-    for (int k = 0; k < N - 1; ++k) {
-      out[(L::AL + k) * nf + t] = G.gm[k];
-      out[(M + k) * nf + t] = G.gp[k];
-    }
-  };
-
-  if (pr.scheme == 1) {
-    FluxPack<N, D> H;
-    first_order(H);
-    store(H);
-    return;
-  }
   double p6[6], u6[6];
 #pragma unroll
   for (int j = 0; j < 6; ++j) {
@@ -461,7 +459,7 @@ __device__ __forceinline__ void face_body(int64_t t, const Nodes6& nd, const dou
   }
   if (pr.limiters && !ok) {
     FluxPack<N, D> G, H;
-    first_order(H);
+    first_order64<N, D, DIR>(nd, V, nc, f, H);
     double Wi[M], Wj[M], Fi[L::NC], Fj[L::NC];
     {
       double Vi[M], Vj[M];
@@ -483,7 +481,7 @@ __device__ __forceinline__ void face_body(int64_t t, const Nodes6& nd, const dou
       G.gp[k] = slot(0, L::AL + k);
     }
     flux_limit<N, D>(Wi, Wj, Fi, Fj, lam, G, H, f, pr);
-    store(G);
+    if (sub == 0) store_flux64<N, D, DIR>(t, G, out, nf);
     group_sync();  // the column is the next midpoint's
     return;
   }
@@ -498,6 +496,34 @@ __device__ __forceinline__ void face_body(int64_t t, const Nodes6& nd, const dou
   }
 }
 
+// Without a list LANES lanes test the six nodes of their midpoint t themselves:
+// whether they are bit-identical (every plane of W), and if so its flux written.
+template <int N, int D, int DIR, int LANES>
+__device__ __forceinline__ bool uniform_midpoint64(int64_t t, const Nodes6& nd, const double* __restrict__ W,
+                                                   const double* __restrict__ V, double* __restrict__ out,
+                                                   const DevGrid& g) {
+  using L = Lay<N, D>;
+  const int lane = threadIdx.x & 31, sub = lane % LANES;
+  bool same = true;
+#pragma unroll
+  for (int m = 0; m < L::M; m += LANES) {
+    const int64_t plane = (int64_t)(m + sub < L::M ? m + sub : 0) * g.ncells;
+    const long long b = __double_as_longlong(W[plane + nd.c[2]]);
+#pragma unroll
+    for (int j = 0; j < 6; ++j)
+      if (j != 2) same = same & (__double_as_longlong(W[plane + nd.c[j]]) == b);
+  }
+  if (!__all_sync(((1u << LANES) - 1u) << (lane / LANES * LANES), same)) return false;
+  if (sub == 0) {
+    const int64_t nf = face_count<DIR>(g);
+    double G[L::NC];
+    uniform_flux64<N, D>(nd.c[2], DIR, W, V, g.ncells, G);
+#pragma unroll
+    for (int m = 0; m < L::M + N - 1; ++m) out[m * nf + t] = m < L::NC ? G[m < L::NC ? m : 0] : 0.0;
+  }
+  return true;
+}
+
 // Sweep of direction DIR over its list (k_mark), a warp of 32 entries at a time
 // taken from a counter: every lane then runs the whole body (the FP64 unit's time
 // does not depend on the active lanes), and the warps end within one entry of one
@@ -509,6 +535,7 @@ __device__ __forceinline__ void face_body(int64_t t, const Nodes6& nd, const dou
 // 12880 815 | 582 | 606 | 758, 20100 1307 | 1028 | 710 | 835, 32896 2048 | 1500 |
 // 1083 | 1043; two: 3080 228 | 228 | 260 | 411, 5256 341 | 351 | 369 | 445, 12210
 // 559 | 420 | 435 | 478, 17030 757 | 633 | 462 | 484, 25760 965 | 701 | 497 | 481.
+// No list (small grids, kListedCells64): every midpoint, by the same rule.
 constexpr uint32_t kSplit8 = 4608, kSplit4 = 13312, kSplit2 = 20480;
 
 template <int N, int D, int DIR, int LANES>
@@ -522,8 +549,9 @@ __device__ __forceinline__ void sweep_split(const double* __restrict__ W, const 
     Nodes6 nd;
     const uint32_t i = k * per + (threadIdx.x & 31) / LANES;
     if (i >= n) continue;
-    const int64_t t = list[i];
+    const int64_t t = list ? list[i] : i;
     if (!face_nodes<DIR>(g, t, nd)) continue;
+    if (!list && uniform_midpoint64<N, D, DIR, LANES>(t, nd, W, V, out, g)) continue;
     const bool lin = gate != nullptr && gate[t] != 0;
     face_body<N, D, DIR, LANES>(t, nd, W, V, AUX, out, g, f, pr, st->lam[DIR], col, lin);
   }
@@ -535,10 +563,10 @@ __global__ void __launch_bounds__(kFaceThreads, 3)
            double* __restrict__ out, DevGrid g, DevFluid f, DevParams pr, const StepState* __restrict__ st,
            const uint8_t* __restrict__ gate, const uint32_t* __restrict__ list, uint32_t* __restrict__ cnt) {
   __shared__ double col[kFaceCol<N, D>];
-  const uint32_t n = cnt[0];
+  const uint32_t n = list ? cnt[0] : (uint32_t)face_count<DIR>(g);
   if (n <= kSplit8) return sweep_split<N, D, DIR, 8>(W, V, AUX, out, g, f, pr, st, gate, list, n, col);
   if (n <= kSplit4) return sweep_split<N, D, DIR, 4>(W, V, AUX, out, g, f, pr, st, gate, list, n, col);
-  if (n <= kSplit2) return sweep_split<N, D, DIR, 2>(W, V, AUX, out, g, f, pr, st, gate, list, n, col);
+  if (n <= kSplit2 || !list) return sweep_split<N, D, DIR, 2>(W, V, AUX, out, g, f, pr, st, gate, list, n, col);
   uint32_t i;
   while (next_entries(cnt, n, i)) {
     Nodes6 nd;
@@ -548,6 +576,18 @@ __global__ void __launch_bounds__(kFaceThreads, 3)
     const bool lin = gate != nullptr && gate[t] != 0;
     face_body<N, D, DIR>(t, nd, W, V, AUX, out, g, f, pr, st->lam[DIR], col, lin);
   }
+}
+
+// The first-order scheme: every midpoint, a thread each.
+template <int N, int D, int DIR>
+__global__ void __launch_bounds__(kFaceThreads)
+    k_face_first(const double* __restrict__ V, double* __restrict__ out, DevGrid g, DevFluid f) {
+  const int64_t t = (int64_t)blockIdx.x * kFaceThreads + threadIdx.x;
+  Nodes6 nd;
+  if (!face_nodes<DIR>(g, t, nd)) return;
+  FluxPack<N, D> H;
+  first_order64<N, D, DIR>(nd, V, g.ncells, f, H);
+  store_flux64<N, D, DIR>(t, H, out, face_count<DIR>(g));
 }
 
 }  // namespace hrm

@@ -18,8 +18,11 @@ void face_l(int precision, const double* W, const double* V, const double* AUX, 
       face32_d2(N, DIR, W, V, AUX, P32, out, g, f, p, st, gate, s);
       return;
     }
-    k_face<N, kD, DIR><<<list_grid(g, DIR, 3, 8), kFaceThreads, 0, s>>>(W, V, AUX, out, g, f, p, st, gate.fixed,
-                                                                     gate.list, gate.list_cnt);
+    if (p.scheme == 1)
+      k_face_first<N, kD, DIR><<<all_grid(g, DIR), kFaceThreads, 0, s>>>(V, out, g, f);
+    else
+      k_face<N, kD, DIR><<<list_grid(g, DIR, 3, 8), kFaceThreads, 0, s>>>(W, V, AUX, out, g, f, p, st, gate.fixed,
+                                                                       gate.list, gate.list_cnt);
   }
 }
 
@@ -32,11 +35,11 @@ void update_l(int mode, int fast, const double* Wn, const double* Wsrc, double* 
     update32_d2(N, Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count, s);
     return;
   }
-  const unsigned gr = grid_for(g.nint, kCellThreads);
+  const unsigned th = cell_threads(g.nint), gr = grid_for(g.nint, th);
   if (mode == 1)
-    k_update<N, kD, 1><<<gr, kCellThreads, 0, s>>>(Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count);
+    k_update<N, kD, 1><<<gr, th, 0, s>>>(Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count);
   else
-    k_update<N, kD, 0><<<gr, kCellThreads, 0, s>>>(Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count,
+    k_update<N, kD, 0><<<gr, th, 0, s>>>(Wn, Wsrc, Wout, F0, F1, F2, g, f, st, a, b, relax, count,
                                                    same, uni, V, src_relaxed);
 }
 

@@ -47,7 +47,8 @@ struct GateArgs {
   const float* R32 = nullptr;
   float zthr = 0.f;
   uint8_t* out_gate = nullptr;
-  // the midpoints to sweep and their counters (SweepLists of the direction)
+  // the midpoints to sweep (nullptr: all of the direction) and their counters
+  // (SweepLists of the direction; without a list, list_cnt[2] must be 0)
   const uint32_t* list = nullptr;
   uint32_t* list_cnt = nullptr;
 };
@@ -161,11 +162,23 @@ void launch_set_dt(StepState* st, double dt, cudaStream_t s);
 
 inline unsigned grid_for(long long n, int threads) { return (unsigned)((n + threads - 1) / threads); }
 
+// Threads per block of a kernel with a thread per cell and FP64 work: 256, or 64
+// where blocks of 256 would leave every other SM idle (a warp alone on its SM issues
+// an FP64 instruction every 64 cycles, eight share the unit at 19 each). Measured us
+// per step with 64 | 256: precision form 90x90 103 | 112, 128x64 175 | 179; 256x128
+// 196 | 190.
+inline unsigned cell_threads(long long n) {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return n < 128ll * sms ? 64u : 256u;
+}
+
 // Uniform faces and the lists of the other midpoints of a stage's source state
 // (hrm_sweep.cuh): two launches. P32 NULL: the FP64 form, from W and V; else the
-// precision form, from its FP32 planes. all: every midpoint is listed.
+// precision form, from its FP32 planes.
 void launch_mark(int N, int D, const double* W, const double* V, const float* P32, const DevGrid& g,
-                 const SweepLists& lists, int all, cudaStream_t s);
+                 const SweepLists& lists, cudaStream_t s);
 
 // Blocks for up to n items of a list that its warps take from a counter: what is
 // resident at per_sm blocks on each SM, or fewer where n needs no more.
@@ -175,6 +188,11 @@ inline unsigned resident_grid(long long n, int threads, int per_sm) {
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const long long all = (n + threads - 1) / threads, fit = (long long)(sms > 0 ? sms : 1) * per_sm;
   return (unsigned)(all < fit ? all : fit);
+}
+
+// Blocks of kFaceThreads with a thread per midpoint of a direction.
+inline unsigned all_grid(const DevGrid& g, int dir) {
+  return grid_for((g.n[0] + (dir == 0)) * (g.n[1] + (dir == 1)) * (g.n[2] + (dir == 2)), 128);
 }
 
 // Blocks of kFaceThreads of a list-driven sweep at `lanes` threads per midpoint.

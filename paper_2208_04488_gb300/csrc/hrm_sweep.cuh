@@ -8,7 +8,8 @@
 // are uniform and appends the other midpoints to a list per direction (k_mark).
 // The sweeps then run the body over full warps of listed midpoints, and the
 // update forms a uniform face's flux from the cell's own state, which the face's
-// nodes equal, so such faces are neither written nor read.
+// nodes equal, so such faces are neither written nor read. (Small grids and the
+// first-order scheme go without: `listed` in hrm_api.cu.)
 #pragma once
 
 #include "hrm_face32.cuh"
@@ -97,8 +98,7 @@ __global__ void __launch_bounds__(kCellThreads)
 }
 
 // uni[c], bits 2 d and 2 d + 1: the faces of cell c on the low and the high side
-// of direction d are uniform (no face is with `all`, the first-order scheme); bit
-// kFluxOverflow as in eq[c]. The
+// of direction d are uniform; bit kFluxOverflow as in eq[c]. The
 // other midpoints go to lists.list[d] in the order of their cells, one atomic per
 // block and direction. With lists.F (every midpoint's flux wanted) the uniform
 // faces' fluxes are written too, and with lists.gate their gate bytes. FP32: the
@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(kCellThreads)
 template <int N, int D, bool FP32>
 __global__ void __launch_bounds__(kCellThreads)
     k_mark(const double* __restrict__ W, const double* __restrict__ V, const float* __restrict__ P32, DevGrid g,
-           SweepLists lists, int all) {
+           SweepLists lists) {
   using L = Lay<N, D>;
   constexpr int kWarps = kCellThreads / 32;
   __shared__ uint32_t base[D][kWarps];
@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(kCellThreads)
   int64_t ijk[3] = {0, 0, 0};
   if (in) cell_index(g, c, ijk);
   unsigned uni = 0;
-  if (in && !all) {
+  if (in) {
 #pragma unroll
     for (int d = 0; d < D; ++d) {
       const int64_t stride = d == 0 ? 1 : (d == 1 ? g.n[0] : g.n[0] * g.n[1]);
