@@ -272,9 +272,9 @@ hrm_status hrm_time(hrm_ctx* ctx, double* t, int64_t* steps);
 
 /* Out-of-range indices met by the kernels of ctx so far, in a library built
  * with -DHRM_BOUNDS_CHECK (HRM_BOUNDS_CHECK=1 in the environment of the build),
- * where every midpoint's node index and every cell's midpoint index is checked
- * against its array and, when outside, counted and replaced by 0; -1 in a
- * release build or on error. A debugging aid in place of a memory checker (the
+ * where every midpoint's node index, every cell's midpoint index and every
+ * position and entry of a work list is checked against its array and, when
+ * outside, counted and replaced by 0; -1 in a release build or on error. A debugging aid in place of a memory checker (the
  * paper has no counterpart). Synchronises. */
 int64_t hrm_bounds_violations(hrm_ctx* ctx);
 
@@ -503,6 +503,8 @@ hrm_status hrm_batch_set_launch(hrm_batch* b, int32_t face_threads, int32_t face
  * resident), restores the states after every trial, keeps the fastest and
  * writes it to best[4] (128, 128, cell_tile, blocks_per_sm). */
 hrm_status hrm_batch_tune(hrm_batch* b, int32_t steps_per_trial, int32_t* best);
+/* As hrm_bounds_violations, over the instances of a batch. */
+int64_t hrm_batch_bounds_violations(hrm_batch* b);
 int64_t hrm_batch_kernel_launches(const hrm_batch* b);
 int64_t hrm_batch_total_cells(const hrm_batch* b);
 

@@ -535,7 +535,8 @@ hrm_status enqueue_persistent_step(hrm_ctx* c, cudaStream_t s) {
     A.listed = c->p_listed;
     A.deferred = c->p_deferred;
     // the segments of this context's species count (the others stay empty)
-    A.seg[1] = A.seg[3] = face_total(c->dg, 0);
+    A.seg[(c->N - 2) * 2 + 1] = face_total(c->dg, 0);
+    for (int key = (c->N - 2) * 2 + 2; key < 5; ++key) A.seg[key] = face_total(c->dg, 0) + face_total(c->dg, 1);
     A.stage = k;
     A.update = 1;
     hrm_status st;

@@ -71,11 +71,11 @@ struct StageArgs {
   GridSync* sync;
   uint64_t limit_ns;      // time limit of one barrier wait
   // listed midpoints: (instance << 40 | midpoint), one segment per species count
-  // and direction starting at seg[key], and those deferred to the full body
+  // and direction, seg[key] to seg[key + 1], and those deferred to the full body
   // (key << 62 | instance << 40 | midpoint)
   uint64_t* listed;
   uint64_t* deferred;
-  int64_t seg[4];
+  int64_t seg[5];
   int stage;              // 0..2: slot of the phase stamps
   int update;             // 1: the update phase runs in this launch (0: the caller runs it after)
 };
@@ -191,8 +191,10 @@ __device__ __forceinline__ bool stage_midpoints(const StageArgs& A, float* xs) {
       }
     }
     __syncthreads();
-    if (!uni)
-      A.listed[A.seg[key] + wbase[warp] + __popc(m & ((1u << lane) - 1u))] = (uint64_t)w.inst << 40 | (uint64_t)t;
+    if (!uni) {
+      const int64_t p = wbase[warp] + __popc(m & ((1u << lane) - 1u));
+      A.listed[A.seg[key] + HRM_IDX(I.g, p, A.seg[key + 1] - A.seg[key])] = (uint64_t)w.inst << 40 | (uint64_t)t;
+    }
   }
   if (!grid_barrier(A.sync, gridDim.x, A.limit_ns)) return false;
   {
@@ -215,9 +217,9 @@ __device__ __forceinline__ bool stage_midpoints(const StageArgs& A, float* xs) {
       bool done = true;
       uint64_t e = 0;
       if (i < n[key]) {
-        e = A.listed[A.seg[key] + i];
-        const BatchInst& I = A.insts[e >> 40];
-        const int64_t t = (int64_t)(e & kMidpoint);
+        e = A.listed[A.seg[key] + HRM_IDX(A.insts[0].g, (int64_t)i, A.seg[key + 1] - A.seg[key])];
+        const BatchInst& I = A.insts[HRM_IDX(A.insts[0].g, (int64_t)(e >> 40), A.ninst)];
+        const int64_t t = HRM_IDX(I.g, (int64_t)(e & kMidpoint), key & 1 ? face_count<1>(I.g) : face_count<0>(I.g));
         if (key == 0)
           done = stage_face<2, D, 0, FP32>(I, t, A.src, A.pr, xs);
         else if (key == 1)
@@ -227,7 +229,10 @@ __device__ __forceinline__ bool stage_midpoints(const StageArgs& A, float* xs) {
         else
           done = stage_face<3, D, 1, FP32>(I, t, A.src, A.pr, xs);
       }
-      if (!done) A.deferred[atomicAdd(&A.sync->deferred, 1u)] = (uint64_t)key << 62 | e;
+      if (!done) {
+        const int64_t p = atomicAdd(&A.sync->deferred, 1u);
+        A.deferred[HRM_IDX(A.insts[0].g, p, A.seg[4])] = (uint64_t)key << 62 | e;
+      }
     }
   }
   if (!grid_barrier(A.sync, gridDim.x, A.limit_ns)) return false;
@@ -236,10 +241,10 @@ __device__ __forceinline__ bool stage_midpoints(const StageArgs& A, float* xs) {
     const unsigned int warps = gridDim.x * (kBatchFace32Threads / 32);
     const unsigned int first = blockIdx.x + gridDim.x * warp;
     for (uint64_t i = first + (uint64_t)lane * warps; i < n; i += 32ull * warps) {
-      const uint64_t e = A.deferred[i];
+      const uint64_t e = A.deferred[HRM_IDX(A.insts[0].g, (int64_t)i, A.seg[4])];
       const int key = (int)(e >> 62);
-      const BatchInst& I = A.insts[e >> 40 & ((1ull << 22) - 1ull)];
-      const int64_t t = (int64_t)(e & kMidpoint);
+      const BatchInst& I = A.insts[HRM_IDX(A.insts[0].g, (int64_t)(e >> 40 & ((1ull << 22) - 1ull)), A.ninst)];
+      const int64_t t = HRM_IDX(I.g, (int64_t)(e & kMidpoint), key & 1 ? face_count<1>(I.g) : face_count<0>(I.g));
       Nodes6 nd;
       if (key == 0 && face_nodes<0>(I.g, t, nd)) face32_full<2, D, 0>(t, nd, I, A.src, A.pr, xs);
       if (key == 1 && face_nodes<1>(I.g, t, nd)) face32_full<2, D, 1>(t, nd, I, A.src, A.pr, xs);

@@ -45,6 +45,7 @@ struct hrm_batch {
   int ncell_items = 0;
   WorkItem* d_tiles = nullptr;   // 128-midpoint tiles, grouped by species count and direction (in pad)
   int ntiles = 0;
+  unsigned long long* oob = nullptr;  // bounds-check builds: count of out-of-range indices
   uint64_t* d_listed = nullptr;  // the stage's non-uniform midpoints, a segment per species count and direction
   uint64_t* d_deferred = nullptr;  // precision form: those left to the full body
   int64_t seg[5] = {};           // segment starts
@@ -164,7 +165,7 @@ hrm_status enqueue_stage(hrm_batch* b, cudaStream_t s, int stage) {
   A.limit_ns = kBarrierLimitNs;
   A.listed = b->d_listed;
   A.deferred = b->d_deferred;
-  for (int k = 0; k < 4; ++k) A.seg[k] = b->seg[k];
+  for (int k = 0; k < 5; ++k) A.seg[k] = b->seg[k];
   A.stage = stage;
   A.update = 1;
   hrm_status st;
@@ -251,6 +252,7 @@ void hrm_batch_destroy(hrm_batch* b) {
   cudaFree(b->d_cells);
   cudaFree(b->d_tiles);
   cudaFree(b->sync);
+  cudaFree(b->oob);
   cudaFree(b->d_listed);
   cudaFree(b->d_deferred);
   if (b->cap) cudaStreamDestroy(b->cap);
@@ -308,6 +310,10 @@ hrm_status hrm_batch_create(hrm_batch** out, int32_t ninst, const hrm_instance* 
   if (b->fit < 1) return bail(bfail(b, HRM_E_CUDA, "persistent stage kernel: no resident block fits an SM"));
   if ((s = bcuda(b, cudaMalloc(&b->sync, sizeof(GridSync)), "alloc grid sync"))) return bail(s);
   if ((s = bcuda(b, cudaMemset(b->sync, 0, sizeof(GridSync)), "clear grid sync"))) return bail(s);
+#ifdef HRM_BOUNDS_CHECK
+  if ((s = bcuda(b, cudaMalloc(&b->oob, sizeof *b->oob), "alloc bounds counter"))) return bail(s);
+  if ((s = bcuda(b, cudaMemset(b->oob, 0, sizeof *b->oob), "clear bounds counter"))) return bail(s);
+#endif
   b->host.resize(ninst);
   b->N.resize(ninst);
   b->relaxed.assign(ninst, 0);
@@ -340,7 +346,7 @@ hrm_status hrm_batch_create(hrm_batch** out, int32_t ninst, const hrm_instance* 
     fill_fluid_f(I.f);
     I.N = N;
     b->N[i] = N;
-    I.g.oob = nullptr;
+    I.g.oob = b->oob;
     I.g.ncells = 1;
     for (int d = 0; d < 3; ++d) {
       const int64_t n = d < 2 ? in.grid.n[d] : 1;
@@ -581,6 +587,15 @@ hrm_status hrm_batch_tune(hrm_batch* b, int32_t steps_per_trial, int32_t* best) 
     best[3] = best_shape.blocks_per_sm;
   }
   return HRM_OK;
+}
+
+int64_t hrm_batch_bounds_violations(hrm_batch* b) {
+  if (!b || !b->oob) return -1;
+  unsigned long long n = 0;
+  if (cudaMemcpyAsync(&n, b->oob, sizeof n, cudaMemcpyDeviceToHost, b->stream) != cudaSuccess ||
+      cudaStreamSynchronize(b->stream) != cudaSuccess)
+    return -1;
+  return (int64_t)n;
 }
 
 int64_t hrm_batch_kernel_launches(const hrm_batch* b) { return b ? b->launches : 0; }

@@ -64,6 +64,7 @@ struct DevGrid {
 
 // Bounds-check builds (-DHRM_BOUNDS_CHECK): an index outside [0, n) is counted
 // in g.oob and replaced by 0 instead of being used; release builds use it as is.
+// Every index that data decide goes through it: list positions and entries too.
 #ifdef HRM_BOUNDS_CHECK
 __device__ __forceinline__ int64_t hrm_checked_index(const DevGrid& g, int64_t i, int64_t n) {
   if (i >= 0 && i < n) return i;
@@ -99,9 +100,6 @@ __device__ __forceinline__ void cell_index(const DevGrid& g, int64_t c, int64_t*
 // groups of 32 taken, deferred midpoints); cells: the cells that the stage's update
 // changes, with the fourth set of counters; F: the flux planes where the uniform
 // faces' fluxes are wanted as well; gate: the gate bytes where they are.
-// A cell between two uniform faces takes its own flux twice, whose difference is
-// zero unless the flux is not finite: such cells carry kFluxOverflow in uni.
-constexpr unsigned kFluxOverflow = 0x40u;
 constexpr int kSweepCounts = 4, kSweepCounters = 4 * kSweepCounts;
 struct SweepLists {
   uint8_t* eq = nullptr;
@@ -112,6 +110,11 @@ struct SweepLists {
   double* F[3] = {nullptr, nullptr, nullptr};
   uint8_t* gate[3] = {nullptr, nullptr, nullptr};
 };
+
+// A cell between two uniform faces takes its own flux twice, whose difference is
+// zero unless the flux is not finite: cells whose flux may overflow carry this bit
+// in eq and uni.
+constexpr unsigned kFluxOverflow = 0x40u;
 
 // Next group of 32 entries of a list for this warp (every lane calls it): the
 // entry of this lane, or an index past the end. False when the list is done.
@@ -125,10 +128,10 @@ __device__ __forceinline__ bool next_entries(uint32_t* __restrict__ cnt, uint32_
   return k < n / 32u + (n % 32u ? 1u : 0u);
 }
 
-// Appends value to a list where `need`, in thread order within the block, with one
-// atomic per block of at most 1024 threads (every thread calls it).
-__device__ __forceinline__ void block_append(bool need, uint32_t value, uint32_t* __restrict__ list,
-                                             uint32_t* __restrict__ count) {
+// Appends value to a list of `room` entries where `need`, in thread order within the
+// block, with one atomic per block of at most 1024 threads (every thread calls it).
+__device__ __forceinline__ void block_append(const DevGrid& g, bool need, uint32_t value, uint32_t* __restrict__ list,
+                                             uint32_t* __restrict__ count, int64_t room) {
   __shared__ uint32_t base[32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
   const unsigned m = __ballot_sync(0xffffffffu, need);
@@ -145,7 +148,7 @@ __device__ __forceinline__ void block_append(bool need, uint32_t value, uint32_t
     }
   }
   __syncthreads();
-  if (need) list[base[warp] + __popc(m & ((1u << lane) - 1u))] = value;
+  if (need) list[HRM_IDX(g, base[warp] + __popc(m & ((1u << lane) - 1u)), room)] = value;
 }
 
 struct DevParams {

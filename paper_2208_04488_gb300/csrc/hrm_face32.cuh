@@ -502,17 +502,17 @@ __device__ __forceinline__ bool uniform_midpoint32(int64_t t, const Nodes6& nd, 
   return true;
 }
 
-// Appends index t to a worklist where `need` (all lanes of the warp call it;
-// warp-aggregated: one atomic per warp; order not significant).
-__device__ __forceinline__ void defer_push(bool need, int64_t t, uint32_t* __restrict__ list,
-                                           uint32_t* __restrict__ count) {
+// Appends index t to a worklist of `room` entries where `need` (all lanes of the
+// warp call it; warp-aggregated: one atomic per warp; order not significant).
+__device__ __forceinline__ void defer_push(const DevGrid& g, bool need, int64_t t, uint32_t* __restrict__ list,
+                                           uint32_t* __restrict__ count, int64_t room) {
   const unsigned m = __ballot_sync(0xffffffffu, need);
   if (m == 0u) return;
   const int lane = threadIdx.x & 31, leader = __ffs(m) - 1;
   uint32_t base = 0;
   if (lane == leader) base = atomicAdd(count, (uint32_t)__popc(m));
   base = __shfl_sync(0xffffffffu, base, leader);
-  if (need) list[base + __popc(m & ((1u << lane) - 1u))] = (uint32_t)t;
+  if (need) list[HRM_IDX(g, base + __popc(m & ((1u << lane) - 1u)), room)] = (uint32_t)t;
 }
 
 // Precision-form update of one RK stage with the next stage's primitives fused
@@ -614,7 +614,7 @@ __global__ void __launch_bounds__(kCellThreads)
 #pragma unroll
   for (int d = 0; d < D; ++d) s[d] = 0.0;
   const bool changed = c < g.nint && !update32p_keep<N, D>(c, A, g, f, tau ? s : nullptr);
-  block_append(changed, (uint32_t)c, cells, cnt);
+  block_append(g, changed, (uint32_t)c, cells, cnt, g.nint);
   if (tau) block_tau_max<D>(s, A.st->tau_bits);
 }
 
@@ -640,7 +640,8 @@ __global__ void __launch_bounds__(kCellThreads, 3)
   uint32_t i;
   while (next_entries(cnt, n, i)) {
     if (i >= n) continue;
-    update32p_change<N, D, true>(cells[i], A, g, f, tau ? sc : nullptr);
+    const int64_t c = HRM_IDX(g, cells[HRM_IDX(g, i, g.nint)], g.nint);
+    update32p_change<N, D, true>(c, A, g, f, tau ? sc : nullptr);
 #pragma unroll
     for (int d = 0; d < D; ++d) s[d] = (sc[d] != sc[d]) ? sc[d] : (sc[d] > s[d] ? sc[d] : s[d]);
   }
@@ -1017,20 +1018,20 @@ __global__ void __launch_bounds__(kFaceThreads, LISTED ? 6 : 4)
       const bool lin = gate != nullptr && gate[t] != 0;
       need = !face32_body<N, D, DIR, true>(t, nd, W, nullptr, nullptr, P32, out, g, f, pr, st->lam[DIR], lin);
     }
-    defer_push(need, t, deferred, &cnt[2]);
+    defer_push(g, need, t, deferred, &cnt[2], face_count<DIR>(g));
     return;
   }
   const uint32_t n = cnt[0];
   uint32_t i;
   while (next_entries(cnt, n, i)) {
-    const int64_t t = i < n ? (int64_t)list[i] : 0;
+    const int64_t t = i < n ? listed_midpoint<DIR>(g, list, i) : 0;
     Nodes6 nd;
     bool need = false;
     if (i < n && face_nodes<DIR>(g, t, nd)) {
       const bool lin = gate != nullptr && gate[t] != 0;
       need = !face32_body<N, D, DIR, true>(t, nd, W, nullptr, nullptr, P32, out, g, f, pr, st->lam[DIR], lin);
     }
-    defer_push(need, t, deferred, &cnt[2]);
+    defer_push(g, need, t, deferred, &cnt[2], face_count<DIR>(g));
   }
 }
 
@@ -1048,7 +1049,7 @@ __global__ void __launch_bounds__(kFaceThreads, 2)
   for (int64_t r = threadIdx.x;; r += blockDim.x) {
     const int64_t i = r * gridDim.x + blockIdx.x;
     if (i >= n) break;
-    const int64_t t = list[i];
+    const int64_t t = listed_midpoint<DIR>(g, list, i);
     Nodes6 nd;
     if (!face_nodes<DIR>(g, t, nd)) continue;
     const bool lin = gate != nullptr && gate[t] != 0;
@@ -1076,7 +1077,7 @@ __global__ void __launch_bounds__(kFaceThreads, 3)
   uint32_t i;
   while (next_entries(cnt, n, i)) {
     if (i >= n) continue;
-    const int64_t t = list[i];
+    const int64_t t = listed_midpoint<DIR>(g, list, i);
     Nodes6 nd;
     if (!face_nodes<DIR>(g, t, nd)) continue;
     const bool lin = gate != nullptr && gate[t] != 0;

@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(kFaceThreads, LISTED ? 5 : 4)
       gate[t] = lin ? 1 : 0;
       need = !face32_body<N, D, DIR, true>(t, nd, W, nullptr, nullptr, P32, out, g, f, pr, st->lam[DIR], lin);
     }
-    defer_push(need, t, deferred, &cnt[2]);
+    defer_push(g, need, t, deferred, &cnt[2], face_count<DIR>(g));
   };
   if constexpr (!LISTED) {
     const int64_t t = (int64_t)blockIdx.x * kFaceThreads + threadIdx.x;
@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(kFaceThreads, LISTED ? 5 : 4)
   const uint32_t n = cnt[0];
   uint32_t i;
   while (next_entries(cnt, n, i)) {
-    const int64_t t = i < n ? (int64_t)list[i] : 0;
+    const int64_t t = i < n ? listed_midpoint<DIR>(g, list, i) : 0;
     Nodes6 nd;
     const bool in = i < n && face_nodes<DIR>(g, t, nd);
     group(t, nd, in);

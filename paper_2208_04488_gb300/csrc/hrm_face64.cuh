@@ -549,7 +549,7 @@ __device__ __forceinline__ void sweep_split(const double* __restrict__ W, const 
     Nodes6 nd;
     const uint32_t i = k * per + (threadIdx.x & 31) / LANES;
     if (i >= n) continue;
-    const int64_t t = list ? list[i] : i;
+    const int64_t t = list ? listed_midpoint<DIR>(g, list, i) : i;
     if (!face_nodes<DIR>(g, t, nd)) continue;
     if (!list && uniform_midpoint64<N, D, DIR, LANES>(t, nd, W, V, out, g)) continue;
     const bool lin = gate != nullptr && gate[t] != 0;
@@ -571,7 +571,7 @@ __global__ void __launch_bounds__(kFaceThreads, 3)
   while (next_entries(cnt, n, i)) {
     Nodes6 nd;
     if (i >= n) continue;
-    const int64_t t = list[i];
+    const int64_t t = listed_midpoint<DIR>(g, list, i);
     if (!face_nodes<DIR>(g, t, nd)) continue;
     const bool lin = gate != nullptr && gate[t] != 0;
     face_body<N, D, DIR>(t, nd, W, V, AUX, out, g, f, pr, st->lam[DIR], col, lin);

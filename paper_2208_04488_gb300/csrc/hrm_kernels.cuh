@@ -22,6 +22,12 @@ __device__ __forceinline__ int64_t face_count(const DevGrid& g) {
   return (g.n[0] + (DIR == 0)) * (g.n[1] + (DIR == 1)) * (g.n[2] + (DIR == 2));
 }
 
+// Entry i of a list of midpoints of direction DIR.
+template <int DIR>
+__device__ __forceinline__ int64_t listed_midpoint(const DevGrid& g, const uint32_t* __restrict__ list, int64_t i) {
+  return HRM_IDX(g, list[HRM_IDX(g, i, face_count<DIR>(g))], face_count<DIR>(g));
+}
+
 // ---------------------------------------------------------------- interpolation limiter
 
 // Positivity-preserving interpolation limiter (Sec. 4.3.2, Alg. interp_limit_densities,

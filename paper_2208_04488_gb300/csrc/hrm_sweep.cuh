@@ -171,18 +171,19 @@ __global__ void __launch_bounds__(kCellThreads)
 #pragma unroll
   for (int d = 0; d < D; ++d) {
     const int64_t f0 = g.n[0] + (d == 0), f1 = g.n[1] + (d == 1);
-    const int64_t t = (ijk[2] * f1 + ijk[1]) * f0 + ijk[0];
-    const int64_t up = t + (d == 0 ? 1 : (d == 1 ? f0 : f0 * f1));
+    const int64_t nf = f0 * f1 * (g.n[2] + (d == 2));
+    const int64_t t = HRM_IDX(g, (ijk[2] * f1 + ijk[1]) * f0 + ijk[0], nf);
+    const int64_t stride = d == 0 ? 1 : (d == 1 ? f0 : f0 * f1);
     const uint32_t p = base[d][warp] + at[d];
-    if (lo[d]) lists.list[d][p] = (uint32_t)t;
-    if (hi[d]) lists.list[d][p + (lo[d] ? 1u : 0u)] = (uint32_t)up;
+    if (lo[d]) lists.list[d][HRM_IDX(g, p, nf)] = (uint32_t)t;
+    if (hi[d]) lists.list[d][HRM_IDX(g, p + (lo[d] ? 1u : 0u), nf)] = (uint32_t)HRM_IDX(g, t + stride, nf);
     const bool last = ijk[d] == g.n[d] - 1 && !hi[d];
+    const int64_t up = last ? HRM_IDX(g, t + stride, nf) : t;
     if (lists.gate[d]) {
       if (!lo[d]) lists.gate[d][t] = 2;
       if (last) lists.gate[d][up] = 2;
     }
     if (lists.F[d] && (!lo[d] || last)) {
-      const int64_t nf = f0 * f1 * (g.n[2] + (d == 2));
       double G[L::NC];
       if constexpr (FP32)
         uniform_flux32<N, D>(c, d, P32, g.ncells, G);

@@ -133,6 +133,8 @@ def lib():
     L.hrm_batch_admissibility.argtypes = [_VP, P(ctypes.c_int64)]
     L.hrm_batch_set_launch.argtypes = [_VP, ctypes.c_int32, ctypes.c_int32, ctypes.c_int32, ctypes.c_int32]
     L.hrm_batch_tune.argtypes = [_VP, ctypes.c_int32, P(ctypes.c_int32)]
+    L.hrm_batch_bounds_violations.argtypes = [_VP]
+    L.hrm_batch_bounds_violations.restype = ctypes.c_int64
     L.hrm_batch_kernel_launches.argtypes = [_VP]
     L.hrm_batch_kernel_launches.restype = ctypes.c_int64
     L.hrm_batch_total_cells.argtypes = [_VP]
@@ -705,6 +707,10 @@ class BatchSolver:
         best = (ctypes.c_int32 * 4)()
         self._check(lib().hrm_batch_tune(self.h, steps_per_trial, best))
         return dict(zip(["face_threads", "face_tile", "cell_tile", "blocks_per_sm"], list(best)))
+
+    def bounds_violations(self) -> int:
+        """Out-of-range indices the kernels met (bounds-check builds; -1 otherwise)."""
+        return int(lib().hrm_batch_bounds_violations(self.h))
 
     def kernel_launches(self) -> int:
         return int(lib().hrm_batch_kernel_launches(self.h))
