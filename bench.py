@@ -249,13 +249,10 @@ def run_reference(args):
 
 
 def time_steps(torch, s, K, flush, ev_stream, dt=0.0):
-    """K single steps, each bracketed by CUDA events on the library's stream,
-    with an L2 flush (a write larger than L2) before each. The step graph
-    carries an event pair around every kernel (hrm_set_profiling), read after
-    each step; dt <= 0: the automatic CFL step. Returns (seconds,
-    {kernel kind: (launches, seconds)})."""
+    """Seconds of K single steps, each bracketed by CUDA events on the library's
+    stream, with an L2 flush (a write larger than L2) before each; dt <= 0: the
+    automatic CFL step."""
     total = 0.0
-    per = {}
     for _ in range(K):
         flush.fill_(1.0)
         e0 = torch.cuda.Event(enable_timing=True)
@@ -265,9 +262,24 @@ def time_steps(torch, s, K, flush, ev_stream, dt=0.0):
         e1.record(ev_stream)
         e1.synchronize()
         total += e0.elapsed_time(e1) * 1e-3
+    return total
+
+
+def kernel_times(torch, s, prim, K, flush, ev_stream, dt=0.0):
+    """The same K steps from the initial condition once more with an event pair
+    around every kernel in the step graph (hrm_set_profiling; the event nodes
+    lengthen a step, 50 us of the precision form's 500, so they stay out of the
+    timed steps). Returns (seconds, {kernel kind: (launches, seconds)})."""
+    s.set_profiling(True)
+    s.step(dt, 1)  # captures the graph
+    s.set_primitive(prim)
+    total, per = 0.0, {}
+    for _ in range(K):
+        total += time_steps(torch, s, 1, flush, ev_stream, dt)
         for kind, ms in s.profile_read():
             n, t = per.get(kind, (0, 0.0))
             per[kind] = (n + 1, t + ms * 1e-3)
+    s.set_profiling(False)
     return total, per
 
 
@@ -461,20 +473,20 @@ def run_form(torch, hrm, pr, precision, det, dt, steps, warmup, flush, stream, t
         s.set_detector(det)
         s.set_params(hrm.params_default(cfl=pr.cfl, check=0, precision=precision, learned=hrm.LEARNED_GATE,
                                         learned_threshold=threshold))
-    s.set_profiling(True)
     for _ in range(warmup):
         s.step(dt, 1)
     s.set_primitive(pr.prim)
     torch.cuda.synchronize()
     l0 = s.kernel_launches()
-    t, per = time_steps(torch, s, steps, flush, stream, dt)
-    out = {"t": t, "per": per, "launches": s.kernel_launches() - l0, "adm": s.admissibility(),
+    t = time_steps(torch, s, steps, flush, stream, dt)
+    out = {"t": t, "launches": s.kernel_launches() - l0, "adm": s.admissibility(),
            "W": s.get(hrm.FIELD_W)}
     # gate bytes: 1 linear weights, 0 full WENO-IS, 2 (precision form) a
     # uniform stencil, which takes the exact node flux
     gb = np.concatenate([s.get_gate(d) for d in range(pr.D)]) if det is not None else np.zeros(1, np.uint8)
     out["gated"] = float(np.mean(gb != 0)) if det is not None else 0.0
     out["gated_uniform"] = float(np.mean(gb == 2)) if det is not None else 0.0
+    out["per"] = kernel_times(torch, s, pr.prim, steps, flush, stream, dt)[1]
     s.close()
     return out
 
@@ -525,11 +537,16 @@ def sweep_time(hrm, per, D):
     return n, t
 
 
-def time_shares(hrm, per, D):
-    """Share of each non-overlapping bracket (the sweeps as one) in their sum."""
+def time_shares(hrm, per, D, wall=None):
+    """Share of each non-overlapping bracket (the sweeps as one) in the time of the steps, `wall` seconds, the rest as
+    "between" (launch gaps, waits for the deferred midpoints); without it, in the brackets' sum."""
     skip = {hrm.KERNEL_FACE_X + d for d in range(D)} if hrm.KERNEL_SWEEPS in per else set()
-    tot = sum(v[1] for k, v in per.items() if k not in skip)
-    return {hrm.KERNEL_NAMES[k]: round(v[1] / tot, 4) for k, v in sorted(per.items()) if k not in skip}
+    skip |= {hrm.KERNEL_KEEP, hrm.KERNEL_FIX}  # they run beside the sweeps and one another
+    tot = wall if wall else sum(v[1] for k, v in per.items() if k not in skip)
+    sh = {hrm.KERNEL_NAMES[k]: round(v[1] / tot, 4) for k, v in sorted(per.items()) if k not in skip}
+    if wall:
+        sh["between"] = round(1.0 - sum(sh.values()), 4)
+    return sh
 
 
 def form_summary(hrm, pr, r, ref_W, steps, face_fl, face_fl_gated, peak, peak_name):
@@ -621,7 +638,6 @@ def main():
 
     flush = torch.empty(256 * 1024 * 1024 // 4, dtype=torch.float32, device="cuda")
     s = make(hrm.FP64)
-    s.set_profiling(True)
     for _ in range(args.warmup):
         s.step(0.0, 1)
     torch.cuda.synchronize()
@@ -631,11 +647,12 @@ def main():
         dist.barrier()
     torch.cuda.synchronize()
     with Clocks(local) as clk:
-        t_dev, per_kernel = time_steps(torch, s, args.steps, flush, stream)
+        t_dev = time_steps(torch, s, args.steps, flush, stream)
     launches = s.kernel_launches() - launches0
     torch.cuda.synchronize()
     adm = s.admissibility()
     W_fp64 = s.get(hrm.FIELD_W)
+    t_prof, per_kernel = kernel_times(torch, s, pr.prim, args.steps, flush, stream)
     from paper_2208_04488_gb300.replicas import whole_job_rate
     value, t_max = whole_job_rate(pr.ncells * args.steps, t_dev, dist, device="cuda")
 
@@ -677,13 +694,13 @@ def main():
     # precision form on the same workload: timed the same way, and its relative
     # L1 error against FP64 after the same number of equal fixed-size steps
     s32 = make(hrm.FP32)
-    s32.set_profiling(True)
     for _ in range(args.warmup):
         s32.step(0.0, 1)
     s32.set_primitive(pr.prim)
     torch.cuda.synchronize()
-    t32, per32 = time_steps(torch, s32, args.steps, flush, stream)
+    t32 = time_steps(torch, s32, args.steps, flush, stream)
     adm32 = s32.admissibility()
+    t32_prof, per32 = kernel_times(torch, s32, pr.prim, args.steps, flush, stream)
     dt0, _ = s.dt(pr.cfl)
     ea, eb = make(hrm.FP64), make(hrm.FP32)
     ea.step(dt0, args.steps)
@@ -724,10 +741,10 @@ def main():
         n_face, t_face = sweep_time(hrm, per_kernel, pr.D)
         achieved = fl_launch / (t_face / n_face)
         frac = achieved / fp64_peak
-        share = time_shares(hrm, per_kernel, pr.D)
+        share = time_shares(hrm, per_kernel, pr.D, t_prof)
         n32, tf32 = sweep_time(hrm, per32, pr.D)
         ach32 = fl_launch / (tf32 / n32)
-        share32 = time_shares(hrm, per32, pr.D)
+        share32 = time_shares(hrm, per32, pr.D, t32_prof)
         # the precision form's sweep finishes a uniform stencil exactly (the node
         # flux) without the method's arithmetic: the share of such midpoints, as
         # the learned form's sweep reports it in its gate bytes (byte 2) at the

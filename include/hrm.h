@@ -298,16 +298,23 @@ enum {
   HRM_KERNEL_PRIM = 0,      /* per-cell primitives (+ CFL reduction at the first stage) */
   HRM_KERNEL_FINALIZE = 1,  /* dt, sigma_d, lambda_d */
   HRM_KERNEL_FACE_X = 2,    /* per-midpoint sweep in x (HRM_KERNEL_FACE_X + d for direction d) */
-  HRM_KERNEL_UPDATE = 5,    /* flux difference, RK combination, relaxation */
+  HRM_KERNEL_UPDATE = 5,    /* flux difference, RK combination, relaxation (precision form with lists: of
+                               the cells the stage changes) */
   HRM_KERNEL_GATE = 6,      /* learned smoothness gate of one direction */
-  HRM_KERNEL_SWEEPS = 7     /* all sweeps of one stage, fork to join: in 2D and 3D the directions run
+  HRM_KERNEL_SWEEPS = 7,    /* all sweeps of one stage, fork to join: in 2D and 3D the directions run
                                concurrently (direction d > 0 on its own stream of the step graph), so
                                their own brackets overlap and this one times them together */
+  HRM_KERNEL_LISTS = 8,     /* the two kernels that find uniform faces and list the other midpoints */
+  HRM_KERNEL_KEEP = 9,      /* precision form: the cells a stage leaves unchanged, beside the sweeps */
+  HRM_KERNEL_FIX = 10       /* precision form: the deferred midpoints of one direction, from the end of
+                               its sweep; the update waits for it */
 };
 
 /* Tracing: with on != 0 the step graph is (re)captured with a CUDA event pair
  * around every kernel and one around the sweeps of each stage
- * (HRM_KERNEL_SWEEPS). Costs one event-record node per bracket boundary. */
+ * (HRM_KERNEL_SWEEPS). Brackets of kernels that run beside others overlap
+ * (HRM_KERNEL_FACE_X.., KEEP, FIX). Costs one event-record node per bracket
+ * boundary. */
 hrm_status hrm_set_profiling(hrm_ctx* ctx, int32_t on);
 
 /* After a step with tracing on: synchronises the stream and writes, for the

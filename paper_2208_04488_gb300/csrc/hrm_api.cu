@@ -23,7 +23,8 @@
 using namespace hrm;
 
 namespace {
-constexpr int kMaxProf = 32;  // brackets of one step: 3 stages x (prim, 3 gates, sweeps, 3 sweeps, update) + finalize
+// brackets of one step: 3 stages x (prim, 3 gates, lists, keep, sweeps, 3 sweeps, 3 fix, update) + finalize
+constexpr int kMaxProf = 48;
 }
 
 struct hrm_ctx {
@@ -220,18 +221,18 @@ void drop_graph(hrm_ctx* c) {
 // concurrent sweeps of a stage); while profiling, bracket it with an event pair
 // on s (captured as event-record nodes) and remember its kind (HRM_KERNEL_*).
 // The slot is taken before launching, so brackets may nest.
+cudaEvent_t* prof_slot(hrm_ctx* c, int kind) {  // the pair, or nullptr while not profiling
+  if (!c->profiling || c->nprof >= kMaxProf) return nullptr;
+  c->prof_kind[c->nprof] = kind;
+  return &c->prof_ev[2 * c->nprof++];
+}
 template <typename F>
 void traced(hrm_ctx* c, cudaStream_t s, int kind, F&& launch) {
-  const int i = c->nprof;
-  const bool on = c->profiling && i < kMaxProf;
+  cudaEvent_t* ev = prof_slot(c, kind);
   // external event-record nodes: recorded each time the graph runs
-  if (on) {
-    ++c->nprof;
-    c->prof_kind[i] = kind;
-    cudaEventRecordWithFlags(c->prof_ev[2 * i], s, cudaEventRecordExternal);
-  }
+  if (ev) cudaEventRecordWithFlags(ev[0], s, cudaEventRecordExternal);
   launch();
-  if (on) cudaEventRecordWithFlags(c->prof_ev[2 * i + 1], s, cudaEventRecordExternal);
+  if (ev) cudaEventRecordWithFlags(ev[1], s, cudaEventRecordExternal);
 }
 
 float gate_logit_threshold(const hrm_ctx* c) {
@@ -365,7 +366,10 @@ int enqueue_stage(hrm_ctx* c, cudaStream_t s, const double* Wsrc, double* Wout, 
       ++k;
     }
   const bool whole = c->params.precision == HRM_FP32 && !fuse_next, lists = listed(c, whole);
-  k += enqueue_mark(c, s, Wsrc, lists, whole);
+  if (lists)
+    traced(c, s, HRM_KERNEL_LISTS, [&] { k += enqueue_mark(c, s, Wsrc, true, whole); });
+  else
+    enqueue_mark(c, s, Wsrc, false, whole);
   Update32Args up{};
   if (fuse_next) {
     up = {c->Wn, Wsrc, Wout, c->F[0], c->F[1], c->F[2], c->st, a, b, relax, count, c->P32, r32_target(c),
@@ -373,7 +377,8 @@ int enqueue_stage(hrm_ctx* c, cudaStream_t s, const double* Wsrc, double* Wout, 
     if (up.uni) {
       cudaEventRecord(c->ev_mark, s);
       cudaStreamWaitEvent(c->keep, c->ev_mark, 0);
-      launch_update32p(c->N, c->D, up, c->dg, c->fl, tau_next ? 1 : 0, c->lists, 0, c->keep);
+      traced(c, c->keep, HRM_KERNEL_KEEP,
+             [&] { launch_update32p(c->N, c->D, up, c->dg, c->fl, tau_next ? 1 : 0, c->lists, 0, c->keep); });
       cudaEventRecord(c->ev_keep, c->keep);
       ++k;
     }
@@ -395,6 +400,10 @@ int enqueue_stage(hrm_ctx* c, cudaStream_t s, const double* Wsrc, double* Wout, 
         ga.ev_fix = c->ev_fix[d];
       }
       traced(c, sd, HRM_KERNEL_FACE_X + d, [&] {
+        if (cudaEvent_t* ev = ga.side ? prof_slot(c, HRM_KERNEL_FIX) : nullptr) {
+          ga.prof_fix[0] = ev[0];
+          ga.prof_fix[1] = ev[1];
+        }
         c->fk->face[d](c->params.precision, Wsrc, c->V, c->AUX, c->P32, c->F[d], c->dg, c->fl, c->dp, c->st, ga,
                        sd);
       });

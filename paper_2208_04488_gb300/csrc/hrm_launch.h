@@ -38,6 +38,7 @@ struct GateArgs {
   // sweep; the caller joins ev_fix before the update
   cudaStream_t side = nullptr;
   cudaEvent_t ev_fast = nullptr, ev_fix = nullptr;
+  cudaEvent_t prof_fix[2] = {nullptr, nullptr};  // profiling: recorded around it
   // precision form with the learned detector (with a worklist): the sweep
   // evaluates the network itself (k_face32_net) from the FP32 planes and their
   // residues R32, with the detector's inference blob (an mlp::GateBlob) and the
@@ -59,10 +60,13 @@ inline cudaStream_t fix_stream(const GateArgs& gate, cudaStream_t s) {
   if (!gate.side) return s;
   cudaEventRecord(gate.ev_fast, s);
   cudaStreamWaitEvent(gate.side, gate.ev_fast, 0);
+  if (gate.prof_fix[0]) cudaEventRecordWithFlags(gate.prof_fix[0], gate.side, cudaEventRecordExternal);
   return gate.side;
 }
 inline void fix_done(const GateArgs& gate) {
-  if (gate.side) cudaEventRecord(gate.ev_fix, gate.side);
+  if (!gate.side) return;
+  if (gate.prof_fix[1]) cudaEventRecordWithFlags(gate.prof_fix[1], gate.side, cudaEventRecordExternal);
+  cudaEventRecord(gate.ev_fix, gate.side);
 }
 
 // Launch shape of the deferred-midpoint kernel: one-warp blocks, 16 per SM.

@@ -30,8 +30,8 @@ RELAX_OFF, RELAX_STAGE, RELAX_STEP = 0, 1, 2
 KERNEL_PRIM, KERNEL_FINALIZE, KERNEL_FACE_X, KERNEL_FACE_Y, KERNEL_FACE_Z, KERNEL_UPDATE = 0, 1, 2, 3, 4, 5
 KERNEL_GATE = 6
 KERNEL_NAMES = {0: "prim", 1: "finalize", 2: "face_x", 3: "face_y", 4: "face_z", 5: "update", 6: "gate",
-                7: "sweeps"}
-KERNEL_SWEEPS = 7
+                7: "sweeps", 8: "lists", 9: "keep", 10: "fix"}
+KERNEL_SWEEPS, KERNEL_LISTS, KERNEL_KEEP, KERNEL_FIX = 7, 8, 9, 10
 LEARNED_OFF, LEARNED_GATE, LEARNED_FIXED = 0, 1, 2
 BC_TRANSMISSIVE, BC_PERIODIC, BC_DIRICHLET = 0, 1, 2
 DETECTOR_PARAMS, DETECTOR_INPUTS = 2081, 30
@@ -496,7 +496,7 @@ class Solver:
     def set_profiling(self, on=True):
         self._check(lib().hrm_set_profiling(self.h, 1 if on else 0))
 
-    def profile_read(self, maxn=32):
+    def profile_read(self, maxn=64):
         """[(kind, ms)] of the kernels of the last traced step."""
         ms = (ctypes.c_float * maxn)()
         kd = (ctypes.c_int32 * maxn)()

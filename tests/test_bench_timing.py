@@ -65,3 +65,14 @@ def test_run_face_flops_means_the_first_and_last_state(mods):
     for d in range(pr.D):
         assert run[d][0] == pytest.approx(0.5 * (first[d][0] + last[d][0]))
         assert last[d][0] > first[d][0]
+
+
+def test_shares_of_the_wall_time_leave_room_for_what_lies_between(mods):
+    """Kernels beside the sweeps (unchanged cells, deferred midpoints) are not added; what no bracket holds is named."""
+    bench, hrm = mods
+    per = {hrm.KERNEL_PRIM: (3, 0.3e-3), hrm.KERNEL_LISTS: (3, 1.2e-3), hrm.KERNEL_KEEP: (3, 2e-3), hrm.KERNEL_FIX: (6, 8e-3),
+           hrm.KERNEL_FACE_X: (3, 6e-3), hrm.KERNEL_FACE_Y: (3, 6e-3), hrm.KERNEL_SWEEPS: (3, 9e-3), hrm.KERNEL_UPDATE: (3, 0.6e-3)}
+    sh = bench.time_shares(hrm, per, 2, 15e-3)
+    assert set(sh) == {"prim", "lists", "sweeps", "update", "between"}
+    assert sh["sweeps"] == pytest.approx(0.6) and sh["lists"] == pytest.approx(0.08)
+    assert sh["between"] == pytest.approx(1.0 - 11.1 / 15.0, abs=1e-3)
