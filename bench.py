@@ -30,12 +30,22 @@ import numpy as np
 ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
-# DRAM traffic per launch of the dominant kernels, dram__bytes_read.sum + dram__bytes_write.sum from one
-# ncu capture on this workload (profiles/k_face_fp64_shock_bubble_1024x512.md and
-# profiles/k_face32_shock_bubble_1024x512.md); to be re-taken whenever those kernels change.
-TRAFFIC_BYTES = {"k_face_fp64": 9.06e6, "k_face32": 6.07e6}
-# FP64-pipe activity of the FP64 sweep in the same ncu capture (fraction of peak sustained)
-FP64_PIPE_ACTIVE = {"k_face_fp64": 0.769}
+# The two sweeps (x, y) of the first stage of step 11 of this workload, from one ncu capture (cold caches, one launch at a
+# time; profiles/launches_shock_bubble_1024x512.md): device time, DRAM bytes read and written, activity of the FP64 and
+# the FMA pipe. A sweep's work grows with the share of non-uniform stencils, so these belong to that step and are
+# combined with no other time; to be taken again when the kernels change.
+CAPTURED = {"k_face_fp64": {"us": [614.9, 454.7], "dram_bytes": [2.696e7, 2.204e7], "fp64_pipe_active": [0.557, 0.599]},
+            "k_face32_fast": {"us": [34.8, 29.0], "dram_bytes": [9.28e6, 4.01e6], "fma_pipe_active": [0.283, 0.193]}}
+
+
+def captured_traffic(name, hbm_gbs):
+    """DRAM bytes of a captured launch (mean of the two sweeps), its bandwidth and share of the measured one."""
+    c = CAPTURED[name]
+    gbs = sum(c["dram_bytes"]) / sum(c["us"]) * 1e-3
+    return {"of": "one captured launch of each sweep, step 11", "traffic_bytes_per_launch": sum(c["dram_bytes"]) / 2,
+            "launch_us": sum(c["us"]) / 2, "achieved_gbs": gbs, "peak_gbs": hbm_gbs, "frac": gbs / hbm_gbs if hbm_gbs else None}
+
+
 METRIC = "cell-updates/s (FP64 plain vs FP32+learned) at stated L1 err; % of roofline"
 UNIT = "cell-updates/s"
 WORKLOAD = "2D three-species shock-bubble, 1024x512 cells, Mach 1.5 shock, water+air+helium, SSP-RK3, CFL 0.4"
@@ -748,10 +758,8 @@ def main():
         # the precision form's sweep finishes a uniform stencil exactly (the node
         # flux) without the method's arithmetic: the share of such midpoints, as
         # the learned form's sweep reports it in its gate bytes (byte 2) at the
-        # end of the same steps, and the bytes a launch moves (ncu capture: the
-        # sweep reads and writes at listed, non-uniform midpoints only)
+        # end of the same steps
         uni = (learned_runs["fp32_learned"].get("gated_uniform") if learned_runs is not None else None)
-        bytes32 = TRAFFIC_BYTES["k_face32"]
         learned_block = None
         if learned_runs is not None:
             faces_g = gated_face_flops(pr, pr.cfl, W_fp64)
@@ -769,9 +777,11 @@ def main():
                                        if ws > 1 else "single GPU")},
             "roofline": {"bound": "alu", "kernel": "k_face (per-midpoint, FP64)",
                          "achieved": achieved / 1e12, "peak": fp64_peak / 1e12, "unit": "TFLOP/s",
-                         "frac": frac, "traffic": TRAFFIC_BYTES["k_face_fp64"],
-                         "traffic_unit": "bytes per launch (ncu capture, y sweep)",
-                         "fp64_pipe_active_ncu": FP64_PIPE_ACTIVE["k_face_fp64"],
+                         "frac": frac, "traffic": sum(CAPTURED["k_face_fp64"]["dram_bytes"]) / 2,
+                         "traffic_unit": "bytes per launch (ncu capture of step 11, mean of the x and y sweeps)",
+                         "hbm": captured_traffic("k_face_fp64", pk.get("hbm_gbs")),
+                         "fp64_pipe_active_ncu": CAPTURED["k_face_fp64"]["fp64_pipe_active"],
+                         "fp64_pipe_active_of": "the x and the y sweep of step 11, captured alone",
                          "peak_source": "measured FP64 FMA-chain probe on this GPU (hrm_probe_fma_peak)",
                          "algorithmic_flops_per_face": [round(x[0], 1) for x in faces],
                          "flops_per_face_first_last_state": [x[2] for x in faces],
@@ -802,19 +812,15 @@ def main():
                                       "peak_fp32": fp32_peak / 1e12, "frac_of_fp32_peak": ach32 / fp32_peak,
                                       "peak_fp64": fp64_peak / 1e12,
                                       "avg_launch_ms": 1e3 * tf32 / n32, "kernel_time_share": share32,
-                                      "traffic": TRAFFIC_BYTES["k_face32"],
+                                      "traffic": sum(CAPTURED["k_face32_fast"]["dram_bytes"]) / 2,
                                       "flops_counted": "the oracle's count over the timed states, as for the "
                                                        "FP64 sweep: the method's arithmetic at non-uniform "
                                                        "midpoints, the node flux at uniform ones (the sweep "
                                                        "takes that flux where its FP32 planes are uniform); "
                                                        "the sweep is bound by the latency of its body, "
-                                                       "not by the FP32 pipe (ncu: FMA pipe 19-23 %)",
+                                                       "not by the FP32 pipe (ncu, step 11: FMA pipe 19-28 %)",
                                       "uniform_share": uni,
-                                      "hbm": {"traffic_bytes_per_launch": bytes32,
-                                              "achieved_gbs": bytes32 / (tf32 / n32) / 1e9,
-                                              "peak_gbs": pk.get("hbm_gbs"),
-                                              "frac": (bytes32 / (tf32 / n32) / 1e9 / pk["hbm_gbs"]
-                                                       if pk.get("hbm_gbs") else None)}}},
+                                      "hbm": captured_traffic("k_face32_fast", pk.get("hbm_gbs"))}},
             },
             "batched": batched,
             "interface_3d": three_d,

@@ -76,3 +76,13 @@ def test_shares_of_the_wall_time_leave_room_for_what_lies_between(mods):
     assert set(sh) == {"prim", "lists", "sweeps", "update", "between"}
     assert sh["sweeps"] == pytest.approx(0.6) and sh["lists"] == pytest.approx(0.08)
     assert sh["between"] == pytest.approx(1.0 - 11.1 / 15.0, abs=1e-3)
+
+
+def test_captured_traffic_is_of_the_captured_launches(mods):
+    """A captured launch's bytes go with its own time, never with that of the timed steps' launches."""
+    bench, _ = mods
+    for name, c in bench.CAPTURED.items():
+        t = bench.captured_traffic(name, 7000.0)
+        assert t["achieved_gbs"] == pytest.approx(sum(c["dram_bytes"]) / sum(c["us"]) / 1e3)
+        assert t["frac"] == pytest.approx(t["achieved_gbs"] / 7000.0) and 0.0 < t["frac"] < 1.0
+        assert t["traffic_bytes_per_launch"] * 2 == pytest.approx(sum(c["dram_bytes"]))
