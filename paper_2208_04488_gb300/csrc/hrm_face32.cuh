@@ -572,16 +572,26 @@ __device__ __forceinline__ bool update32p_keep(int64_t c, const Update32Args& A,
   return true;
 }
 
-// Any other cell.
+// kFluxOverflow where dt / dx_d is not finite in some direction: a flux difference of
+// zero then counts as well.
+template <int D>
+__device__ __forceinline__ unsigned undefined_step(const DevGrid& g, double dt) {
+  bool odd = false;
+#pragma unroll
+  for (int d = 0; d < D; ++d) odd = odd | (((uint32_t)__double2hiint(dt * g.inv_dx[d]) & 0x7ff00000u) == 0x7ff00000u);
+  return odd ? kFluxOverflow : 0u;
+}
+
+// Any other cell. odd: undefined_step of the stage's dt (with A.uni).
 template <int N, int D, bool SOFT = false>
 __device__ __forceinline__ void update32p_change(int64_t c, const Update32Args& A, const DevGrid& g, const DevFluid& f,
-                                                 double* s) {
+                                                 double* s, unsigned odd = 0u) {
   constexpr int M = Lay<N, D>::M;
   const int64_t nc = g.ncells;
   double Ws[M], Wo[M];
 #pragma unroll
   for (int m = 0; m < M; ++m) Ws[m] = A.Wsrc[m * nc + c];
-  fast_combine<N, D>(c, A.Wn, Ws, A.F0, A.F1, A.F2, g, A.st->dt, A.a, A.b, Wo, A.uni ? A.uni[c] : 0u, A.P32);
+  fast_combine<N, D>(c, A.Wn, Ws, A.F0, A.F1, A.F2, g, A.st->dt, A.a, A.b, Wo, A.uni ? A.uni[c] | odd : 0u, A.P32);
   double rho, Re;
   if (A.relax)
     relax_fast<N, D, SOFT>(Wo, f, rho, Re);
@@ -637,11 +647,12 @@ __global__ void __launch_bounds__(kCellThreads, 3)
 #pragma unroll
   for (int d = 0; d < D; ++d) s[d] = sc[d] = 0.0;
   const uint32_t n = cnt[0];
+  const unsigned odd = undefined_step<D>(g, A.st->dt);
   uint32_t i;
   while (next_entries(cnt, n, i)) {
     if (i >= n) continue;
     const int64_t c = HRM_IDX(g, cells[HRM_IDX(g, i, g.nint)], g.nint);
-    update32p_change<N, D, true>(c, A, g, f, tau ? sc : nullptr);
+    update32p_change<N, D, true>(c, A, g, f, tau ? sc : nullptr, odd);
 #pragma unroll
     for (int d = 0; d < D; ++d) s[d] = (sc[d] != sc[d]) ? sc[d] : (sc[d] > s[d] ? sc[d] : s[d]);
   }

@@ -513,8 +513,8 @@ __device__ __forceinline__ void uniform_flux32(int64_t c, int d, const float* __
 // b = 1 - a, so their combination is formed as acc + a (W^n - acc): two
 // operations as before, and exactly acc when W^n equals acc. ub: the cell's
 // uniform faces (k_mark), whose flux comes from the cell's own planes P32; two
-// of them leave acc as it is (acc + cd 0 with cd < 0), unless their flux or cd is
-// not finite.
+// of them leave acc as it is (acc + cd 0 with cd < 0), unless kFluxOverflow says
+// that their flux or cd may not be finite.
 template <int N, int D>
 __device__ __forceinline__ void fast_combine(int64_t c, const double* Wn, const double* Ws,
                                              const double* __restrict__ F0, const double* __restrict__ F1,
@@ -530,11 +530,12 @@ __device__ __forceinline__ void fast_combine(int64_t c, const double* Wn, const 
   double acc[M];
 #pragma unroll
   for (int m = 0; m < M; ++m) acc[m] = Ws[m];
+  const unsigned both = (ub & kFluxOverflow) ? 0u : ub & ub >> 1;  // bit 2 d: both faces, their difference zero
 #pragma unroll
   for (int d = 0; d < D; ++d) {
     const unsigned u = ub >> (2 * d) & 3u;
+    if (both >> (2 * d) & 1u) continue;
     const double cd = -dt * g.inv_dx[d];
-    if (u == 3u && !(ub & kFluxOverflow) && ((uint32_t)__double2hiint(cd) & 0x7ff00000u) != 0x7ff00000u) continue;
     const double* F = d == 0 ? F0 : (d == 1 ? F1 : F2);
     const int64_t f0 = g.n[0] + (d == 0), f1 = g.n[1] + (d == 1), f2 = g.n[2] + (d == 2);
     const int64_t nf = f0 * f1 * f2;
@@ -696,7 +697,7 @@ __device__ __forceinline__ void update_body(int64_t c, const double* Wn, const d
   double rhs[M];
 #pragma unroll
   for (int m = 0; m < M; ++m) rhs[m] = 0.0;
-  const unsigned ub = uni ? uni[c] : 0u;
+  const unsigned ub = uni ? uni[c] : 0u, both = (ub & kFluxOverflow) ? 0u : ub & ub >> 1;
   // flat: every flux difference is exactly +0 (the two faces' values bit-equal and finite)
   bool flat = true;
   auto differ = [](double x, double y) {
@@ -706,8 +707,7 @@ __device__ __forceinline__ void update_body(int64_t c, const double* Wn, const d
 #pragma unroll
   for (int d = 0; d < D; ++d) {
     const unsigned u = ub >> (2 * d) & 3u;
-    // both faces uniform: the cell's own flux twice, and rhs - 0 / dx = rhs
-    if (u == 3u && !(ub & kFluxOverflow)) continue;
+    if (both >> (2 * d) & 1u) continue;  // the cell's own flux twice, and rhs - 0 / dx = rhs
     const double* F = d == 0 ? F0 : (d == 1 ? F1 : F2);
     const int64_t f0 = g.n[0] + (d == 0), f1 = g.n[1] + (d == 1), f2 = g.n[2] + (d == 2);
     const int64_t nf = f0 * f1 * f2;

@@ -58,28 +58,33 @@ __global__ void __launch_bounds__(kCellThreads)
   int64_t ijk[3];
   cell_index(g, c, ijk);
   constexpr int kBias = sizeof(T) == 8 ? 1023 : 127, kMant = sizeof(T) == 8 ? 20 : 23;
-  auto magnitude = [](T x) -> uint32_t {  // ordered as |x|, exponent field on top
+  // larger magnitude: bits ordered as |x|, exponent field on top (float: one
+  // instruction, which passes NaN over -- a cell that holds one equals no other)
+  auto larger = [](uint32_t h, T x) -> uint32_t {
     if constexpr (sizeof(T) == 8)
-      return (uint32_t)__double2hiint(x) & 0x7fffffffu;
+      return max(h, (uint32_t)__double2hiint(x) & 0x7fffffffu);
     else
-      return __float_as_uint(x) & 0x7fffffffu;
+      return __float_as_uint(fmaxf(__uint_as_float(h), fabsf(x)));
   };
   T w[M];
   uint32_t hw = 0, hu = 0;
 #pragma unroll
   for (int m = 0; m < M; ++m) {
     w[m] = W[m * g.ncells + c];
-    hw = max(hw, magnitude(w[m]));
+    // what a flux multiplies or adds (uniform_flux64, uniform_flux32)
+    using L = Lay<N, D>;
+    const bool factor = sizeof(T) == 8 ? m < L::AL : (m < N || m == L::EN || (m >= L::M + 3 && m <= L::M + 3 + D));
+    if (factor) hw = larger(hw, w[m]);
   }
 #pragma unroll
   for (int d = 0; d < D; ++d) {
     constexpr int u = Lay<N, D>::MOM;
     if constexpr (sizeof(T) == 8)
-      hu = max(hu, magnitude(V[(u + d) * g.ncells + c]));
+      hu = larger(hu, V[(u + d) * g.ncells + c]);
     else
-      hu = max(hu, magnitude(w[u + d]));
+      hu = larger(hu, w[u + d]);
   }
-  if constexpr (sizeof(T) == 8) hw = max(hw, magnitude(V[Lay<N, D>::EN * g.ncells + c]));
+  if constexpr (sizeof(T) == 8) hw = larger(hw, V[Lay<N, D>::EN * g.ncells + c]);
   const int ew = (int)(hw >> kMant), eu = (int)(hu >> kMant);  // 2 kBias + 1 for infinities and NaN
   unsigned bits = (ew > 2 * kBias - 4 || eu > 2 * kBias || ew + eu > 3 * kBias - 4) ? kFluxOverflow : 0u;
 #pragma unroll
@@ -171,19 +176,19 @@ __global__ void __launch_bounds__(kCellThreads)
 #pragma unroll
   for (int d = 0; d < D; ++d) {
     const int64_t f0 = g.n[0] + (d == 0), f1 = g.n[1] + (d == 1);
-    const int64_t nf = f0 * f1 * (g.n[2] + (d == 2));
-    const int64_t t = HRM_IDX(g, (ijk[2] * f1 + ijk[1]) * f0 + ijk[0], nf);
-    const int64_t stride = d == 0 ? 1 : (d == 1 ? f0 : f0 * f1);
+    const int64_t t = (ijk[2] * f1 + ijk[1]) * f0 + ijk[0];
+    const int64_t up = t + (d == 0 ? 1 : (d == 1 ? f0 : f0 * f1));
     const uint32_t p = base[d][warp] + at[d];
-    if (lo[d]) lists.list[d][HRM_IDX(g, p, nf)] = (uint32_t)t;
-    if (hi[d]) lists.list[d][HRM_IDX(g, p + (lo[d] ? 1u : 0u), nf)] = (uint32_t)HRM_IDX(g, t + stride, nf);
+    if (lo[d]) lists.list[d][HRM_IDX(g, p, f0 * f1 * (g.n[2] + (d == 2)))] = (uint32_t)t;
+    if (hi[d]) lists.list[d][HRM_IDX(g, p + (lo[d] ? 1u : 0u), f0 * f1 * (g.n[2] + (d == 2)))] = (uint32_t)up;
     const bool last = ijk[d] == g.n[d] - 1 && !hi[d];
-    const int64_t up = last ? HRM_IDX(g, t + stride, nf) : t;
     if (lists.gate[d]) {
-      if (!lo[d]) lists.gate[d][t] = 2;
-      if (last) lists.gate[d][up] = 2;
+      const int64_t nf = f0 * f1 * (g.n[2] + (d == 2));
+      if (!lo[d]) lists.gate[d][HRM_IDX(g, t, nf)] = 2;
+      if (last) lists.gate[d][HRM_IDX(g, up, nf)] = 2;
     }
     if (lists.F[d] && (!lo[d] || last)) {
+      const int64_t nf = f0 * f1 * (g.n[2] + (d == 2));
       double G[L::NC];
       if constexpr (FP32)
         uniform_flux32<N, D>(c, d, P32, g.ncells, G);
@@ -192,8 +197,8 @@ __global__ void __launch_bounds__(kCellThreads)
 #pragma unroll
       for (int m = 0; m < L::M + N - 1; ++m) {
         const double v = m < L::NC ? G[m < L::NC ? m : 0] : 0.0;
-        if (!lo[d]) lists.F[d][m * nf + t] = v;
-        if (last) lists.F[d][m * nf + up] = v;
+        if (!lo[d]) lists.F[d][m * nf + HRM_IDX(g, t, nf)] = v;
+        if (last) lists.F[d][m * nf + HRM_IDX(g, up, nf)] = v;
       }
     }
   }
