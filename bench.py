@@ -34,8 +34,8 @@ sys.path.insert(0, ROOT)
 # time; profiles/launches_shock_bubble_1024x512.md): device time, DRAM bytes read and written, activity of the FP64 and
 # the FMA pipe. A sweep's work grows with the share of non-uniform stencils, so these belong to that step and are
 # combined with no other time; to be taken again when the kernels change.
-CAPTURED = {"k_face_fp64": {"us": [614.9, 454.7], "dram_bytes": [2.696e7, 2.204e7], "fp64_pipe_active": [0.557, 0.599]},
-            "k_face32_fast": {"us": [34.8, 29.0], "dram_bytes": [9.28e6, 4.01e6], "fma_pipe_active": [0.283, 0.193]}}
+CAPTURED = {"k_face_fp64": {"us": [610.2, 469.3], "dram_bytes": [2.698e7, 2.206e7], "fp64_pipe_active": [0.557, 0.604]},
+            "k_face32_fast": {"us": [34.9, 29.4], "dram_bytes": [9.33e6, 4.01e6], "fma_pipe_active": [0.285, 0.196]}}
 
 
 def captured_traffic(name, hbm_gbs):

@@ -827,7 +827,8 @@ hrm_status hrm_create(hrm_ctx** out, const hrm_grid* grid, int32_t N, const doub
     if ((s = cuda_check(c, ctx_malloc(c, &c->F[d], sizeof(double) * nf * (M + N - 1)), "alloc faces"))) return bail(s);
     if ((int64_t)nf > c->defer_cap) c->defer_cap = (int64_t)nf;
   }
-  if (c->defer_cap >= (int64_t)0xffffffffll)  // (its flux planes alone would exceed the device)
+  // (32-bit list entries; the planes allocated above are at least 236 bytes a cell, a terabyte by then)
+  if (c->defer_cap >= (int64_t)0xffffffffll)
     return bail(fail(c, HRM_E_NOMEM, "2^32 - 1 midpoints or more in one direction"));
   // the lists, their counters and flags, and the worklist of the precision form's deferred midpoints: one
   // allocation (a new context pays for each)

@@ -515,13 +515,6 @@ __device__ __forceinline__ void defer_push(const DevGrid& g, bool need, int64_t 
   if (need) list[HRM_IDX(g, base + __popc(m & ((1u << lane) - 1u)), room)] = (uint32_t)t;
 }
 
-// Precision-form update of one RK stage with the next stage's primitives fused
-// in: the flux difference and SSP-RK combination (fast_combine), the
-// relaxation (relax_fast), the admissibility count, the store of W_out, then
-// the FP32 planes of W_out (prim32_store) that the next stage's sweeps read --
-// in place of a separate k_prim32 pass over W_out. Interior cells only: the
-// planes of Dirichlet slices keep what the stage's first primitive pass wrote
-// (their states do not change).
 // The cell's five-equation CFL speeds (|u_d| + c) / dx_d, as k_prim32 forms them.
 template <int D>
 __device__ __forceinline__ void speeds32(const DevGrid& g, const float* u, float cs, double* s) {
@@ -582,7 +575,12 @@ __device__ __forceinline__ unsigned undefined_step(const DevGrid& g, double dt) 
   return odd ? kFluxOverflow : 0u;
 }
 
-// Any other cell. odd: undefined_step of the stage's dt (with A.uni).
+// Any other cell: the flux difference and SSP-RK combination (fast_combine), the
+// relaxation (relax_fast), the admissibility count, the store of W_out, then the
+// FP32 planes of W_out (prim32_store) that the next stage's sweeps read, in place of
+// a separate k_prim32 pass. Interior cells only: the planes of Dirichlet slices keep
+// what the stage's first primitive pass wrote (their states do not change). odd:
+// undefined_step of the stage's dt (with A.uni).
 template <int N, int D, bool SOFT = false>
 __device__ __forceinline__ void update32p_change(int64_t c, const Update32Args& A, const DevGrid& g, const DevFluid& f,
                                                  double* s, unsigned odd = 0u) {

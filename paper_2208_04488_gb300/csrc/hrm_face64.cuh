@@ -16,8 +16,8 @@
 // Measured, a pass of one step: shock-bubble 1024x512 6.18 -> 3.97 ms, 72x60x50
 // interface 7.10 -> 2.57 (with the lists of hrm_sweep.cuh), smooth advection
 // 250x250 (no stencil uniform) 1.61 -> 1.13. Three blocks per SM at 168 registers
-// against four at 128: the same within 4 % on large grids, 20 % faster where the
-// listed midpoints are few.
+// against four at 128, us a pass: 301x151 jet 1191 against 1455, 72x60x50 box 2497
+// against 2568, shock-bubble 3819 against 3784, 250x250 advection 1129 against 1049.
 #pragma once
 
 #include "hrm_kernels.cuh"
@@ -535,7 +535,7 @@ __device__ __forceinline__ bool uniform_midpoint64(int64_t t, const Nodes6& nd, 
 // 12880 815 | 582 | 606 | 758, 20100 1307 | 1028 | 710 | 835, 32896 2048 | 1500 |
 // 1083 | 1043; two: 3080 228 | 228 | 260 | 411, 5256 341 | 351 | 369 | 445, 12210
 // 559 | 420 | 435 | 478, 17030 757 | 633 | 462 | 484, 25760 965 | 701 | 497 | 481.
-// No list (small grids, kListedCells64): every midpoint, by the same rule.
+// No list (small grids, `listed` in hrm_api.cu): every midpoint, by the same rule.
 constexpr uint32_t kSplit8 = 4608, kSplit4 = 13312, kSplit2 = 20480;
 
 template <int N, int D, int DIR, int LANES>

@@ -484,9 +484,10 @@ __device__ __forceinline__ void count_bits(StepState* st, int b) {
 // The precision form's FP64 arithmetic writes its multiply-adds as explicit
 // fma(): its translation units are built without FMA contraction, so that every
 // FP32 expression rounds as written whichever kernel it is inlined into.
-// The same flux in the precision form, where every FP32 plane holds the same value
-// at the six nodes (uniform_stencil), from the planes of one of the cells (the HCS
-// node-flux expression). Formed directly instead of through rounded steps that
+
+// Flux of a midpoint in the precision form where every FP32 plane holds the same
+// value at the six nodes (as uniform_flux64 below for the FP64 form), from the planes
+// of one of the cells (the HCS node-flux expression). Formed directly instead of through rounded steps that
 // would only cancel; every FP32 sweep takes it, so they stay bit-identical.
 // Planes as in P32Lay: V, then c, rho, rho c^2, rho u_d, E.
 template <int N, int D>
